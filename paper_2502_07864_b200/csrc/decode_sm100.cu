@@ -5,13 +5,18 @@
 // One CTA = one (partition, block of 32 query rows); it walks its segments page by page.
 //
 // Tile plan per 64-token page
-//   S  [128 x 64]   = Q_hat (tensor memory, the 32 rows replicated into the four 32-lane quadrants)
-//                     x K_hat^T (the page in shared memory, K-major, 128-byte swizzle), K = 576
+//   S  [32 x 64]    = Q_hat (tensor memory, the 32 rows replicated into the four 32-lane quadrants)
+//                     x K_hat^T (the page in shared memory, K-major, 128-byte swizzle), K = 576, by
+//                     tcgen05.mma.ws with M = 32, whose accumulator puts tokens 16w..16w+15 of the 32 rows in
+//                     quadrant w (16 columns).  The M = 128 form on the replicated rows gives the same values and
+//                     takes about as many cycles (34 against 31 an instruction), but it multiplies every row four
+//                     times: at the 1000 W limit that energy was what bound long steps (SM clock 1.4 GHz at
+//                     B = 128 x 8192 cached tokens; step 274 us, with M = 32 at 1.9 GHz 239 us).
 //   O^T[512 x 32]  += C^T (the same shared-memory page read MN-major, four 128-row tiles)
 //                     x P^T (32 rows x 64 tokens, bf16, shared memory, K-major)
 // O is kept transposed (latent index on the tensor-memory lanes, query rows on the columns) so that
 // the accumulator costs 4 x 32 columns instead of 512, which leaves room for Q_hat (288 columns) and
-// S (64 columns) in the 512-column tensor memory, and so that no padded query row costs PV work.
+// S (16 columns) in the 512-column tensor memory, and so that no padded query row costs PV work.
 //
 // Warp roles: warps 0-3 softmax + epilogue (warp w owns tensor-memory lanes 32w..32w+31, i.e. replica w
 // of the 32 query rows, and the probabilities of tokens 16w..16w+15 of every page); warp 4 lane 0
@@ -220,7 +225,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
       // Q_READY, which also tells when the ring has ended) and runs QK^T for a page as soon as it has landed.
       // Issuing an instruction costs this warp about as many cycles as a small one occupies the pipe, so the 36
       // score instructions and the 16 product instructions of a page are issued by two warps side by side.
-      constexpr uint32_t idesc_qk = instr_desc(kPage, false);
+      constexpr uint32_t idesc_qk = instr_desc(kPage, false, kRowBlock);
       int g = 0, n = 0, seg = 0;  // ring items, pages, segments handled so far
       while (true) {
         // a segment begins (or the ring ends): the softmax warps say which
@@ -240,7 +245,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
               if (elect_one())
-                mma_ts(tmem + kColS, tmem + kColQ + c * 32 + kk * 8, desc_advance(k0, c * kSubTileBytes + kk * 32),
+                mma_ws_ts(tmem + kColS, tmem + kColQ + c * 32 + kk * 8, desc_advance(k0, c * kSubTileBytes + kk * 32),
                        idesc_qk, (c | kk) ? 1u : 0u);
             }
           }
@@ -357,7 +362,7 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
           mbar_wait(bar(BAR_S_FULL), n & 1, abort_flag, dev_status);
           tc_fence_after();
           uint32_t sq[16];  // this warp's 16 tokens of its row
-          tmem_ld16(tmem + lane_base + kColS + warp * 16, sq);
+          tmem_ld16(tmem + lane_base + kColS, sq);
           tc_wait_ld();
           tc_fence_before();
           mbar_arrive(bar(BAR_S_FREE));

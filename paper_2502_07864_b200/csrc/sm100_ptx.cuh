@@ -53,6 +53,14 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a_desc, uint64_t b_d
       ::"r"(d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// The weight-stationary form, M = 32: D[tmem] (+)= A[tmem] * B[smem desc].  A's 32 rows are replicated in the four 32-lane
+// quadrants; quadrant w of D holds the 32 rows x columns w*N/4 .. (w+1)*N/4-1 of the product, in N/4 tensor-memory columns.
+__device__ __forceinline__ void mma_ws_ts(uint32_t d, uint32_t a, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.ws.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
+      ::"r"(d), "r"(a), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
 
 #define TM_R4(v, i) "=r"(v[i]), "=r"(v[i + 1]), "=r"(v[i + 2]), "=r"(v[i + 3])
 #define TM_R16(v, i) TM_R4(v, i), TM_R4(v, i + 4), TM_R4(v, i + 8), TM_R4(v, i + 12)
@@ -98,10 +106,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
 // The same descriptor `bytes` further on (bytes is a multiple of 16; the tile stays inside the 256 KB window,
 // so the 14-bit address field cannot carry).
 __device__ __forceinline__ uint64_t desc_advance(uint64_t desc, uint32_t bytes) { return desc + (bytes >> 4); }
-// Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, M = 128.
-__host__ __device__ constexpr uint32_t instr_desc(int n, bool a_mn_major) {
+// Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B.
+__host__ __device__ constexpr uint32_t instr_desc(int n, bool a_mn_major, int m = 128) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn_major ? 1u : 0u) << 15) | (static_cast<uint32_t>(n >> 3) << 17) |
-         (static_cast<uint32_t>(128 >> 4) << 24);
+         (static_cast<uint32_t>(m >> 4) << 24);
 }
 
 // ---------------------------------------------------------------------------------------------- host
