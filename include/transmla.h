@@ -83,7 +83,8 @@ typedef struct {
   int32_t max_pages_per_seq; /* row stride of page_table */
   int32_t batch;             /* B */
   int32_t num_partitions;    /* G: how many pieces the batch's pages are split into; 0 = library chooses
-                                (SMs / row blocks, at most batch * max_pages_per_seq / 4).  With an explicit G
+                                (SMs / row blocks of 32 query rows, 64 where S*H > 32
+                                and r = 512; at most batch * max_pages_per_seq / 4).  With an explicit G
                                 every partition handles exactly the page range of the plan and a rerun gives
                                 the same bits.  With 0, r = 512, dR = 64 and at least 8 partitions per
                                 sequence, the CTAs that share a sequence take its pages from a counter as they
@@ -269,7 +270,8 @@ transmla_status_t transmla_decode_step_host(const transmla_params_t* params, con
  * until the process ends.  The call allocates and frees nothing on the device.
  *
  * Limits and rules:
- *   - transmla_workspace_layout(params).total_bytes must not exceed the capacity, otherwise the call
+ *   - transmla_workspace_layout(params).total_bytes must not exceed the capacity (with num_partitions == 0
+ *     the call tries half the library's own partition count before it gives up), otherwise the call
  *     returns TRANSMLA_ERR_WORKSPACE and launches nothing.  The size grows with
  *     (num_partitions + B - 1) * S * H * r * 4 bytes; pass a smaller params->num_partitions to fit.
  *   - The first call on each device looks up the array's device address (with that device current)

@@ -110,7 +110,8 @@ transmla_status_t transmla_workspace_layout(const transmla_params_t* p, transmla
     int sms = 0;
     st = check_device(&sms);
     if (st != TRANSMLA_OK) return st;
-    const int row_blocks = (p->q_len * p->num_heads + kRowBlock - 1) / kRowBlock;
+    const int rows = decode_row_block(*p);
+    const int row_blocks = (p->q_len * p->num_heads + rows - 1) / rows;
     G = sms / row_blocks;
     // Small problems: no more partitions than a quarter of the pages the batch can hold, so that a partition
     // keeps at least about four pages and a sequence is not cut into dozens of one-page partials.
@@ -189,7 +190,8 @@ static transmla_status_t launch_split_kv(const transmla_params_t* p, const trans
   cudaEvent_t ev0 = tl_prof_start, ev1 = tl_prof_stop;
   tl_prof_start = tl_prof_stop = nullptr;
   if (ev0 != nullptr && cudaEventRecord(ev0, s) != cudaSuccess) return TRANSMLA_ERR_CUDA;
-  auto launch = decode_sm100_supported(*p) ? launch_decode_sm100 : launch_decode_generic;
+  auto launch = !decode_sm100_supported(*p) ? launch_decode_generic
+                : decode_row_block(*p) == 64 ? launch_decode_rows64 : launch_decode_sm100;
   if (launch(*p, lay.num_partitions, reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset),
              static_cast<const __nv_bfloat16*>(cache), page_table, seqlens,
              reinterpret_cast<int32_t*>(ws + lay.cum_pages_offset), reinterpret_cast<int32_t*>(ws + lay.plan_offset),

@@ -11,7 +11,7 @@
 namespace transmla {
 
 constexpr int kPage = 64;       // tokens per cache page (P)
-constexpr int kRowBlock = 32;   // query rows (s*H + h) one CTA works on
+constexpr int kRowBlock = 32;   // query rows (s*H + h) of a block; the page counters are sized for blocks of this many
 constexpr int kSegCost = TRANSMLA_SEGMENT_COST_PAGES;  // virtual slots in front of every non-empty sequence
 // Dynamic page claims of the split-KV kernel (r = 512, dR = 64, partition count chosen by the library): the CTAs
 // whose partitions hold pages of a sequence take that sequence's pages one by one from a counter instead of
@@ -203,6 +203,10 @@ cudaError_t launch_decode_generic(const transmla_params_t& p, int G, const __nv_
                                   const int32_t* cum, const int32_t* plan, float* partial_o, float* partial_lse,
                                   int32_t* dev_status, cudaStream_t stream);
 bool decode_sm100_supported(const transmla_params_t& p);
+int decode_row_block(const transmla_params_t& p);  // query rows one split-KV CTA works on: 32, or 64
+cudaError_t launch_decode_rows64(const transmla_params_t& p, int G, const __nv_bfloat16* q_hat, const __nv_bfloat16* cache,
+                                 const int32_t* page_table, const int32_t* seqlens, const int32_t* cum, const int32_t* plan,
+                                 float* partial_o, float* partial_lse, int32_t* dev_status, cudaStream_t stream);
 cudaError_t launch_decode_sm100(const transmla_params_t& p, int G, const __nv_bfloat16* q_hat,
                                 const __nv_bfloat16* cache, const int32_t* page_table, const int32_t* seqlens,
                                 const int32_t* cum, const int32_t* plan, float* partial_o, float* partial_lse,

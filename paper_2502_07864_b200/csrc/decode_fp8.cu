@@ -19,6 +19,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "partition_walk.cuh"
 #include "sm100_ptx.cuh"
 
 namespace transmla {
@@ -99,7 +100,7 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
                     const int32_t* page_table, const int32_t* seqlens,
                     const int32_t* cum, const int32_t* plan, float* partial_o,
                     float* partial_lse, int32_t* dev_status, int S, int H, int num_pages, int max_pages,
-                    float scale_log2, int B, int dynamic, int32_t* next) {
+                    float scale_log2, int B, int dynamic, int32_t* next, int G, int merge) {
   extern __shared__ unsigned char smem_unaligned[];
   const uint32_t raw = smem_u32(smem_unaligned);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -114,7 +115,7 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
   auto bar = [&](int i) -> uint32_t { return base + kOffBar + 8 * i; };
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int part = blockIdx.x, rb = blockIdx.y;
+  const int rb = blockIdx.y;
   const int SH = S * H;
   pdl_trigger();
 
@@ -146,8 +147,8 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
   tc_fence_after();
   const uint32_t tmem = *tmem_base_s;
   pdl_wait();  // the plan, the absorbed queries and the appended cache rows come from the kernel before this one
-  const int4 pl = reinterpret_cast<const int4*>(plan)[part];
-  const bool has_home = pl.y > pl.x;
+  const int part = blockIdx.x * merge, parts = min(merge, G - part);
+  const bool has_home = reinterpret_cast<const int4*>(plan)[part + parts - 1].y > reinterpret_cast<const int4*>(plan)[part].x;
 
   if (has_home) {
     if (warp == 4) {
@@ -193,66 +194,9 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
         __syncwarp();
         ++g;
       };
-      // ---- the partition's sequences in turn
-      // Page-table entries [lo, hi) of sequence b are asked into L1 ahead of their use (one 128-byte line per lane
-      // and round), so that the look-up in front of every page load does not cost a trip to L2.
-      auto prefetch_table = [&](int b, int lo, int hi) {
-        const int32_t* row = page_table + static_cast<size_t>(b) * max_pages;
-        for (int i = (lo & ~31) + lane * 32; i < hi; i += 32 * 32)
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(row + max(i, lo)));
-      };
-      // The last sequence in which this partition owns pages: there it claims until the counter runs dry.  In the
-      // sequences before it (a partition that straddles two or more) it takes no more pages than the plan gave it,
-      // so that every sequence gets the share of CTA time that the plan meant it to have.
-      int last_home = pl.w;
-      if (dynamic) {
-        const int cw = cum[pl.w], cw1 = cum[pl.w + 1];
-        if (min(pl.y, cw1) <= max(pl.x, cw + kSegCost)) --last_home;
-      }
-      for (int b = pl.z; b <= pl.w; ++b) {
-        const int cb = cum[b], cb1 = cum[b + 1];  // one round trip for the three of them
-        const int L = clamped_len(seqlens[b], max_pages, nullptr);  // the plan block has already reported a bad length
-        const int c0s = cb + kSegCost;  // slot of page 0 of sequence b
-        const int pg_lo = max(pl.x, c0s) - c0s, pg_hi = min(pl.y, cb1) - c0s;
-        if (pg_hi <= pg_lo) continue;
-        if (!dynamic) {  // exactly the plan's range
-          prefetch_table(b, pg_lo, pg_hi);
-          issue_queries(b, part + b, L);
-          for (int pj = pg_lo; pj < pg_hi; ++pj) issue_page(b, pj, pj == pg_lo, pj == pg_hi - 1);
-          continue;
-        }
-        // Pages of sequence b from its counter until it runs dry.  Three are claimed in one go (one atomic
-        // instruction, lanes 0..2) so that the stages fill at once.  After that the next two page numbers are
-        // always in hand and the claim behind them is in flight while a page waits for its stage, which keeps the
-        // counter's round trip off the critical path and tells at issue time whether a page is the segment's
-        // last one: it is exactly when the claim behind it is past the end (claims only grow).
-        const int n_b = cb1 - c0s;
-        int32_t* counter = next + static_cast<size_t>(rb) * B + b;
-        int left = b < last_home ? pg_hi - pg_lo : 0x7fffffff;  // claims this partition may still make here
-        const int take = min(kStages, left);
-        left -= take;
-        int head = 0x7fffffff;
-        if (lane < take) head = atomicAdd(counter, 1);
-        prefetch_table(b, 0, n_b);  // in flight together with the claim
-        int c0 = __shfl_sync(0xffffffffu, head, 0), c1 = __shfl_sync(0xffffffffu, head, 1), c2 = __shfl_sync(0xffffffffu, head, 2);
-        { int t; if (c0 > c1) { t = c0; c0 = c1; c1 = t; } if (c1 > c2) { t = c1; c1 = c2; c2 = t; } if (c0 > c1) { t = c0; c0 = c1; c1 = t; } }
-        if (c0 >= n_b) {  // the others have taken everything: the combine still expects a partial from this slot
-          if (rb * kRowBlock + lane < SH) partial_lse[static_cast<size_t>(part + b) * SH + rb * kRowBlock + lane] = -INFINITY;
-          continue;
-        }
-        issue_queries(b, part + b, L);
-        bool first = true;
-        while (c0 < n_b) {
-          int pend = 0x7fffffff;
-          const bool ahead = c2 < n_b && left > 0;
-          if (ahead) { --left; if (lane == 0) pend = atomicAdd(counter, 1); }
-          issue_page(b, c0, first, c1 >= n_b);
-          first = false;
-          c0 = c1;
-          c1 = c2;
-          c2 = ahead ? __shfl_sync(0xffffffffu, pend, 0) : 0x7fffffff;
-        }
-      }
+      const PartitionWalk walk = {page_table, seqlens, cum, next + static_cast<size_t>(rb) * B, partial_lse, part, parts,
+                                  rb * kRowBlock, kRowBlock, SH, max_pages, dynamic};
+      walk_partition(walk, lane < parts ? reinterpret_cast<const int4*>(plan)[part + lane] : make_int4(0, 0, -1, -1), lane, issue_queries, issue_page);
       {  // closing item
         const uint32_t stage = acquire(g);
         if (elect_one()) {
@@ -667,11 +611,16 @@ cudaError_t launch_decode_fp8(const transmla_params_t& p, int G, const __nv_bflo
     return cudaErrorInvalidValue;
   static PerDeviceFlag smem_set;
   if (cudaError_t e = ensure_dynamic_smem(decode_fp8_kernel, kSmemBytes, smem_set); e != cudaSuccess) return e;
-  dim3 grid(G, (SH + kRowBlock - 1) / kRowBlock);
+  // The library's own partition count suits the bf16 kernels, which take 64 query rows a CTA from 33 rows on; here a CTA
+  // takes 32, so that each works on as many partitions as bring the grid back to one wave (two waves measured
+  // 290 us a step instead of 267 at B=30, S=2, 11K to 20K tokens).
+  const int blocks = (SH + kRowBlock - 1) / kRowBlock, bf16_blocks = (SH + decode_row_block(p) - 1) / decode_row_block(p);
+  const int merge = p.num_partitions == 0 && G > 1 ? (blocks + bf16_blocks - 1) / bf16_blocks : 1;
+  dim3 grid((G + merge - 1) / merge, blocks);
   int32_t* next = const_cast<int32_t*>(cum) + 3 * p.batch + 1;  // page counters, zeroed by the plan
   return launch_pdl(decode_fp8_kernel, grid, dim3(kThreads), static_cast<size_t>(kSmemBytes), stream, map, smap, qmap,
                     page_table, seqlens, cum, plan, partial_o, partial_lse, dev_status, p.q_len, p.num_heads,
-                    p.num_pages, p.max_pages_per_seq, p.softmax_scale * kLog2e, p.batch, dynamic_claims(p, G) ? 1 : 0, next);
+                    p.num_pages, p.max_pages_per_seq, p.softmax_scale * kLog2e, p.batch, dynamic_claims(p, G) ? 1 : 0, next, G, merge);
 }
 
 }  // namespace transmla

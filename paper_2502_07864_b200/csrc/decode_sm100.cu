@@ -26,6 +26,7 @@
 // TRANSMLA_DEV_TIMEOUT, every later wait returns at once, and control flow stays identical, so the CTA
 // still reaches its teardown and frees its tensor memory.
 #include "common.cuh"
+#include "partition_walk.cuh"
 #include "sm100_ptx.cuh"
 
 namespace transmla {
@@ -151,66 +152,9 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
         __syncwarp();
         ++g;
       };
-      // ---- the partition's sequences in turn
-      // Page-table entries [lo, hi) of sequence b are asked into L1 ahead of their use (one 128-byte line per lane
-      // and round), so that the look-up in front of every page load does not cost a trip to L2.
-      auto prefetch_table = [&](int b, int lo, int hi) {
-        const int32_t* row = page_table + static_cast<size_t>(b) * max_pages;
-        for (int i = (lo & ~31) + lane * 32; i < hi; i += 32 * 32)
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(row + max(i, lo)));
-      };
-      // The last sequence in which this partition owns pages: there it claims until the counter runs dry.  In the
-      // sequences before it (a partition that straddles two or more) it takes no more pages than the plan gave it,
-      // so that every sequence gets the share of CTA time that the plan meant it to have.
-      int last_home = pl.w;
-      if (dynamic) {
-        const int cw = cum[pl.w], cw1 = cum[pl.w + 1];
-        if (min(pl.y, cw1) <= max(pl.x, cw + kSegCost)) --last_home;
-      }
-      for (int b = pl.z; b <= pl.w; ++b) {
-        const int cb = cum[b], cb1 = cum[b + 1];  // one round trip for the three of them
-        const int L = clamped_len(seqlens[b], max_pages, nullptr);  // the plan block has already reported a bad length
-        const int c0s = cb + kSegCost;  // slot of page 0 of sequence b
-        const int pg_lo = max(pl.x, c0s) - c0s, pg_hi = min(pl.y, cb1) - c0s;
-        if (pg_hi <= pg_lo) continue;
-        if (!dynamic) {  // exactly the plan's range
-          prefetch_table(b, pg_lo, pg_hi);
-          issue_queries(b, part + b, L);
-          for (int pj = pg_lo; pj < pg_hi; ++pj) issue_page(b, pj, pj == pg_lo, pj == pg_hi - 1);
-          continue;
-        }
-        // Pages of sequence b from its counter until it runs dry.  Three are claimed in one go (one atomic
-        // instruction, lanes 0..2) so that the stages fill at once.  After that the next two page numbers are
-        // always in hand and the claim behind them is in flight while a page waits for its stage, which keeps the
-        // counter's round trip off the critical path and tells at issue time whether a page is the segment's
-        // last one: it is exactly when the claim behind it is past the end (claims only grow).
-        const int n_b = cb1 - c0s;
-        int32_t* counter = next + static_cast<size_t>(rb) * B + b;
-        int left = b < last_home ? pg_hi - pg_lo : 0x7fffffff;  // claims this partition may still make here
-        const int take = min(kStages, left);
-        left -= take;
-        int head = 0x7fffffff;
-        if (lane < take) head = atomicAdd(counter, 1);
-        prefetch_table(b, 0, n_b);  // in flight together with the claim
-        int c0 = __shfl_sync(0xffffffffu, head, 0), c1 = __shfl_sync(0xffffffffu, head, 1), c2 = __shfl_sync(0xffffffffu, head, 2);
-        { int t; if (c0 > c1) { t = c0; c0 = c1; c1 = t; } if (c1 > c2) { t = c1; c1 = c2; c2 = t; } if (c0 > c1) { t = c0; c0 = c1; c1 = t; } }
-        if (c0 >= n_b) {  // the others have taken everything: the combine still expects a partial from this slot
-          if (rb * kRowBlock + lane < SH) partial_lse[static_cast<size_t>(part + b) * SH + rb * kRowBlock + lane] = -INFINITY;
-          continue;
-        }
-        issue_queries(b, part + b, L);
-        bool first = true;
-        while (c0 < n_b) {
-          int pend = 0x7fffffff;
-          const bool ahead = c2 < n_b && left > 0;
-          if (ahead) { --left; if (lane == 0) pend = atomicAdd(counter, 1); }
-          issue_page(b, c0, first, c1 >= n_b);
-          first = false;
-          c0 = c1;
-          c1 = c2;
-          c2 = ahead ? __shfl_sync(0xffffffffu, pend, 0) : 0x7fffffff;
-        }
-      }
+      const PartitionWalk walk = {page_table, seqlens, cum, next + static_cast<size_t>(rb) * B, partial_lse, part, 1,
+                                  rb * kRowBlock, kRowBlock, SH, max_pages, dynamic};
+      walk_partition(walk, lane < 1 ? pl : make_int4(0, 0, -1, -1), lane, issue_queries, issue_page);
       {  // closing item
         const uint32_t stage = acquire(g);
         if (elect_one()) {
@@ -503,6 +447,20 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
 }  // namespace sm100
 
 bool decode_sm100_supported(const transmla_params_t& p) { return p.kv_lora_rank == sm100::R && p.qk_rope_dim == sm100::DR; }
+
+// Query rows per CTA.  Every row block streams the pages and pays a page's tensor instructions, so with more than 32 rows
+// per sequence half as many blocks win (decode_rows64.cu; step, 32 -> 64 rows a CTA: 64 heads S=2 B=64 x 2K-8K 255 -> 193
+// us, 32 heads S=2 B=32 x 4K-8K 101 -> 75 us) - unless the batch is so small that a 32-row CTA handles no more than about
+// 16 pages (12 with more than two row blocks) anyway: then the shorter start and end of the 32-row kernel count (32 heads
+// S=2 B=4 x 4K-8K: 34.1 us against 37.3, B=8 39.8 against 41.3; 64 heads S=2 B=4 x 1K-2K 30.4 against 32.4, x 2K-4K 34.3
+// against 34.9, x 4K-8K 42.1 against 40.5).  Like the partition count the rule goes by the page table's capacity.
+int decode_row_block(const transmla_params_t& p) {
+  constexpr int kSms = 148;
+  if (!decode_sm100_supported(p) || p.q_len * p.num_heads <= kRowBlock) return kRowBlock;
+  const long long blocks = (p.q_len * p.num_heads + kRowBlock - 1) / kRowBlock;
+  const long long ctas = (static_cast<long long>(p.batch) * p.max_pages_per_seq + 3) / 4 * blocks;  // of four pages each
+  return ctas <= (blocks <= 2 ? 4 : 3) * kSms ? kRowBlock : 64;
+}
 
 // Pages are handed out at run time only when the library chose the partition count itself (a caller who fixes the
 // count gets the plan's page ranges, and with them results that do not depend on timing) and only when a sequence

@@ -51,6 +51,14 @@ transmla_status_t transmla_mla_attention_static(const transmla_params_t* params,
   transmla_workspace_layout_t lay;
   transmla_status_t st = transmla_workspace_layout(params, &lay);
   if (st != TRANSMLA_OK) return st;
+  transmla_params_t fitted = *params;
+  if (lay.total_bytes > kStaticWorkspaceBytes && params->num_partitions == 0) {
+    // The library's own partition count is chosen for speed; half as many partitions need about half the partials.
+    fitted.num_partitions = (lay.num_partitions + 1) / 2;
+    st = transmla_workspace_layout(&fitted, &lay);
+    if (st != TRANSMLA_OK) return st;
+    params = &fitted;
+  }
   if (lay.total_bytes > kStaticWorkspaceBytes) return TRANSMLA_ERR_WORKSPACE;  // problem too large for the built-in array
   void* ws = nullptr;
   st = static_workspace_ptr(&ws);

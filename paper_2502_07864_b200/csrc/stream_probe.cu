@@ -1,6 +1,6 @@
 // Read-only streaming probe: what the split-KV kernel's access pattern costs when nothing is computed.
 //
-// Same grid (one CTA per partition and block of 32 query rows), same split plan, same ring of three 73 728-byte
+// Same grid (one CTA per partition and block of query rows), same split plan, same ring of three 73 728-byte
 // stages filled by the same TMA boxes (nine 64-token x 64-column boxes per page, 128-byte swizzle, evict-first),
 // but the consumer is a single warp that hands every stage back as soon as it has landed: no tensor-core work,
 // no softmax, no output.  Its duration is the ceiling that launch, ramp-up and the memory system put on any kernel
@@ -85,7 +85,8 @@ cudaError_t launch_stream_probe(const transmla_params_t& p, int G, const __nv_bf
   static PerDeviceFlag smem_set;
   if (cudaError_t e = ensure_dynamic_smem(stream_probe_kernel, kProbeSmem, smem_set); e != cudaSuccess) return e;
   const int SH = p.q_len * p.num_heads;
-  dim3 grid(G, (SH + kRowBlock - 1) / kRowBlock);
+  const int rows = decode_row_block(p);
+  dim3 grid(G, (SH + rows - 1) / rows);
   return launch_pdl(stream_probe_kernel, grid, dim3(64), static_cast<size_t>(kProbeSmem), stream, map, page_table, cum, plan,
                     dev_status, p.num_pages, p.max_pages_per_seq);
 }

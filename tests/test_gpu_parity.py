@@ -22,9 +22,17 @@ def _lib():
     gu.ensure_built()
 
 
-def _run_and_compare(shape, seqlens, seed, G=0, scale=None, nan_tails=True, check_internals=False):
+def _widen_table(case, columns):
+    # a page table with room for longer sequences: what the library goes by when it picks a kernel for the batch
+    pt = case['page_table']
+    case['page_table'] = torch.cat([pt, torch.full((pt.shape[0], columns - pt.shape[1]), -1, dtype=torch.int32)], dim=1)
+
+
+def _run_and_compare(shape, seqlens, seed, G=0, scale=None, nan_tails=True, check_internals=False, columns=0):
     scale = scale if scale is not None else gu.mla_scale(shape)
     case = synth.make_decode_case(shape, seqlens, seed, nan_tails=nan_tails)
+    if columns:
+        _widen_table(case, columns)
     out, lse, status, views, lay = gu.gpu_decode(shape, gu.to_dev(case), scale, G=G, want_views=check_internals,
                                                  fixed_plan=check_internals)
     assert status == 0
@@ -102,6 +110,28 @@ def test_production_latent_with_row_counts_that_do_not_fill_a_block(H, S):
     # r = 512, dR = 64 goes through the TMA/tcgen05 kernel; S*H = 8, 40, 48 leave the last 32-row block ragged
     shape = synth.MLAShape(H=H, dn=128, dR=64, dv=128, r=512, D=4096, S=S)
     _run_and_compare(shape, [300, 64, 2, 1100], seed=17, G=5, check_internals=True)
+
+
+@pytest.mark.parametrize('H,S,G', [(33, 1, 3), (64, 1, 0), (65, 1, 2), (32, 2, 7), (16, 8, 1), (96, 3, 3), (256, 4, 2)])
+def test_row_blocks_of_64(H, S, G):
+    # More than 32 query rows take 64 a CTA unless the page table has room for a small batch only: 33, 64, 65, 128 and
+    # 288 rows, and 1024, the most that is allowed; lengths with one token, full pages, ragged tails, a query position that sees nothing (L < S), and enough pages per
+    # partition for the two-stage ring to wrap.  (With S*H > 64 the last case compares the heads at the block edges.)
+    shape = synth.MLAShape(H=H, dn=128, dR=64, dv=128, r=512, D=4096, S=S)
+    seqlens = [64 * 7 + 3, max(S - 1, 1), 128, 65, 900]
+    if S * H <= 128:
+        _run_and_compare(shape, seqlens, seed=18, G=G, check_internals=S * H <= 65, columns=600)
+        return
+    case = synth.make_decode_case(shape, seqlens, 18, nan_tails=True)
+    _widen_table(case, 600)
+    out, lse, status, _, _ = gu.gpu_decode(shape, gu.to_dev(case), gu.mla_scale(shape), G=G)
+    assert status == 0
+    rows = sorted({r for e in range(0, S * H, 64) for r in (e, e + 31, e + 32, e + 63)} & set(range(S * H)) | {S * H - 1})
+    only = [(b, r // H, r % H) for b in range(len(seqlens)) for r in rows]
+    want, want_lse = gu.oracle_decode(shape, case, gu.mla_scale(shape), only=only)
+    idx = tuple(np.array(only).T)
+    gu.assert_close(lifts.f64(out)[idx], want[idx], 'row blocks of 64')
+    gu.assert_lse_close(lifts.f64(lse)[idx], want_lse[idx], 'lse')
 
 
 def test_wide_heads_and_many_sequences():
@@ -434,19 +464,21 @@ def test_dynamic_page_claims_match_the_oracle(shape, seqlens):
         gu.assert_lse_close(lifts.f64(lse)[idx], want_lse[idx], 'dynamic claims lse')
 
 
-@pytest.mark.parametrize('G', [0, 37])
-def test_many_serialized_launches_never_time_out(G):
+@pytest.mark.parametrize('shape,G', [(synth.LLAMA2_7B, 0), (synth.LLAMA2_7B, 37), (synth.QWEN25_72B, 0), (synth.QWEN25_72B, 10)])
+def test_many_serialized_launches_never_time_out(shape, G):
     # Launches bracketed by events start all CTAs at once with cold instruction caches, which is when the softmax
     # warps can get a whole page ahead of the MMA warp; every bounded wait must still be satisfied.
-    shape = synth.LLAMA2_7B
     seqlens = [1024] * 4
-    case = gu.to_dev(synth.make_decode_case(shape, seqlens, seed=24))
+    case = synth.make_decode_case(shape, seqlens, seed=24)
+    if shape.S * shape.H > 32:
+        _widen_table(case, 600)  # so that the kernel for 64 query rows is the one that runs
+    case = gu.to_dev(case)
     B = len(seqlens)
     params = binding.make_params(shape, B, case['cache'].shape[0], case['page_table'].shape[1], gu.mla_scale(shape),
                                  num_partitions=G)
     ws, lay = binding.alloc_workspace(params)
     status = torch.zeros(1, dtype=torch.int32, device='cuda')
-    out = torch.empty(B, 1, shape.H, shape.dv, dtype=torch.bfloat16, device='cuda')
+    out = torch.empty(B, shape.S, shape.H, shape.dv, dtype=torch.bfloat16, device='cuda')
     evs = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
     for e in evs:
         e.record()
