@@ -5,16 +5,26 @@
 // is the bf16 split-KV kernel with three differences:
 //   - scores: the page's codes are the B operand of native FP8 products (kind::f8f6f4, K = 32).  The absorbed
 //     queries are split, row by row, into two e4m3 terms q ~ sq * (hi + lo) when they are moved into tensor memory
-//     (two terms carry about the 8 bits a bf16 query has); the rope part runs as bf16 products on k^R / scale and
-//     q^R / sq.  All of it lands in one accumulator and a score is sq * scale_j times that sum.
-//   - products: four more warps turn the codes of a page into scale_j * code as fp16 (the code's fp16 image is exact,
-//     the product with the fp16-rounded scale is rounded once more) in a second buffer with the layout the bf16 kernel reads its pages in, and
-//     zero-fill the rows beyond the sequence; P is fp16 too (operands of one product must agree in type).
+//     (two terms carry about the 8 bits a bf16 query has), and the 32 high and 32 low rows are the 64 rows of one
+//     weight-stationary product, so that a page's codes are read once; the rope part runs as bf16 products on
+//     k^R / scale and (q^R / sq, 0).  A score is sq * scale_j times the sum of its high and its low row.
+//   - products: eight more warps transpose the codes of a page on their way (ldmatrix) and put them into tensor memory
+//     as fp16 (exactly), latents on the lanes: the A operand of O^T += V^T P'^T.  A token's scale goes into its
+//     probability instead: P' = scale_j * p_j in fp16 (operands of one product must agree in type), with the reference
+//     maximum taken over score + log2 scale so that P' keeps the range p had.
 //   - a page's stage goes back to the TMA warp when three parties are done with it: the scores, the converters,
 //     and the softmax warps (they read the scales).
-// Tensor-memory map: Q hi 0-127, Q lo 128-255 (four codes a column), q^R / sq 256-287, S 288-351, O^T 352-479.
+// Tensor-memory map: Q 0-127 (four codes a column; high rows in quadrants 0 and 2, low rows in 1 and 3), q^R / sq 128-159,
+// S 160-191, O^T 192-319, V^T 320-511 (three buffers of half a page: 4 tiles of 128 latents x 32 tokens, two a column).
+// Lane i of a group of 16 holds latent 2 i (i < 8) or 2 (i - 8) + 1 of its 16: ldmatrix hands out pairs.
 //
-// Warp roles: warps 0-3 softmax + epilogue, warp 4 TMA, warp 5 score products, warp 6 PV products, warps 7-10
+// What bounds it: HBM, 1800 cycles a page at 148 SMs (a TMA-only loop over such pages reaches 6.1 TB/s whatever the stage
+// count).  The codes as fp16 in shared memory (written by the converters, read again by the products) cost 1000 cycles
+// of its 128 bytes a page and held a page at 2500 cycles; now about 1000 are left in all and a page
+// takes 2100, of which the converters are busy 1700.  B=64 x 4K-8K: kernel 110 -> 66 us (4.0 TB/s), step 145 -> 112 us;
+// S=2 B=30 x 11K-20K: step 266 -> 180 us.
+//
+// Warp roles: warps 0-3 softmax + epilogue, warp 4 TMA, warp 5 score products, warp 6 PV products, warps 8-15
 // converters.  All waits are bounded as in the bf16 kernel.
 #include <cuda_fp16.h>
 
@@ -34,56 +44,58 @@ constexpr int kSubTileBytes = kPage * 128;            // 8192
 constexpr int kOffRope = kCodeTiles * kSubTileBytes;  // 32768: 64 tokens x 64 bf16
 constexpr int kOffScale = kOffRope + kSubTileBytes;   // 40960: 64 tokens x 16 bytes (the scale is the first 4)
 constexpr int kStageBytes = kOffScale + kPage * 16;   // 41984
-constexpr int kStages = 3;
-constexpr int kVBytes = 8 * kSubTileBytes;            // 65536: the page's latent part as fp16, 8 sub-tiles of 64 x 64
+constexpr int kStages = 4;
 constexpr int kPBytes = kRowBlock * 128;              // 4096: P[32 rows][64 tokens] fp16
 constexpr int kQTileBytes = kRowBlock * 128;          // 4096: one 64-column sub-tile of the 32 query rows (bf16)
 constexpr int kQChunks = K / 64;                      // 9
-constexpr int kThreads = 352;
+constexpr int kThreads = 512, kConverters = 256;
+constexpr int kVBufs = 3;                             // V^T buffers, half a page each
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMetaRing = 16;
 enum { ITEM_QUERIES = 1, ITEM_PAGE = 2, ITEM_END = 3 };
-constexpr uint32_t kColQhi = 0, kColQlo = 128, kColQr = 256, kColS = 288, kColO = 352;
+constexpr uint32_t kColQ = 0, kColQr = 128, kColS = 160, kColO = 192, kColV = 320;
 
 // shared-memory map (offsets from a 1024-byte aligned base)
 constexpr int kOffStage = 0;
-constexpr int kOffV = kStages * kStageBytes;      // 125952 (a multiple of 1024)
-constexpr int kOffP = kOffV + kVBytes;            // 2 buffers
-constexpr int kOffBar = kOffP + 2 * kPBytes;      // mbarriers (8 bytes each)
-constexpr int kOffMisc = kOffBar + 128;
-// misc: pmax_s[2][4][32] f32, alpha_s[32] f32, inv_l[32] f32, meta[16] int4, tmem base, abort, ring_done
-constexpr int kMiscBytes = 1024 + 128 + 128 + 16 * kMetaRing + 16;
+constexpr int kOffP = kStages * kStageBytes;      // 167936 (a multiple of 1024), 2 buffers
+constexpr int kOffX = kOffP + 2 * kPBytes;        // halves of the scores on their way between warps: [4][16][32] f32
+constexpr int kOffBar = kOffX + 8192;             // mbarriers (8 bytes each)
+constexpr int kOffMisc = kOffBar + 256;
+// misc: pmax_s[2][4][32] f32, alpha_s[32], inv_l[32], qmax_s[4][32] f32, meta[16] int4, tmem base, abort, ring_done, v_flags[3]
+constexpr int kMiscBytes = 1024 + 128 + 128 + 512 + 16 * kMetaRing + 32;
 constexpr int kSmemBytes = kOffMisc + kMiscBytes + 1024;  // + slack for the 1024-byte alignment
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 static_assert(kStageBytes % 1024 == 0 && kQChunks * kQTileBytes <= kStageBytes, "stage layout");
 
-enum { BAR_KV_FULL = 0, BAR_KV_EMPTY = kStages, BAR_Q_READY = 2 * kStages, BAR_S_FULL, BAR_S_FREE, BAR_P_READY0, BAR_P_READY1,
-       BAR_PV_DONE0, BAR_PV_DONE1, BAR_V_FULL, BAR_V_EMPTY };
+enum { BAR_KV_FULL = 0, BAR_KV_EMPTY = kStages, BAR_Q_READY = 2 * kStages, BAR_S_FULL, BAR_S_FREE, BAR_P_READY0,
+       BAR_P_READY1, BAR_PV_DONE0, BAR_PV_DONE1, BAR_V_FULL, BAR_V_EMPTY = BAR_V_FULL + kVBufs, BAR_COUNT = BAR_V_EMPTY + kVBufs };
+static_assert(BAR_COUNT <= 24 && kOffBar % 256 == 0, "barrier block");
 
-// D[tmem] (+)= A[tmem] * B[smem desc], both operands e4m3 (K = 32 per instruction)
-__device__ __forceinline__ void mma_ts_f8(uint32_t d, uint32_t a, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+// D[tmem] (+)= A[tmem] * B[smem desc], both operands e4m3 (K = 32 per instruction), weight-stationary, M = 64 (layout of
+// A and D as for mma_ws_ss; A replicated in the two halves of the lanes)
+__device__ __forceinline__ void mma_ws_ts_f8(uint32_t d, uint32_t a, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n}"
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.ws.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n}"
       ::"r"(d), "r"(a), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Instruction descriptors: fp32 accumulator, M = 128; e4m3 x e4m3 (both K-major), and fp16 x fp16 with A MN-major.
+// Instruction descriptors, fp32 accumulator: e4m3 x e4m3 (both K-major), M = 64; fp16 x fp16, M = 128.
 __host__ __device__ constexpr uint32_t instr_desc_e4m3(int n) {
-  return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
+  return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(64 >> 4) << 24);
 }
-__host__ __device__ constexpr uint32_t instr_desc_f16_a_mn(int n) {
-  return (1u << 4) | (1u << 15) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
+__host__ __device__ constexpr uint32_t instr_desc_f16(int n) {
+  return (1u << 4) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
 }
 // Two floats -> two e4m3 codes (nearest, ties to even, saturating), first argument in the low byte.
 __device__ __forceinline__ uint32_t pack_e4m3x2(float lo, float hi) {
   uint16_t r;
-  asm volatile("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
+  asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
   return r;
 }
 // Two e4m3 codes (low 16 bits) -> two fp16 values, exactly.
 __device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t v) {
   uint32_t r;
-  asm volatile("{\n.reg .b16 t;\nmov.b32 {t, _}, %1;\ncvt.rn.f16x2.e4m3x2 %0, t;\n}" : "=r"(r) : "r"(v));
+  asm("{\n.reg .b16 t;\nmov.b32 {t, _}, %1;\ncvt.rn.f16x2.e4m3x2 %0, t;\n}" : "=r"(r) : "r"(v));
   return r;
 }
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<__half2*>(&v); }
@@ -93,10 +105,17 @@ __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// 16 lanes x 16 columns: thread 4 i + k of the warp gives column 4 j + k of lanes i (v[2 j]) and i + 8 (v[2 j + 1]), j = 0..3.
+__device__ __forceinline__ void tmem_st_16x128b_x4(uint32_t taddr, const uint32_t* v) {
+  asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};"
+               ::TM_W4(v, 0), TM_W4(v, 4), "r"(taddr)
+               : "memory");
+}
+
 // ---------------------------------------------------------------------------------------------- kernel
 __global__ void __launch_bounds__(kThreads, 1)
 decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_constant__ CUtensorMap scale_map,
-                  const __grid_constant__ CUtensorMap q_map,
+                  const __grid_constant__ CUtensorMap q_map, const unsigned char* cache,
                     const int32_t* page_table, const int32_t* seqlens,
                     const int32_t* cum, const int32_t* plan, float* partial_o,
                     float* partial_lse, int32_t* dev_status, int S, int H, int num_pages, int max_pages,
@@ -108,10 +127,12 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
   float* pmax_s = reinterpret_cast<float*>(sm + kOffMisc);         // [2][4][32]: per page parity, warp, row
   float* alpha_s = pmax_s + 256;                                   // [32]
   float* inv_l = alpha_s + 32;                                     // [32]
-  int4* meta = reinterpret_cast<int4*>(inv_l + 32);                // [kMetaRing]: what each ring item is
+  float* qmax_s = inv_l + 32;                                    // [4][32]: parts of the query rows' maxima
+  int4* meta = reinterpret_cast<int4*>(qmax_s + 128);            // [kMetaRing]: what each ring item is
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(meta + kMetaRing);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_s + 1);
   volatile int* ring_done = abort_flag + 1;
+  volatile int* v_flags = ring_done + 1;  // [3]: what the converters put into each V buffer
   auto bar = [&](int i) -> uint32_t { return base + kOffBar + 8 * i; };
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -123,12 +144,11 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&cache_map)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&q_map)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&scale_map)) : "memory");
-    for (int i = 0; i < kStages; ++i) { mbar_init(bar(BAR_KV_FULL + i), 1); mbar_init(bar(BAR_KV_EMPTY + i), 3); }
-    mbar_init(bar(BAR_V_FULL), 1);
-    mbar_init(bar(BAR_V_EMPTY), 1);
-    mbar_init(bar(BAR_Q_READY), 128);
+    for (int i = 0; i < kStages; ++i) { mbar_init(bar(BAR_KV_FULL + i), 1); mbar_init(bar(BAR_KV_EMPTY + i), 2 + kConverters); }
+    for (int i = 0; i < kVBufs; ++i) { mbar_init(bar(BAR_V_FULL + i), kConverters); mbar_init(bar(BAR_V_EMPTY + i), 1); }
     mbar_init(bar(BAR_S_FULL), 1);
     mbar_init(bar(BAR_S_FREE), 128);
+    mbar_init(bar(BAR_Q_READY), 128);
     mbar_init(bar(BAR_P_READY0), 128);
     mbar_init(bar(BAR_P_READY1), 128);
     mbar_init(bar(BAR_PV_DONE0), 1);
@@ -179,6 +199,10 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
         int idx = page_table[static_cast<size_t>(b) * max_pages + pj];
         const bool ok = idx >= 0 && idx < num_pages;
         if (!ok) { if (lane == 0) set_status(dev_status, TRANSMLA_DEV_BAD_PAGE); idx = 0; }
+        // A page is one contiguous piece of memory: it is asked into L2 while its stage is still in use.
+        if (elect_one())
+          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(cache + static_cast<size_t>(idx) * (kPage * kRowBytes)),
+                       "r"(kPage * kRowBytes) : "memory");
         const uint32_t stage = acquire(g);
         if (!*abort_flag && elect_one()) {
           meta[g & (kMetaRing - 1)] = make_int4(ITEM_PAGE, pj, ok ? 1 : 0, (first ? 1 : 0) | (last ? 2 : 0));
@@ -209,10 +233,10 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
       // ======================================================================== MMA issuer, scores
       // Follows the ring: skips query items (the softmax warps move them to tensor memory and report through
       // Q_READY, which also tells when the ring has ended) and runs the score products of a page as soon as it has
-      // landed: per 32 codes two e4m3 products (the queries' high and low term) on the page's codes as they came
-      // from memory, then four bf16 products on the rope part, all into one accumulator.
+      // landed: one e4m3 product per 32 codes on the page's codes as they came from memory, then four bf16 products on
+      // the rope part, all into one accumulator.
       constexpr uint32_t idesc_f8 = instr_desc_e4m3(kPage);
-      constexpr uint32_t idesc_rope = instr_desc(kPage, false);
+      constexpr uint32_t idesc_rope = instr_desc(kPage, false, 64);
       int g = 0, n = 0, seg = 0;  // ring items, pages, segments handled so far
       while (true) {
         // a segment begins (or the ring ends): the softmax warps say which
@@ -229,21 +253,17 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
           if (n > 0) mbar_wait(bar(BAR_S_FREE), (n - 1) & 1, abort_flag, dev_status);
           tc_fence_after();
           const uint64_t k0 = smem_desc(base + kOffStage + stage * kStageBytes, 16, 1024);
-#pragma unroll
-          for (int c = 0; c < kCodeTiles; ++c) {
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              const uint64_t bd = desc_advance(k0, c * kSubTileBytes + kk * 32);
-              if (elect_one()) mma_ts_f8(tmem + kColS, tmem + kColQhi + c * 32 + kk * 8, bd, idesc_f8, (c | kk) ? 1u : 0u);
-              if (elect_one()) mma_ts_f8(tmem + kColS, tmem + kColQlo + c * 32 + kk * 8, bd, idesc_f8, 1u);
-            }
-          }
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            if (elect_one())
-              mma_ts(tmem + kColS, tmem + kColQr + kk * 8, desc_advance(k0, kOffRope + kk * 32), idesc_rope, 1u);
-          }
           if (elect_one()) {
+#pragma unroll
+            for (int c = 0; c < kCodeTiles; ++c) {
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk)
+                mma_ws_ts_f8(tmem + kColS, tmem + kColQ + c * 32 + kk * 8, desc_advance(k0, c * kSubTileBytes + kk * 32), idesc_f8,
+                             (c | kk) ? 1u : 0u);
+            }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              mma_ws_ts(tmem + kColS, tmem + kColQr + kk * 8, desc_advance(k0, kOffRope + kk * 32), idesc_rope, 1u);
             tc_commit(bar(BAR_KV_EMPTY + stage));  // one of the three parties that hand the stage back
             tc_commit(bar(BAR_S_FULL));
           }
@@ -254,101 +274,95 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
       }
     } else if (warp == 6) {
       // ======================================================================== MMA issuer, products
-      // O^T += V^T P^T for a page as soon as its probabilities and its fp16 copy are there.  It follows the ring only
-      // to learn where segments begin and end.
-      constexpr uint32_t idesc_pv = instr_desc_f16_a_mn(kRowBlock);
-      int g = 0, n = 0, seg = 0;
-      while (true) {
-        mbar_wait(bar(BAR_Q_READY), seg & 1, abort_flag, dev_status);
-        ++seg;
-        if (__any_sync(0xffffffffu, *abort_flag != 0) || *ring_done != 0) break;
-        ++g;
-        while (true) {
-          const int stage = g % kStages, use = g / kStages;
-          mbar_wait(bar(BAR_KV_FULL + stage), use & 1, abort_flag, dev_status);
-          const int4 m = meta[g & (kMetaRing - 1)];
-          mbar_wait(bar(BAR_V_FULL), n & 1, abort_flag, dev_status);
-          mbar_wait(bar(BAR_P_READY0 + (n & 1)), (n >> 1) & 1, abort_flag, dev_status);
-          tc_fence_after();
-          const uint64_t a0 = smem_desc(base + kOffV, kSubTileBytes, 1024);
-          const uint64_t b0 = smem_desc(base + kOffP + (n & 1) * kPBytes, 16, 1024);
-          const uint32_t acc0 = (m.w & 1) != 0 ? 0u : 1u;  // the segment's first page starts the accumulator afresh
+      // O^T += V^T P'^T, half a page (32 tokens) at a time, as soon as the page's probabilities and the half's V^T are
+      // there.  V^T comes with the half's place in its segment (1 = the segment starts here, 4 = nothing more): this warp
+      // does not look at the ring, whose stages may be pages further.
+      constexpr uint32_t idesc_pv = instr_desc_f16(kRowBlock);
+      for (int h = 0;; ++h) {
+        const int vb = h % kVBufs, n = h >> 1;
+        mbar_wait(bar(BAR_V_FULL + vb), (h / kVBufs) & 1, abort_flag, dev_status);
+        const int flags = v_flags[vb];
+        if (__any_sync(0xffffffffu, *abort_flag != 0) || (flags & 4) != 0) break;
+        if ((h & 1) == 0) mbar_wait(bar(BAR_P_READY0 + (n & 1)), (n >> 1) & 1, abort_flag, dev_status);
+        tc_fence_after();
+        const uint64_t b0 = smem_desc(base + kOffP + (n & 1) * kPBytes + (h & 1) * 64, 16, 1024);
+        const uint32_t v0 = tmem + kColV + vb * 64;
+        const uint32_t acc0 = (flags & 1) != 0 ? 0u : 1u;
+        if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
+          for (int kk = 0; kk < 2; ++kk) {
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              if (elect_one())
-                mma_ss(tmem + kColO + t * 32, desc_advance(a0, (2 * t) * kSubTileBytes + kk * 2048),
-                       desc_advance(b0, kk * 32), idesc_pv, kk == 0 ? acc0 : 1u);
-            }
+            for (int t = 0; t < 4; ++t)
+              mma_ts(tmem + kColO + t * 32, v0 + t * 16 + kk * 8, desc_advance(b0, kk * 32), idesc_pv, kk == 0 ? acc0 : 1u);
           }
-          if (elect_one()) {
-            tc_commit(bar(BAR_V_EMPTY));
-            tc_commit(bar(BAR_PV_DONE0 + (n & 1)));
-          }
-          __syncwarp();
-          ++g; ++n;
-          if ((m.w & 2) != 0 || m.x != ITEM_PAGE || __any_sync(0xffffffffu, *abort_flag != 0)) break;
+          tc_commit(bar(BAR_V_EMPTY + vb));
+          if (h & 1) tc_commit(bar(BAR_PV_DONE0 + (n & 1)));
         }
+        __syncwarp();
       }
-    } else if (warp >= 7) {
-      // ======================================================================== converters (warps 7-10)
-      // Per page: scale_j * code -> fp16 into the V buffer, in the layout of a bf16 page's latent sub-tiles (64
-      // tokens x 64 columns, 128-byte rows, 128-byte swizzle); rows beyond the sequence become zeros.  They hand a
-      // query item back too (their third of it), so that no stage can be
-      // used twice before they have seen it.
-      const int c = tid - 224;
-      int g = 0, n = 0, L_seg = 0;
-      while (true) {
+    } else if (warp >= 8) {
+      // ======================================================================== converters (warps 8-15)
+      // Per half page (32 tokens): the codes of quadrant `quad`'s latents, transposed by ldmatrix (8 tokens x 8 pairs of
+      // codes a matrix; a thread gets a pair of latents for two tokens), as fp16 into that quadrant's lanes of a V^T
+      // buffer; tokens beyond the sequence become zeros.  They hand a query item back too, so that no stage can be used
+      // twice before they have seen it.
+      const int quad = warp & 3, t0 = (warp - 8) >> 2 << 1;   // a quadrant's two warps take two tiles of 128 latents each
+      const uint32_t lane_base = static_cast<uint32_t>(quad * 32) << 16;
+      int g = 0, h = 0, L_seg = 0;
+      bool run = true;
+      while (run) {
         const int stage = g % kStages, use = g / kStages;
         mbar_wait(bar(BAR_KV_FULL + stage), use & 1, abort_flag, dev_status);
         const int4 m = meta[g & (kMetaRing - 1)];
-        int stop;
-        asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 3, 128, q;\nselp.s32 %0, 1, 0, p;\n}"
-                     : "=r"(stop) : "r"(static_cast<int>(*abort_flag != 0 || m.x == ITEM_END)) : "memory");
-        if (stop) break;
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
         if (m.x == ITEM_QUERIES) {
           L_seg = m.w;  // the sequence's length, for the pages that follow
-          if (c == 0) mbar_arrive(bar(BAR_KV_EMPTY + stage));
+          mbar_arrive(bar(BAR_KV_EMPTY + stage));
           ++g;
           continue;
         }
-        if (n > 0) mbar_wait(bar(BAR_V_EMPTY), (n - 1) & 1, abort_flag, dev_status);
-        const unsigned char* st = sm + kOffStage + stage * kStageBytes;
-        unsigned char* vb = sm + kOffV;
-        const int valid = m.z != 0 ? min(kPage, L_seg - m.y * kPage) : 0;  // rows [valid, 64) must read as zero
-        // 16 rounds; in a round a warp takes 4 consecutive rows x the 8 16-byte chunks of one 128-code sub-tile, so that
-        // its loads sweep whole 128-byte rows (the swizzle only permutes the chunks inside a row)
+        run = m.x == ITEM_PAGE;
+        const uint32_t st = base + kOffStage + stage * kStageBytes;
+        const int valid = m.z != 0 ? min(kPage, L_seg - m.y * kPage) : 0;  // tokens [valid, 64) must read as zero
 #pragma unroll 1
-        for (int rblk = 0; rblk < 4; ++rblk) {
-          const int r = rblk * 16 + (c >> 3), j = c & 7;
-          const __half2 sc2 = __half2half2(__float2half_rn(r < valid ? *reinterpret_cast<const float*>(st + kOffScale + r * 16) : 0.f));
+        for (int half = 0; half < (run ? 2 : 1); ++half, ++h) {
+          const int vb = h % kVBufs;
+          if (h >= kVBufs) mbar_wait(bar(BAR_V_EMPTY + vb), (h / kVBufs - 1) & 1, abort_flag, dev_status);
+          if (tid == 256) v_flags[vb] = !run ? 4 : half == 0 ? (m.w & 1) : 0;
+          if (run) {
+            tc_fence_after();
+            const int tok = half * 32 + lane;
+            const int left = valid - half * 32 - 2 * (lane & 3);  // of this thread's token pairs 8 j + (0, 1): visible if 8 j (+ 1) < left
+            uint32_t x[4][4];
 #pragma unroll
-          for (int ct = 0; ct < kCodeTiles; ++ct) {  // code sub-tile: columns 128 ct .. 128 ct + 127
-            const uint4 x = *reinterpret_cast<const uint4*>(st + ct * kSubTileBytes + r * 128 + ((j ^ (r & 7)) << 4));
-            const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-            uint32_t o[8];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const __half2 lo = __hmul2(as_half2(e4m3x2_to_f16x2(w[k] & 0xffffu)), sc2);
-              const __half2 hi = __hmul2(as_half2(e4m3x2_to_f16x2(w[k] >> 16)), sc2);
-              o[2 * k] = r < valid ? as_u32(lo) : 0u;  // (a NaN code times a zero scale would still be NaN)
-              o[2 * k + 1] = r < valid ? as_u32(hi) : 0u;
+            for (int i = 0; i < 4; ++i) {  // tile t0 + i / 2, 16 of this quadrant's latents: one 16-byte chunk of the token rows
+              const uint32_t addr = st + (t0 + (i >> 1)) * kSubTileBytes + tok * 128 + (((quad * 2 + (i & 1)) ^ (tok & 7)) << 4);
+              asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                           : "=r"(x[i][0]), "=r"(x[i][1]), "=r"(x[i][2]), "=r"(x[i][3]) : "r"(addr) : "memory");
             }
-            // columns 128 ct + 16 j .. + 15 -> V sub-tile 2 ct + j / 4, 16-byte chunks 2 (j % 4) and 2 (j % 4) + 1
-            unsigned char* dst = vb + (2 * ct + (j >> 2)) * kSubTileBytes + r * 128;
-            const int ch = 2 * (j & 3);
-            *reinterpret_cast<uint4*>(dst + ((ch ^ (r & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
-            *reinterpret_cast<uint4*>(dst + (((ch + 1) ^ (r & 7)) << 4)) = make_uint4(o[4], o[5], o[6], o[7]);
+            if (valid < kPage) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) x[i][j] = 8 * j + 1 < left ? x[i][j] : 8 * j < left ? x[i][j] & 0xffffu : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              uint32_t o[8];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                o[2 * j] = e4m3x2_to_f16x2(__byte_perm(x[i][j], 0, 0x4420));      // the even latent, tokens 2 k and 2 k + 1
+                o[2 * j + 1] = e4m3x2_to_f16x2(__byte_perm(x[i][j], 0, 0x4431));  // the odd one
+              }
+              tmem_st_16x128b_x4(tmem + lane_base + (static_cast<uint32_t>((i & 1) * 16) << 16) + kColV + vb * 64 + (t0 + (i >> 1)) * 16, o);
+            }
+            tc_wait_st();
+            tc_fence_before();
           }
+          mbar_arrive(bar(BAR_V_FULL + vb));
         }
-        fence_proxy_async();
-        asm volatile("bar.sync 3, 128;" ::: "memory");
-        if (c == 0) {
-          mbar_arrive(bar(BAR_V_FULL));
-          mbar_arrive(bar(BAR_KV_EMPTY + stage));
-        }
-        ++g; ++n;
+        mbar_arrive(bar(BAR_KV_EMPTY + stage));
+        ++g;
       }
     } else if (warp < 4) {
       // ======================================================================== softmax + epilogue (warps 0-3)
@@ -374,56 +388,77 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
           mbar_arrive(bar(BAR_Q_READY));
           return m;
         }
-        const unsigned char* qrow = sm + kOffStage + stage * kStageBytes + lane * 128;
-        // This row's absorbed query q (512 bf16): q ~ sq * (hi + lo) with hi, lo e4m3 and sq = max|q| / 448.
+        unsigned char* qrow = sm + kOffStage + stage * kStageBytes + lane * 128;
+        // This row's absorbed query q (512 bf16): q ~ sq * (hi + lo) with hi, lo e4m3 and sq = max|q| / 448.  All four
+        // warps need all of it in their quadrant, so each works out a quarter (two sub-tiles of 64 values) and leaves the
+        // codes where the bf16 values were: 64 bytes of high terms, then 64 bytes of low terms.
         float amax = 0.f;
 #pragma unroll 1
-        for (int c = 0; c < kCodeTiles * 2; ++c) {
+        for (int c = 0; c < 2; ++c) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const uint4 x = *reinterpret_cast<const uint4*>(qrow + c * kQTileBytes + ((j ^ (lane & 7)) << 4));
+            const uint4 x = *reinterpret_cast<const uint4*>(qrow + (2 * warp + c) * kQTileBytes + ((j ^ (lane & 7)) << 4));
             const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) amax = fmaxf(amax, fmaxf(fabsf(bf16_lo(w[k])), fabsf(bf16_hi(w[k]))));
           }
         }
+        qmax_s[warp * 32 + lane] = amax;
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        amax = fmaxf(fmaxf(qmax_s[lane], qmax_s[32 + lane]), fmaxf(qmax_s[64 + lane], qmax_s[96 + lane]));
         sq_row = amax > 0.f ? amax * (1.f / 448.f) : 1.f;
         const float inv_sq = 1.f / sq_row;
 #pragma unroll 1
-        for (int c = 0; c < kCodeTiles * 2; ++c) {  // 64 query values -> 16 columns of four codes, high and low term
-          uint32_t hi[16], lo[16];
+        for (int c = 0; c < 2; ++c) {
+          unsigned char* tile = qrow + (2 * warp + c) * kQTileBytes;
+          uint32_t qv[32];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const uint4 x = *reinterpret_cast<const uint4*>(qrow + c * kQTileBytes + ((j ^ (lane & 7)) << 4));
-            const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-            uint32_t h2[4], l2[4];
+            const uint4 x = *reinterpret_cast<const uint4*>(tile + ((j ^ (lane & 7)) << 4));
+            qv[4 * j] = x.x; qv[4 * j + 1] = x.y; qv[4 * j + 2] = x.z; qv[4 * j + 3] = x.w;
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {  // 16 values -> 16 bytes of each term
+            uint32_t h[4], l[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              const float a = bf16_lo(w[k]) * inv_sq, b = bf16_hi(w[k]) * inv_sq;
-              h2[k] = pack_e4m3x2(a, b);
-              const float2 back = __half22float2(as_half2(e4m3x2_to_f16x2(h2[k])));
-              l2[k] = pack_e4m3x2(a - back.x, b - back.y);
+              const uint32_t w0 = qv[8 * j + 2 * k], w1 = qv[8 * j + 2 * k + 1];
+              const float a0 = bf16_lo(w0) * inv_sq, a1 = bf16_hi(w0) * inv_sq, a2 = bf16_lo(w1) * inv_sq, a3 = bf16_hi(w1) * inv_sq;
+              const uint32_t h0 = pack_e4m3x2(a0, a1), h1 = pack_e4m3x2(a2, a3);
+              const float2 b0 = __half22float2(as_half2(e4m3x2_to_f16x2(h0))), b1 = __half22float2(as_half2(e4m3x2_to_f16x2(h1)));
+              h[k] = h0 | (h1 << 16);
+              l[k] = pack_e4m3x2(a0 - b0.x, a1 - b0.y) | (pack_e4m3x2(a2 - b1.x, a3 - b1.y) << 16);
             }
-            hi[2 * j] = h2[0] | (h2[1] << 16); hi[2 * j + 1] = h2[2] | (h2[3] << 16);
-            lo[2 * j] = l2[0] | (l2[1] << 16); lo[2 * j + 1] = l2[2] | (l2[3] << 16);
+            *reinterpret_cast<uint4*>(tile + ((j ^ (lane & 7)) << 4)) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(tile + (((j + 4) ^ (lane & 7)) << 4)) = make_uint4(l[0], l[1], l[2], l[3]);
           }
-          tmem_st16(tmem + lane_base + kColQhi + c * 16, hi);
-          tmem_st16(tmem + lane_base + kColQlo + c * 16, lo);
         }
-        {  // the rope part, divided by sq, stays bf16
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+#pragma unroll 1
+        for (int c = 0; c < kCodeTiles * 2; ++c) {  // 64 query values -> 16 columns of four codes, this quadrant's term
+          uint32_t v[16];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint4 x = *reinterpret_cast<const uint4*>(qrow + c * kQTileBytes + (((j + 4 * (warp & 1)) ^ (lane & 7)) << 4));
+            v[4 * j] = x.x; v[4 * j + 1] = x.y; v[4 * j + 2] = x.z; v[4 * j + 3] = x.w;
+          }
+          tmem_st16(tmem + lane_base + kColQ + c * 16, v);
+        }
+        {  // the rope part, divided by sq, stays bf16; the low rows have none
           uint32_t v[32];
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const uint4 x = *reinterpret_cast<const uint4*>(qrow + 8 * kQTileBytes + ((j ^ (lane & 7)) << 4));
             const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) v[4 * j + k] = pack_bf16(bf16_lo(w[k]) * inv_sq, bf16_hi(w[k]) * inv_sq);
+            for (int k = 0; k < 4; ++k) v[4 * j + k] = (warp & 1) ? 0u : pack_bf16(bf16_lo(w[k]) * inv_sq, bf16_hi(w[k]) * inv_sq);
           }
           tmem_st32(tmem + lane_base + kColQr, v);
         }
         tc_wait_st();
         tc_fence_before();
         mbar_arrive(bar(BAR_Q_READY));
+        fence_proxy_async();  // the stage was written here; its next contents come through the async proxy
         asm volatile("bar.sync 1, 128;" ::: "memory");
         if (tid == 0) mbar_arrive(bar(BAR_KV_EMPTY + stage));  // one of three: the score warp and the converters see it too
         ++g;
@@ -448,26 +483,42 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
           const bool first = (pm.w & 1) != 0;
           const int buf = n & 1;
 
+          // Quadrants 0 and 2 hold the high rows' sums for 32 tokens, 1 and 3 the low rows' for the same: each warp keeps
+          // 16 of them (even warps the first), gets the other row's for those from its neighbour and adds.
           mbar_wait(bar(BAR_S_FULL), n & 1, abort_flag, dev_status);
           tc_fence_after();
           uint32_t sq[16];  // this warp's 16 tokens of its row
-          tmem_ld16(tmem + lane_base + kColS + warp * 16, sq);
-          tc_wait_ld();
-          tc_fence_before();
-          mbar_arrive(bar(BAR_S_FREE));
+          {
+            uint32_t other[16];
+            tmem_ld16(tmem + lane_base + kColS + (warp & 1) * 16, sq);
+            tmem_ld16(tmem + lane_base + kColS + (~warp & 1) * 16, other);
+            tc_wait_ld();
+            tc_fence_before();
+            mbar_arrive(bar(BAR_S_FREE));
+            float* mine = reinterpret_cast<float*>(sm + kOffX) + warp * 512 + lane;
+            const float* theirs = reinterpret_cast<const float*>(sm + kOffX) + (warp ^ 1) * 512 + lane;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) mine[j * 32] = __uint_as_float(other[j]);
+            asm volatile("bar.sync %0, 64;" ::"r"(2 + (warp >> 1)) : "memory");
+#pragma unroll
+            for (int j = 0; j < 16; ++j) sq[j] = __float_as_uint(__uint_as_float(sq[j]) + theirs[j * 32]);
+          }
+          float sc[16];
           {
             // a score is sq (row) * scale_j (token) * the accumulated sum; tokens beyond the visible range are dropped
-            // by selection, so whatever their scale holds does not matter
+            // by selection, so whatever their scale holds does not matter.  The reference maximum is that of score +
+            // log2 scale (its whole part, from the exponent bits; not below -60, so that exp2 of the rest stays finite).
             const unsigned char* scl = sm + kOffStage + stage * kStageBytes + kOffScale + warp * 16 * 16;
             const float row_factor = sq_row * scale_log2;
             float pmax = -INFINITY;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              const float x = warp * 16 + j < tok_end
-                                  ? __uint_as_float(sq[j]) * (row_factor * *reinterpret_cast<const float*>(scl + j * 16))
-                                  : -INFINITY;
+              const bool seen = warp * 16 + j < tok_end;
+              sc[j] = *reinterpret_cast<const float*>(scl + j * 16);
+              const float x = seen ? __uint_as_float(sq[j]) * (row_factor * sc[j]) : -INFINITY;
+              sc[j] = seen ? sc[j] : 0.f;
               sq[j] = __float_as_uint(x);
-              pmax = fmaxf(pmax, x);
+              pmax = fmaxf(pmax, x + static_cast<float>(max(static_cast<int>(__float_as_uint(sc[j]) >> 23) - 127, -60)));
             }
             pmax_s[(buf * 4 + warp) * 32 + lane] = pmax;
           }
@@ -494,18 +545,16 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
               l_run *= alpha;
             }
           }
-          const float m_ref = m_used;
+          const float m_ref = m_used == -INFINITY ? 0.f : m_used;
 
           // ---- probabilities of tokens 16*warp .. 16*warp+15
           uint32_t pk[8];
           float psum = 0.f;
 #pragma unroll
           for (int j = 0; j < 16; j += 2) {
-            const int t0 = warp * 16 + j;
-            const float p0 = t0 < tok_end ? exp2f(__uint_as_float(sq[j]) - m_ref) : 0.f;
-            const float p1 = t0 + 1 < tok_end ? exp2f(__uint_as_float(sq[j + 1]) - m_ref) : 0.f;
+            const float p0 = ex2_approx(__uint_as_float(sq[j]) - m_ref), p1 = ex2_approx(__uint_as_float(sq[j + 1]) - m_ref);
             psum += p0 + p1;
-            pk[j >> 1] = pack_f16(p0, p1);
+            pk[j >> 1] = pack_f16(p0 * sc[j], p1 * sc[j + 1]);
           }
           l_run += psum;
 
@@ -558,21 +607,16 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
         const int n_last = n - 1;
         mbar_wait(bar(BAR_PV_DONE0 + (n_last & 1)), (n_last >> 1) & 1, abort_flag, dev_status);
         tc_fence_after();
-        float* dst = o_rows + warp * 32 + lane;
+        // lane -> latent, see the tensor-memory map
+        float* dst = o_rows + warp * 32 + (lane & 16) + ((lane & 15) < 8 ? 2 * (lane & 15) : 2 * (lane & 7) + 1);
 #pragma unroll 1
-        for (int t = 0; t < 4; t += 2) {  // two 128-row tiles per round trip to tensor memory
-          uint32_t ov[64];
+        for (int t = 0; t < 4; ++t) {
+          uint32_t ov[32];
           tmem_ld32(tmem + lane_base + kColO + t * 32, ov);
-          tmem_ld32(tmem + lane_base + kColO + (t + 1) * 32, ov + 32);
           tc_wait_ld();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (rb * kRowBlock + j < SH) {
-              const float sc = inv_l[j];
-              dst[static_cast<size_t>(j) * R + t * 128] = __uint_as_float(ov[j]) * sc;
-              dst[static_cast<size_t>(j) * R + (t + 1) * 128] = __uint_as_float(ov[32 + j]) * sc;
-            }
-          }
+          for (int j = 0; j < 32; ++j)
+            if (rb * kRowBlock + j < SH) dst[static_cast<size_t>(j) * R + t * 128] = __uint_as_float(ov[j]) * inv_l[j];
         }
         tc_fence_before();
         asm volatile("bar.sync 1, 128;" ::: "memory");  // inv_l and the row sums are reused by the next segment
@@ -619,7 +663,7 @@ cudaError_t launch_decode_fp8(const transmla_params_t& p, int G, const __nv_bflo
   dim3 grid((G + merge - 1) / merge, blocks);
   int32_t* next = const_cast<int32_t*>(cum) + 3 * p.batch + 1;  // page counters, zeroed by the plan
   return launch_pdl(decode_fp8_kernel, grid, dim3(kThreads), static_cast<size_t>(kSmemBytes), stream, map, smap, qmap,
-                    page_table, seqlens, cum, plan, partial_o, partial_lse, dev_status, p.q_len, p.num_heads,
+                    static_cast<const unsigned char*>(cache_fp8), page_table, seqlens, cum, plan, partial_o, partial_lse, dev_status, p.q_len, p.num_heads,
                     p.num_pages, p.max_pages_per_seq, p.softmax_scale * kLog2e, p.batch, dynamic_claims(p, G) ? 1 : 0, next, G, merge);
 }
 

@@ -28,10 +28,11 @@ def pack_fp8_cache(codes, k_pe, scale):
     return out
 
 
-def fp8_case(shape, seqlens, seed, poison=True):
+def fp8_case(shape, seqlens, seed, poison=True, factor=None):
     case = synth.make_decode_case(shape, seqlens, seed)
     rng = np.random.default_rng(seed)
-    rows = lifts.f64(case['cache']) * rng.uniform(0.5, 2.0, size=case['cache'].shape[:2] + (1,))
+    size = case['cache'].shape[:2] + (1,)
+    rows = lifts.f64(case['cache']) * (rng.uniform(0.5, 2.0, size=size) if factor is None else factor(rng, size))
     codes, k_pe, scale = orc.quantize_latent_rows(rows, shape.r)
     if poison:   # rows that no sequence owns: NaN codes, NaN k_pe, NaN scale
         owned = np.zeros(codes.shape[:2], bool)
@@ -100,6 +101,20 @@ def test_fp8_decode_two_query_positions_and_many_rows():
     idx = tuple(np.array(only).T)
     gu.assert_close(lifts.f64(out)[idx], want[idx], 'fp8 cache, S = 2')
     gu.assert_lse_close(lifts.f64(lse)[idx], want_lse[idx], 'fp8 cache lse, S = 2')
+
+
+def test_fp8_rows_of_very_different_size():
+    # A token's scale multiplies its probability in fp16, with the reference maximum taken over both: rows 2^-14 to 1 times
+    # the usual size, zero rows among them (scale 1 by definition, far above their neighbours').
+    gu.ensure_built()
+    shape = synth.LLAMA2_7B
+    seqlens = [330, 64, 1500]
+    case = fp8_case(shape, seqlens, seed=28, factor=lambda rng, size: 2.0 ** rng.uniform(-14, 0, size) * (rng.random(size) > 0.05))
+    out, lse, status = run_fp8(shape, case, gu.mla_scale(shape), 0)
+    assert status == 0
+    want, want_lse = oracle_fp8(shape, case, gu.mla_scale(shape))
+    gu.assert_close(lifts.f64(out), want, 'rows of very different size')
+    gu.assert_lse_close(lifts.f64(lse), want_lse, 'rows of very different size, lse')
 
 
 @pytest.mark.parametrize('seqlens,columns', [([64 * 40 + 5, 1, 700, 0, 333], 600), ([2900], 1200)])
