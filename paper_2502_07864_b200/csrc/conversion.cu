@@ -123,15 +123,6 @@ __global__ void __launch_bounds__(256) gemm_kernel(int ta, int tb, int M, int N,
   }
 }
 
-cudaError_t gemm_f32(int ta, int tb, int M, int N, int K, float alpha, const float* A, int lda, long long strideA,
-                     const float* B, int ldb, long long strideB, float* C, int ldc, long long strideC, int batch,
-                     cudaStream_t stream) {
-  if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
-  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch);
-  gemm_kernel<float><<<grid, 256, 0, stream>>>(ta, tb, M, N, K, alpha, A, lda, strideA, B, ldb, strideB, C, ldc, strideC, 0);
-  return cudaGetLastError();
-}
-
 // G [r,r] (fp64) = Y^T Y for Y [m,r]: the long sum over m is cut into kGramSlices slices, one batch entry each
 // (16 tiles alone would leave most SMs idle), and the partial sums are added in a fixed order.
 constexpr int kGramSlices = kGramPartials;
