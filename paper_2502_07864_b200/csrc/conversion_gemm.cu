@@ -14,8 +14,12 @@
 // shared memory - K-major where K is contiguous in memory (64-byte swizzle), MN-major where it is not (128-byte swizzle,
 // 64-wide pieces).  All sixteen drain the accumulators (two, in tensor memory) in between.  One warp of the pair's first
 // CTA issues the products.
-// Rates (fp32 products): 8192 x 4096 x 4096 132 TFLOP/s, X^T X of 8192 x 8064 239 (half of it mirrored), 8064 x 512 x 8064
-// 116; the fp32 multiply-add kernel this one replaced reached 48, 50 and 42.
+// Rates (fp32 products): 8192 x 4096 x 4096 185 TFLOP/s, X^T X of 8192 x 8064 303 (half of it mirrored), 8064 x 512 x 8064
+// 161; the fp32 multiply-add kernel this one replaced reached 48, 50 and 42.  What bounds it: a chunk takes about 3000
+// cycles, 1540 of them the tensor pipe's, in a ring of waits: sums drained (650) and reported to the issuer, products,
+// stages freed, pieces converted (900).  (With arrivals that release to the other CTA in every worker, which wait for the
+// thread's loads in flight, it took 4400; with the jobs split over converting and adding warps and the fp32 pieces fetched
+// through shared memory 2900 at more shared-memory traffic and no gain.)
 #include "conversion.cuh"
 #include "sm100_ptx.cuh"
 
@@ -28,7 +32,7 @@ namespace {
 
 constexpr int kRows = 128, kKc = 32;           // rows of op(A) and columns of op(B) a CTA converts; K per chunk
 constexpr int kStages = 4;
-constexpr int kWorkers = 512, kThreads = kWorkers + 128;   // the issuer's warpgroup has one warp at work
+constexpr int kWorkers = 512, kThreads = kWorkers + 128;   // the last warpgroup has one warp at work: issuer or messenger
 constexpr int kPlane = kRows * kKc * 2;        // 8192 bytes: one term of one operand's chunk
 constexpr int kStageBytes = 6 * kPlane;
 constexpr int kOffBar = kStages * kStageBytes;
@@ -36,7 +40,9 @@ constexpr int kSmemBytes = kOffBar + 256 + 1024;
 constexpr int kLaunchRegs = 96, kWorkerRegs = 112, kIssuerRegs = 24;
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 static_assert(kThreads * kLaunchRegs <= 65536 && kWorkers * kWorkerRegs + 128 * kIssuerRegs <= kThreads * kLaunchRegs, "register split");
-enum { BAR_FULL = 0, BAR_EMPTY = kStages, BAR_D_FULL = 2 * kStages, BAR_D_FREE = BAR_D_FULL + 2 };
+enum { BAR_FULL = 0, BAR_EMPTY = kStages, BAR_D_FULL = 2 * kStages, BAR_D_FREE = BAR_D_FULL + 2,
+       BAR_FULL2 = BAR_D_FREE + 2, BAR_D_FREE2 = BAR_FULL2 + kStages, BAR_COUNT = BAR_D_FREE2 + 2 };  // ..2: the second CTA's word
+static_assert(BAR_COUNT <= 24, "barrier block");
 
 // The pair's instructions.  The first CTA issues for both: A and B descriptors address the same offsets in both CTAs (128
 // rows of A and half of B's columns each), and each CTA's tensor memory gets its 128 rows of D.
@@ -53,6 +59,12 @@ __device__ __forceinline__ void tc_commit2(uint32_t bar) {  // arrives on the ba
 // Arrives on the first CTA's barrier at this offset.
 __device__ __forceinline__ void mbar_arrive_first(uint32_t bar) {
   asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, 0;\nmbarrier.arrive.release.cluster.shared::cluster.b64 _, [a];\n}"
+               ::"r"(bar) : "memory");
+}
+
+// The same without a release: for an arrival that hands over tensor memory (the reads have completed), nothing in memory.
+__device__ __forceinline__ void mbar_arrive_first_relaxed(uint32_t bar) {
+  asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, 0;\nmbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [a];\n}"
                ::"r"(bar) : "memory");
 }
 
@@ -130,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
   const uint32_t raw = smem_u32(smem_unaligned);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* sm = smem_unaligned + (base - raw);
-  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(sm + kOffBar + 128);
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(sm + kOffBar + 192);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_s + 1);
   auto bar = [&](int i) -> uint32_t { return base + kOffBar + 8 * i; };
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -152,13 +164,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
     if (kCtas == 2) asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     else __syncthreads();
   };
-  auto arrive_issuer = [&](int i) {
-    if (kCtas == 2) mbar_arrive_first(bar(i)); else mbar_arrive(bar(i));
-  };
 
   if (tid == 0) {
-    for (int i = 0; i < kStages; ++i) { mbar_init(bar(BAR_FULL + i), 8 * kCtas); mbar_init(bar(BAR_EMPTY + i), 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(bar(BAR_D_FULL + i), 1); mbar_init(bar(BAR_D_FREE + i), 16 * kCtas); }
+    for (int i = 0; i < kStages; ++i) { mbar_init(bar(BAR_FULL + i), 8); mbar_init(bar(BAR_EMPTY + i), 1); mbar_init(bar(BAR_FULL2 + i), 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar(BAR_D_FULL + i), 1); mbar_init(bar(BAR_D_FREE + i), 16); mbar_init(bar(BAR_D_FREE2 + i), 16); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -184,8 +193,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
       constexpr uint32_t idesc = instr_desc(kTile, !kAContig, kTile) | (kBContig ? 0u : 1u << 16);
       for (int c = 0; c < chunks; ++c) {
         const int stage = c % kStages, buf = c & 1;
-        if (c >= 2) mbar_wait_cluster(bar(BAR_D_FREE + buf), ((c >> 1) - 1) & 1, abort_flag);
-        mbar_wait_cluster(bar(BAR_FULL + stage), (c / kStages) & 1, abort_flag);
+        if (c >= 2) {
+          mbar_wait(bar(BAR_D_FREE + buf), ((c >> 1) - 1) & 1, abort_flag, nullptr);
+          if (kCtas == 2) mbar_wait_cluster(bar(BAR_D_FREE2 + buf), ((c >> 1) - 1) & 1, abort_flag);
+        }
+        mbar_wait(bar(BAR_FULL + stage), (c / kStages) & 1, abort_flag, nullptr);
+        if (kCtas == 2) mbar_wait_cluster(bar(BAR_FULL2 + stage), (c / kStages) & 1, abort_flag);
         tc_fence_after();
         const uint64_t a0 = operand_desc<kAContig>(base + stage * kStageBytes);
         const uint64_t b0 = operand_desc<kBContig>(base + stage * kStageBytes + 3 * kPlane);
@@ -204,6 +217,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
           if (kCtas == 2) { tc_commit2(bar(BAR_EMPTY + stage)); tc_commit2(bar(BAR_D_FULL + buf)); }
           else { tc_commit(bar(BAR_EMPTY + stage)); tc_commit(bar(BAR_D_FULL + buf)); }
         }
+        __syncwarp();
+      }
+    } else if (rank == 1 && warp == kWorkers / 32) {
+      // The second CTA's messenger tells the issuer of written stages: an arrival that releases to the other CTA waits for
+      // everything its thread has in flight, which the workers must not.
+      for (int c = 0; c < chunks; ++c) {
+        mbar_wait(bar(BAR_FULL + c % kStages), (c / kStages) & 1, abort_flag, nullptr);
+        if (elect_one()) mbar_arrive_first(bar(BAR_FULL2 + c % kStages));
         __syncwarp();
       }
     }
@@ -232,12 +253,31 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) arrive_issuer(BAR_D_FREE + buf);
+      if (lane == 0) { if (rank == 0) mbar_arrive(bar(BAR_D_FREE + buf)); else mbar_arrive_first_relaxed(bar(BAR_D_FREE2 + buf)); }
     };
     const int gtid = tid & 255;                         // thread of its group: two pieces of A and two of B a chunk
     const int nb0 = n0 + rank * kRows;                  // this CTA's columns of op(B)
     float xa[2][8], xb[2][8];
+    // Away from the edges a thread's pieces sit at fixed distances from one address per operand.
+    const bool inside = vec_a && vec_b && m0 + kRows <= M && nb0 + kRows <= N;
+    const float* next_a = A + (kAContig ? static_cast<size_t>(m0 + (gtid >> 2)) * args.lda + (gtid & 3) * 8
+                                        : static_cast<size_t>(gtid >> 3) * args.lda + m0 + (gtid & 7) * 8);
+    const float* next_b = B + (kBContig ? static_cast<size_t>(nb0 + (gtid >> 2)) * args.ldb + (gtid & 3) * 8
+                                        : static_cast<size_t>(gtid >> 3) * args.ldb + nb0 + (gtid & 7) * 8);
+    auto load8 = [](float (&x)[8], const float* src) {
+      const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
+      x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+    };
     auto load = [&](int c) {
+      if (inside && (c + 1) * kKc <= K) {
+        const float* a = next_a + (kAContig ? static_cast<size_t>(c) * kKc : static_cast<size_t>(c) * kKc * args.lda);
+        const float* b = next_b + (kBContig ? static_cast<size_t>(c) * kKc : static_cast<size_t>(c) * kKc * args.ldb);
+        load8(xa[0], a);
+        load8(xa[1], a + (kAContig ? static_cast<size_t>(64) * args.lda : 64));
+        load8(xb[0], b);
+        load8(xb[1], b + (kBContig ? static_cast<size_t>(64) * args.ldb : 64));
+        return;
+      }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         load_group<kAContig>(xa[u], A, vec_a, args.lda, m0, M, c * kKc, K, gtid + u * 256);
@@ -258,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
       }
       fence_proxy_async();
       __syncwarp();
-      if (lane == 0) arrive_issuer(BAR_FULL + stage);
+      if (lane == 0) mbar_arrive(bar(BAR_FULL + stage));
       if (c + 2 < chunks) load(c + 2);
       while (drained + 2 <= c) drain(drained++);
     }

@@ -40,6 +40,24 @@ def test_gemm_all_storage_orders_with_ragged_edges(ta, tb):
     assert _rel(_f64(c), want) < 1e-6
 
 
+@pytest.mark.parametrize('M,N,K,ta,tb', [(128, 128, 32, 0, 1), (129, 127, 33, 1, 0), (1, 1, 1, 0, 0), (20000, 301, 100, 0, 1),
+                                         (301, 20000, 65, 1, 0), (5001, 5001, 300, 1, 0), (200, 200, 300, 1, 0), (333, 333, 40, 0, 1)])
+def test_gemm_tiles_pairs_and_symmetric_products(M, N, K, ta, tb):
+    # one tile and one past it; enough tiles for the two-CTA kernel (row strides that are and are not whole 16 bytes); X^T X
+    # and X X^T, whose upper half is mirrored.  Per chunk of 32 at most 12 truncations of 2^-23 in the accumulator, then
+    # rounded sums: below 1e-6 of the norm for random signs.
+    gu.ensure_built()
+    gen = torch.Generator(device='cuda'); gen.manual_seed(M + K)
+    a = torch.randn((K, M) if ta else (M, K), generator=gen, device='cuda')
+    b = a if M == N and ta != tb and M > 129 else torch.randn((N, K) if tb else (K, N), generator=gen, device='cuda')
+    c = torch.full((M, N), float('nan'), device='cuda')
+    binding.transmla_conv_gemm(a, b, c, ta=bool(ta), tb=bool(tb))
+    want = (a.double().T if ta else a.double()) @ (b.double().T if tb else b.double())
+    assert float((c - want).norm() / want.norm()) < 1e-6
+    if b is a:
+        assert torch.equal(c, c.T)
+
+
 @pytest.mark.parametrize('g,d,fold', [(4, 16, 1), (4, 16, 2), (32, 128, 4), (3, 8, 4)])
 def test_rorope_covariance_matches_the_oracle(g, d, fold):
     gu.ensure_built()
