@@ -1,146 +1,10 @@
-// Kernels of the GQA -> MLA conversion on calibration activations (Sec. 4.2, 4.3; App. B, C, D).
-// fp32 SIMT arithmetic (fp64 where the orthonormalisation needs it): the results are eigenvectors and low-rank
-// bases, and the step is a one-off per model, bound by the two large contractions (the joint second moment and
-// the subspace iteration's products).
+// Kernels of the GQA -> MLA conversion on calibration activations (Sec. 4.2, 4.3; App. B, C, D): rotations, balancing and
+// eigenvectors in fp32 arithmetic.  The matrix products are in conversion_gemm.cu, the orthonormalisation of the subspace
+// iteration in conversion_qr.cu.
 #include "conversion.cuh"
 
 namespace transmla {
 namespace conv {
-
-// ------------------------------------------------------------------------------------------------ GEMM
-// 128 x 128 tile, 256 threads x (8 x 8) outputs, k in steps of 16 through two shared-memory buffers: the next
-// tile's global loads (16 bytes each where the storage allows, element by element at ragged edges or odd strides)
-// are in flight while the current tile is multiplied.  Any of the four storage combinations, no shape restriction.
-constexpr int BM = 128, BN = 128, BK = 16;
-
-// One operand tile [128 x BK] as two float4 per thread.  `rows_major`: the operand is stored [rows, K] (k contiguous),
-// otherwise [K, rows] (rows contiguous).  r0 = first row of the tile, R = row count, ld = storage stride.
-struct TileRegs { float4 v[2]; };
-__device__ __forceinline__ void fetch_tile(TileRegs& t, const float* P, bool rows_major, bool vec, int ld, int r0, int R, int k0,
-                                           int K, int tid) {
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int f = tid + 256 * u;
-    float x[4] = {0.f, 0.f, 0.f, 0.f};
-    if (rows_major) {
-      const int rr = r0 + f / 4, k = k0 + (f % 4) * 4;
-      if (rr < R) {
-        const float* src = P + static_cast<size_t>(rr) * ld + k;
-        if (vec && k + 3 < K) { const float4 q = *reinterpret_cast<const float4*>(src); x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w; }
-        else {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) if (k + c < K) x[c] = src[c];
-        }
-      }
-    } else {
-      const int k = k0 + f / 32, rr = r0 + (f % 32) * 4;
-      if (k < K) {
-        const float* src = P + static_cast<size_t>(k) * ld + rr;
-        if (vec && rr + 3 < R) { const float4 q = *reinterpret_cast<const float4*>(src); x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w; }
-        else {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) if (rr + c < R) x[c] = src[c];
-        }
-      }
-    }
-    t.v[u] = make_float4(x[0], x[1], x[2], x[3]);
-  }
-}
-__device__ __forceinline__ void stash_tile(const TileRegs& t, float (*S)[BM + 4], bool rows_major, int tid) {
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int f = tid + 256 * u;
-    if (rows_major) {
-      const int rr = f / 4, kq = (f % 4) * 4;
-      S[kq][rr] = t.v[u].x; S[kq + 1][rr] = t.v[u].y; S[kq + 2][rr] = t.v[u].z; S[kq + 3][rr] = t.v[u].w;
-    } else {
-      *reinterpret_cast<float4*>(&S[f / 32][(f % 32) * 4]) = t.v[u];
-    }
-  }
-}
-
-template <typename TOut>
-__global__ void __launch_bounds__(256) gemm_kernel(int ta, int tb, int M, int N, int K, float alpha, const float* A, int lda,
-                                                   long long strideA, const float* B, int ldb, long long strideB, TOut* C,
-                                                   int ldc, long long strideC, int k_total) {
-  __shared__ __align__(16) float As[2][BK][BM + 4];
-  __shared__ __align__(16) float Bs[2][BK][BN + 4];
-  A += strideA * blockIdx.z;
-  B += strideB * blockIdx.z;
-  C += strideC * blockIdx.z;
-  if (k_total > 0) K = max(0, min(K, k_total - static_cast<int>(blockIdx.z) * K));  // batch = slices of one long K
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const bool a_rows = !ta, b_rows = tb != 0;   // stored [rows, K]?
-  const bool vec_a = (lda & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
-  const bool vec_b = (ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
-  TOut acc[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = TOut(0);
-  TileRegs ra, rb;
-  if (K > 0) {
-    fetch_tile(ra, A, a_rows, vec_a, lda, m0, M, 0, K, tid);
-    fetch_tile(rb, B, b_rows, vec_b, ldb, n0, N, 0, K, tid);
-    stash_tile(ra, As[0], a_rows, tid);
-    stash_tile(rb, Bs[0], b_rows, tid);
-  }
-  __syncthreads();
-  for (int k0 = 0; k0 < K; k0 += BK) {
-    const int buf = (k0 / BK) & 1;
-    const bool more = k0 + BK < K;
-    if (more) {
-      fetch_tile(ra, A, a_rows, vec_a, lda, m0, M, k0 + BK, K, tid);
-      fetch_tile(rb, B, b_rows, vec_b, ldb, n0, N, k0 + BK, K, tid);
-    }
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]), a1 = *reinterpret_cast<const float4*>(&As[buf][kk][64 + ty * 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]), b1 = *reinterpret_cast<const float4*>(&Bs[buf][kk][64 + tx * 4]);
-      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] += static_cast<TOut>(a[i]) * static_cast<TOut>(b[j]);
-    }
-    if (more) {
-      stash_tile(ra, As[buf ^ 1], a_rows, tid);
-      stash_tile(rb, Bs[buf ^ 1], b_rows, tid);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int m = m0 + ty * 4 + (i & 3) + (i >> 2) * 64;
-    if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int n = n0 + tx * 4 + (j & 3) + (j >> 2) * 64;
-      if (n < N) C[static_cast<size_t>(m) * ldc + n] = static_cast<TOut>(alpha) * acc[i][j];
-    }
-  }
-}
-
-// G [r,r] (fp64) = Y^T Y for Y [m,r]: the long sum over m is cut into kGramSlices slices, one batch entry each
-// (16 tiles alone would leave most SMs idle), and the partial sums are added in a fixed order.
-constexpr int kGramSlices = kGramPartials;
-__global__ void sum_slices_kernel(const double* part, int count, int slices, double* out) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= count) return;
-  double s = 0.0;
-  for (int i = 0; i < slices; ++i) s += part[static_cast<size_t>(i) * count + e];
-  out[e] = s;
-}
-cudaError_t gram_f64(const float* Y, int m, int r, double* partial, double* G, cudaStream_t stream) {
-  const int ks = (m + kGramSlices - 1) / kGramSlices;
-  dim3 grid((r + BN - 1) / BN, (r + BM - 1) / BM, kGramSlices);
-  gemm_kernel<double><<<grid, 256, 0, stream>>>(1, 0, r, r, ks, 1.f, Y, r, static_cast<long long>(ks) * r, Y, r,
-                                                static_cast<long long>(ks) * r, partial, r, static_cast<long long>(r) * r, m);
-  sum_slices_kernel<<<(r * r + 255) / 256, 256, 0, stream>>>(partial, r * r, kGramSlices, G);
-  return cudaGetLastError();
-}
 
 // ------------------------------------------------------------------------------------------------ RoRoPE helpers
 // Position in the merged key of segment entry i of group G (i = p*g + j: frequency G*fold + p, head j), real part.
@@ -372,101 +236,5 @@ cudaError_t sym_eig(float* a, int batch, int m, float* eigvals, float* eigvecs, 
   jacobi_eigh_kernel<<<batch, kEigThreads, smem, stream>>>(a, m, eigvals, eigvecs, dev_status);
   return cudaGetLastError();
 }
-// ------------------------------------------------------------------------------------------------ orthonormalisation
-// Cholesky QR: G = Y^T Y = L L^T, Q = Y L^-T.
-// cholesky_kernel: blocked right-looking factorisation of the fp64 Gram matrix in place, one block.  Panels of 32
-// columns are factored in shared memory (all rows below the diagonal block with them); the trailing matrix then takes
-// one rank-32 update per panel, so that an element of G is read and written 16 times instead of 512.  L is also
-// written as fp32 for the solve.
-constexpr int kCholMax = 1024, kCholNb = 32;
-__global__ void __launch_bounds__(1024) cholesky_kernel(double* G, int r, float* L32, int32_t* dev_status) {
-  extern __shared__ double ps[];  // panel [r - kb][kCholNb + 1]
-  __shared__ int bad;
-  constexpr int ld = kCholNb + 1;
-  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-  if (tid == 0) bad = 0;
-  __syncthreads();
-  for (int kb = 0; kb < r; kb += kCholNb) {
-    const int nb = min(kCholNb, r - kb), rows = r - kb;
-    for (int e = tid; e < rows * nb; e += 1024) { const int i = e / nb, j = e % nb; ps[i * ld + j] = G[static_cast<size_t>(kb + i) * r + kb + j]; }
-    __syncthreads();
-    for (int k = 0; k < nb; ++k) {
-      if (tid == 0) {
-        double d = ps[k * ld + k];
-        if (!(d > 0.0)) { bad = 1; d = 1.0; }
-        ps[k * ld + k] = sqrt(d);
-      }
-      __syncthreads();
-      const double dk = ps[k * ld + k];
-      for (int i = k + 1 + tid; i < rows; i += 1024) ps[i * ld + k] /= dk;
-      __syncthreads();
-      for (int e = tid; e < (rows - k - 1) * (nb - k - 1); e += 1024) {
-        const int i = k + 1 + e / (nb - k - 1), j = k + 1 + e % (nb - k - 1);
-        ps[i * ld + j] -= ps[i * ld + k] * ps[j * ld + k];
-      }
-      __syncthreads();
-    }
-    for (int e = tid; e < rows * nb; e += 1024) {
-      const int i = e / nb, j = e % nb;
-      const double v = (kb + j <= kb + i) ? ps[i * ld + j] : 0.0;
-      G[static_cast<size_t>(kb + i) * r + kb + j] = v;
-      L32[static_cast<size_t>(kb + i) * r + kb + j] = static_cast<float>(v);
-    }
-    // trailing update: G[i][j] -= sum_k P[i][k] P[j][k] for i >= j >= kb + nb
-    for (int i = nb + ty; i < rows; i += 32) {
-      for (int j = nb + tx; j <= i; j += 32) {
-        double acc = 0.0;
-#pragma unroll 8
-        for (int k = 0; k < nb; ++k) acc += ps[i * ld + k] * ps[j * ld + k];
-        G[static_cast<size_t>(kb + i) * r + kb + j] -= acc;
-      }
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < r * r; e += 1024) { if (e % r > e / r) L32[e] = 0.f; }
-  if (tid == 0 && bad && dev_status != nullptr) atomicOr(dev_status, TRANSMLA_DEV_NUMERIC);
-}
-
-// Q[row] L^T = Y[row]: forward substitution along the row, one warp per row (the dot product of step j is split
-// over the lanes), 8 rows per block kept in shared memory.  Q may alias Y.
-__global__ void __launch_bounds__(256) trsm_rows_kernel(const float* Y, int m, int r, const float* L32, float* Q) {
-  extern __shared__ float qs[];  // [8][r]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = blockIdx.x * 8 + warp;
-  if (row >= m) return;
-  float* q = qs + warp * r;
-  for (int c = lane; c < r; c += 32) q[c] = Y[static_cast<size_t>(row) * r + c];
-  __syncwarp();
-  for (int j = 0; j < r; ++j) {
-    const float* lj = L32 + static_cast<size_t>(j) * r;
-    float s = 0.f;
-    for (int k = lane; k < j; k += 32) s = fmaf(q[k], lj[k], s);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) q[j] = (q[j] - s) / lj[j];
-    __syncwarp();
-  }
-  for (int c = lane; c < r; c += 32) Q[static_cast<size_t>(row) * r + c] = q[c];
-}
-
-cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G, float* L32, float* Q, int32_t* dev_status,
-                        cudaStream_t stream) {
-  if (r > kCholMax) return cudaErrorInvalidValue;
-  if (cudaError_t e = gram_f64(Y, m, r, partial, G, stream); e != cudaSuccess) return e;
-  const size_t chol_smem = static_cast<size_t>(r) * (kCholNb + 1) * sizeof(double);
-  if (cudaError_t e = cudaFuncSetAttribute(cholesky_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(chol_smem));
-      e != cudaSuccess)
-    return e;
-  cholesky_kernel<<<1, 1024, chol_smem, stream>>>(G, r, L32, dev_status);
-  const size_t smem = static_cast<size_t>(8) * r * sizeof(float);
-  if (smem > 48 * 1024) {
-    if (cudaError_t e = cudaFuncSetAttribute(trsm_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        e != cudaSuccess)
-      return e;
-  }
-  trsm_rows_kernel<<<(m + 7) / 8, 256, smem, stream>>>(Y, m, r, L32, Q);
-  return cudaGetLastError();
-}
-
 }  // namespace conv
 }  // namespace transmla

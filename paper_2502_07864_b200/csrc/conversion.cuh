@@ -11,7 +11,7 @@ namespace transmla {
 namespace conv {
 
 // C[M,N] = alpha * op(A) op(B); op(A) is A [M,K] (ta = 0, row stride lda) or the transpose of A [K,M] (ta = 1), likewise
-// op(B) from B [K,N] or B [N,K].  `batch` problems, strides in elements.  TOut = float or double (fp64 accumulation).
+// op(B) from B [K,N] or B [N,K].  `batch` problems, strides in elements.
 cudaError_t gemm_f32(int ta, int tb, int M, int N, int K, float alpha, const float* A, int lda, long long strideA,
                      const float* B, int ldb, long long strideB, float* C, int ldc, long long strideC, int batch,
                      cudaStream_t stream);
@@ -24,11 +24,11 @@ cudaError_t row_norm_ratio(const float* k_nope, int n, int mk, const float* v, i
                            cudaStream_t stream);
 cudaError_t balance_concat(const float* k_nope, int n, int mk, const float* v, int mv, const float* alpha, float* Z,
                            cudaStream_t stream);
-// Cholesky QR: Q [m,r] = Y L^-T with Y^T Y = L L^T (Gram matrix G [r,r] and its factor in fp64; L32 [r,r] the factor
-// in fp32 for the solve).  r <= 1024.  Q may alias Y.  Sets TRANSMLA_DEV_NUMERIC if the Gram matrix is not positive definite.
-constexpr int kGramPartials = 8;  // partial Gram matrices [r,r] fp64 that `partial` must hold
-cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G, float* L32, float* Q, int32_t* dev_status,
-                        cudaStream_t stream);
+// Cholesky QR: Q [m,r] = Y L^-T with Y^T Y = L L^T, r <= 1024.  Scratch: partial [gram_slices(r)][r,r], G [r,r] and X [r,r]
+// in fp64, X32 [r,r] (L^-T in fp32).  Q must not alias Y.  Sets TRANSMLA_DEV_NUMERIC if the Gram matrix is not positive definite.
+int gram_slices(int r);
+cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G, double* X, float* X32, float* Q,
+                        int32_t* dev_status, cudaStream_t stream);
 
 }  // namespace conv
 }  // namespace transmla

@@ -67,9 +67,27 @@ transmla_status_t transmla_conv_balance_concat(const float* k_nope, int n, int m
   return done(conv::balance_concat(k_nope, n, mk, v, mv, alpha, Z, static_cast<cudaStream_t>(stream)));
 }
 
+// Scratch of the subspace iteration: a second basis, and what the orthonormalisation needs.
+namespace {
+struct SubspaceLayout { size_t partial, g, x, x32, y, total; };
+SubspaceLayout subspace_layout(int m, int r) {
+  const size_t rr = static_cast<size_t>(r) * r;
+  SubspaceLayout l;
+  size_t off = 0;
+  auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 255) & ~size_t(255); return at; };
+  l.partial = take(conv::gram_slices(r) * rr * sizeof(double));
+  l.g = take(rr * sizeof(double));
+  l.x = take(rr * sizeof(double));
+  l.x32 = take(rr * sizeof(float));
+  l.y = take(static_cast<size_t>(m) * r * sizeof(float));
+  l.total = off;
+  return l;
+}
+}  // namespace
+
 size_t transmla_conv_subspace_scratch_bytes(int m, int r) {
   if (m < 1 || r < 1 || r > m || r > 1024) return 0;
-  return static_cast<size_t>(m) * r * sizeof(float) + static_cast<size_t>(r) * r * ((conv::kGramPartials + 1) * sizeof(double) + sizeof(float)) + 512;
+  return subspace_layout(m, r).total;
 }
 
 transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, int iters, float* Q, void* scratch,
@@ -79,21 +97,22 @@ transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, in
   if (!al16(Cmat) || !al16(Q) || (reinterpret_cast<uintptr_t>(scratch) & 255)) return TRANSMLA_ERR_ALIGN;
   if (scratch_bytes < transmla_conv_subspace_scratch_bytes(m, r)) return TRANSMLA_ERR_WORKSPACE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const SubspaceLayout l = subspace_layout(m, r);
   char* w = static_cast<char*>(scratch);
-  double* partial = reinterpret_cast<double*>(w);
-  double* G = partial + static_cast<size_t>(conv::kGramPartials) * r * r;
-  float* L32 = reinterpret_cast<float*>(G + static_cast<size_t>(r) * r);
-  float* Y = reinterpret_cast<float*>(
-      w + ((static_cast<size_t>(r) * r * ((conv::kGramPartials + 1) * sizeof(double) + sizeof(float)) + 255) & ~size_t(255)));
+  float* Y = reinterpret_cast<float*>(w + l.y);
   // Orthogonal iteration: Q <- orth(C Q).  One Cholesky QR per round keeps the columns independent; the basis is made
   // orthonormal to fp32 resolution by the two passes at the start and the extra pass at the end.
-  auto orth = [&](float* y, float* q) { return conv::cholesky_qr(y, m, r, partial, G, L32, q, dev_status, s) == cudaSuccess; };
-  if (!orth(Q, Q) || !orth(Q, Q)) return TRANSMLA_ERR_CUDA;
+  auto orth = [&](const float* from, float* to) {
+    return conv::cholesky_qr(from, m, r, reinterpret_cast<double*>(w + l.partial), reinterpret_cast<double*>(w + l.g),
+                             reinterpret_cast<double*>(w + l.x), reinterpret_cast<float*>(w + l.x32), to, dev_status, s) == cudaSuccess;
+  };
+  if (!orth(Q, Y) || !orth(Y, Q)) return TRANSMLA_ERR_CUDA;
   for (int it = 0; it < iters; ++it) {
     if (conv::gemm_f32(0, 0, m, r, m, 1.f, Cmat, m, 0, Q, r, 0, Y, r, 0, 1, s) != cudaSuccess) return TRANSMLA_ERR_CUDA;
     if (!orth(Y, Q)) return TRANSMLA_ERR_CUDA;
   }
-  return orth(Q, Q) ? TRANSMLA_OK : TRANSMLA_ERR_CUDA;
+  if (!orth(Q, Y)) return TRANSMLA_ERR_CUDA;
+  return done(cudaMemcpyAsync(Q, Y, static_cast<size_t>(m) * r * sizeof(float), cudaMemcpyDeviceToDevice, s));
 }
 
 }  // extern "C"

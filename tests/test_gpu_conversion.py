@@ -135,9 +135,10 @@ def test_alpha_and_balanced_concatenation():
     assert _rel(z[:, :mk], k.astype(np.float64) / float(alpha.item())) < 1e-6 and np.array_equal(z[:, mk:], v.astype(np.float64))
 
 
-@pytest.mark.parametrize('m,r', [(96, 24), (300, 64)])
+@pytest.mark.parametrize('m,r', [(96, 24), (300, 64), (333, 33), (40, 1), (200, 129), (1100, 1024)])
 def test_top_subspace_captures_what_the_leading_eigenvectors_capture(m, r):
     gu.ensure_built()
+    # (orders that do and do not fill the factor's blocks of 32, up to the largest)
     rng = np.random.default_rng(60 + m)
     basis = np.linalg.qr(rng.standard_normal((m, m)))[0]
     lam = np.concatenate([np.linspace(50.0, 10.0, r), np.linspace(4.0, 0.01, m - r)])   # a clear gap after r
