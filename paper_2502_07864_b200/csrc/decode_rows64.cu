@@ -52,9 +52,9 @@ constexpr int kOffRope = kStages * kStageBytes;       // rope part of a page, th
 constexpr int kOffQ = kOffRope + kRopeStages * kSubTileBytes;
 constexpr int kOffBar = kOffQ + 2 * kSubTileBytes;
 constexpr int kOffMisc = kOffBar + 256;
-// misc: pmax_s[2][8][32] bf16, meta[8][2] int4, tmem base, abort
-constexpr int kMiscBytes = 1024 + 32 * kMetaRing + 16;
-constexpr int kSmemBytes = kOffMisc + kMiscBytes + 1024;  // + slack for the 1024-byte alignment
+// misc: pmax_s[2][8][32] f32, meta[8][2] int4, tmem base, abort
+constexpr int kMiscBytes = 2048 + 32 * kMetaRing + 16;
+constexpr int kSmemBytes = kOffMisc + kMiscBytes;
 static_assert(kSmemBytes <= 232448 && kOffBar % 256 == 0, "shared memory budget");
 static_assert(kRows * 256 * 4 <= kStageBytes, "half of a segment's result passes through a stage");
 
@@ -68,12 +68,12 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
                      const int32_t* page_table, const int32_t* seqlens, const int32_t* cum, const int32_t* plan,
                      float* partial_o, float* partial_lse, int32_t* dev_status, int S, int H, int num_pages, int max_pages,
                      float scale_log2, int B, int dynamic, int32_t* next) {
-  extern __shared__ unsigned char smem_unaligned[];
-  const uint32_t raw = smem_u32(smem_unaligned);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  unsigned char* sm = smem_unaligned + (base - raw);
-  __nv_bfloat16* pmax_s = reinterpret_cast<__nv_bfloat16*>(sm + kOffMisc);  // [2][8][32]: per page parity, warp, lane
-  int4* meta = reinterpret_cast<int4*>(pmax_s + 512);                           // [kMetaRing][2]: what each ring item is; its segment
+  extern __shared__ __align__(1024) unsigned char smem_aligned[];  // no room to align by hand
+  unsigned char* sm = smem_aligned;
+  const uint32_t base = smem_u32(sm);
+  if ((base & 1023u) != 0) { set_status(dev_status, TRANSMLA_DEV_TIMEOUT); return; }
+  float* pmax_s = reinterpret_cast<float*>(sm + kOffMisc);  // [2][8][32]: per page parity, warp, lane
+  int4* meta = reinterpret_cast<int4*>(pmax_s + 512);           // [kMetaRing][2]: what each ring item is; its segment
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(meta + 2 * kMetaRing);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_s + 1);
   auto bar = [&](int i) -> uint32_t { return base + kOffBar + 8 * i; };
@@ -344,7 +344,7 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
 #pragma unroll
               for (int j = 0; j < 16; ++j) a = fmaxf(a, j < tok_end ? __uint_as_float(sq[j]) * scale_log2 : -INFINITY);
             }
-            pmax_s[(buf * 8 + sw) * 32 + lane] = __float2bfloat16_rn(a);
+            pmax_s[(buf * 8 + sw) * 32 + lane] = a;
           }
           // One barrier per page: the four parts of a row's maximum meet, and all 256 threads learn together whether the
           // CTA gave up.
@@ -352,12 +352,11 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
           asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 1, 256, q;\nselp.s32 %0, 1, 0, p;\n}"
                        : "=r"(aborted) : "r"(*abort_flag) : "memory");
           more = !last && pm.x == ITEM_PAGE && !aborted;
-          // The maximum is only the reference that keeps the exponents in range, so it may be rounded (to bf16, to spare
-          // shared memory) as long as the row's four threads use the same value.  Their warps: quadrants quad and quad ^ 2.
+          // The row's four threads: both warps of quadrants quad and quad ^ 2.
           float rowmax = -INFINITY;
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            rowmax = fmaxf(rowmax, __bfloat162float(pmax_s[(buf * 8 + (quad & 1) + 2 * i) * 32 + lane]));
+            rowmax = fmaxf(rowmax, pmax_s[(buf * 8 + (quad & 1) + 2 * i) * 32 + lane]);
           // Lazy rescale: the reference maximum only moves when some row's new maximum exceeds it by 2^8.  The warps that
           // share 32 rows see the same maxima and decide alike.
           bool rescale = false;
