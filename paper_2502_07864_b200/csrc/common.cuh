@@ -99,10 +99,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait.  Returns at once when the CTA has already given up.  For diagnosis, bit 8 + i of the status word
+// One look at a barrier, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bounded wait.  Returns at once when the phase is complete or the CTA has already given up.  For diagnosis, bit 8 + i of the status word
 // is set for every barrier slot i (position within its 256-byte block) on which a wait was still pending when the
 // CTA gave up; the first of them is the one whose limit expired.
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* dev_status) {
+  if (mbar_test(bar, parity)) return;
   if (*abort_flag) return;
   if (mbar_try_wait(bar, parity)) return;
   const long long t0 = clock64();
