@@ -54,9 +54,11 @@ def test_decompressed_store_matches_the_oracle_row_by_row():
             assert torch.all(store[pg].view(torch.int16) == 0x7fc1), 'a page nobody names was written'
 
 
-@pytest.mark.parametrize('S,seqlens', [(130, [130, 257, 64, 1000]), (1, [1, 64, 65]), (64, [64, 200]), (300, [320, 1100])])
+@pytest.mark.parametrize('S,seqlens', [(130, [130, 257, 64, 1000]), (1, [1, 64, 65]), (64, [64, 200]), (300, [320, 1100]),
+                                       (129, [129, 700]), (256, [256, 300]), (257, [100, 260, 130]), (385, [200, 390])])
 def test_prefill_all_outputs_small_head_count(S, seqlens):
     # every output and lse; S = 130 and 300 leave the last 128-row tile ragged, L = S is a pure prefill,
+    # (a CTA takes two tiles: 129 .. 257 and 385 leave one of them short, empty or without anything to see)
     # L = 64 < S = 130 leaves the first positions with nothing to see (zeros, lse = -inf)
     gu.ensure_built()
     shape = synth.MLAShape(H=2, dn=128, dR=64, dv=128, r=512, D=4096, S=S)
