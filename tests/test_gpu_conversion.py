@@ -97,6 +97,27 @@ def test_symmetric_eigendecomposition(m, batch):
             assert abs(cv.captured_energy(a[b], v[b][:, :keep]) - want[:keep].sum()) < 1e-4 * top
 
 
+@pytest.mark.parametrize('m,batch', [(3, 2), (66, 2), (97, 1), (127, 2)])
+def test_symmetric_eigendecomposition_of_odd_orders(m, batch):
+    # odd orders get an index of zeros, and odd numbers of pairs split the triangle of blocks unevenly
+    gu.ensure_built()
+    rng = np.random.default_rng(130 + m)
+    x = rng.standard_normal((batch, 3 * m + 2, m)) * (np.arange(1, m + 1) ** -0.7)
+    a = np.einsum('bni,bnj->bij', x, x).astype(np.float32)
+    w = torch.empty(batch, m, device='cuda'); v = torch.empty(batch, m, m, device='cuda')
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    binding.transmla_conv_sym_eig(_dev(a), w, v, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    w, v = _f64(w), _f64(v)
+    for b in range(batch):
+        want, _ = cv.sorted_eigh(a[b])
+        # bounds as for the even orders: at most 10 (m - 1) fp32 rotations of a column
+        assert np.abs(w[b] - want).max() < 2e-5 * want[0]
+        assert np.abs(v[b].T @ v[b] - np.eye(m)).max() < 1e-4
+        assert np.abs(a[b].astype(np.float64) @ v[b] - v[b] * w[b]).max() < 1e-4 * want[0]
+
+
 @pytest.mark.parametrize('fold', [1, 2])
 def test_rorope_apply_matches_the_oracle_and_keeps_the_rope_inner_product(fold):
     gu.ensure_built()
