@@ -4,7 +4,7 @@
 // cholesky_kernel   L^-T in fp64 by one cluster of CTAs, rounded to fp32
 // gemm_f32          Q = Y L^-T, with the products exact to fp32 (conversion_gemm.cu)
 // For a basis of 512 columns of length 8064: 0.24 + 1.86 + 0.74 ms in the form this one replaced (whole G, one block for the
-// factor, a triangular solve per row), now 0.13 + 0.36 + 0.03.
+// factor, a triangular solve per row), now 0.13 + 0.22 + 0.03.
 #include "conversion.cuh"
 #include "common.cuh"
 
@@ -125,8 +125,10 @@ __global__ void sum_slices_kernel(const double* part, int r, int slices, double*
 //              its share of the blocks behind column p
 //   each CTA   P(R,p) = B(R,p) L(p,p)^-T for its blocks R of column p: G rows below p, and X rows up to p
 // and one cluster barrier.  What bounds it is the chain of r square roots and the updates between them, about 300 cycles
-// each.  Rows and columns beyond r behave as an identity.
-constexpr int NB = 32, kCluster = 8, kCholThreads = 256, kPitch = NB + 1, kBlock = NB * kPitch;
+// each, with the fp64 units beside it: a block's product takes one SM's units 1000 cycles, and a panel has about 100 of them.
+// At r = 512: 359 us by 8 CTAs with the own blocks one a warp, 221 us by 16 (the cluster's size limit with the opt-in), four
+// rows of a block a warp and whole lines moved.  Rows and columns beyond r behave as an identity.
+constexpr int NB = 32, kCluster = 16, kCholThreads = 256, kPitch = NB + 1, kBlock = NB * kPitch;
 constexpr int kMaxBlocks = 1024 / NB, kMaxOwn = kMaxBlocks / kCluster;
 // doubles: D, W, P(p,p-1), col[2][32], the CTA's blocks of column p, two operands for each of warps 1-7
 constexpr int kCholSmem = (3 * kBlock + 2 * NB + kMaxOwn * kBlock + 14 * kBlock) * 8;
@@ -136,6 +138,8 @@ struct CholView {
   double* G;   // [r, r], lower
   double* X;   // [r, r], upper
   int r, n;    // n block rows of each
+  bool even;   // pairs of elements are aligned
+  __device__ __forceinline__ bool next(int c, int j) const { return c * NB + j + 1 < r; }
   // element (i, j) of block (R, c): R < n rows of G, otherwise rows of X
   __device__ __forceinline__ double* at(int R, int c, int i, int j, bool& in) const {
     const int row = (R < n ? R : R - n) * NB + i, col = c * NB + j;
@@ -155,36 +159,55 @@ __device__ __forceinline__ void load_block(const CholView& v, int R, int c, doub
 #pragma unroll
   for (int i = 0; i < NB; ++i) dst[i * kPitch + lane] = x[i];
 }
-// The lane's elements of block (R, c), at the places of its elements of a product: rows l/4 + 8a, columns l%4 + 4b.
-__device__ __forceinline__ void load_elements(const CholView& v, int R, int c, bool fresh, double (&x)[4][8], int lane) {
+// A lane's elements of a product: rows l/8 + 4i for i from `from`, columns 2 (l%8) + {0, 1} + 16h: eight lanes move one line.
+template <int kRows>
+__device__ __forceinline__ void load_elements(const CholView& v, int R, int c, int from, double (&x)[kRows][4], int lane) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < kRows; ++i) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int h = 0; h < 2; ++h) {
       bool in;
-      const double* p = v.at(R, c, (lane >> 2) + 8 * i, (lane & 3) + 4 * j, in);
-      x[i][j] = in && !fresh ? __ldcg(p) : 0.0;
+      const double* p = v.at(R, c, (lane >> 3) + 4 * (from + i), 2 * (lane & 7) + 16 * h, in);
+      double2 e = make_double2(0.0, 0.0);
+      if (in && v.even) e = __ldcg(reinterpret_cast<const double2*>(p));  // an even order has both or neither
+      else if (in) { e.x = __ldcg(p); if (v.next(c, 2 * (lane & 7) + 16 * h)) e.y = __ldcg(p + 1); }
+      x[i][2 * h] = e.x;
+      x[i][2 * h + 1] = e.y;
     }
   }
 }
-// acc[a][b] -= sum_k A[row][k] B[col][k] for the lane's rows l/4 + 8a and columns l%4 + 4b
-__device__ __forceinline__ void warp_product(double (&acc)[4][8], const double* A, const double* B, int lane) {
-  const double* ar = A + (lane >> 2) * kPitch;
-  const double* br = B + (lane & 3) * kPitch;
-#pragma unroll 4
-  for (int k = 0; k < NB; ++k) {
-    double a[4], b[8];
+template <int kRows>
+__device__ __forceinline__ void store_elements(const CholView& v, int R, int c, const double (&x)[kRows][4], int lane) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = ar[8 * i * kPitch + k];
+  for (int i = 0; i < kRows; ++i) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) b[j] = br[4 * j * kPitch + k];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc[i][j] = fma(-a[i], b[j], acc[i][j]);
+    for (int h = 0; h < 2; ++h) {
+      bool in;
+      double* p = v.at(R, c, (lane >> 3) + 4 * i, 2 * (lane & 7) + 16 * h, in);
+      if (in && v.even) __stcg(reinterpret_cast<double2*>(p), make_double2(x[i][2 * h], x[i][2 * h + 1]));
+      else if (in) { __stcg(p, x[i][2 * h]); if (v.next(c, 2 * (lane & 7) + 16 * h)) __stcg(p + 1, x[i][2 * h + 1]); }
+    }
   }
 }
-__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kCholThreads, 1)
+// acc -= A B^T at the lane's elements; A's first row is that of acc's
+template <int kRows>
+__device__ __forceinline__ void warp_product(double (&acc)[kRows][4], const double* A, const double* B, int lane) {
+  const double* ar = A + (lane >> 3) * kPitch;
+  const double* br = B + 2 * (lane & 7) * kPitch;
+#pragma unroll 4
+  for (int k = 0; k < NB; ++k) {
+    double a[kRows], b[4];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) a[i] = ar[4 * i * kPitch + k];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) b[j] = br[((j & 1) + 16 * (j >> 1)) * kPitch + k];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = fma(-a[i], b[j], acc[i][j]);
+  }
+}
+__global__ void __launch_bounds__(kCholThreads, 1)
 cholesky_kernel(double* G, double* X, int r, float* X32, int32_t* dev_status) {
   extern __shared__ __align__(16) double cs[];
   double* D = cs;                     // the panel's diagonal block
@@ -193,8 +216,8 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int32_t* dev_status) {
   double* col = Pp + kBlock;          // [2][32]
   double* Bs = col + 2 * NB;          // [kMaxOwn] blocks of column p
   double* ops = Bs + kMaxOwn * kBlock;  // [7][2]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = blockIdx.x;
-  const CholView v = {G, X, r, (r + NB - 1) / NB};
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = blockIdx.x, ctas = gridDim.x;
+  const CholView v = {G, X, r, (r + NB - 1) / NB, (r & 1) == 0};
   const int n = v.n;
   double* opA = ops + (warp - 1) * 2 * kBlock;  // warps 1-7
   double* opB = opA + kBlock;
@@ -202,22 +225,42 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int32_t* dev_status) {
 
   for (int p = 0; p < n; ++p) {
     // ---- D, by all warps: 4 elements a thread
-    if (p > 0) {
-      if (warp == 0) load_block(v, p, p - 1, Pp, lane);
-      __syncthreads();
-    }
-    for (int e = tid; e < NB * NB; e += kCholThreads) {
-      const int i = e >> 5, j = e & 31, hi = max(i, j), lo = min(i, j);
-      bool in;
-      const double* g = v.at(p, p, hi, lo, in);
-      double d = in ? __ldcg(g) : (i == j ? 1.0 : 0.0);
+    const int lo = tid & 15, up = tid >> 4;  // rows and columns lo, lo + 16, up, up + 16 of a block
+    {
+      double d[2][2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int a = up + 16 * i, b = lo + 16 * j;
+          bool in;
+          const double* g = v.at(p, p, max(a, b), min(a, b), in);
+          d[i][j] = in ? __ldcg(g) : (a == b ? 1.0 : 0.0);
+        }
       if (p > 0) {
-        double s = 0.0;
+        double x[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          bool in;
+          const double* g = v.at(p, p - 1, warp * 4 + i, lane, in);
+          x[i] = in ? __ldcg(g) : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) Pp[(warp * 4 + i) * kPitch + lane] = x[i];
+        __syncthreads();
+        const double* a = Pp + up * kPitch;
+        const double* b = Pp + lo * kPitch;
 #pragma unroll 8
-        for (int k = 0; k < NB; ++k) s = fma(Pp[i * kPitch + k], Pp[j * kPitch + k], s);
-        d -= s;
+        for (int k = 0; k < NB; ++k) {
+          const double a0 = a[k], a1 = a[16 * kPitch + k], b0 = b[k], b1 = b[16 * kPitch + k];
+          d[0][0] = fma(-a0, b0, d[0][0]); d[0][1] = fma(-a0, b1, d[0][1]);
+          d[1][0] = fma(-a1, b0, d[1][0]); d[1][1] = fma(-a1, b1, d[1][1]);
+        }
       }
-      D[i * kPitch + j] = d;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) D[(up + 16 * i) * kPitch + lo + 16 * j] = d[i][j];
     }
     __syncthreads();
     if (warp == 0) {
@@ -225,12 +268,14 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int32_t* dev_status) {
       double a[NB], x[NB];
 #pragma unroll
       for (int j = 0; j < NB; ++j) { a[j] = D[lane * kPitch + j]; x[j] = j == lane ? 1.0 : 0.0; }
+      double pivot = a[0];
 #pragma unroll
       for (int k = 0; k < NB; ++k) {
-        double d = __shfl_sync(0xffffffffu, a[k], k);
+        double d = __shfl_sync(0xffffffffu, pivot, k);
         if (!(d > 0.0)) { bad = true; d = 1.0; }
         const double inv = rsqrt(d);
         const double l = a[k] * inv;
+        if (k + 1 < NB) pivot = fma(-l, l, a[k + 1]);  // in lane k + 1: the next step need not wait for the exchange
         x[k] *= inv;
         col[(k & 1) * NB + lane] = l;
         __syncwarp();
@@ -244,53 +289,52 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int32_t* dev_status) {
 #pragma unroll
       for (int j = 0; j < NB; ++j) W[lane * kPitch + j] = x[j];
     } else {
-      // ---- this CTA's blocks of column p: list entry e is G row p + 1 + e, then X rows 0 .. p
+      // ---- this CTA's blocks of column p, four rows a warp: list entry e is G row p + 1 + e, then X rows 0 .. p
       int own = 0;
-      for (int e = cta; e < n; e += kCluster, ++own) {
-        if (own % 7 != warp - 1) continue;
+      for (int e = cta; e < n; e += ctas, ++own) {
         const int R = e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p), q = R - n;  // (q < 0 for G rows)
         double* B = Bs + own * kBlock;
-        double acc[4][8];
-        // nothing stored yet in X rows p - 1 (zeros) and p (the identity's block)
-        load_elements(v, R, p, R >= n && q >= p - 1, acc, lane);
-        if (q == p) {
+        for (int slab = warp - 1; slab < NB / 4; slab += 7) {
+          double acc[1][4] = {{0.0, 0.0, 0.0, 0.0}};
+          const int row = 4 * slab + (lane >> 3);
+          if (q == p) {  // nothing stored yet in X rows p - 1 (zeros) and p (the identity's block)
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < 4; ++j) acc[0][j] = row == 2 * (lane & 7) + (j & 1) + 16 * (j >> 1) ? 1.0 : 0.0;
+          } else {
+            if (R < n || q < p - 1) load_elements(v, R, p, slab, acc, lane);
+            if (p > 0) {
+              double x[4];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[i][j] = (lane >> 2) + 8 * i == (lane & 3) + 4 * j ? 1.0 : 0.0;
-        } else if (p > 0) {
-          load_block(v, R, p - 1, opA, lane);
-          __syncwarp();
-          warp_product(acc, opA, Pp, lane);
+              for (int i = 0; i < 4; ++i) {
+                bool in;
+                const double* g = v.at(R, p - 1, 4 * slab + i, lane, in);
+                x[i] = in ? __ldcg(g) : 0.0;
+              }
+#pragma unroll
+              for (int i = 0; i < 4; ++i) opA[i * kPitch + lane] = x[i];
+              __syncwarp();
+              warp_product(acc, opA, Pp, lane);
+              __syncwarp();
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) B[row * kPitch + 2 * (lane & 7) + (j & 1) + 16 * (j >> 1)] = acc[0][j];
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) B[((lane >> 2) + 8 * i) * kPitch + (lane & 3) + 4 * j] = acc[i][j];
-        __syncwarp();
       }
       // ---- panel p - 1 on the blocks behind column p: column j takes G rows j .. n-1 and X rows 0 .. p-1
       if (p > 0) {
         int t = cta * 7 + warp - 1;
         for (int j = p + 1; j < n; ++j) {
           const int count = n - j + p;
-          for (; t < count; t += kCluster * 7) {
+          for (; t < count; t += ctas * 7) {
             const int R = t < n - j ? j + t : n + t - (n - j);
-            double acc[4][8];
-            load_elements(v, R, j, R >= n && R - n == p - 1, acc, lane);
+            double acc[8][4] = {};
+            if (R != n + p - 1) load_elements(v, R, j, 0, acc, lane);
             load_block(v, R, p - 1, opA, lane);
             load_block(v, j, p - 1, opB, lane);
             __syncwarp();
             warp_product(acc, opA, opB, lane);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-#pragma unroll
-              for (int jj = 0; jj < 8; ++jj) {
-                bool in;
-                double* g = v.at(R, j, (lane >> 2) + 8 * i, (lane & 3) + 4 * jj, in);
-                if (in) __stcg(g, acc[i][jj]);
-              }
-            }
+            store_elements(v, R, j, acc, lane);
             __syncwarp();
           }
           t -= count;
@@ -298,26 +342,34 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int32_t* dev_status) {
       }
     }
     __syncthreads();
-    // ---- P(R,p) = B W: one warp a block, the product with W's columns as rows of its transpose
+    // ---- P(R,p) = B W.  W is an upper triangle: a warp's four columns need only the rows of W up to the last of them
     {
       int own = 0;
-      for (int e = cta; e < n; e += kCluster, ++own) {
+      for (int e = cta; e < n; e += ctas, ++own) {
         const int R = e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p);
         const double* B = Bs + own * kBlock;
-        for (int o = tid; o < NB * NB; o += kCholThreads) {
-          const int row = o >> 5, c = o & 31;
-          double s = 0.0;
-#pragma unroll 8
-          for (int k = 0; k < NB; ++k) s = fma(B[row * kPitch + k], W[k * kPitch + c], s);
-          bool in;
-          double* g = v.at(R, p, row, c, in);
-          if (in) __stcg(g, s);
+        const double* b = B + lo * kPitch;
+        const double* w = W + 2 * up;
+        double o[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll 4
+        for (int k = 0; k < 4 * warp + 4; ++k) {
+          const double b0 = b[k], b1 = b[16 * kPitch + k], w0 = w[k * kPitch], w1 = w[k * kPitch + 1];
+          o[0][0] = fma(b0, w0, o[0][0]); o[0][1] = fma(b0, w1, o[0][1]);
+          o[1][0] = fma(b1, w0, o[1][0]); o[1][1] = fma(b1, w1, o[1][1]);
         }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            bool in;
+            double* g = v.at(R, p, lo + 16 * i, 2 * up + j, in);
+            if (in) __stcg(g, o[i][j]);
+          }
       }
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
-  for (int e = cta * kCholThreads + tid; e < r * r; e += kCluster * kCholThreads) {
+  for (int e = cta * kCholThreads + tid; e < r * r; e += ctas * kCholThreads) {
     const int row = e / r, c = e % r;
     X32[e] = c < row ? 0.f : static_cast<float>(__ldcg(X + e));
   }
@@ -338,12 +390,25 @@ cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G
   static PerDeviceFlag gram_set, chol_set;
   if (cudaError_t e = ensure_dynamic_smem(gram_kernel, kGramSmem, gram_set); e != cudaSuccess) return e;
   if (cudaError_t e = ensure_dynamic_smem(cholesky_kernel, kCholSmem, chol_set); e != cudaSuccess) return e;
+  if (cudaError_t e = cudaFuncSetAttribute(cholesky_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); e != cudaSuccess) return e;
   const int t = (r + GT - 1) / GT, slices = gram_slices(r);
   const int ks = ((m + slices - 1) / slices + GK - 1) / GK * GK;
   gram_kernel<<<dim3(t * (t + 1) / 2, slices), 256, kGramSmem, stream>>>(Y, m, r, ks, partial);
   sum_slices_kernel<<<dim3((r + 127) / 128, r), 128, 0, stream>>>(partial, r, slices, G);
-  cholesky_kernel<<<kCluster, kCholThreads, kCholSmem, stream>>>(G, X, r, X32, dev_status);
-  if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) return e;
+  int ctas = 1;  // one cluster, of no more CTAs than a panel has blocks for
+  while (ctas < kCluster && ctas < (r + NB - 1) / NB) ctas *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kCholThreads);
+  cfg.dynamicSmemBytes = kCholSmem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaError_t e = cudaLaunchKernelEx(&cfg, cholesky_kernel, G, X, r, X32, dev_status); e != cudaSuccess) return e;
   return gemm_f32(0, 0, m, r, r, 1.f, Y, r, 0, X32, r, 0, Q, r, 0, 1, stream);
 }
 
