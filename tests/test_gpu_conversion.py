@@ -139,6 +139,18 @@ def test_rorope_apply_matches_the_oracle_and_keeps_the_rope_inner_product(fold):
             assert abs(got_ip - want_ip) < 1e-4 * max(1.0, abs(want_ip))
 
 
+@pytest.mark.parametrize('g,d,fold,C', [(32, 128, 4, 192), (3, 16, 4, 68), (5, 4, 2, 65), (1, 2, 1, 3)])
+def test_rorope_apply_at_the_edges_of_its_tiles(g, d, fold, C):
+    # the largest order, orders off the 8 values of a thread, columns off the tile of 64 and off the 4 of a thread
+    gu.ensure_built()
+    rng = np.random.default_rng(41)
+    X = rng.standard_normal((g * d, C)).astype(np.float32)
+    U = rng.standard_normal((d // 2 // fold, g * fold, g * fold)).astype(np.float32)
+    Y = torch.full((g * d, C), float('nan'), device='cuda')
+    binding.transmla_conv_rorope_apply(_dev(X), _dev(U), g, d, fold, Y)
+    assert _rel(_f64(Y), cv.rorope_apply(X, U, g, d, fold)) < 1e-6     # at most 128 fp32 roundings that average out
+
+
 def test_alpha_and_balanced_concatenation():
     gu.ensure_built()
     rng = np.random.default_rng(50)
