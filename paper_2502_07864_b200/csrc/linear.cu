@@ -1,8 +1,6 @@
 // Linear maps either side of the attention (Eq. 8 right column: queries; Eq. 9 last line: W_O), as skinny GEMMs
 // y[M, N] = x[M, K] w[N, K]^T with M = the step's new tokens.  They stream their weights once; a block owns 8
 // output features (see skinny_gemm.cuh).  One launch may hold two jobs (q^C and q^R share their input).
-#include <algorithm>
-
 #include "append_block.cuh"
 #include "common.cuh"
 #include "linear_args.cuh"
@@ -81,15 +79,6 @@ size_t transmla_layer_scratch_bytes(const transmla_params_t* p, int32_t q_lora_r
   off = round_up(off + M * H * p->qk_nope_dim * 2, kAlign);
   off = round_up(off + M * H * p->qk_rope_dim * 2 + 16, kAlign);
   off = round_up(off + M * H * p->v_dim * 2, kAlign);
-  // tcgen05 linear maps: partial results of the K slices (largest of the three launches) and arrival counters
-  const int Mi = static_cast<int>(M), D = p->hidden_dim, Kq = q_lora_rank ? q_lora_rank : D;
-  const int tiles_dq = q_lora_rank / 128, tiles_q = static_cast<int>(H) * (p->qk_nope_dim + p->qk_rope_dim) / 128, tiles_o = D / 128;
-  size_t partial = 0;
-  if (tiles_dq > 0) partial = std::max(partial, linear_sm100_partial_bytes(tiles_dq, D, Mi));
-  if (tiles_q > 0) partial = std::max(partial, linear_sm100_partial_bytes(tiles_q, Kq, Mi));
-  if (tiles_o > 0) partial = std::max(partial, linear_sm100_partial_bytes(tiles_o, static_cast<int>(H) * p->v_dim, Mi));
-  off = round_up(off + partial, kAlign);
-  off = round_up(off + linear_sm100_counter_bytes(std::max(tiles_dq, std::max(tiles_q, tiles_o)) + 1, Mi), kAlign);
   return off;
 }
 
@@ -119,26 +108,16 @@ transmla_status_t transmla_layer_decode_step(const transmla_params_t* p, const t
   auto* q_pe = reinterpret_cast<__nv_bfloat16*>(base + off);    off = round_up(off + static_cast<size_t>(M) * H * p->qk_rope_dim * 2 + 16, kAlign);
   auto* attn = reinterpret_cast<__nv_bfloat16*>(base + off);                          off = round_up(off + static_cast<size_t>(M) * H * p->v_dim * 2, kAlign);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // tcgen05 linear maps (feature counts that are multiples of 128): scratch for the K slices and their counters
-  const int tiles_dq = rq / 128, tiles_q = H * (p->qk_nope_dim + p->qk_rope_dim) / 128, tiles_o = D / 128;
-  size_t partial_bytes = 0;
-  if (tiles_dq > 0) partial_bytes = std::max(partial_bytes, linear_sm100_partial_bytes(tiles_dq, D, M));
-  if (tiles_q > 0) partial_bytes = std::max(partial_bytes, linear_sm100_partial_bytes(tiles_q, Kq, M));
-  if (tiles_o > 0) partial_bytes = std::max(partial_bytes, linear_sm100_partial_bytes(tiles_o, Ko, M));
-  auto* lin_partial = reinterpret_cast<float*>(base + off);                          off = round_up(off + partial_bytes, kAlign);
-  auto* lin_counters = reinterpret_cast<int32_t*>(base + off);
-  const size_t counter_bytes = linear_sm100_counter_bytes(std::max(tiles_dq, std::max(tiles_q, tiles_o)) + 1, M);
-  bool counters_cleared = false;
-  // One linear launch: the tcgen05 kernel where the shapes allow it, the mma.sync tiles otherwise.  The counters
-  // of the tcgen05 kernel must be zero before its first launch of this call; every launch leaves them at zero.
+  // One linear launch: the tcgen05 kernel where the shapes allow it, the mma.sync tiles otherwise.  These also where a few
+  // tokens meet three short maps in a row: their blocks start beside those of the kernel before and have their weights on the
+  // way to L2 by then, which is all that counts there.  Full step, mma.sync / tcgen05: 33 M weights (LLaMA-2-7B, rank 1536)
+  // 49.0 / 50.6 us at 1 token, 51.7 / 52.8 at 8, 58.4 / 54.2 at 16; 99 M (Qwen2.5-72B) 102 / 75 at 3; full rank, two longer
+  // maps, 42 M: 49.3 / 47.8 at 1, 53.0 / 50.0 at 8.
+  const size_t map_weights = static_cast<size_t>(rq) * D + static_cast<size_t>(H) * (p->qk_nope_dim + p->qk_rope_dim) * Kq + static_cast<size_t>(D) * Ko;
+  const bool short_maps = low_rank && M <= 8 && map_weights <= (size_t(40) << 20);
+  auto on_sm100 = [&](const LinearArgs& la) { return !short_maps && linear_sm100_supported(la); };
   auto run_linear = [&](const LinearArgs& la) -> cudaError_t {
-    if (!linear_sm100_supported(la)) return launch_linear(la, dev_status, s);
-    if (!counters_cleared) {
-      cudaError_t e = cudaMemsetAsync(lin_counters, 0, counter_bytes, s);
-      if (e != cudaSuccess) return e;
-      counters_cleared = true;
-    }
-    return launch_linear_sm100(la, lin_partial, lin_counters, dev_status, s);
+    return on_sm100(la) ? launch_linear_sm100(la, dev_status, s) : launch_linear(la, dev_status, s);
   };
   const auto* xin = static_cast<const __nv_bfloat16*>(x);
 
@@ -148,9 +127,8 @@ transmla_status_t transmla_layer_decode_step(const transmla_params_t* p, const t
 
   LinearArgs a = {};
   a.M = M; a.S = p->q_len; a.t_splits = token_splits(M); a.pos_base = seqlens; a.pos_shift = -p->q_len; a.theta = p->rope_theta;
-  // The append (Eq. 7 left) is one more linear map of x: where the layer's first launch runs on the mma.sync tiles
-  // its blocks ride in that launch, off the chain queries -> absorb -> attention; otherwise it stays in the
-  // attention step's prologue.
+  // The append (Eq. 7 left) is one more linear map of x: it rides in the layer's first launch, off the chain queries ->
+  // absorb -> attention, or stays in the attention step's prologue where that launch cannot take it.
   AppendJob ap = {};
   ap.x = xin; ap.w = static_cast<const __nv_bfloat16*>(w->w_dkv_kr); ap.page_table = page_table;
   ap.cache = static_cast<__nv_bfloat16*>(cache);
@@ -159,7 +137,7 @@ transmla_status_t transmla_layer_decode_step(const transmla_params_t* p, const t
   ap.blocks = (ap.r + ap.dR) / (ap.wide ? 32 : 8) * ap.t_splits;
   bool appended = false;
   auto with_append = [&](LinearArgs& la) {  // the first launch takes the append along if it can
-    if (!appended && !linear_sm100_supported(la)) { la.append = ap; appended = true; }
+    if (!on_sm100(la) || linear_sm100_takes_append(ap, la)) { la.append = ap; appended = true; }
   };
   if (low_rank) {  // c^Q = W_DQ x
     a.n_jobs = 1;

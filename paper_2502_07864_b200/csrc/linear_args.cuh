@@ -31,10 +31,7 @@ struct LinearArgs {
 
 // tcgen05 implementation (linear_sm100.cu): needs N a multiple of 128 and K a multiple of 64 in every job.
 bool linear_sm100_supported(const LinearArgs& a);
-int linear_sm100_splits(int n_tiles, int K);
-size_t linear_sm100_partial_bytes(int n_tiles, int K, int M);   // scratch for the K slices' partial results
-size_t linear_sm100_counter_bytes(int n_tiles, int M);          // per-tile arrival counters (zero before a launch)
-cudaError_t launch_linear_sm100(const LinearArgs& a, float* partial, int32_t* counters, int32_t* dev_status,
-                                cudaStream_t stream);
+bool linear_sm100_takes_append(const AppendJob& ap, const LinearArgs& a);
+cudaError_t launch_linear_sm100(const LinearArgs& a, int32_t* dev_status, cudaStream_t stream);
 
 }  // namespace transmla

@@ -12,13 +12,20 @@
 // The slices of a tile are the CTAs of one thread-block cluster: each leaves its fp32 partial in its own shared
 // memory (the ring is free by then), and after a cluster barrier every CTA adds the slices of its share of the
 // tokens in slice order, reading the others' shared memory directly, applies RoPE where asked and writes bf16 (no
-// float atomics: reruns give the same bits).  If the clusters do not all fit on the device at once, or there are
-// more than 8 slices, the partials go through a scratch buffer instead and the CTA that arrives last at the tile's
-// counter adds them.
+// float atomics: reruns give the same bits).
+// What bounds it: the 31 bytes a cycle that an SM gets from L2, 585 cycles a stage at 16 tokens, and what stands at either
+// end of the stream.  The ring takes the whole shared memory and is filled with weights before the CTA waits for the kernel
+// before it (half the ring beside that kernel's CTAs, with the rest requested for L2, was 6 to 30 us slower a layer: the
+// requests go through the same path as the loads).  The code behind the stream is small: unrolled over the tokens, with its
+// sine at 16 places, its fetch from memory took 9 to 12 thousand cycles of a launch's 28 to 35 thousand, now 4.
+// The layer step of LLaMA-2-7B, 16 x 8192 tokens: 86 -> 71 us with the append among the tiles (75 without), 128 short
+// sequences 130 -> 102; Qwen2.5-72B, 40 sequences: 244 -> 144 (both against the mma.sync tiles below 48 tokens and the
+// unrolled epilogue).
 //
 // Warps: 0 TMA producer, 1 MMA issuer, 2-5 epilogue (each owns the 32 tensor-memory lanes of its quadrant).
 #include "common.cuh"
 #include "linear_args.cuh"
+#include "skinny_gemm.cuh"
 #include "sm100_ptx.cuh"
 
 namespace transmla {
@@ -29,7 +36,7 @@ constexpr int kLinBK = 64;                       // contracted elements per ring
 constexpr int kLinMaxT = 256;                    // tokens per CTA at most (MMA N)
 constexpr int kLinMaxStages = 12;
 constexpr int kLinWBytes = kLinBM * 128;         // 16384
-constexpr int kLinRingBytes = 196608;            // stages of (weight tile + activation tile); as many as fit, at most 12
+constexpr int kLinRingBytes = 221184;            // stages of (weight tile + activation tile); as many as fit, at most 12
 constexpr int kLinThreads = 192;
 constexpr int kLinSmemBytes = kLinRingBytes + 256 + 1024;
 enum { LB_FULL = 0, LB_EMPTY = kLinMaxStages, LB_DONE = 2 * kLinMaxStages };
@@ -37,85 +44,56 @@ enum { LB_FULL = 0, LB_EMPTY = kLinMaxStages, LB_DONE = 2 * kLinMaxStages };
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// fp32 at the same shared-memory offset in the CTA of rank `rank` of this cluster
-__device__ __forceinline__ float ld_cluster_f32(const float* local, uint32_t rank) {
+// four floats at the same shared-memory offset in the CTA of rank `rank` of this cluster
+__device__ __forceinline__ float4 ld_cluster_f32x4(const float* local, uint32_t rank) {
   uint32_t remote;
-  float v;
+  float4 v;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)), "r"(rank));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(remote) : "memory");
   return v;
 }
-
 struct LinSm100Params {
-  __nv_bfloat16* out[2];   // [M, N_j]
-  int N[2];                // output features of job j (multiples of 128)
+  __nv_bfloat16* out[3];   // [M, N_j]; job 2 is the append (Eq. 7 left): the cache
+  int N[3];                // output features of job j (multiples of 128, but for the append's r + dR)
   int rope_d[2];           // > 0: consecutive blocks of rope_d features are rotated (Eq. 1, d := rope_d)
-  int n_jobs, M, S, K, splits;
+  int tiles01[2];          // tiles of jobs 0 and 1; those behind belong to the append
+  int M, S, K, splits;
+  const int32_t* page_table;
+  int r, dR, num_pages, max_pages;
   int stages;              // ring depth: as many (weight tile + activation box) stages as fit
-  int cluster;             // 1: the slices of a tile are the CTAs of one cluster and meet through distributed shared memory
-  int x_box_rows;          // rows of the activation box (tokens of a full block, padded to 16); also the row stride of `partial`
+  int x_box_rows;          // rows of the activation box (tokens of a full block, padded to 16)
   const int32_t* pos_base; // position of token (b, s) = pos_base[b] + pos_shift + s (rotated jobs only)
   int pos_shift;
   float theta;
-  float* partial;          // [token block][tile][split][T][128] fp32 (splits > 1)
-  int32_t* counters;       // [token block][tile], zero before the launch; left at zero
 };
 
-// RoPE of Eq. 1 in the epilogue, rounding and the store.  The even lane of a pair holds the real part, the odd one
-// the imaginary part.  Angle = position x theta^(-2l/d), reduced to [-pi, pi] before sine and cosine.  The
+// RoPE of Eq. 1 in the epilogue.  Angle = position x theta^(-2l/d), reduced to [-pi, pi] before sine and cosine.  The
 // reduction runs in fp32 with the frequency as a (hi, lo) pair and 2*pi as three constants whose products with the
 // turn count are formed exactly inside the fused multiply-adds (positions up to 2^20 keep an angle error below
-// 1e-5 rad); the double-precision units of this chip are too slow to do it for every (token, pair).  Tokens are
-// taken two at a time: the even lane works out the angle of the first, the odd lane that of the second, and they
-// swap.
-struct LinRope {
-  float f_hi = 0.f, f_lo = 0.f;
-  int rope_d, S, pos_shift;
-  const int32_t* pos_base;
-  __device__ LinRope(const LinSm100Params& p, int feature, int rope_d_)
-      : rope_d(rope_d_), S(p.S), pos_shift(p.pos_shift), pos_base(p.pos_base) {
-    if (rope_d > 0) {
-      const double inv_freq = exp2(-2.0 * ((feature % rope_d) >> 1) / rope_d * log2(static_cast<double>(p.theta)));
-      f_hi = static_cast<float>(inv_freq);
-      f_lo = static_cast<float>(inv_freq - static_cast<double>(f_hi));
-    }
-  }
-  __device__ void sincos_at(int tok, float& sn, float& cs) const {
-    const float pos = static_cast<float>(pos_base[tok / S] + pos_shift + tok % S);
-    const float a = pos * f_hi;
-    const float e = fmaf(pos, f_hi, -a) + pos * f_lo;          // what the rounded product left out
-    const float k = rintf(a * 0.15915494309189535f);          // whole turns
-    float r = fmaf(-k, 6.28125f, a);                           // 2*pi = 6.28125 + 0.001934051513671875 + 1.2556659146e-6
-    r = fmaf(-k, 0.001934051513671875f, r);
-    r = fmaf(-k, 1.2556659146e-6f, r) + e;
-    sincosf(r, &sn, &cs);
-  }
-  // values of `feature` for tokens t0 + t and t0 + t + 1 (the second only if has_b): rotate, round, store.
-  // Called by all 32 lanes of a warp together.
-  __device__ void finish2(__nv_bfloat16* out, int N, int feature, int t0, int t, float va, float vb, bool has_b, int lane) const {
-    const float oa = __shfl_xor_sync(0xffffffffu, va, 1), ob = __shfl_xor_sync(0xffffffffu, vb, 1);
-    const bool odd = (lane & 1) != 0;
-    float re_a = odd ? oa : va, im_a = odd ? va : oa, re_b = odd ? ob : vb, im_b = odd ? vb : ob;
-    if (rope_d > 0) {
-      float sn = 0.f, cs = 1.f;
-      sincos_at(t0 + t + ((odd && has_b) ? 1 : 0), sn, cs);    // even lane: first token; odd lane: second
-      const float sn_o = __shfl_xor_sync(0xffffffffu, sn, 1), cs_o = __shfl_xor_sync(0xffffffffu, cs, 1);
-      const float sn_a = odd ? sn_o : sn, cs_a = odd ? cs_o : cs;
-      const float sn_b = (odd || !has_b) ? sn : sn_o, cs_b = (odd || !has_b) ? cs : cs_o;
-      const float ra = re_a * cs_a - im_a * sn_a, ia = im_a * cs_a + re_a * sn_a;
-      const float rb = re_b * cs_b - im_b * sn_b, ib = im_b * cs_b + re_b * sn_b;
-      re_a = ra; im_a = ia; re_b = rb; im_b = ib;
-    }
-    if (!odd) {
-      *reinterpret_cast<uint32_t*>(out + static_cast<size_t>(t0 + t) * N + feature) = pack_bf16(re_a, im_a);
-      if (has_b) *reinterpret_cast<uint32_t*>(out + static_cast<size_t>(t0 + t + 1) * N + feature) = pack_bf16(re_b, im_b);
-    }
-  }
-};
+// 1e-5 rad); the double-precision units of this chip are too slow to do it for every (token, pair).
+struct LinFreq { float hi, lo; };
+__device__ __forceinline__ LinFreq lin_freq(int feature, int rope_d, float theta) {
+  const double f = exp2(-2.0 * ((feature % rope_d) >> 1) / rope_d * log2(static_cast<double>(theta)));
+  const float hi = static_cast<float>(f);
+  return {hi, static_cast<float>(f - static_cast<double>(hi))};
+}
+__device__ __forceinline__ void lin_rotate(float& re, float& im, float pos, const LinFreq& f) {
+  const float a = pos * f.hi;
+  const float e = fmaf(pos, f.hi, -a) + pos * f.lo;          // what the rounded product left out
+  const float k = rintf(a * 0.15915494309189535f);          // whole turns
+  float r = fmaf(-k, 6.28125f, a);                           // 2*pi = 6.28125 + 0.001934051513671875 + 1.2556659146e-6
+  r = fmaf(-k, 0.001934051513671875f, r);
+  r = fmaf(-k, 1.2556659146e-6f, r) + e;
+  float sn, cs;
+  sincosf(r, &sn, &cs);
+  const float x = re * cs - im * sn, y = im * cs + re * sn;
+  re = x;
+  im = y;
+}
 
 __global__ void __launch_bounds__(kLinThreads, 1)
 linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant__ CUtensorMap w_map1,
-                    const __grid_constant__ CUtensorMap x_map, const LinSm100Params p, int32_t* dev_status) {
+                    const __grid_constant__ CUtensorMap w_map2, const __grid_constant__ CUtensorMap x_map, const LinSm100Params p, int32_t* dev_status) {
   extern __shared__ unsigned char smem_unaligned[];
   const uint32_t raw = smem_u32(smem_unaligned);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -126,20 +104,19 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_con
   const int kLinStages = p.stages;
   const uint32_t kLinStageBytes = kLinWBytes + static_cast<uint32_t>(p.x_box_rows) * 128u;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_s + 1);
-  volatile int* last_flag = abort_flag + 1;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tiles0 = p.N[0] / kLinBM, tiles = tiles0 + (p.n_jobs > 1 ? p.N[1] / kLinBM : 0);
   const int tile = blockIdx.x / p.splits, split = blockIdx.x % p.splits;
-  const int job = tile >= tiles0 ? 1 : 0;
-  const int f0 = (job ? tile - tiles0 : tile) * kLinBM;       // first output feature of the tile within its job
+  const int tiles0 = p.tiles01[0], tiles1 = p.tiles01[1];
+  const int job = tile < tiles0 ? 0 : tile < tiles0 + tiles1 ? 1 : 2;
+  const int f0 = (tile - (job == 0 ? 0 : job == 1 ? tiles0 : tiles0 + tiles1)) * kLinBM;  // first output feature within the job
   const int t0 = blockIdx.y * kLinMaxT;                        // first token of the block
   const int T = min(kLinMaxT, p.M - t0);                       // tokens of this block
   const int TP = (T + 15) & ~15;                               // MMA N
   const int ktiles = p.K / kLinBK;
   const int kt0 = static_cast<int>(static_cast<long long>(split) * ktiles / p.splits);
   const int kt1 = static_cast<int>(static_cast<long long>(split + 1) * ktiles / p.splits);
-  const CUtensorMap* w_map = job ? &w_map1 : &w_map0;
+  const CUtensorMap* w_map = job == 0 ? &w_map0 : job == 1 ? &w_map1 : &w_map2;
   uint32_t tmem_cols = 32;
   while (tmem_cols < static_cast<uint32_t>(TP)) tmem_cols <<= 1;
   pdl_trigger();
@@ -150,7 +127,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_con
     for (int i = 0; i < kLinMaxStages; ++i) { mbar_init(bar(LB_FULL + i), 1); mbar_init(bar(LB_EMPTY + i), 1); }
     mbar_init(bar(LB_DONE), 1);
     *abort_flag = 0;
-    *last_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -215,101 +191,71 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_con
     const int quad = warp & 3;                                 // tensor-memory lanes 32*quad .. 32*quad+31
     const int fl = quad * 32 + lane;                           // feature of this thread within the tile
     const uint32_t lane_base = static_cast<uint32_t>(quad * 32) << 16;
-    const int N = p.N[job], rope_d = p.rope_d[job];
-    __nv_bfloat16* out = p.out[job];
-    pdl_wait();  // the scratch buffer, the counters and the output may still be in use by earlier kernels
+    const int N = p.N[job], rope_d = job < 2 ? p.rope_d[job] : 0;
+    float* part_s = reinterpret_cast<float*>(sm);              // [T][128]: the ring is free when every MMA has retired
+    const int f = f0 + 4 * lane;                               // the lane's four features in the second half
+    LinFreq freq[2] = {};
+    if (rope_d > 0) { freq[0] = lin_freq(f, rope_d, p.theta); freq[1] = lin_freq(f + 2, rope_d, p.theta); }
+    double key_freq[2] = {};                                   // the append keeps its angles in fp64
+    if (job == 2 && f >= p.r && f < N)
+      for (int i = 0; i < 2; ++i) key_freq[i] = rope_freq(((f - p.r) >> 1) + i, p.dR, p.theta);
+    pdl_wait();  // the output may still be in use by earlier kernels
     mbar_wait(bar(LB_DONE), 0, abort_flag, dev_status);
     tc_fence_after();
-    LinRope rope(p, f0 + fl, rope_d);
-    auto finish2 = [&](int t, float va, float vb, bool has_b) { rope.finish2(out, N, f0 + fl, t0, t, va, vb, has_b, lane); };
-    const size_t tile_id = static_cast<size_t>(blockIdx.y) * tiles + tile;
-    const size_t slice_elems = static_cast<size_t>(p.x_box_rows) * kLinBM;
-    float* my_partial = p.partial + (tile_id * p.splits + split) * slice_elems;
-    for (int c = 0; c < TP; c += 32) {
-      uint32_t v[32];
-      tmem_ld32(tmem + lane_base + c, v);
+#pragma unroll 1
+    for (int c = 0; c < TP; c += 16) {
+      uint32_t v[16];
+      tmem_ld16(tmem + lane_base + c, v);
       tc_wait_ld();
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) {
-        if (c + j < T) {  // uniform over the warp
-          const bool has_b = c + j + 1 < T;
-          if (p.splits == 1) {
-            finish2(c + j, __uint_as_float(v[j]), __uint_as_float(v[j + 1]), has_b);
-          } else if (p.cluster) {  // the ring is free: every MMA of this CTA has retired
-            float* part_s = reinterpret_cast<float*>(sm);
-            part_s[(c + j) * kLinBM + fl] = __uint_as_float(v[j]);
-            if (has_b) part_s[(c + j + 1) * kLinBM + fl] = __uint_as_float(v[j + 1]);
-          } else {
-            my_partial[static_cast<size_t>(c + j) * kLinBM + fl] = __uint_as_float(v[j]);
-            if (has_b) my_partial[static_cast<size_t>(c + j + 1) * kLinBM + fl] = __uint_as_float(v[j + 1]);
-          }
-        }
-      }
-    }
-    if (p.splits > 1 && !p.cluster) {
-      // the slice that arrives last at the tile's counter adds all slices, in slice order
-      __threadfence();
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (tid == 64) {
-        const int old = atomicAdd(p.counters + tile_id, 1);
-        *last_flag = (old == p.splits - 1) ? 1 : 0;
-        if (old == p.splits - 1) p.counters[tile_id] = 0;  // ready for the next launch
-      }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      if (*last_flag) {
-        __threadfence();
-        const float* tile_partial = p.partial + tile_id * p.splits * slice_elems;
-        for (int tb = 0; tb < T; tb += 8) {  // eight tokens' slices in flight together
-          float acc[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u] = 0.f;
-          for (int s = 0; s < p.splits; ++s) {
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-              v[u] = tb + u < T ? __ldcg(tile_partial + s * slice_elems + static_cast<size_t>(tb + u) * kLinBM + fl) : 0.f;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) acc[u] += v[u];
-          }
-#pragma unroll
-          for (int u = 0; u < 8; u += 2)
-            if (tb + u < T) finish2(tb + u, acc[u], acc[u + 1], tb + u + 1 < T);
-        }
-      }
+      for (int j = 0; j < 16; ++j) part_s[(c + j) * kLinBM + fl] = __uint_as_float(v[j]);
     }
     tc_fence_before();
-  }
-
-  if (p.cluster && p.splits > 1) {
-    // ---- the slices of the tile meet: every CTA of the cluster has its partial [T][128] in its own shared memory;
-    // CTA `split` adds the slices of its share of the tokens in slice order, reading the others' memory directly
+    // The slices of the tile meet: CTA `split` adds the slices of its share of the tokens, a warp a token.
     cluster_sync_all();
-    if (warp >= 2) {
-      const int quad = warp & 3, fl = quad * 32 + lane;
-      const int N = p.N[job], rope_d = p.rope_d[job];
-      __nv_bfloat16* out = p.out[job];
-      const float* part_s = reinterpret_cast<const float*>(sm);
-      const int share = (((T + p.splits - 1) / p.splits) + 1) & ~1;  // even, so that token pairs stay together
-      const int ts = split * share, te = min(T, ts + share);
-      LinRope rope(p, f0 + fl, rope_d);
-      for (int tb = ts; tb < te; tb += 8) {
-        float acc[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc[u] = 0.f;
-        for (int s = 0; s < p.splits; ++s) {
-          float v[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) v[u] = tb + u < te ? ld_cluster_f32(part_s + (tb + u) * kLinBM + fl, s) : 0.f;
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u] += v[u];
-        }
-#pragma unroll
-        for (int u = 0; u < 8; u += 2)
-          if (tb + u < te) rope.finish2(out, N, f0 + fl, t0, tb + u, acc[u], acc[u + 1], tb + u + 1 < te, lane);
+    const int share = (T + p.splits - 1) / p.splits, te = min(T, (split + 1) * share);
+#pragma unroll 1
+    for (int t = split * share + quad; t < te; t += 4) {
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+      for (int s = 0; s < p.splits; ++s) {
+        const float4 v = ld_cluster_f32x4(part_s + t * kLinBM + 4 * lane, s);
+        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
       }
+      const int tok = t0 + t;
+      if (rope_d > 0) {
+        const float pos = static_cast<float>(p.pos_base[tok / p.S] + p.pos_shift + tok % p.S);
+#pragma unroll 1
+        for (int i = 0; i < 2; ++i) {  // one copy of the sine's code
+          lin_rotate(acc.x, acc.y, pos, freq[0]);
+          const float4 o = acc;
+          acc = make_float4(o.z, o.w, o.x, o.y);
+          const LinFreq g = freq[0];
+          freq[0] = freq[1];
+          freq[1] = g;
+        }
+      }
+      size_t row = tok;
+      if (job == 2) {  // the token's slot of the cache
+        const int b = tok / p.S, pos = p.pos_base[b] + p.pos_shift + tok % p.S, pj = pos / kPage;
+        int page = -1;
+        if (pos >= 0 && pj < p.max_pages) page = p.page_table[static_cast<size_t>(b) * p.max_pages + pj];
+        if (page < 0 || page >= p.num_pages) {
+          if (lane == 0) set_status(dev_status, TRANSMLA_DEV_BAD_PAGE);
+          continue;
+        }
+        if (f >= N) continue;
+        row = static_cast<size_t>(page) * kPage + pos % kPage;
+        if (f >= p.r) {
+          rope_pair_at(acc.x, acc.y, pos, key_freq[0]);
+          rope_pair_at(acc.z, acc.w, pos, key_freq[1]);
+        }
+      }
+      *reinterpret_cast<uint2*>(p.out[job] + row * N + f) = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
     }
-    cluster_sync_all();  // nobody leaves while its memory may still be read
   }
+  if (warp < 2) cluster_sync_all();
+  cluster_sync_all();  // nobody leaves while its memory may still be read
 
   // ---- teardown
   tc_fence_before();
@@ -324,28 +270,23 @@ static bool encode_2d(CUtensorMap* map, const void* ptr, int rows, int cols, int
 
 }  // namespace sm100
 
-// Slices of K per 128-feature tile: enough CTAs for every SM to stream weights, at least 4 stages of K per slice.
-int linear_sm100_splits(int n_tiles, int K) {
-  // one CTA per SM (the ring takes the whole shared memory) and one wave: as many slices as keep tiles x slices
-  // within the SM count of a B200, each at least four ring stages long
+// Slices of K per 128-feature tile wanted: as many as keep tiles x slices within the SM count of a B200, each at least four
+// stages long, at most the portable size of a cluster.
+static int linear_sm100_splits(int n_tiles, int K) {
   const int ktiles = K / sm100::kLinBK;
   int s = 148 / n_tiles;
-  if (s > 12) s = 12;
+  if (s > 8) s = 8;
   if (s > ktiles / 4) s = ktiles / 4;
   return s < 1 ? 1 : s;
 }
 
-// Where this kernel is used.  Its CTAs take the whole shared memory, so they cannot start while blocks of the kernel
-// before them are still resident, and the slices of a tile have to meet at the end; the mma.sync tiles of linear.cu
-// have neither cost but re-read the activations once per 32 features.  Measured on the LLaMA-2-7B shape (layer
-// step, pipelined) the tcgen05 kernel wins from about 48 tokens on, with long rows of weights (K >= 2048) and at
-// least 24 tiles of 128 features: B = 128: 108 -> 70 us for the layer's two large maps; at 16 tokens it is level
-// with the mma.sync tiles and at 1 token 13 us slower.
+// Where this kernel can be used: whole tiles of 128 features, whole ring stages, enough of both to be worth a launch of
+// this kind (smaller maps are not measured).
 bool linear_sm100_supported(const LinearArgs& a) {
-  if (a.n_jobs < 1 || a.n_jobs > 2 || a.M < 48 || a.job[0].K < 2048) return false;
+  if (a.n_jobs < 1 || a.n_jobs > 2 || a.job[0].K < 512) return false;
   int tiles = 0;
   for (int j = 0; j < a.n_jobs; ++j) tiles += a.job[j].N / sm100::kLinBM;
-  if (tiles < 24) return false;
+  if (tiles < 4) return false;
   for (int j = 0; j < a.n_jobs; ++j) {
     if (a.job[j].N % sm100::kLinBM || a.job[j].K % sm100::kLinBK || a.job[j].K != a.job[0].K || a.job[j].x != a.job[0].x) return false;
     if (a.job[j].rope_d % 2) return false;
@@ -353,46 +294,45 @@ bool linear_sm100_supported(const LinearArgs& a) {
   return true;
 }
 
-size_t linear_sm100_partial_bytes(int n_tiles, int K, int M) {
-  const int splits = linear_sm100_splits(n_tiles, K);
-  if (splits == 1) return 0;
-  const size_t blocks = (M + sm100::kLinMaxT - 1) / sm100::kLinMaxT;
-  const size_t rows = ((M < sm100::kLinMaxT ? M : sm100::kLinMaxT) + 15) & ~15;
-  return blocks * n_tiles * splits * rows * sm100::kLinBM * sizeof(float);
+// The append can ride along: a lane's four features are all latent or all rope key.
+bool linear_sm100_takes_append(const AppendJob& ap, const LinearArgs& a) {
+  return ap.x == a.job[0].x && ap.D == a.job[0].K && ap.r % 4 == 0 && ap.dR % 4 == 0;
 }
 
-size_t linear_sm100_counter_bytes(int n_tiles, int M) {
-  return static_cast<size_t>((M + sm100::kLinMaxT - 1) / sm100::kLinMaxT) * n_tiles * sizeof(int32_t);
-}
-
-cudaError_t launch_linear_sm100(const LinearArgs& a, float* partial, int32_t* counters, int32_t* dev_status,
-                                cudaStream_t stream) {
+cudaError_t launch_linear_sm100(const LinearArgs& a, int32_t* dev_status, cudaStream_t stream) {
   using namespace sm100;
   LinSm100Params p = {};
-  CUtensorMap wmap[2], xmap;
+  CUtensorMap wmap[3], xmap;
   int tiles = 0;
   for (int j = 0; j < a.n_jobs; ++j) {
     p.out[j] = a.job[j].out; p.N[j] = a.job[j].N; p.rope_d[j] = a.job[j].rope_d;
     if (!encode_2d(&wmap[j], a.job[j].w, a.job[j].N, a.job[j].K, kLinBM)) return cudaErrorInvalidValue;
-    tiles += a.job[j].N / kLinBM;
+    p.tiles01[j] = a.job[j].N / kLinBM;
+    tiles += p.tiles01[j];
   }
   if (a.n_jobs == 1) wmap[1] = wmap[0];
+  wmap[2] = wmap[0];
+  if (a.append.blocks > 0) {
+    const AppendJob& ap = a.append;
+    p.out[2] = ap.cache; p.N[2] = ap.r + ap.dR; p.page_table = ap.page_table;
+    p.r = ap.r; p.dR = ap.dR; p.num_pages = ap.num_pages; p.max_pages = ap.max_pages;
+    if (!encode_2d(&wmap[2], ap.w, p.N[2], ap.D, kLinBM)) return cudaErrorInvalidValue;
+    tiles += (p.N[2] + kLinBM - 1) / kLinBM;
+  }
   const int T = a.M < kLinMaxT ? a.M : kLinMaxT;
   p.x_box_rows = (T + 15) & ~15;
   p.stages = kLinRingBytes / (kLinWBytes + p.x_box_rows * 128);
   if (p.stages > kLinMaxStages) p.stages = kLinMaxStages;
   if (!encode_2d(&xmap, a.job[0].x, a.M, a.job[0].K, p.x_box_rows)) return cudaErrorInvalidValue;
-  p.n_jobs = a.n_jobs; p.M = a.M; p.S = a.S; p.K = a.job[0].K;
+  p.M = a.M; p.S = a.S; p.K = a.job[0].K;
   p.splits = linear_sm100_splits(tiles, p.K);
   p.pos_base = a.pos_base; p.pos_shift = a.pos_shift; p.theta = a.theta;
-  p.partial = partial; p.counters = counters;
   static PerDeviceFlag smem_set;  // zero-initialised; one slot per device
   if (cudaError_t e = ensure_dynamic_smem(linear_sm100_kernel, kLinSmemBytes, smem_set); e != cudaSuccess) return e;
   const int token_blocks = (a.M + kLinMaxT - 1) / kLinMaxT;
-  // The K slices of a tile are launched as one thread-block cluster (they are neighbours in blockIdx.x); they then
-  // meet through distributed shared memory and need neither the scratch buffer nor the counters.  All clusters have
-  // to fit on the device at once (a cluster lives inside one GPC, so fewer fit than SMs / size suggests): the
-  // slice count is lowered until they do; if no size from 2 to 8 fits, the wanted count runs through the scratch.
+  // The K slices of a tile are launched as one thread-block cluster (they are neighbours in blockIdx.x).  All clusters
+  // have to fit on the device at once, one CTA per SM (a cluster lives inside one GPC, so fewer fit than SMs / size
+  // suggests): the slice count is lowered until they do.
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kLinThreads);
   cfg.dynamicSmemBytes = kLinSmemBytes;
@@ -403,27 +343,24 @@ cudaError_t launch_linear_sm100(const LinearArgs& a, float* partial, int32_t* co
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  p.cluster = 0;
+  cfg.numAttrs = 2;
   static PerDeviceFlag max_clusters[9];  // co-resident clusters of each size on each device, asked once (0 = not yet)
   const int slot = current_device_slot();
-  for (int s = p.splits < 8 ? p.splits : 8; s >= 2 && !p.cluster; --s) {
-    attr[1].val.clusterDim.x = s;
-    cfg.gridDim = dim3(tiles * s, token_blocks);
-    cfg.numAttrs = 2;
-    int fit = slot >= 0 ? max_clusters[s].value[slot].load(std::memory_order_acquire) : 0;
+  for (; p.splits > 1; --p.splits) {
+    attr[1].val.clusterDim.x = p.splits;
+    cfg.gridDim = dim3(tiles * p.splits, token_blocks);
+    int fit = slot >= 0 ? max_clusters[p.splits].value[slot].load(std::memory_order_acquire) : 0;
     if (fit == 0) {
       int n = 0;
       if (cudaOccupancyMaxActiveClusters(&n, linear_sm100_kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = -1; }
       fit = n > 0 ? n : -1;
-      if (slot >= 0) max_clusters[s].value[slot].store(fit, std::memory_order_release);
+      if (slot >= 0) max_clusters[p.splits].value[slot].store(fit, std::memory_order_release);
     }
-    if (fit >= tiles * token_blocks) { p.cluster = 1; p.splits = s; }
+    if (fit >= tiles * token_blocks) break;
   }
-  if (!p.cluster) {
-    cfg.gridDim = dim3(tiles * p.splits, token_blocks);
-    cfg.numAttrs = 1;
-  }
-  return cudaLaunchKernelEx(&cfg, linear_sm100_kernel, wmap[0], wmap[1], xmap, p, dev_status);
+  attr[1].val.clusterDim.x = p.splits;
+  cfg.gridDim = dim3(tiles * p.splits, token_blocks);
+  return cudaLaunchKernelEx(&cfg, linear_sm100_kernel, wmap[0], wmap[1], wmap[2], xmap, p, dev_status);
 }
 
 }  // namespace transmla

@@ -13,14 +13,18 @@ __device__ __forceinline__ uint4 ld_u128(const __nv_bfloat16* p) { return *reint
 
 // RoPE of Eq. 1 on the pair (re, im) = elements (2l, 2l+1) of a d-vector at position pos.  The angle is formed
 // and reduced to [-pi, pi] in fp64 so that positions of 10^5 keep their phase; sine and cosine are fp32.
-__device__ __forceinline__ void rope_pair(float& re, float& im, int pos, int l, int d, float theta) {
-  const double ang = static_cast<double>(pos) * exp2(-2.0 * l / d * log2(static_cast<double>(theta)));
+__device__ __forceinline__ double rope_freq(int l, int d, float theta) { return exp2(-2.0 * l / d * log2(static_cast<double>(theta))); }
+__device__ __forceinline__ void rope_pair_at(float& re, float& im, int pos, double freq) {
+  const double ang = static_cast<double>(pos) * freq;
   const double red_ang = ang - 6.283185307179586476925 * rint(ang * 0.15915494309189533577);
   float sn, cs;
   sincosf(static_cast<float>(red_ang), &sn, &cs);
   const float nre = re * cs - im * sn, nim = im * cs + re * sn;
   re = nre;
   im = nim;
+}
+__device__ __forceinline__ void rope_pair(float& re, float& im, int pos, int l, int d, float theta) {
+  rope_pair_at(re, im, pos, rope_freq(l, d, theta));
 }
 
 constexpr int kAppendMaxMT = 8;  // 16-token tiles per pass

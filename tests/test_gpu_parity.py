@@ -408,6 +408,40 @@ def test_layer_decode_step(shape, seqlens, rq):
     err, rel = gu.assert_close(lifts.f64(y), want, f'layer output rq={rq}')
 
 
+@pytest.mark.parametrize('B,rq,dR,r', [(1, 0, 16, 64), (9, 0, 16, 64), (17, 512, 16, 64), (70, 0, 0, 128), (259, 512, 16, 64)])
+def test_layer_step_with_the_append_among_the_tiles(B, rq, dR, r):
+    """The append's r + dR features fill its last tile of 128 in part; token counts off the padding of 16, more than one
+    block of 256, no rope part; the slices of a tile in clusters of 2 to 3 CTAs."""
+    shape = synth.MLAShape(H=16, dn=64, dR=dR, dv=64, r=r, D=768)
+    seqlens = [3 + 7 * (i % 21) for i in range(B)]
+    scale = gu.mla_scale(shape)
+    dc = synth.make_decode_case(shape, seqlens, 51)
+    ac = synth.make_append_case(shape, [L - 1 for L in seqlens], 52)
+    lw = synth.make_layer_weights(shape, 53, q_lora_rank=rq)
+    weights = {k: v.cuda() for k, v in lw.items()}
+    weights.update(w_dkv_kr=ac['w_dkv_kr'].cuda(), w_uk=dc['w_uk'].cuda(), w_uv=dc['w_uv'].cuda())
+    params = binding.make_params(shape, B, dc['cache'].shape[0], dc['page_table'].shape[1], scale)
+    ws, _ = binding.alloc_workspace(params)
+    scratch = torch.empty(binding.transmla_layer_scratch_bytes(params, rq), dtype=torch.uint8, device='cuda')
+    y = torch.full((B, 1, shape.D), float('nan'), dtype=torch.bfloat16, device='cuda')
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    cache, alone = dc['cache'].cuda(), dc['cache'].cuda()
+    table = dc['page_table'].cuda()
+    binding.transmla_layer_decode_step(params, weights, ac['x'].cuda(), table, dc['seqlens'].cuda(), cache, ws, scratch, y, status)
+    binding.transmla_latent_append(params, ac['x'].cuda(), weights['w_dkv_kr'],
+                                   torch.tensor([L - 1 for L in seqlens], dtype=torch.int32, device='cuda'), table, alone, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    # the same rows in another order of summation: one bf16 step of the value, at most
+    a, b = cache.float(), alone.float()
+    assert float(((a - b).abs() / b.abs().clamp(min=b.abs().mean().item())).max()) <= 2.0 ** -7
+    want = orc.mla_layer_decode(lifts.f64(ac['x']), lifts.f64(lw['w_uq']), lifts.f64(lw['w_qr']), lifts.f64(ac['w_dkv_kr']),
+                                lifts.f64(dc['w_uk']), lifts.f64(dc['w_uv']), lifts.f64(lw['w_o']), lifts.f64(dc['cache']),
+                                dc['page_table'].numpy(), seqlens, scale, shape.r,
+                                w_dq=None if not rq else lifts.f64(lw['w_dq']))
+    gu.assert_close(lifts.f64(y), want, f'layer output B={B} rq={rq}')
+
+
 @pytest.mark.parametrize('shape,seqlens', [(synth.QWEN25_72B, [131, 700]), (synth.LLAMA2_7B, [300, 65, 1024])])
 def test_layer_step_repeated_on_a_poisoned_workspace(shape, seqlens):
     """Nothing may be read before the kernel that produces it has finished.  From the second call on every kernel is
