@@ -174,3 +174,32 @@ def test_fp8_append_writes_the_quantised_row():
         g_k = torch.tensor(row[512:640].copy()).view(torch.bfloat16).to(torch.float64).numpy() * g_scale
         assert np.all(np.abs(g_k - k_pe[page, off] * sc[page, off]) <= 2.0 ** -7 * np.abs(g_k) + 2e-3)
     assert np.all(got[~touched] == 0xA5)                                       # no other byte of the pool changed
+
+
+@pytest.mark.parametrize('B', [49, 64, 65, 130])
+def test_fp8_append_of_many_tokens_writes_the_bytes_of_few(B):
+    # the block's share of features and tokens changes at 48 and 64 tokens; a value's sum and its order do not
+    gu.ensure_built()
+    shape = synth.LLAMA2_7B
+    positions = [3 + 5 * (i % 40) for i in range(B)]
+    ac = synth.make_append_case(shape, positions, 45)
+    cols = max(positions) // 64 + 1
+    table = torch.arange(B * cols, dtype=torch.int32, device='cuda').reshape(B, cols)
+    x, w = ac['x'].cuda(), ac['w_dkv_kr'].cuda()
+    pos = torch.tensor(positions, dtype=torch.int32, device='cuda')
+    pages = B * cols
+    caches = []
+    for chunk in (B, 32):
+        cache = torch.zeros(pages, 64, synth.FP8_ROW_BYTES, dtype=torch.uint8, device='cuda')
+        status = torch.zeros(1, dtype=torch.int32, device='cuda')
+        for i in range(0, B, chunk):
+            n = min(chunk, B - i)
+            params = binding.make_params(shape, n, pages, cols, 1.0)
+            scratch = torch.full((n, shape.r + shape.dR), float('nan'), dtype=torch.float32, device='cuda')
+            binding.transmla_latent_append_fp8(params, x[i:i + n].contiguous(), w, pos[i:i + n].contiguous(),
+                                               table[i:i + n].contiguous(), cache, scratch, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        caches.append(cache)
+    assert torch.equal(caches[0], caches[1])
+    assert int((caches[0] != 0).sum()) > 500 * B
