@@ -397,7 +397,9 @@ def measure_conversion(args, name, shape, seqlens, seed, rank, world, local):
         return None
     f_sm = 2.0 * n * mz * mz
     sm_mhz = (clocks or {}).get('sm_mhz') or 1965.0
-    peak = 148 * 128 * 2 * 1965.0e6 / 1e12     # fp32 FMA lanes x 2 flop x the maximum SM clock
+    # an fp32 product is six bf16 products (three exact terms a value), and half of Z^T Z is mirrored
+    tpeak, tpeak_kind = measured_tensor_peak()
+    peak = tpeak / 6 * 2
     return {
         'metric': 'conversion of one layer: calibration tokens/s (RoRoPE + FreqFold + balanced joint PCA, synthetic activations)',
         'value': n * world / (ms_step * 1e-3), 'unit': 'tokens/s', 'n_gpus': world, 'steps': steps, 'warmup': 3,
@@ -407,12 +409,12 @@ def measure_conversion(args, name, shape, seqlens, seed, rank, world, local):
                    'parallelism': f'replicas x{world}, no data-path collective'},
         'decode_kernel_us': None, 'cache_gbs_pct_of_8tbs': None,
         'conversion_ms': part_ms,
-        'roofline': {'bound': 'alu', 'kernel': 'gemm_kernel<float> (second moment Z^T Z)', 'achieved': f_sm / part_ms['second_moment'] / 1e9,
+        'roofline': {'bound': 'tensor', 'kernel': 'gemm_split_kernel (second moment Z^T Z)', 'achieved': f_sm / part_ms['second_moment'] / 1e9,
                      'peak': peak, 'unit': 'TFLOP/s', 'frac': f_sm / part_ms['second_moment'] / 1e9 / peak,
-                     'peak_kind': 'derived: 148 SMs x 128 fp32 lanes x 2 flop x 1965 MHz', 'traffic': None, 'flops_per_launch': f_sm,
+                     'peak_kind': f'{tpeak_kind} bf16 GEMM / 6 products x 2 for the mirrored half', 'traffic': None, 'flops_per_launch': f_sm,
                      'sm_mhz_sampled': sm_mhz},
-        # gemm 6, gather 1, Jacobi 1, rotation 1, norms 3, concat 1, and (iters + 3) Cholesky QRs of three launches each
-        'gpu_launches': (13 + iters + 3 * (iters + 3)) * steps, 'clocks': clocks,
+        # gemm 6, gather 1, Jacobi 1, rotation 1, norms 3, concat 1, and (iters + 3) Cholesky QRs of four launches each
+        'gpu_launches': (13 + iters + 4 * (iters + 3)) * steps, 'clocks': clocks,
     }
 
 
@@ -579,7 +581,7 @@ def measure(args, name, shape, seqlens, seed, rank, world, local, full):
         layer_ms = replicas.max_over_ranks([l0.elapsed_time(l1)], device='cuda')[0] / steps
         lbytes = sum(t.numel() * t.element_size() for t in lws[0].values())
         layer = {'ms_per_step': layer_ms, 'tokens_per_s': B * S * world / (layer_ms * 1e-3), 'weight_bytes': lbytes,
-                 'q_lora_rank': args.q_lora_rank, 'launches_per_step': 6 + (1 if args.q_lora_rank else 0),
+                 'q_lora_rank': args.q_lora_rank, 'launches_per_step': 5 + (1 if args.q_lora_rank else 0),
                  'gbs_weights_plus_cache': (lbytes + sum(seqlens) * shape.row * 2) / (layer_ms * 1e-3) / 1e9}
 
     ms_total, e2e_ms = replicas.max_over_ranks([ms_total, e2e_s * 1e3], device='cuda')

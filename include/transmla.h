@@ -214,8 +214,7 @@ typedef struct {
   const void* w_o;       /* [D, H*dv]:  y = W_O [o_1; ...; o_H]  (Eq. 9, last line) */
 } transmla_layer_weights_t;
 
-/* Bytes of device scratch transmla_layer_decode_step needs: c^Q, q^C, q^R and the attention output (bf16), plus
- * the partial sums and arrival counters of the K-sliced linear maps used from 48 new tokens on. */
+/* Bytes of device scratch transmla_layer_decode_step needs: c^Q, q^C, q^R and the attention output (bf16). */
 size_t transmla_layer_scratch_bytes(const transmla_params_t* params /* host */, int32_t q_lora_rank);
 
 /* The whole attention layer for the S newest tokens of every sequence, x [B, S, D] -> y [B, S, D] (device bf16):
@@ -305,7 +304,7 @@ transmla_status_t transmla_selftest_bounded_wait(int32_t* dev_status, long long*
  *     bytes 640..643   scale_t = max_i |c_t[i]| / 448 as fp32 (1.0 for an all-zero row); bytes 644..655 unused
  * and the cache is [num_pages, P, 656] bytes, 128-byte aligned.  What the attention sees is the dequantised row
  * scale_t * code, scale_t * (k^R_t / scale_t); results are Eq. 9 on those values.  |c| must stay below 65504 (the
- * products run on fp16 copies of scale_t * code).
+ * products run in fp16: the codes themselves against probabilities that carry scale_t).
  *
  * transmla_latent_append_fp8: transmla_latent_append into such a cache.  `scratch` is device memory of at least
  * B * S * (r + dR) * 4 bytes, 16-byte aligned (the rows in fp32 between the projection and the quantisation: a row's
