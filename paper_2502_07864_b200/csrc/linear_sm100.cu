@@ -67,30 +67,6 @@ struct LinSm100Params {
   float theta;
 };
 
-// RoPE of Eq. 1 in the epilogue.  Angle = position x theta^(-2l/d), reduced to [-pi, pi] before sine and cosine.  The
-// reduction runs in fp32 with the frequency as a (hi, lo) pair and 2*pi as three constants whose products with the
-// turn count are formed exactly inside the fused multiply-adds (positions up to 2^20 keep an angle error below
-// 1e-5 rad); the double-precision units of this chip are too slow to do it for every (token, pair).
-struct LinFreq { float hi, lo; };
-__device__ __forceinline__ LinFreq lin_freq(int feature, int rope_d, float theta) {
-  const double f = exp2(-2.0 * ((feature % rope_d) >> 1) / rope_d * log2(static_cast<double>(theta)));
-  const float hi = static_cast<float>(f);
-  return {hi, static_cast<float>(f - static_cast<double>(hi))};
-}
-__device__ __forceinline__ void lin_rotate(float& re, float& im, float pos, const LinFreq& f) {
-  const float a = pos * f.hi;
-  const float e = fmaf(pos, f.hi, -a) + pos * f.lo;          // what the rounded product left out
-  const float k = rintf(a * 0.15915494309189535f);          // whole turns
-  float r = fmaf(-k, 6.28125f, a);                           // 2*pi = 6.28125 + 0.001934051513671875 + 1.2556659146e-6
-  r = fmaf(-k, 0.001934051513671875f, r);
-  r = fmaf(-k, 1.2556659146e-6f, r) + e;
-  float sn, cs;
-  sincosf(r, &sn, &cs);
-  const float x = re * cs - im * sn, y = im * cs + re * sn;
-  re = x;
-  im = y;
-}
-
 __global__ void __launch_bounds__(kLinThreads, 1)
 linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_constant__ CUtensorMap w_map1,
                     const __grid_constant__ CUtensorMap w_map2, const __grid_constant__ CUtensorMap x_map, const LinSm100Params p, int32_t* dev_status) {
@@ -194,11 +170,11 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_con
     const int N = p.N[job], rope_d = job < 2 ? p.rope_d[job] : 0;
     float* part_s = reinterpret_cast<float*>(sm);              // [T][128]: the ring is free when every MMA has retired
     const int f = f0 + 4 * lane;                               // the lane's four features in the second half
-    LinFreq freq[2] = {};
-    if (rope_d > 0) { freq[0] = lin_freq(f, rope_d, p.theta); freq[1] = lin_freq(f + 2, rope_d, p.theta); }
-    double key_freq[2] = {};                                   // the append keeps its angles in fp64
-    if (job == 2 && f >= p.r && f < N)
-      for (int i = 0; i < 2; ++i) key_freq[i] = rope_freq(((f - p.r) >> 1) + i, p.dR, p.theta);
+    const int rot_d = job < 2 ? rope_d : p.dR, rot_from = job < 2 ? 0 : p.r;
+    const bool rotated = rot_d > 0 && f >= rot_from && f < N;
+    double freq[2] = {};                                       // angles in fp64, as in the mma.sync tiles
+    if (rotated)
+      for (int i = 0; i < 2; ++i) freq[i] = rope_freq(((f - rot_from + 2 * i) % rot_d) >> 1, rot_d, p.theta);
     pdl_wait();  // the output may still be in use by earlier kernels
     mbar_wait(bar(LB_DONE), 0, abort_flag, dev_status);
     tc_fence_after();
@@ -222,22 +198,20 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_con
         const float4 v = ld_cluster_f32x4(part_s + t * kLinBM + 4 * lane, s);
         acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
       }
-      const int tok = t0 + t;
-      if (rope_d > 0) {
-        const float pos = static_cast<float>(p.pos_base[tok / p.S] + p.pos_shift + tok % p.S);
+      const int tok = t0 + t, pos = rot_d > 0 || job == 2 ? p.pos_base[tok / p.S] + p.pos_shift + tok % p.S : 0;
+      if (rotated) {
 #pragma unroll 1
         for (int i = 0; i < 2; ++i) {  // one copy of the sine's code
-          lin_rotate(acc.x, acc.y, pos, freq[0]);
-          const float4 o = acc;
-          acc = make_float4(o.z, o.w, o.x, o.y);
-          const LinFreq g = freq[0];
+          rope_pair_at(acc.x, acc.y, pos, freq[0]);
+          acc = make_float4(acc.z, acc.w, acc.x, acc.y);
+          const double g = freq[0];
           freq[0] = freq[1];
           freq[1] = g;
         }
       }
       size_t row = tok;
       if (job == 2) {  // the token's slot of the cache
-        const int b = tok / p.S, pos = p.pos_base[b] + p.pos_shift + tok % p.S, pj = pos / kPage;
+        const int b = tok / p.S, pj = pos / kPage;
         int page = -1;
         if (pos >= 0 && pj < p.max_pages) page = p.page_table[static_cast<size_t>(b) * p.max_pages + pj];
         if (page < 0 || page >= p.num_pages) {
@@ -246,10 +220,6 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_con
         }
         if (f >= N) continue;
         row = static_cast<size_t>(page) * kPage + pos % kPage;
-        if (f >= p.r) {
-          rope_pair_at(acc.x, acc.y, pos, key_freq[0]);
-          rope_pair_at(acc.z, acc.w, pos, key_freq[1]);
-        }
       }
       *reinterpret_cast<uint2*>(p.out[job] + row * N + f) = make_uint2(pack_bf16(acc.x, acc.y), pack_bf16(acc.z, acc.w));
     }
