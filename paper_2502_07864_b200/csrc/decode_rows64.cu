@@ -60,7 +60,7 @@ static_assert(kRows * 256 * 4 <= kStageBytes, "half of a segment's result passes
 
 enum { BAR_LAT_FULL = 0, BAR_LAT_EMPTY = kHalves * kStages, BAR_ROPE_FULL = BAR_LAT_EMPTY + kStages,
        BAR_ROPE_EMPTY = BAR_ROPE_FULL + kRopeStages, BAR_Q_READY = BAR_ROPE_EMPTY + kRopeStages, BAR_Q_EMPTY, BAR_S_FULL,
-       BAR_S_FREE, BAR_P_READY, BAR_PV_DONE = BAR_P_READY + 2, BAR_COUNT };
+       BAR_S_FREE, BAR_P_READY, BAR_PV_DONE = BAR_P_READY + 2, BAR_COUNT = BAR_PV_DONE + 2 };
 static_assert(BAR_COUNT <= 24, "barrier block");
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -93,8 +93,7 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
     mbar_init(bar(BAR_Q_EMPTY), 1);
     mbar_init(bar(BAR_S_FULL), 1);
     mbar_init(bar(BAR_S_FREE), kSoftmaxThreads);
-    for (int i = 0; i < 2; ++i) mbar_init(bar(BAR_P_READY + i), kSoftmaxThreads);
-    mbar_init(bar(BAR_PV_DONE), 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(bar(BAR_P_READY + i), kSoftmaxThreads); mbar_init(bar(BAR_PV_DONE + i), 1); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -265,7 +264,7 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
             tc_commit(bar(BAR_LAT_EMPTY + stage));
             tc_commit(bar(BAR_ROPE_EMPTY + slot));
           }
-          tc_commit(bar(BAR_PV_DONE));
+          tc_commit(bar(BAR_PV_DONE + (n & 1)));
         }
         __syncwarp();
         ++n;
@@ -326,6 +325,11 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
           const bool full = __all_sync(0xffffffffu, tok_end >= 16) && pos_scale;   // no masking
 
           uint32_t sq[16];
+          // The products of page n-2 are done before the scores of page n (whose rope part is loaded after them), so this
+          // wait costs nothing; it sees to it that every phase of the two barriers is looked at in turn.  With one barrier
+          // for all pages the wait for a segment's last products could meet the phase of the page before, whose parity
+          // reads as done: the softmax can be a whole page ahead of the products.
+          if (n >= 2) mbar_wait(bar(BAR_PV_DONE + buf), ((n >> 1) - 1) & 1, abort_flag, dev_status);
           mbar_wait(bar(BAR_S_FULL), n & 1, abort_flag, dev_status);
           tc_fence_after();
           tmem_ld16(tmem + lane_base + kColS + 16 * sub, sq);
@@ -410,9 +414,8 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
             }
           }
           if (rescale) {  // warp-uniform; each of a quadrant's two warps takes half of its 256 columns
-            // O is at rest once the products of the page before are done (those of the page before that are: this page's
-            // rope part was loaded after them, so the parity cannot be mistaken)
-            if (n >= 1) mbar_wait(bar(BAR_PV_DONE), (n - 1) & 1, abort_flag, dev_status);
+            // O is at rest once the products of the page before are done
+            if (n >= 1) mbar_wait(bar(BAR_PV_DONE + (buf ^ 1)), ((n - 1) >> 1) & 1, abort_flag, dev_status);
             tc_fence_after();
 #pragma unroll 1
             for (int t = 0; t < 4; ++t) {
@@ -438,7 +441,7 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
         const int last_stage = (g - 1) % kStages, last_slot = (n - 1) % kRopeStages;
         const int out_slot = meta[2 * ((g - 1) & (kMetaRing - 1)) + 1].x;
         open = open_segment();
-        mbar_wait(bar(BAR_PV_DONE), (n - 1) & 1, abort_flag, dev_status);
+        mbar_wait(bar(BAR_PV_DONE + ((n - 1) & 1)), ((n - 1) >> 1) & 1, abort_flag, dev_status);
         tc_fence_after();
         float* l_s = reinterpret_cast<float*>(sm + kOffRope + last_slot * kSubTileBytes);  // [8][32]
         l_s[stid] = l_run;
