@@ -52,8 +52,8 @@ constexpr int kOffRope = kStages * kStageBytes;       // rope part of a page, th
 constexpr int kOffQ = kOffRope + kRopeStages * kSubTileBytes;
 constexpr int kOffBar = kOffQ + 2 * kSubTileBytes;
 constexpr int kOffMisc = kOffBar + 256;
-// misc: pmax_s[2][8][32] f32, meta[8][2] int4, tmem base, abort
-constexpr int kMiscBytes = 2048 + 32 * kMetaRing + 16;
+// misc: pmax_s[2][8][32] f32, meta[8] int4, tmem base, abort
+constexpr int kMiscBytes = 2048 + 16 * kMetaRing + 16;
 constexpr int kSmemBytes = kOffMisc + kMiscBytes;
 static_assert(kSmemBytes <= 232448 && kOffBar % 256 == 0, "shared memory budget");
 static_assert(kRows * 256 * 4 <= kStageBytes, "half of a segment's result passes through a stage");
@@ -73,8 +73,8 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
   const uint32_t base = smem_u32(sm);
   if ((base & 1023u) != 0) { set_status(dev_status, TRANSMLA_DEV_TIMEOUT); return; }
   float* pmax_s = reinterpret_cast<float*>(sm + kOffMisc);  // [2][8][32]: per page parity, warp, lane
-  int4* meta = reinterpret_cast<int4*>(pmax_s + 512);           // [kMetaRing][2]: what each ring item is; its segment
-  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(meta + 2 * kMetaRing);
+  int4* meta = reinterpret_cast<int4*>(pmax_s + 512);       // [kMetaRing]: what each ring item is
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(meta + kMetaRing);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_s + 1);
   auto bar = [&](int i) -> uint32_t { return base + kOffBar + 8 * i; };
 
@@ -113,23 +113,18 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
     if (warp == 4) {
       // ======================================================================== TMA producer
       int g = 0, n = 0, segs = 0;   // ring items, pages and segments issued so far
-      int2 seg = make_int2(0, 0);
       const uint64_t stream_policy = l2_evict_first_policy();
       auto acquire = [&]() -> int {
         const int stage = g % kStages, use = g / kStages;
         mbar_wait(bar(BAR_LAT_EMPTY + stage), (use & 1) ^ 1, abort_flag, dev_status);
         return stage;
       };
-      auto describe = [&](int4 item) {
-        meta[2 * (g & (kMetaRing - 1))] = item;
-        meta[2 * (g & (kMetaRing - 1)) + 1] = make_int4(seg.x, seg.y, 0, 0);
-      };
+      auto describe = [&](int4 item) { meta[g & (kMetaRing - 1)] = item; };
       auto issue_queries = [&](int b, int slot, int L) {
-        seg = make_int2(slot, L);
         const int stage = acquire();
         mbar_wait(bar(BAR_Q_EMPTY), (segs & 1) ^ 1, abort_flag, dev_status);  // the segment before has its last scores
         if (!*abort_flag && elect_one()) {
-          describe(make_int4(ITEM_QUERIES, 0, 0, 0));
+          describe(make_int4(ITEM_QUERIES, slot, L, 0));
           const uint32_t full = bar(BAR_LAT_FULL + kHalves * stage);
           mbar_arrive_expect_tx(full, (kLatChunks + 1) * kSubTileBytes);
           const uint32_t dst = base + kOffLat + stage * kStageBytes;
@@ -186,7 +181,7 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
       for (int g = 0;; ++g) {
         const int stage = g % kStages, use = g / kStages;
         mbar_wait(bar(BAR_LAT_FULL + kHalves * stage), use & 1, abort_flag, dev_status);
-        const int4 m = meta[2 * (g & (kMetaRing - 1))];
+        const int4 m = meta[g & (kMetaRing - 1)];
         if (__any_sync(0xffffffffu, *abort_flag != 0) || m.x == ITEM_END) break;
         if (m.x == ITEM_QUERIES) {
           mbar_wait(bar(BAR_Q_READY), segs & 1, abort_flag, dev_status);  // moved to tensor memory
@@ -237,7 +232,7 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
       for (int g = 0;; ++g) {
         const int stage = g % kStages, use = g / kStages;
         mbar_wait(bar(BAR_LAT_FULL + kHalves * stage), use & 1, abort_flag, dev_status);
-        const int4 m = meta[2 * (g & (kMetaRing - 1))];
+        const int4 m = meta[g & (kMetaRing - 1)];
         if (__any_sync(0xffffffffu, *abort_flag != 0) || m.x == ITEM_END) break;
         if (m.x == ITEM_QUERIES) {
           mbar_wait(bar(BAR_Q_READY), segs & 1, abort_flag, dev_status);
@@ -281,16 +276,17 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
       const bool pos_scale = scale_log2 >= 0.f;
       int g = 0, n = 0;
       // Looks at ring item g, all 256 threads together.  Queries: this thread's row goes to tensor memory, sub-tile by
-      // sub-tile (each of a quadrant's two warps takes some), the issuers are told, and true is returned.  They give the
-      // stage back.  Otherwise the ring has ended or the CTA gave up.
-      auto open_segment = [&]() -> bool {
+      // sub-tile (each of a quadrant's two warps takes some), the issuers are told, `seg` gets the segment's slot and length,
+      // and true is returned.  They give the stage back.  Otherwise the ring has ended or the CTA gave up.
+      auto open_segment = [&](int2& seg) -> bool {
         const int stage = g % kStages;
         mbar_wait(bar(BAR_LAT_FULL + kHalves * stage), (g / kStages) & 1, abort_flag, dev_status);
-        const int4 m = meta[2 * (g & (kMetaRing - 1))];
+        const int4 m = meta[g & (kMetaRing - 1)];
         int stop;
         asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 1, 256, q;\nselp.s32 %0, 1, 0, p;\n}"
                      : "=r"(stop) : "r"(static_cast<int>(*abort_flag != 0 || m.x != ITEM_QUERIES)) : "memory");
         if (stop) return false;
+        seg = make_int2(m.y, m.z);
         const unsigned char* qrow = sm + kOffLat + stage * kStageBytes + row * 128;
 #pragma unroll 1
         for (int c = sub * 4; c < (sub ? kQTmemChunks : 4); ++c) {
@@ -308,19 +304,19 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
         ++g;
         return true;
       };
-      bool open = open_segment();
+      int2 seg, next_seg;   // slot of the segment's partial and length of its sequence
+      bool open = open_segment(seg);
       while (open) {
         float m_used = -INFINITY, l_run = 0.f;
         bool more = true;
         while (more) {
           const int stage = g % kStages, slot = n % kRopeStages, buf = n & 1;
           mbar_wait(bar(BAR_LAT_FULL + kHalves * stage), (g / kStages) & 1, abort_flag, dev_status);
-          const int4 pm = meta[2 * (g & (kMetaRing - 1))], seg = meta[2 * (g & (kMetaRing - 1)) + 1];
+          const int4 pm = meta[g & (kMetaRing - 1)];
           const int L = seg.y, pj = pm.y;
           const bool page_ok = pm.x == ITEM_PAGE && pm.z != 0;
           const int n_vis = my_row < SH ? L - behind : 0;
           const int tok_end = page_ok ? n_vis - pj * kPage - tok0 : 0;   // of this thread's 16 tokens, [0, tok_end) are visible
-          const int valid = page_ok ? min(kPage, L - pj * kPage) : 0;    // rows [valid, 64) of the page must read as zero
           const bool first = (pm.w & 1) != 0, last = (pm.w & 2) != 0;
           const bool full = __all_sync(0xffffffffu, tok_end >= 16) && pos_scale;   // no masking
 
@@ -356,6 +352,8 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
           asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 1, 256, q;\nselp.s32 %0, 1, 0, p;\n}"
                        : "=r"(aborted) : "r"(*abort_flag) : "memory");
           more = !last && pm.x == ITEM_PAGE && !aborted;
+          // rows [valid, 64) of the page must read as zero; once the CTA has given up, what `pm` says may never have been written
+          const int valid = aborted ? kPage : page_ok ? min(kPage, L - pj * kPage) : 0;
           // The row's four threads: both warps of quadrants quad and quad ^ 2.
           float rowmax = -INFINITY;
 #pragma unroll
@@ -439,8 +437,9 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
         // the place of its last P and the last page's stage are free: the four parts of a row's sum meet in the first;
         // O, normalised, passes through the second, 256 latents of the 64 rows at a time, and leaves in whole lines.
         const int last_stage = (g - 1) % kStages, last_slot = (n - 1) % kRopeStages;
-        const int out_slot = meta[2 * ((g - 1) & (kMetaRing - 1)) + 1].x;
-        open = open_segment();
+        const int out_slot = seg.x;
+        open = open_segment(next_seg);
+        seg = next_seg;
         mbar_wait(bar(BAR_PV_DONE + ((n - 1) & 1)), ((n - 1) >> 1) & 1, abort_flag, dev_status);
         tc_fence_after();
         float* l_s = reinterpret_cast<float*>(sm + kOffRope + last_slot * kSubTileBytes);  // [8][32]

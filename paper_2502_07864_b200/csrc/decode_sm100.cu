@@ -299,7 +299,6 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
           const int pj = pm.y;
           const bool page_ok = pm.z != 0;
           const int tok_end = page_ok ? n_vis - pj * kPage : 0;           // tokens [0, tok_end) of the page are visible
-          const int valid = page_ok ? min(kPage, L - pj * kPage) : 0;      // rows [valid, 64) must read as zero
           const bool first = (pm.w & 1) != 0;
           const int buf = n & 1;
 
@@ -322,6 +321,8 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
           asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 1, 128, q;\nselp.s32 %0, 1, 0, p;\n}"
                        : "=r"(aborted) : "r"(*abort_flag) : "memory");
           more = (pm.w & 2) == 0 && pm.x == ITEM_PAGE && !aborted;
+          // rows [valid, 64) of the page must read as zero; once the CTA has given up, what `pm` says may never have been written
+          const int valid = aborted ? kPage : page_ok ? min(kPage, L - pj * kPage) : 0;
           const float rowmax = fmaxf(fmaxf(pmax_s[(buf * 4 + 0) * 32 + lane], pmax_s[(buf * 4 + 1) * 32 + lane]),
                                      fmaxf(pmax_s[(buf * 4 + 2) * 32 + lane], pmax_s[(buf * 4 + 3) * 32 + lane]));
           // Lazy rescale: the reference maximum only moves when some row's new maximum exceeds it by 2^8.  Every
