@@ -147,6 +147,7 @@ linear_sm100_kernel(const __grid_constant__ CUtensorMap w_map0, const __grid_con
     // ======================================================================== MMA issuer
     const uint32_t idesc = instr_desc(TP, false);
     const int n_it = kt1 - kt0;
+    pdl_wait();  // no activations arrive before: the bounded waits below must not count the kernel before this one
     for (int i = 0; i < n_it; ++i) {
       const int stage = i % kLinStages, use = i / kLinStages;
       mbar_wait(bar(LB_FULL + stage), use & 1, abort_flag, dev_status);

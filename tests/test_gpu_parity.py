@@ -442,6 +442,33 @@ def test_layer_step_with_the_append_among_the_tiles(B, rq, dR, r):
     gu.assert_close(lifts.f64(y), want, f'layer output B={B} rq={rq}')
 
 
+def test_linear_maps_wait_for_a_long_kernel_before_them():
+    """One partition walks 400 000 page-table entries (8 pages in turn) for about 0.4 s, beside the resident blocks of W_O,
+    whose own waits are bounded at 0.2 s: those must not begin to count before the attention is done."""
+    shape = synth.LLAMA2_7B
+    entries, pages = 400_000, 8
+    dc = synth.make_decode_case(shape, [pages * 64], 61)
+    ac = synth.make_append_case(shape, [0], 62)
+    weights = {k: v.cuda() for k, v in synth.make_layer_weights(shape, 63).items()}
+    weights.update(w_dkv_kr=ac['w_dkv_kr'].cuda(), w_uk=dc['w_uk'].cuda(), w_uv=dc['w_uv'].cuda())
+    table = dc['page_table'][:, :pages].repeat(1, entries // pages).cuda()
+    seqlens = torch.tensor([entries * 64], dtype=torch.int32, device='cuda')
+    got = []
+    for G in (1, 0):
+        params = binding.make_params(shape, 1, dc['cache'].shape[0], entries, gu.mla_scale(shape), num_partitions=G)
+        ws, _ = binding.alloc_workspace(params)
+        scratch = torch.empty(binding.transmla_layer_scratch_bytes(params, 0), dtype=torch.uint8, device='cuda')
+        y = torch.full((1, 1, shape.D), float('nan'), dtype=torch.bfloat16, device='cuda')
+        status = torch.zeros(1, dtype=torch.int32, device='cuda')
+        binding.transmla_layer_decode_step(params, weights, ac['x'].cuda(), table, seqlens, dc['cache'].cuda(), ws, scratch, y, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        got.append(lifts.f64(y))
+    # One partial adds 4 products a page to an fp32 accumulator that truncates: at most 4 x 400 000 x 2^-23 = 0.19 of the value
+    # against the 148 partials' 0.0013 (0.03 was seen; activations that had not arrived would be another vector).
+    assert np.all(np.isfinite(got[0])) and lifts.rel_l2(got[0], got[1]) < 0.19
+
+
 @pytest.mark.parametrize('shape,seqlens', [(synth.QWEN25_72B, [131, 700]), (synth.LLAMA2_7B, [300, 65, 1024])])
 def test_layer_step_repeated_on_a_poisoned_workspace(shape, seqlens):
     """Nothing may be read before the kernel that produces it has finished.  From the second call on every kernel is
