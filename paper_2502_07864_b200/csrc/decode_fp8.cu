@@ -112,6 +112,42 @@ __device__ __forceinline__ void tmem_st_16x128b_x4(uint32_t taddr, const uint32_
                : "memory");
 }
 
+// An all-zero row adds nothing to O, but its scale is 1 by definition and may be far above its neighbours': if the reference
+// maximum followed it, their P' would leave fp16's range.  So whenever the reference is about to move (rarely: a segment's
+// first page, a new maximum far above) the softmax warps look for such rows and leave them out.  In functions of their own:
+// the same code inside the page loop cost 240 cycles a page.
+// Which of the warp's 16 tokens have all-zero rows; rows with a scale of exactly 1 are rare, and only their codes are read.
+__device__ __noinline__ uint32_t find_zero_rows(const unsigned char* page_s, int warp, int lane) {
+  uint32_t zero = 0;
+  uint32_t ones = __ballot_sync(0xffffffffu, lane < 16 && *reinterpret_cast<const uint32_t*>(page_s + kOffScale + (warp * 16 + (lane & 15)) * 16) == 0x3f800000u);
+#pragma unroll 1
+  for (; ones != 0; ones &= ones - 1) {
+    const int j = __ffs(ones) - 1;
+    const uint4 c = *reinterpret_cast<const uint4*>(page_s + (lane >> 3) * kSubTileBytes + (warp * 16 + j) * 128 + (lane & 7) * 16);
+    if (!__any_sync(0xffffffffu, ((c.x | c.y | c.z | c.w) & 0x7f7f7f7fu) != 0)) zero |= 1u << j;
+  }
+  return zero;
+}
+// The row's maximum of score + log2 scale over the warp's 16 tokens (scores in `x`, 32 apart; tokens from `seen` on do not
+// count), a zero row's scale taken as the smallest there is.
+__device__ __noinline__ float maximum_without(uint32_t zero, const float* x, const unsigned char* scl, int seen) {
+  float pmax = -INFINITY;
+#pragma unroll 1
+  for (int j = 0; j < seen && j < 16; ++j) {
+    const int e = static_cast<int>(*reinterpret_cast<const uint32_t*>(scl + j * 16) >> 23) - 127;
+    pmax = fmaxf(pmax, x[j * 32] + static_cast<float>(zero >> j & 1u ? -60 : max(e, -60)));
+  }
+  return pmax;
+}
+// Zero rows' probabilities become zeros in this row of P (they may be beyond fp16's range, and infinity times zero is not zero).
+__device__ __noinline__ void clear_zero_rows(uint32_t zero, unsigned char* prow, int warp, int sw) {
+#pragma unroll 1
+  for (; zero != 0; zero &= zero - 1) {
+    const int t = warp * 16 + __ffs(zero) - 1;
+    *reinterpret_cast<uint16_t*>(prow + (((t >> 3) ^ sw) << 4) + (t & 7) * 2) = 0;
+  }
+}
+
 // ---------------------------------------------------------------------------------------------- kernel
 __global__ void __launch_bounds__(kThreads, 1)
 decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_constant__ CUtensorMap scale_map,
@@ -527,17 +563,34 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
           asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 1, 128, q;\nselp.s32 %0, 1, 0, p;\n}"
                        : "=r"(aborted) : "r"(*abort_flag) : "memory");
           more = (pm.w & 2) == 0 && pm.x == ITEM_PAGE && !aborted;
-          if (tid == 0) mbar_arrive(bar(BAR_KV_EMPTY + stage));  // the scales have been read: the softmax warps' share
-          const float rowmax = fmaxf(fmaxf(pmax_s[(buf * 4 + 0) * 32 + lane], pmax_s[(buf * 4 + 1) * 32 + lane]),
+          float rowmax = fmaxf(fmaxf(pmax_s[(buf * 4 + 0) * 32 + lane], pmax_s[(buf * 4 + 1) * 32 + lane]),
                                      fmaxf(pmax_s[(buf * 4 + 2) * 32 + lane], pmax_s[(buf * 4 + 3) * 32 + lane]));
           // Lazy rescale: the reference maximum only moves when some row's new maximum exceeds it by 2^8.  Every
           // warp holds all 32 rows, so the four warps take the same decision without talking to each other.
           float alpha = 1.f;
-          bool rescale = false;
+          bool rescale = !first && __any_sync(0xffffffffu, rowmax > m_used + 8.f);
+          uint32_t zero_rows = 0;
+          if (first || rescale) {
+            const unsigned char* page_s = sm + kOffStage + stage * kStageBytes;
+            zero_rows = find_zero_rows(page_s, warp, lane);
+            int again;
+            asm volatile("{\n.reg .pred p, q;\nsetp.ne.b32 q, %1, 0;\nbar.red.or.pred p, 1, 128, q;\nselp.s32 %0, 1, 0, p;\n}"
+                         : "=r"(again) : "r"(static_cast<int>(zero_rows)) : "memory");
+            if (again) {
+              float* x = reinterpret_cast<float*>(sm + kOffX) + warp * 512 + lane;  // the neighbour has read its halves
+#pragma unroll
+              for (int j = 0; j < 16; ++j) x[j * 32] = __uint_as_float(sq[j]);
+              pmax_s[(buf * 4 + warp) * 32 + lane] = maximum_without(zero_rows, x, page_s + kOffScale + warp * 16 * 16, tok_end - warp * 16);
+              asm volatile("bar.sync 1, 128;" ::: "memory");
+              rowmax = fmaxf(fmaxf(pmax_s[(buf * 4 + 0) * 32 + lane], pmax_s[(buf * 4 + 1) * 32 + lane]),
+                             fmaxf(pmax_s[(buf * 4 + 2) * 32 + lane], pmax_s[(buf * 4 + 3) * 32 + lane]));
+              rescale = !first && __any_sync(0xffffffffu, rowmax > m_used + 8.f);
+            }
+          }
+          if (tid == 0) mbar_arrive(bar(BAR_KV_EMPTY + stage));  // scales (and codes) have been read: the softmax warps' share
           if (first) {
             m_used = rowmax;
           } else {
-            rescale = __any_sync(0xffffffffu, rowmax > m_used + 8.f);
             if (rescale) {
               const float m_new = fmaxf(m_used, rowmax);
               alpha = (m_new == -INFINITY) ? 1.f : exp2f(m_used - m_new);
@@ -565,6 +618,7 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
             const int c0w = 2 * warp, sw = lane & 7;
             *reinterpret_cast<uint4*>(prow + ((c0w ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             *reinterpret_cast<uint4*>(prow + (((c0w + 1) ^ sw) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+            if (zero_rows != 0) clear_zero_rows(zero_rows, prow, warp, sw);
           }
           // ---- rescale O^T by alpha (columns = query rows) once the previous PV has landed
           if (rescale) {

@@ -117,6 +117,21 @@ def test_fp8_rows_of_very_different_size():
     gu.assert_lse_close(lifts.f64(lse), want_lse, 'rows of very different size, lse')
 
 
+@pytest.mark.parametrize('octave', [-14, -18, -30])
+def test_fp8_small_rows_beside_zero_rows(octave):
+    # Every row is small (scales near 2^(octave - 8)) but for zero rows, whose scale is 1 by definition: those must not push
+    # the others' fp16 products into the denormals.  (Codes of a zero row may be -0.)
+    gu.ensure_built()
+    shape = synth.LLAMA2_7B
+    seqlens = [330, 64, 1500, 65]
+    case = fp8_case(shape, seqlens, seed=31, factor=lambda rng, size: 2.0 ** rng.uniform(octave, octave + 2, size) * np.where(rng.random(size) > 0.05, 1.0, -0.0))
+    out, lse, status = run_fp8(shape, case, gu.mla_scale(shape), 0)
+    assert status == 0
+    want, want_lse = oracle_fp8(shape, case, gu.mla_scale(shape))
+    gu.assert_close(lifts.f64(out), want, 'small rows beside zero rows')
+    gu.assert_lse_close(lifts.f64(lse), want_lse, 'small rows beside zero rows, lse')
+
+
 @pytest.mark.parametrize('seqlens,columns', [([64 * 40 + 5, 1, 700, 0, 333], 600), ([2900], 1200)])
 def test_fp8_two_partitions_a_cta(seqlens, columns):
     # 64 query rows and a page table with room for many pages: the library picks its partition count for 64 rows a CTA,
