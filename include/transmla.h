@@ -296,6 +296,12 @@ transmla_status_t transmla_mla_attention_static(const transmla_params_t* params 
  * usable.  cycles_out (device int64[2], may be NULL) receives the SM cycles spent in the two waits. */
 transmla_status_t transmla_selftest_bounded_wait(int32_t* dev_status, long long* cycles_out, void* stream);
 
+/* Diagnostic: the kernel of transmla_conv_gemm on dense A [M,K] and B [K,N], by single CTAs or by CTA pairs, with barrier
+ * waits that give up at once.  Shows what that leaves behind: TRANSMLA_DEV_TIMEOUT in *dev_status (device int32, required)
+ * and NaN in C [M,N]. */
+transmla_status_t transmla_selftest_conv_gemm(int pairs, int M, int N, int K, const float* A, const float* B, float* C,
+                                              int32_t* dev_status, void* stream);
+
 /* FP8 latent cache (the paper's abstract names FP8 quantisation as combinable with the method and gives no detail; the
  * stored format is this library's own).  Only r = 512, dR = 64.  A token's row is TRANSMLA_FP8_ROW_BYTES = 656 bytes:
  *     bytes   0..511   e4m3 codes (OCP 8-bit float: 1 sign, 4 exponent bits with bias 7, 3 mantissa bits, largest
@@ -359,6 +365,8 @@ transmla_status_t transmla_mla_prefill(const transmla_params_t* params /* host *
  * head j and dimension c; RoPE pair l of a head is (2l, 2l+1) = (real, imaginary).  `fold` = M of App. C: group G
  * holds frequencies G*M .. G*M+M-1 and has g*M real and g*M imaginary entries, entry i = p*g + j for frequency
  * G*M + p and head j.
+ * The matrix products wait on barriers inside the kernel, each wait bounded at about 0.2 s: one that expires raises
+ * TRANSMLA_DEV_TIMEOUT where the call has a dev_status, and leaves NaN instead of unfinished sums everywhere.
  *   transmla_conv_gemm: C[M,N] = alpha * op(A) op(B); op(A) = A [M,K] (ta = 0) or the transpose of A [K,M]
  *     (ta = 1), op(B) from B [K,N] (tb = 0) or B [N,K] (tb = 1); lda/ldb/ldc are row strides in elements.  Serves
  *     the calibration activations (K = X W^T), second moments (Z^T Z) and the low-rank rewrite of App. D.2

@@ -5,16 +5,21 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "common.cuh"
 #include "transmla.h"
 
 namespace transmla {
 namespace conv {
 
 // C[M,N] = alpha * op(A) op(B); op(A) is A [M,K] (ta = 0, row stride lda) or the transpose of A [K,M] (ta = 1), likewise
-// op(B) from B [K,N] or B [N,K].  `batch` problems, strides in elements.
+// op(B) from B [K,N] or B [N,K].  `batch` problems, strides in elements.  A barrier wait that gives up
+// sets TRANSMLA_DEV_TIMEOUT in *dev_status (if there is one) and leaves NaN in the tiles of C that it concerns.
 cudaError_t gemm_f32(int ta, int tb, int M, int N, int K, float alpha, const float* A, int lda, long long strideA,
                      const float* B, int ldb, long long strideB, float* C, int ldc, long long strideC, int batch,
-                     cudaStream_t stream);
+                     int32_t* dev_status, cudaStream_t stream);
+// The same of dense matrices by the kernel for single CTAs or pairs, with waits that give up at once (for a test).
+cudaError_t gemm_f32_gives_up(int pairs, int M, int N, int K, const float* A, const float* B, float* C, int32_t* dev_status,
+                              cudaStream_t stream);
 // seg[G][2n][g*fold]: rows 0..n-1 the real parts, n..2n-1 the imaginary parts of group G's dimensions (App. B, C)
 cudaError_t gather_segments(const float* K, int n, int g, int d, int fold, float* seg, cudaStream_t stream);
 // Symmetric eigendecomposition of `batch` matrices of order m <= 128 (parallel cyclic Jacobi, one block each).

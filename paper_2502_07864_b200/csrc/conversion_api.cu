@@ -17,7 +17,14 @@ transmla_status_t transmla_conv_gemm(int ta, int tb, int M, int N, int K, float 
                                      int ldb, float* C, int ldc, void* stream) {
   if (!A || !B || !C) return TRANSMLA_ERR_NULL;
   if (M < 1 || N < 1 || K < 1 || lda < (ta ? M : K) || ldb < (tb ? K : N) || ldc < N) return TRANSMLA_ERR_SHAPE;
-  return done(conv::gemm_f32(ta, tb, M, N, K, alpha, A, lda, 0, B, ldb, 0, C, ldc, 0, 1, static_cast<cudaStream_t>(stream)));
+  return done(conv::gemm_f32(ta, tb, M, N, K, alpha, A, lda, 0, B, ldb, 0, C, ldc, 0, 1, nullptr, static_cast<cudaStream_t>(stream)));
+}
+
+transmla_status_t transmla_selftest_conv_gemm(int pairs, int M, int N, int K, const float* A, const float* B, float* C,
+                                              int32_t* dev_status, void* stream) {
+  if (!A || !B || !C || !dev_status) return TRANSMLA_ERR_NULL;
+  if (M < 1 || N < 1 || K < 1) return TRANSMLA_ERR_SHAPE;
+  return done(conv::gemm_f32_gives_up(pairs, M, N, K, A, B, C, dev_status, static_cast<cudaStream_t>(stream)));
 }
 
 size_t transmla_conv_rorope_scratch_bytes(int n, int g, int d, int fold) {
@@ -37,7 +44,7 @@ transmla_status_t transmla_conv_rorope_covariance(const float* K, int n, int g, 
   if (cudaError_t e = conv::gather_segments(K, n, g, d, fold, seg, s); e != cudaSuccess) return TRANSMLA_ERR_CUDA;
   // sigma_x + sigma_y = [K_x ; K_y]^T [K_x ; K_y] per group
   return done(conv::gemm_f32(1, 0, m, m, 2 * n, 1.f, seg, m, static_cast<long long>(2) * n * m, seg, m,
-                             static_cast<long long>(2) * n * m, cov, m, static_cast<long long>(m) * m, groups, s));
+                             static_cast<long long>(2) * n * m, cov, m, static_cast<long long>(m) * m, groups, nullptr, s));
 }
 
 transmla_status_t transmla_conv_sym_eig(float* a, int batch, int m, float* eigvals, float* eigvecs, int32_t* dev_status,
@@ -108,7 +115,7 @@ transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, in
   };
   if (!orth(Q, Y) || !orth(Y, Q)) return TRANSMLA_ERR_CUDA;
   for (int it = 0; it < iters; ++it) {
-    if (conv::gemm_f32(0, 0, m, r, m, 1.f, Cmat, m, 0, Q, r, 0, Y, r, 0, 1, s) != cudaSuccess) return TRANSMLA_ERR_CUDA;
+    if (conv::gemm_f32(0, 0, m, r, m, 1.f, Cmat, m, 0, Q, r, 0, Y, r, 0, 1, dev_status, s) != cudaSuccess) return TRANSMLA_ERR_CUDA;
     if (!orth(Y, Q)) return TRANSMLA_ERR_CUDA;
   }
   if (!orth(Q, Y)) return TRANSMLA_ERR_CUDA;

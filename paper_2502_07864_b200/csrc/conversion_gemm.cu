@@ -7,6 +7,9 @@
 // one chunk of K (32) only, then the worker threads add it to fp32 sums in their registers, rounding to nearest.  Relative
 // error of a sum of 8192 products 2.6e-7 (a chain of fp32 multiply-adds: 1.4e-6; four chunks an accumulator: 8.8e-7).
 // (|x| below the largest bf16 value, 3.39e38.)
+// A barrier wait that gives up (which no launch should see) raises TRANSMLA_DEV_TIMEOUT where the caller has a status word,
+// and what the CTA has not finished becomes NaN: the issuer stops then, so that everybody whose sums are not complete gives
+// up as well.
 //
 // A CTA pair (cta_group::2) works on a 256 x 256 tile of C, or a single CTA on a 128 x 128 one; either way a CTA converts
 // 128 rows of op(A) and 128 columns of op(B) a chunk.  Two groups of eight worker warps take the chunks in turn: they read
@@ -41,7 +44,7 @@ constexpr int kLaunchRegs = 96, kWorkerRegs = 112, kIssuerRegs = 24;
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 static_assert(kThreads * kLaunchRegs <= 65536 && kWorkers * kWorkerRegs + 128 * kIssuerRegs <= kThreads * kLaunchRegs, "register split");
 enum { BAR_FULL = 0, BAR_EMPTY = kStages, BAR_D_FULL = 2 * kStages, BAR_D_FREE = BAR_D_FULL + 2,
-       BAR_FULL2 = BAR_D_FREE + 2, BAR_D_FREE2 = BAR_FULL2 + kStages, BAR_COUNT = BAR_D_FREE2 + 2 };  // ..2: the second CTA's word
+       BAR_FULL2 = BAR_D_FREE + 2, BAR_D_FREE2 = BAR_FULL2 + kStages, BAR_LAST = BAR_D_FREE2 + 2, BAR_COUNT };  // ..2: the second CTA's word
 static_assert(BAR_COUNT <= 24, "barrier block");
 
 // The pair's instructions.  The first CTA issues for both: A and B descriptors address the same offsets in both CTAs (128
@@ -68,17 +71,25 @@ __device__ __forceinline__ void mbar_arrive_first_relaxed(uint32_t bar) {
                ::"r"(bar) : "memory");
 }
 
-// Bounded wait as mbar_wait, for a barrier on which the other CTA's threads arrive too.
-__device__ __forceinline__ void mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+// Bounded wait as mbar_wait; kCluster: the other CTA's threads arrive on the barrier too.
+template <bool kCluster>
+__device__ __forceinline__ bool try_wait(uint32_t bar, uint32_t parity) {
+  if (!kCluster) return mbar_try_wait(bar, parity);
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+template <bool kCluster, long long kLimit>  // a limit of 0: whatever is not there at the first look
+__device__ __forceinline__ void wait_for(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  if (!kCluster && mbar_test(bar, parity)) return;
+  if (*abort_flag) return;
+  if (kLimit == 0) { *abort_flag = 1; return; }
+  if (try_wait<kCluster>(bar, parity)) return;
   const long long t0 = clock64();
-  while (true) {
-    if (*abort_flag) return;
-    uint32_t ok;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return;
-    if (clock64() - t0 > kWaitCycles) { *abort_flag = 1; return; }
+  while (!try_wait<kCluster>(bar, parity)) {
+    if (*abort_flag || clock64() - t0 > kLimit) { *abort_flag = 1; return; }
   }
 }
 
@@ -89,6 +100,7 @@ struct GemmArgs {
   long long stride_a, stride_b, stride_c;
   int M, N, K, lda, ldb, ldc, tiles_n, symmetric;
   float alpha;
+  int32_t* dev_status;    // may be null
 };
 
 // Eight consecutive values along the operand's contiguous dimension, zeros beyond its edges.  Group g of a chunk: with K
@@ -135,8 +147,8 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t addr) {
   return (smem_desc(addr, 16, 512) & ~(7ull << 61)) | (4ull << 61);  // 64-byte swizzle
 }
 
-template <int kCtas, bool kAContig, bool kBContig>
-__global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs args) {
+template <int kCtas, bool kAContig, bool kBContig, long long kLimit>
+__global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_constant__ GemmArgs args) {
   extern __shared__ unsigned char smem_unaligned[];
   constexpr int kTile = kRows * kCtas;   // tile of C, both ways
   const uint32_t raw = smem_u32(smem_unaligned);
@@ -168,6 +180,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
   if (tid == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(bar(BAR_FULL + i), 8); mbar_init(bar(BAR_EMPTY + i), 1); mbar_init(bar(BAR_FULL2 + i), 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(bar(BAR_D_FULL + i), 1); mbar_init(bar(BAR_D_FREE + i), 16); mbar_init(bar(BAR_D_FREE2 + i), 16); }
+    mbar_init(bar(BAR_LAST), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -185,6 +198,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
   sync_ctas();
   tc_fence_after();
   const uint32_t tmem = *tmem_base_s;
+  auto wait = [&](uint32_t b, uint32_t parity) { wait_for<false, kLimit>(b, parity, abort_flag); };
+  auto wait_cluster = [&](uint32_t b, uint32_t parity) { wait_for<true, kLimit>(b, parity, abort_flag); };
 
   if (warp >= kWorkers / 32) {
     // ========================================================================== MMA issuer
@@ -194,11 +209,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
       for (int c = 0; c < chunks; ++c) {
         const int stage = c % kStages, buf = c & 1;
         if (c >= 2) {
-          mbar_wait(bar(BAR_D_FREE + buf), ((c >> 1) - 1) & 1, abort_flag, nullptr);
-          if (kCtas == 2) mbar_wait_cluster(bar(BAR_D_FREE2 + buf), ((c >> 1) - 1) & 1, abort_flag);
+          wait(bar(BAR_D_FREE + buf), ((c >> 1) - 1) & 1);
+          if (kCtas == 2) wait_cluster(bar(BAR_D_FREE2 + buf), ((c >> 1) - 1) & 1);
         }
-        mbar_wait(bar(BAR_FULL + stage), (c / kStages) & 1, abort_flag, nullptr);
-        if (kCtas == 2) mbar_wait_cluster(bar(BAR_FULL2 + stage), (c / kStages) & 1, abort_flag);
+        wait(bar(BAR_FULL + stage), (c / kStages) & 1);
+        if (kCtas == 2) wait_cluster(bar(BAR_FULL2 + stage), (c / kStages) & 1);
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) break;  // no further products: those who wait for them give up too
         tc_fence_after();
         const uint64_t a0 = operand_desc<kAContig>(base + stage * kStageBytes);
         const uint64_t b0 = operand_desc<kBContig>(base + stage * kStageBytes + 3 * kPlane);
@@ -219,11 +235,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
         }
         __syncwarp();
       }
+      // Every product has retired before the CTA goes on to its end, also where a wait gave up.
+      if (elect_one()) { if (kCtas == 2) tc_commit2(bar(BAR_LAST)); else tc_commit(bar(BAR_LAST)); }
+      __syncwarp();
+      for (const long long t0 = clock64(); !mbar_try_wait(bar(BAR_LAST), 0) && clock64() - t0 < kWaitCycles;) {}
     } else if (rank == 1 && warp == kWorkers / 32) {
       // The second CTA's messenger tells the issuer of written stages: an arrival that releases to the other CTA waits for
       // everything its thread has in flight, which the workers must not.
       for (int c = 0; c < chunks; ++c) {
-        mbar_wait(bar(BAR_FULL + c % kStages), (c / kStages) & 1, abort_flag, nullptr);
+        wait(bar(BAR_FULL + c % kStages), (c / kStages) & 1);
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
         if (elect_one()) mbar_arrive_first(bar(BAR_FULL2 + c % kStages));
         __syncwarp();
       }
@@ -241,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
     for (int j = 0; j < kCols; ++j) acc[j] = 0.f;
     auto drain = [&](int d) {
       const int buf = d & 1;
-      mbar_wait(bar(BAR_D_FULL + buf), (d >> 1) & 1, abort_flag, nullptr);
+      wait(bar(BAR_D_FULL + buf), (d >> 1) & 1);
       tc_fence_after();
 #pragma unroll
       for (int j0 = 0; j0 < kCols; j0 += 16) {
@@ -289,7 +310,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
     if (group < chunks) load(group);
     for (int c = group; c < chunks; c += 2) {
       const int stage = c % kStages;
-      if (c >= kStages) mbar_wait(bar(BAR_EMPTY + stage), (c / kStages - 1) & 1, abort_flag, nullptr);
+      if (c >= kStages) wait(bar(BAR_EMPTY + stage), (c / kStages - 1) & 1);
       unsigned char* st = sm + stage * kStageBytes;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
@@ -304,6 +325,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
     }
     while (drained < chunks) drain(drained++);
 
+    if (*abort_flag) {
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) acc[j] = __int_as_float(0x7fffffff);
+    }
     // ---- write-out through shared memory (every product has completed), in whole lines
     constexpr int kPitch = kCols + 4;
     float* mine = reinterpret_cast<float*>(sm) + warp * 32 * kPitch;
@@ -333,6 +358,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
   }
   tc_fence_before();
   __syncthreads();
+  if (tid == 0 && *abort_flag) set_status(args.dev_status, TRANSMLA_DEV_TIMEOUT);
   sync_ctas();  // neither CTA leaves while the other may still reach its barriers
   tc_fence_after();
   if (warp == 0) {
@@ -341,10 +367,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const GemmArgs 
   }
 }
 
-template <int kCtas, bool kAContig, bool kBContig>
+template <int kCtas, bool kAContig, bool kBContig, long long kLimit = kWaitCycles>
 cudaError_t launch(GemmArgs args, int batch, cudaStream_t stream) {
   static PerDeviceFlag smem_set;
-  auto kernel = gemm_split_kernel<kCtas, kAContig, kBContig>;
+  auto kernel = gemm_split_kernel<kCtas, kAContig, kBContig, kLimit>;
   if (cudaError_t e = ensure_dynamic_smem(kernel, kSmemBytes, smem_set); e != cudaSuccess) return e;
   constexpr int kTile = kRows * kCtas;
   const long long tiles_m = (args.M + kTile - 1) / kTile;
@@ -380,13 +406,19 @@ cudaError_t launch_size(const GemmArgs& args, int batch, cudaStream_t stream) {
 
 cudaError_t gemm_f32(int ta, int tb, int M, int N, int K, float alpha, const float* A, int lda, long long strideA,
                      const float* B, int ldb, long long strideB, float* C, int ldc, long long strideC, int batch,
-                     cudaStream_t stream) {
+                     int32_t* dev_status, cudaStream_t stream) {
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   // X^T X (or X X^T) is symmetric: the tiles above the diagonal are mirrored instead of computed
   const int symmetric = A == B && ta != tb && M == N && lda == ldb && strideA == strideB;
-  const GemmArgs args = {A, B, C, strideA, strideB, strideC, M, N, K, lda, ldb, ldc, 0, symmetric, alpha};
+  const GemmArgs args = {A, B, C, strideA, strideB, strideC, M, N, K, lda, ldb, ldc, 0, symmetric, alpha, dev_status};
   if (!ta) return tb ? launch_size<true, true>(args, batch, stream) : launch_size<true, false>(args, batch, stream);
   return tb ? launch_size<false, true>(args, batch, stream) : launch_size<false, false>(args, batch, stream);
+}
+
+cudaError_t gemm_f32_gives_up(int pairs, int M, int N, int K, const float* A, const float* B, float* C, int32_t* dev_status,
+                              cudaStream_t stream) {
+  const GemmArgs args = {A, B, C, 0, 0, 0, M, N, K, K, N, N, 0, 0, 1.f, dev_status};
+  return pairs ? launch<2, true, false, 0>(args, 1, stream) : launch<1, true, false, 0>(args, 1, stream);
 }
 
 }  // namespace conv

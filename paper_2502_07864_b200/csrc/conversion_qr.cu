@@ -409,7 +409,7 @@ cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (cudaError_t e = cudaLaunchKernelEx(&cfg, cholesky_kernel, G, X, r, X32, dev_status); e != cudaSuccess) return e;
-  return gemm_f32(0, 0, m, r, r, 1.f, Y, r, 0, X32, r, 0, Q, r, 0, 1, stream);
+  return gemm_f32(0, 0, m, r, r, 1.f, Y, r, 0, X32, r, 0, Q, r, 0, 1, dev_status, stream);
 }
 
 }  // namespace conv

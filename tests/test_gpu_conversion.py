@@ -58,6 +58,21 @@ def test_gemm_tiles_pairs_and_symmetric_products(M, N, K, ta, tb):
         assert torch.equal(c, c.T)
 
 
+@pytest.mark.parametrize('pairs,M,N,K', [(0, 100, 90, 500), (0, 300, 1000, 40), (1, 100, 90, 500), (1, 1000, 700, 300)])
+def test_gemm_that_gives_up_leaves_no_unfinished_sums(pairs, M, N, K):
+    # one CTA a tile and CTA pairs, with waits that expire in every CTA; the launch ends normally
+    gu.ensure_built()
+    a = torch.randn(M, K, device='cuda'); b = torch.randn(K, N, device='cuda')
+    c = torch.zeros(M, N, device='cuda')
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    binding.transmla_selftest_conv_gemm(pairs, a, b, c, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) & 2                    # TRANSMLA_DEV_TIMEOUT
+    assert bool(torch.isnan(c).all())
+    binding.transmla_conv_gemm(a, b, c)
+    assert _rel(_f64(c), _f64(a) @ _f64(b)) < 1e-6
+
+
 @pytest.mark.parametrize('g,d,fold', [(4, 16, 1), (4, 16, 2), (32, 128, 4), (3, 8, 4)])
 def test_rorope_covariance_matches_the_oracle(g, d, fold):
     gu.ensure_built()
