@@ -325,10 +325,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
     }
     while (drained < chunks) drain(drained++);
 
-    if (*abort_flag) {
-#pragma unroll
-      for (int j = 0; j < kCols; ++j) acc[j] = __int_as_float(0x7fffffff);
-    }
+    // (After a give-up other warps may still be writing terms over these sums' staging place: NaN goes straight to C.)
+    const bool bad = __any_sync(0xffffffffu, *abort_flag != 0);
     // ---- write-out through shared memory (every product has completed), in whole lines
     constexpr int kPitch = kCols + 4;
     float* mine = reinterpret_cast<float*>(sm) + warp * 32 * kPitch;
@@ -345,14 +343,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
 #pragma unroll
       for (int j = lane; j < kCols; j += 32) {
         const int n = nw + j;
-        if (n < N && (!args.symmetric || n <= m)) C[static_cast<size_t>(m) * args.ldc + n] = mine[r * kPitch + j];
+        if (n < N && (!args.symmetric || n <= m)) C[static_cast<size_t>(m) * args.ldc + n] = bad ? __int_as_float(0x7fffffff) : mine[r * kPitch + j];
       }
     }
     if (args.symmetric) {
       const int m = mw + lane;
       for (int j = 0; j < kCols; ++j) {
         const int n = nw + j;
-        if (n < m && m < M) C[static_cast<size_t>(n) * args.ldc + m] = mine[lane * kPitch + j];
+        if (n < m && m < M) C[static_cast<size_t>(n) * args.ldc + m] = bad ? __int_as_float(0x7fffffff) : mine[lane * kPitch + j];
       }
     }
   }

@@ -65,10 +65,11 @@ def test_gemm_that_gives_up_leaves_no_unfinished_sums(pairs, M, N, K):
     a = torch.randn(M, K, device='cuda'); b = torch.randn(K, N, device='cuda')
     c = torch.zeros(M, N, device='cuda')
     status = torch.zeros(1, dtype=torch.int32, device='cuda')
-    binding.transmla_selftest_conv_gemm(pairs, a, b, c, status)
-    torch.cuda.synchronize()
-    assert int(status.item()) & 2                    # TRANSMLA_DEV_TIMEOUT
-    assert bool(torch.isnan(c).all())
+    for _ in range(50):
+        c.zero_()
+        binding.transmla_selftest_conv_gemm(pairs, a, b, c, status)
+        assert int(status.item()) & 2                    # TRANSMLA_DEV_TIMEOUT
+        assert bool(torch.isnan(c).all())
     binding.transmla_conv_gemm(a, b, c)
     assert _rel(_f64(c), _f64(a) @ _f64(b)) < 1e-6
 
