@@ -367,6 +367,8 @@ transmla_status_t transmla_mla_prefill(const transmla_params_t* params /* host *
  * G*M + p and head j.
  * The matrix products wait on barriers inside the kernel, each wait bounded at about 0.2 s: one that expires raises
  * TRANSMLA_DEV_TIMEOUT where the call has a dev_status, and leaves NaN instead of unfinished sums everywhere.
+ * Infinities and NaN take part as in fp32 arithmetic; operand values below 2^-110 keep an absolute accuracy of 2^-134 only,
+ * where their products reach 2^-63.
  *   transmla_conv_gemm: C[M,N] = alpha * op(A) op(B); op(A) = A [M,K] (ta = 0) or the transpose of A [K,M]
  *     (ta = 1), op(B) from B [K,N] (tb = 0) or B [N,K] (tb = 1); lda/ldb/ldc are row strides in elements.  Serves
  *     the calibration activations (K = X W^T), second moments (Z^T Z) and the low-rank rewrite of App. D.2

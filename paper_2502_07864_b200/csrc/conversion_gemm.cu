@@ -6,7 +6,7 @@
 // core adds into its fp32 accumulator by truncation, which over thousands of steps would be a bias: an accumulator takes
 // one chunk of K (32) only, then the worker threads add it to fp32 sums in their registers, rounding to nearest.  Relative
 // error of a sum of 8192 products 2.6e-7 (a chain of fp32 multiply-adds: 1.4e-6; four chunks an accumulator: 8.8e-7).
-// (|x| below the largest bf16 value, 3.39e38.)
+// The terms are exact for 2^-110 <= |x| < 3.39e38 (the largest bf16 value): beyond, see the write-out.
 // A barrier wait that gives up (which no launch should see) raises TRANSMLA_DEV_TIMEOUT where the caller has a status word,
 // and what the CTA has not finished becomes NaN: the issuer stops then, so that everybody whose sums are not complete gives
 // up as well.
@@ -145,6 +145,18 @@ template <bool kContig>
 __device__ __forceinline__ uint64_t operand_desc(uint32_t addr) {
   if (!kContig) return smem_desc(addr, 4096, 1024);
   return (smem_desc(addr, 16, 512) & ~(7ull << 61)) | (4ull << 61);  // 64-byte swizzle
+}
+
+// One element of op(A) op(B) as a chain of fp32 multiply-adds.
+template <bool kAContig, bool kBContig>
+__device__ __forceinline__ float plain_sum(const GemmArgs& args, int m, int n) {
+  const float* a = args.A + args.stride_a * blockIdx.y + (kAContig ? static_cast<size_t>(m) * args.lda : m);
+  const float* b = args.B + args.stride_b * blockIdx.y + (kBContig ? static_cast<size_t>(n) * args.ldb : n);
+  float s = 0.f;
+#pragma unroll 1
+  for (int k = 0; k < args.K; ++k)
+    s = fmaf(a[kAContig ? k : static_cast<size_t>(k) * args.lda], b[kBContig ? k : static_cast<size_t>(k) * args.ldb], s);
+  return s;
 }
 
 template <int kCtas, bool kAContig, bool kBContig, long long kLimit>
@@ -334,10 +346,34 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
     for (int j = 0; j < kCols; j += 4)
       *reinterpret_cast<float4*>(mine + lane * kPitch + j) =
           make_float4(acc[j] * args.alpha, acc[j + 1] * args.alpha, acc[j + 2] * args.alpha, acc[j + 3] * args.alpha);
+    // Where the split does not hold the sum is taken once more, by fp32 multiply-adds: an infinite or too large operand value
+    // has no exact terms and made its sums NaN, and operands so small that all of the warp's sums stay below 2^-63 may have
+    // lost their last terms.
+    float size[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < kCols; ++j) size[j & 3] += fabsf(acc[j]);
+    const float all = (size[0] + size[1]) + (size[2] + size[3]);
+    const bool small = __all_sync(0xffffffffu, all < 0x1p-63f) && __any_sync(0xffffffffu, all > 0.f);
+    if (small || __any_sync(0xffffffffu, !(all < INFINITY))) {
+#pragma unroll 1
+      for (int j = 0; j < kCols; ++j) {
+        const int m = m0 + quad * 32 + lane, n = n0 + quarter * kCols + j;
+        if (m < M && n < N && (small || !isfinite(mine[lane * kPitch + j])))
+          mine[lane * kPitch + j] = args.alpha * plain_sum<kAContig, kBContig>(args, m, n);
+      }
+    }
     __syncwarp();
     float* C = args.C + args.stride_c * blockIdx.y;
     const int mw = m0 + quad * 32, nw = n0 + quarter * kCols;
-    for (int r = 0; r < 32; ++r) {
+    const bool whole = !bad && !args.symmetric && n0 + kTile <= N && (args.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+    if (whole) {  // 16 bytes a lane
+      constexpr int kLanes = kCols / 4, kAtOnce = 32 / kLanes;   // of a row; rows
+      const int j = lane % kLanes * 4;
+#pragma unroll 4
+      for (int r = lane / kLanes; r < 32; r += kAtOnce)
+        if (mw + r < M) *reinterpret_cast<float4*>(C + static_cast<size_t>(mw + r) * args.ldc + nw + j) = *reinterpret_cast<const float4*>(mine + r * kPitch + j);
+    }
+    for (int r = 0; r < 32 && !whole; ++r) {
       const int m = mw + r;
       if (m >= M) break;
 #pragma unroll

@@ -58,6 +58,41 @@ def test_gemm_tiles_pairs_and_symmetric_products(M, N, K, ta, tb):
         assert torch.equal(c, c.T)
 
 
+@pytest.mark.parametrize('M,N,K,ta,tb', [(200, 150, 100, 0, 0), (200, 150, 100, 1, 1), (6000, 5000, 40, 0, 1)])
+def test_gemm_of_infinities_and_of_values_at_the_ends_of_fp32(M, N, K, ta, tb):
+    # one CTA a tile and CTA pairs: values that bf16 terms cannot hold take part as in fp32 arithmetic
+    gu.ensure_built()
+    gen = torch.Generator(device='cuda'); gen.manual_seed(M)
+    a = torch.randn((K, M) if ta else (M, K), generator=gen, device='cuda'); b = torch.randn((N, K) if tb else (K, N), generator=gen, device='cuda')
+    op_a, op_b = (a.T if ta else a), (b.T if tb else b)
+    c = torch.empty(M, N, device='cuda')
+
+    def run(alpha=1.0):
+        binding.transmla_conv_gemm(a, b, c, ta=bool(ta), tb=bool(tb), alpha=alpha)
+        return op_a.double() @ op_b.double()
+
+    keep = a.clone()
+    op_a[3, 5], op_a[130, 7], op_a[131, 0] = float('inf'), float('-inf'), float('nan')
+    op_b[5, 9] = 0.0                                   # inf * 0
+    want = run().float()
+    assert torch.equal(torch.isnan(c), torch.isnan(want)) and torch.equal(torch.isinf(c), torch.isinf(want))
+    assert torch.equal(c.sign()[torch.isinf(c)], want.sign()[torch.isinf(want)])
+    ok = torch.isfinite(want)
+    assert float((c[ok] - want[ok]).norm() / want[ok].norm()) < 1e-6
+    a.copy_(keep); op_a[2], op_b[:, 4] = 3.4e38, 1e-3  # finite, above the largest bf16 value
+    want = run(alpha=1e-4)
+    got, ref = c[2].double(), want[2] * 1e-4
+    fin = torch.isfinite(got)                          # (sums beyond 3.4e38 overflow, as fp32 sums do)
+    assert bool(fin[4]) and abs(float(got[4] / ref[4]) - 1) < 1e-5 and float((got[fin] / ref[fin] - 1).abs().max()) < 1e-3
+    # small operands: exact terms down to 2^-110, plain sums below; each row's error against its own norm, where a chain of
+    # K fp32 multiply-adds keeps K 2^-24 at most
+    for scale in (2.0 ** -100, 2.0 ** -112, 2.0 ** -120):
+        a.copy_(keep * scale)
+        want = run(alpha=2.0 ** 90)
+        rel = ((c.double() * 2.0 ** -90 - want).norm(dim=1) / want.norm(dim=1)).max()
+        assert float(rel) < K * 2.0 ** -24, scale
+
+
 @pytest.mark.parametrize('pairs,M,N,K', [(0, 100, 90, 500), (0, 300, 1000, 40), (1, 100, 90, 500), (1, 1000, 700, 300)])
 def test_gemm_that_gives_up_leaves_no_unfinished_sums(pairs, M, N, K):
     # one CTA a tile and CTA pairs, with waits that expire in every CTA; the launch ends normally
