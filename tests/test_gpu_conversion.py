@@ -109,6 +109,21 @@ def test_gemm_that_gives_up_leaves_no_unfinished_sums(pairs, M, N, K):
     assert _rel(_f64(c), _f64(a) @ _f64(b)) < 1e-6
 
 
+@pytest.mark.parametrize('ta,tb', [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize('M,N,K', [(1, 1, 1), (129, 260, 1), (300, 131, 4), (128, 128, 16), (130, 257, 17)])
+def test_gemm_of_short_sums(M, N, K, ta, tb):
+    # up to 16 products a sum: every element within the rounding of K fp32 multiply-adds, K 2^-24 of the sum of sizes
+    gu.ensure_built()
+    gen = torch.Generator(device='cuda'); gen.manual_seed(M + K)
+    a = torch.randn((K, M) if ta else (M, K), generator=gen, device='cuda'); b = torch.randn((N, K) if tb else (K, N), generator=gen, device='cuda')
+    c = torch.full((M, N), float('nan'), device='cuda')
+    binding.transmla_conv_gemm(a, b, c, ta=bool(ta), tb=bool(tb), alpha=0.5)
+    op_a, op_b = (a.T if ta else a).double(), (b.T if tb else b).double()
+    # (17 products pass through the split: 12 truncations of 2^-23)
+    bound = (K * 2.0 ** -24 if K <= 16 else 12 * 2.0 ** -23) * 0.5 * (op_a.abs() @ op_b.abs())
+    assert bool(((c.double() - 0.5 * (op_a @ op_b)).abs() <= bound).all())
+
+
 @pytest.mark.parametrize('g,d,fold', [(4, 16, 1), (4, 16, 2), (32, 128, 4), (3, 8, 4)])
 def test_rorope_covariance_matches_the_oracle(g, d, fold):
     gu.ensure_built()
