@@ -34,6 +34,9 @@ cudaError_t balance_concat(const float* k_nope, int n, int mk, const float* v, i
 int gram_slices(int r);
 cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G, double* X, float* X32, float* Q,
                         int32_t* dev_status, cudaStream_t stream);
+// The pass that leaves the result, in place: Q <- Q L^-T, rounded once.  P [m,r] is scratch; the rest as above.
+cudaError_t cholesky_qr_last(float* Q, int m, int r, double* partial, double* G, double* X, float* X32, float* P,
+                             int32_t* dev_status, cudaStream_t stream);
 
 }  // namespace conv
 }  // namespace transmla

@@ -118,8 +118,8 @@ transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, in
     if (conv::gemm_f32(0, 0, m, r, m, 1.f, Cmat, m, 0, Q, r, 0, Y, r, 0, 1, dev_status, s) != cudaSuccess) return TRANSMLA_ERR_CUDA;
     if (!orth(Y, Q)) return TRANSMLA_ERR_CUDA;
   }
-  if (!orth(Q, Y)) return TRANSMLA_ERR_CUDA;
-  return done(cudaMemcpyAsync(Q, Y, static_cast<size_t>(m) * r * sizeof(float), cudaMemcpyDeviceToDevice, s));
+  return done(conv::cholesky_qr_last(Q, m, r, reinterpret_cast<double*>(w + l.partial), reinterpret_cast<double*>(w + l.g),
+                                     reinterpret_cast<double*>(w + l.x), reinterpret_cast<float*>(w + l.x32), Y, dev_status, s));
 }
 
 }  // extern "C"

@@ -208,7 +208,7 @@ __device__ __forceinline__ void warp_product(double (&acc)[kRows][4], const doub
   }
 }
 __global__ void __launch_bounds__(kCholThreads, 1)
-cholesky_kernel(double* G, double* X, int r, float* X32, int32_t* dev_status) {
+cholesky_kernel(double* G, double* X, int r, float* X32, int diagonal, int32_t* dev_status) {
   extern __shared__ __align__(16) double cs[];
   double* D = cs;                     // the panel's diagonal block
   double* W = D + kBlock;             // L(p,p)^-T
@@ -371,9 +371,21 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int32_t* dev_status) {
   }
   for (int e = cta * kCholThreads + tid; e < r * r; e += ctas * kCholThreads) {
     const int row = e / r, c = e % r;
-    X32[e] = c < row ? 0.f : static_cast<float>(__ldcg(X + e));
+    X32[e] = c < row || (c == row && !diagonal) ? 0.f : static_cast<float>(__ldcg(X + e));
   }
   if (bad && tid == 0 && cta == 0 && dev_status != nullptr) atomicOr(dev_status, TRANSMLA_DEV_NUMERIC);
+}
+
+// Q <- P + Q diag(X), in fp64 per element: the rest of the last pass (see cholesky_qr_last).
+__global__ void __launch_bounds__(256) add_diagonal_kernel(const float* P, float* Q, int m, int r, const double* X) {
+  const int c = blockIdx.x * 256 + threadIdx.x;
+  if (c >= r) return;
+  const double d = X[static_cast<size_t>(c) * r + c];
+#pragma unroll 8
+  for (int i = blockIdx.y; i < m; i += gridDim.y) {
+    const size_t e = static_cast<size_t>(i) * r + c;
+    Q[e] = static_cast<float>(fma(static_cast<double>(Q[e]), d, static_cast<double>(P[e])));
+  }
 }
 
 }  // namespace
@@ -384,8 +396,9 @@ int gram_slices(int r) {  // slices of the sum over rows: what fills the device 
   return s < 1 ? 1 : s > 16 ? 16 : s;
 }
 
-cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G, double* X, float* X32, float* Q,
-                        int32_t* dev_status, cudaStream_t stream) {
+// X = L^-T of Y^T Y = L L^T, in fp64, and X32 in fp32, with its diagonal or without.
+static cudaError_t inverse_factor(const float* Y, int m, int r, double* partial, double* G, double* X, float* X32, int diagonal,
+                                  int32_t* dev_status, cudaStream_t stream) {
   if (r > kMaxBlocks * NB) return cudaErrorInvalidValue;
   static PerDeviceFlag gram_set, chol_set;
   if (cudaError_t e = ensure_dynamic_smem(gram_kernel, kGramSmem, gram_set); e != cudaSuccess) return e;
@@ -408,8 +421,25 @@ cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaError_t e = cudaLaunchKernelEx(&cfg, cholesky_kernel, G, X, r, X32, dev_status); e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&cfg, cholesky_kernel, G, X, r, X32, diagonal, dev_status);
+}
+
+cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G, double* X, float* X32, float* Q,
+                        int32_t* dev_status, cudaStream_t stream) {
+  if (cudaError_t e = inverse_factor(Y, m, r, partial, G, X, X32, 1, dev_status, stream); e != cudaSuccess) return e;
   return gemm_f32(0, 0, m, r, r, 1.f, Y, r, 0, X32, r, 0, Q, r, 0, 1, dev_status, stream);
+}
+
+// A column of Q = Y X is its own diagonal product and little else, and a product through the split is up to 2^-23 short (the
+// accumulator truncates): the columns came out 4.5e-8 short, all alike, which made Q^T Q differ from I by 9.5e-8 of sqrt(r)
+// (a triangular solve: 6.1e-8).  So the diagonal is left out of the matrix product and added in fp64: 3.4e-8.
+cudaError_t cholesky_qr_last(float* Q, int m, int r, double* partial, double* G, double* X, float* X32, float* P,
+                             int32_t* dev_status, cudaStream_t stream) {
+  if (cudaError_t e = inverse_factor(Q, m, r, partial, G, X, X32, 0, dev_status, stream); e != cudaSuccess) return e;
+  if (cudaError_t e = gemm_f32(0, 0, m, r, r, 1.f, Q, r, 0, X32, r, 0, P, r, 0, 1, dev_status, stream); e != cudaSuccess) return e;
+  const int columns = (r + 255) / 256, rows = 1184 / columns;
+  add_diagonal_kernel<<<dim3(columns, m < rows ? m : rows), 256, 0, stream>>>(P, Q, m, r, X);
+  return cudaGetLastError();
 }
 
 }  // namespace conv

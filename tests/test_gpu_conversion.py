@@ -255,6 +255,20 @@ def test_top_subspace_captures_what_the_leading_eigenvectors_capture(m, r):
     assert np.linalg.norm(q @ q.T - R @ R.T) < 1e-2 * np.sqrt(r)      # the same subspace (projectors agree)
 
 
+@pytest.mark.parametrize('m,r', [(1000, 128), (700, 33), (600, 301), (50, 1)])
+def test_the_basis_is_orthonormal_to_one_rounding_an_element(m, r):
+    # rounding q_i and q_j to fp32 moves their product by 2 x 2^-24 at most (the pass itself works in fp64 or on differences)
+    gu.ensure_built()
+    rng = np.random.default_rng(80 + m)
+    x = rng.standard_normal((2 * m, m)) * np.arange(1, m + 1) ** -0.5
+    Q = _dev(rng.standard_normal((m, r)))
+    scratch = torch.empty(binding.transmla_conv_subspace_scratch_bytes(m, r), dtype=torch.uint8, device='cuda')
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    binding.transmla_conv_top_subspace(_dev(x.T @ x), Q, 5, scratch, status)
+    q = _f64(Q)
+    assert int(status.item()) == 0 and np.abs(q.T @ q - np.eye(r)).max() < 2.0 ** -23
+
+
 def test_whole_conversion_step_by_step_against_the_oracle():
     # activations -> per-group covariances -> rotations -> rotated W_K -> alpha -> joint second moment -> basis -> rewrite
     gu.ensure_built()
