@@ -302,6 +302,11 @@ transmla_status_t transmla_selftest_bounded_wait(int32_t* dev_status, long long*
 transmla_status_t transmla_selftest_conv_gemm(int pairs, int M, int N, int K, const float* A, const float* B, float* C,
                                               int32_t* dev_status, void* stream);
 
+/* Diagnostic: transmla_conv_top_subspace with the cluster of its Cholesky factor limited to most_ctas CTAs (1, 2, 4, 8 or
+ * 16), as on a device or partition that holds no larger one. */
+transmla_status_t transmla_selftest_conv_subspace(const float* Cmat, int m, int r, int iters, float* Q, void* scratch,
+                                                  size_t scratch_bytes, int most_ctas, int32_t* dev_status, void* stream);
+
 /* FP8 latent cache (the paper's abstract names FP8 quantisation as combinable with the method and gives no detail; the
  * stored format is this library's own).  Only r = 512, dR = 64.  A token's row is TRANSMLA_FP8_ROW_BYTES = 656 bytes:
  *     bytes   0..511   e4m3 codes (OCP 8-bit float: 1 sign, 4 exponent bits with bias 7, 3 mantissa bits, largest

@@ -31,12 +31,14 @@ cudaError_t balance_concat(const float* k_nope, int n, int mk, const float* v, i
                            cudaStream_t stream);
 // Cholesky QR: Q [m,r] = Y L^-T with Y^T Y = L L^T, r <= 1024.  Scratch: partial [gram_slices(r)][r,r], G [r,r] and X [r,r]
 // in fp64, X32 [r,r] (L^-T in fp32).  Q must not alias Y.  Sets TRANSMLA_DEV_NUMERIC if the Gram matrix is not positive definite.
+// most_ctas: the factor's cluster is no larger (a power of two).
+constexpr int kOrthCluster = 16;
 int gram_slices(int r);
 cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G, double* X, float* X32, float* Q,
-                        int32_t* dev_status, cudaStream_t stream);
+                        int32_t* dev_status, cudaStream_t stream, int most_ctas = kOrthCluster);
 // The pass that leaves the result, in place: Q <- Q L^-T, rounded once.  P [m,r] is scratch; the rest as above.
 cudaError_t cholesky_qr_last(float* Q, int m, int r, double* partial, double* G, double* X, float* X32, float* P,
-                             int32_t* dev_status, cudaStream_t stream);
+                             int32_t* dev_status, cudaStream_t stream, int most_ctas = kOrthCluster);
 
 }  // namespace conv
 }  // namespace transmla

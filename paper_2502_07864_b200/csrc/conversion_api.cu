@@ -97,8 +97,8 @@ size_t transmla_conv_subspace_scratch_bytes(int m, int r) {
   return subspace_layout(m, r).total;
 }
 
-transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, int iters, float* Q, void* scratch,
-                                             size_t scratch_bytes, int32_t* dev_status, void* stream) {
+static transmla_status_t top_subspace(const float* Cmat, int m, int r, int iters, float* Q, void* scratch, size_t scratch_bytes,
+                                      int most_ctas, int32_t* dev_status, void* stream) {
   if (!Cmat || !Q || !scratch) return TRANSMLA_ERR_NULL;
   if (m < 1 || r < 1 || r > m || r > 1024 || iters < 1) return TRANSMLA_ERR_SHAPE;
   if (!al16(Cmat) || !al16(Q) || (reinterpret_cast<uintptr_t>(scratch) & 255)) return TRANSMLA_ERR_ALIGN;
@@ -111,7 +111,7 @@ transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, in
   // orthonormal to fp32 resolution by the two passes at the start and the extra pass at the end.
   auto orth = [&](const float* from, float* to) {
     return conv::cholesky_qr(from, m, r, reinterpret_cast<double*>(w + l.partial), reinterpret_cast<double*>(w + l.g),
-                             reinterpret_cast<double*>(w + l.x), reinterpret_cast<float*>(w + l.x32), to, dev_status, s) == cudaSuccess;
+                             reinterpret_cast<double*>(w + l.x), reinterpret_cast<float*>(w + l.x32), to, dev_status, s, most_ctas) == cudaSuccess;
   };
   if (!orth(Q, Y) || !orth(Y, Q)) return TRANSMLA_ERR_CUDA;
   for (int it = 0; it < iters; ++it) {
@@ -119,7 +119,18 @@ transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, in
     if (!orth(Y, Q)) return TRANSMLA_ERR_CUDA;
   }
   return done(conv::cholesky_qr_last(Q, m, r, reinterpret_cast<double*>(w + l.partial), reinterpret_cast<double*>(w + l.g),
-                                     reinterpret_cast<double*>(w + l.x), reinterpret_cast<float*>(w + l.x32), Y, dev_status, s));
+                                     reinterpret_cast<double*>(w + l.x), reinterpret_cast<float*>(w + l.x32), Y, dev_status, s, most_ctas));
+}
+
+transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, int iters, float* Q, void* scratch,
+                                             size_t scratch_bytes, int32_t* dev_status, void* stream) {
+  return top_subspace(Cmat, m, r, iters, Q, scratch, scratch_bytes, conv::kOrthCluster, dev_status, stream);
+}
+
+transmla_status_t transmla_selftest_conv_subspace(const float* Cmat, int m, int r, int iters, float* Q, void* scratch,
+                                                  size_t scratch_bytes, int most_ctas, int32_t* dev_status, void* stream) {
+  if (most_ctas < 1 || most_ctas > conv::kOrthCluster || (most_ctas & (most_ctas - 1))) return TRANSMLA_ERR_SHAPE;
+  return top_subspace(Cmat, m, r, iters, Q, scratch, scratch_bytes, most_ctas, dev_status, stream);
 }
 
 }  // extern "C"

@@ -126,9 +126,10 @@ __global__ void sum_slices_kernel(const double* part, int r, int slices, double*
 //   each CTA   P(R,p) = B(R,p) L(p,p)^-T for its blocks R of column p: G rows below p, and X rows up to p
 // and one cluster barrier.  What bounds it is the chain of r square roots and the updates between them, about 300 cycles
 // each, with the fp64 units beside it: a block's product takes one SM's units 1000 cycles, and a panel has about 100 of them.
+// (A device that cannot hold 16 such CTAs in a cluster gets 8, 4, .. of them: what it holds at once is asked.)
 // At r = 512: 359 us by 8 CTAs with the own blocks one a warp, 221 us by 16 (the cluster's size limit with the opt-in), four
 // rows of a block a warp and whole lines moved.  Rows and columns beyond r behave as an identity.
-constexpr int NB = 32, kCluster = 16, kCholThreads = 256, kPitch = NB + 1, kBlock = NB * kPitch;
+constexpr int NB = 32, kCluster = kOrthCluster, kCholThreads = 256, kPitch = NB + 1, kBlock = NB * kPitch;
 constexpr int kMaxBlocks = 1024 / NB, kMaxOwn = kMaxBlocks / kCluster;
 // doubles: D, W, P(p,p-1), col[2][32], the CTA's blocks of column p, two operands for each of warps 1-7
 constexpr int kCholSmem = (3 * kBlock + 2 * NB + kMaxOwn * kBlock + 14 * kBlock) * 8;
@@ -223,6 +224,66 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int diagonal, int32_t* 
   double* opB = opA + kBlock;
   bool bad = false;
 
+  // The blocks of column p of this CTA: list entry e is G row p + 1 + e, then X rows 0 .. p.  At most kMaxOwn at a time,
+  // entries `first`, first + ctas ..: formed in Bs by warps 1-7, four rows a warp, then multiplied by W by all.
+  auto form_blocks = [&](int p, int first) {
+    for (int own = 0, e = first; own < kMaxOwn && e < n; e += ctas, ++own) {
+      const int R = e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p), q = R - n;  // (q < 0 for G rows)
+      double* B = Bs + own * kBlock;
+      for (int slab = warp - 1; slab < NB / 4; slab += 7) {
+        double acc[1][4] = {{0.0, 0.0, 0.0, 0.0}};
+        const int row = 4 * slab + (lane >> 3);
+        if (q == p) {  // nothing stored yet in X rows p - 1 (zeros) and p (the identity's block)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[0][j] = row == 2 * (lane & 7) + (j & 1) + 16 * (j >> 1) ? 1.0 : 0.0;
+        } else {
+          if (R < n || q < p - 1) load_elements(v, R, p, slab, acc, lane);
+          if (p > 0) {
+            double x[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              bool in;
+              const double* g = v.at(R, p - 1, 4 * slab + i, lane, in);
+              x[i] = in ? __ldcg(g) : 0.0;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) opA[i * kPitch + lane] = x[i];
+            __syncwarp();
+            warp_product(acc, opA, Pp, lane);
+            __syncwarp();
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) B[row * kPitch + 2 * (lane & 7) + (j & 1) + 16 * (j >> 1)] = acc[0][j];
+      }
+    }
+  };
+  // P(R,p) = B W.  W is an upper triangle: a warp's four columns need only the rows of W up to the last of them
+  auto finish_blocks = [&](int p, int first) {
+    const int lo = tid & 15, up = tid >> 4;
+    for (int own = 0, e = first; own < kMaxOwn && e < n; e += ctas, ++own) {
+      const int R = e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p);
+      const double* B = Bs + own * kBlock;
+      const double* b = B + lo * kPitch;
+      const double* w = W + 2 * up;
+      double o[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll 4
+      for (int k = 0; k < 4 * warp + 4; ++k) {
+        const double b0 = b[k], b1 = b[16 * kPitch + k], w0 = w[k * kPitch], w1 = w[k * kPitch + 1];
+        o[0][0] = fma(b0, w0, o[0][0]); o[0][1] = fma(b0, w1, o[0][1]);
+        o[1][0] = fma(b1, w0, o[1][0]); o[1][1] = fma(b1, w1, o[1][1]);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          bool in;
+          double* g = v.at(R, p, lo + 16 * i, 2 * up + j, in);
+          if (in) __stcg(g, o[i][j]);
+        }
+    }
+  };
+
   for (int p = 0; p < n; ++p) {
     // ---- D, by all warps: 4 elements a thread
     const int lo = tid & 15, up = tid >> 4;  // rows and columns lo, lo + 16, up, up + 16 of a block
@@ -289,38 +350,7 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int diagonal, int32_t* 
 #pragma unroll
       for (int j = 0; j < NB; ++j) W[lane * kPitch + j] = x[j];
     } else {
-      // ---- this CTA's blocks of column p, four rows a warp: list entry e is G row p + 1 + e, then X rows 0 .. p
-      int own = 0;
-      for (int e = cta; e < n; e += ctas, ++own) {
-        const int R = e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p), q = R - n;  // (q < 0 for G rows)
-        double* B = Bs + own * kBlock;
-        for (int slab = warp - 1; slab < NB / 4; slab += 7) {
-          double acc[1][4] = {{0.0, 0.0, 0.0, 0.0}};
-          const int row = 4 * slab + (lane >> 3);
-          if (q == p) {  // nothing stored yet in X rows p - 1 (zeros) and p (the identity's block)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[0][j] = row == 2 * (lane & 7) + (j & 1) + 16 * (j >> 1) ? 1.0 : 0.0;
-          } else {
-            if (R < n || q < p - 1) load_elements(v, R, p, slab, acc, lane);
-            if (p > 0) {
-              double x[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                bool in;
-                const double* g = v.at(R, p - 1, 4 * slab + i, lane, in);
-                x[i] = in ? __ldcg(g) : 0.0;
-              }
-#pragma unroll
-              for (int i = 0; i < 4; ++i) opA[i * kPitch + lane] = x[i];
-              __syncwarp();
-              warp_product(acc, opA, Pp, lane);
-              __syncwarp();
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) B[row * kPitch + 2 * (lane & 7) + (j & 1) + 16 * (j >> 1)] = acc[0][j];
-        }
-      }
+      form_blocks(p, cta);
       // ---- panel p - 1 on the blocks behind column p: column j takes G rows j .. n-1 and X rows 0 .. p-1
       if (p > 0) {
         int t = cta * 7 + warp - 1;
@@ -342,30 +372,12 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int diagonal, int32_t* 
       }
     }
     __syncthreads();
-    // ---- P(R,p) = B W.  W is an upper triangle: a warp's four columns need only the rows of W up to the last of them
-    {
-      int own = 0;
-      for (int e = cta; e < n; e += ctas, ++own) {
-        const int R = e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p);
-        const double* B = Bs + own * kBlock;
-        const double* b = B + lo * kPitch;
-        const double* w = W + 2 * up;
-        double o[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll 4
-        for (int k = 0; k < 4 * warp + 4; ++k) {
-          const double b0 = b[k], b1 = b[16 * kPitch + k], w0 = w[k * kPitch], w1 = w[k * kPitch + 1];
-          o[0][0] = fma(b0, w0, o[0][0]); o[0][1] = fma(b0, w1, o[0][1]);
-          o[1][0] = fma(b1, w0, o[1][0]); o[1][1] = fma(b1, w1, o[1][1]);
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            bool in;
-            double* g = v.at(R, p, lo + 16 * i, 2 * up + j, in);
-            if (in) __stcg(g, o[i][j]);
-          }
-      }
+    finish_blocks(p, cta);
+    for (int first = cta + kMaxOwn * ctas; first < n; first += kMaxOwn * ctas) {  // (a cluster below its full size)
+      __syncthreads();
+      if (warp > 0) form_blocks(p, first);
+      __syncthreads();
+      finish_blocks(p, first);
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
@@ -398,35 +410,53 @@ int gram_slices(int r) {  // slices of the sum over rows: what fills the device 
 
 // X = L^-T of Y^T Y = L L^T, in fp64, and X32 in fp32, with its diagonal or without.
 static cudaError_t inverse_factor(const float* Y, int m, int r, double* partial, double* G, double* X, float* X32, int diagonal,
-                                  int32_t* dev_status, cudaStream_t stream) {
+                                  int most_ctas, int32_t* dev_status, cudaStream_t stream) {
   if (r > kMaxBlocks * NB) return cudaErrorInvalidValue;
   static PerDeviceFlag gram_set, chol_set;
   if (cudaError_t e = ensure_dynamic_smem(gram_kernel, kGramSmem, gram_set); e != cudaSuccess) return e;
   if (cudaError_t e = ensure_dynamic_smem(cholesky_kernel, kCholSmem, chol_set); e != cudaSuccess) return e;
-  if (cudaError_t e = cudaFuncSetAttribute(cholesky_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); e != cudaSuccess) return e;
   const int t = (r + GT - 1) / GT, slices = gram_slices(r);
   const int ks = ((m + slices - 1) / slices + GK - 1) / GK * GK;
   gram_kernel<<<dim3(t * (t + 1) / 2, slices), 256, kGramSmem, stream>>>(Y, m, r, ks, partial);
   sum_slices_kernel<<<dim3((r + 127) / 128, r), 128, 0, stream>>>(partial, r, slices, G);
-  int ctas = 1;  // one cluster, of no more CTAs than a panel has blocks for
-  while (ctas < kCluster && ctas < (r + NB - 1) / NB) ctas *= 2;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctas);
   cfg.blockDim = dim3(kCholThreads);
   cfg.dynamicSmemBytes = kCholSmem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ctas;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  // One cluster, of no more CTAs than a panel has blocks for, and no more than the device holds at once in a cluster.
+  static PerDeviceFlag fits[kMaxBlocks];  // by size: 1 it does, -1 it does not, 0 not asked yet
+  const int slot = current_device_slot();
+  int ctas = 1;
+  while (ctas < most_ctas && ctas < (r + NB - 1) / NB) ctas *= 2;
+  for (; ctas > 1; ctas /= 2) {
+    int known = slot >= 0 ? fits[ctas].value[slot].load(std::memory_order_acquire) : 0;
+    if (known == 0) {
+      int clusters = 0;
+      cfg.gridDim = dim3(ctas);
+      attr[0].val.clusterDim.x = ctas;
+      if ((ctas > 8 && cudaFuncSetAttribute(cholesky_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+          cudaOccupancyMaxActiveClusters(&clusters, cholesky_kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        clusters = 0;
+      }
+      known = clusters > 0 ? 1 : -1;
+      if (slot >= 0) fits[ctas].value[slot].store(known, std::memory_order_release);
+    }
+    if (known > 0) break;
+  }
+  cfg.gridDim = dim3(ctas);
+  attr[0].val.clusterDim.x = ctas;
   return cudaLaunchKernelEx(&cfg, cholesky_kernel, G, X, r, X32, diagonal, dev_status);
 }
 
 cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G, double* X, float* X32, float* Q,
-                        int32_t* dev_status, cudaStream_t stream) {
-  if (cudaError_t e = inverse_factor(Y, m, r, partial, G, X, X32, 1, dev_status, stream); e != cudaSuccess) return e;
+                        int32_t* dev_status, cudaStream_t stream, int most_ctas) {
+  if (cudaError_t e = inverse_factor(Y, m, r, partial, G, X, X32, 1, most_ctas, dev_status, stream); e != cudaSuccess) return e;
   return gemm_f32(0, 0, m, r, r, 1.f, Y, r, 0, X32, r, 0, Q, r, 0, 1, dev_status, stream);
 }
 
@@ -434,8 +464,8 @@ cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G
 // accumulator truncates): the columns came out 4.5e-8 short, all alike, which made Q^T Q differ from I by 9.5e-8 of sqrt(r)
 // (a triangular solve: 6.1e-8).  So the diagonal is left out of the matrix product and added in fp64: 3.4e-8.
 cudaError_t cholesky_qr_last(float* Q, int m, int r, double* partial, double* G, double* X, float* X32, float* P,
-                             int32_t* dev_status, cudaStream_t stream) {
-  if (cudaError_t e = inverse_factor(Q, m, r, partial, G, X, X32, 0, dev_status, stream); e != cudaSuccess) return e;
+                             int32_t* dev_status, cudaStream_t stream, int most_ctas) {
+  if (cudaError_t e = inverse_factor(Q, m, r, partial, G, X, X32, 0, most_ctas, dev_status, stream); e != cudaSuccess) return e;
   if (cudaError_t e = gemm_f32(0, 0, m, r, r, 1.f, Q, r, 0, X32, r, 0, P, r, 0, 1, dev_status, stream); e != cudaSuccess) return e;
   const int columns = (r + 255) / 256, rows = 1184 / columns;
   add_diagonal_kernel<<<dim3(columns, m < rows ? m : rows), 256, 0, stream>>>(P, Q, m, r, X);

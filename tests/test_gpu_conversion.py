@@ -255,6 +255,22 @@ def test_top_subspace_captures_what_the_leading_eigenvectors_capture(m, r):
     assert np.linalg.norm(q @ q.T - R @ R.T) < 1e-2 * np.sqrt(r)      # the same subspace (projectors agree)
 
 
+@pytest.mark.parametrize('most', [1, 2, 4, 8])
+@pytest.mark.parametrize('m,r', [(400, 70), (700, 512), (1100, 1024)])
+def test_the_factor_in_smaller_clusters(m, r, most):
+    # a CTA then owns more blocks of a panel than it holds at once; every block is the same sum in the same order
+    gu.ensure_built()
+    rng = np.random.default_rng(90 + m)
+    x = rng.standard_normal((2 * m, m)) * np.arange(1, m + 1) ** -0.5
+    C, q0 = _dev(x.T @ x), _dev(rng.standard_normal((m, r)))
+    scratch = torch.empty(binding.transmla_conv_subspace_scratch_bytes(m, r), dtype=torch.uint8, device='cuda')
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    full, part = q0.clone(), q0.clone()
+    binding.transmla_conv_top_subspace(C, full, 2, scratch, status)
+    binding.transmla_selftest_conv_subspace(C, part, 2, scratch, most, status)
+    assert int(status.item()) == 0 and torch.equal(full, part)
+
+
 @pytest.mark.parametrize('m,r', [(1000, 128), (700, 33), (600, 301), (50, 1)])
 def test_the_basis_is_orthonormal_to_one_rounding_an_element(m, r):
     # rounding q_i and q_j to fp32 moves their product by 2 x 2^-24 at most (the pass itself works in fp64 or on differences)
