@@ -33,23 +33,27 @@ cudaError_t gather_segments(const float* K, int n, int g, int d, int fold, float
 }
 
 // Y[(q / fold, 2 (G fold + q % fold) + im), c] = sum_i U_G[i, q] X[seg_pos(G, i) + im, c]   (Eq. 18)
-// U_G and 64 columns of X's rows in shared memory, a thread has 8 values of q x 4 columns.  Bound by the fp32 units: 32
-// multiply-adds a thread and step against three 16-byte reads.  g = 32, d = 128, fold = 4, C = 4096: 1.2 ms with one column a
-// thread and X read again for every 8 q, now 187 us.
-constexpr int kRotMax = 128, kRotCols = 64, kRotThreads = 256;
+// U_G and some columns of X's rows in shared memory, a thread has 8 values of q x 4 columns: a block of order 128 has 64
+// columns, one of order 64 has 128, .. of order 8 1024, so that no thread is without values of q.  Bound by the fp32 units (32
+// multiply-adds a thread and step against three 16-byte reads), small orders by memory.  d = 128, C = 4096: g = 32, fold = 4
+// 1.2 ms with one column a thread and X read again for every 8 q, now 180 us; g = 8, fold = 1 16.5 us, now 7.8 (43 with 64 columns
+// a block whatever the order).
+constexpr int kRotMax = 128, kRotThreads = 256;
 
+template <int cols>  // of X a block
 __global__ void __launch_bounds__(kRotThreads) rorope_apply_kernel(const float* X, int C, const float* U, int g, int d, int fold, float* Y) {
-  const int m = g * fold, mp = (m + 7) & ~7, G = blockIdx.y, im = blockIdx.z, c0 = blockIdx.x * kRotCols;
-  const int tid = threadIdx.x, tx = tid & 15, q0 = (tid >> 4) * 8, c = c0 + tx * 4;
+  const int m = g * fold, mp = (m + 7) & ~7, G = blockIdx.y, im = blockIdx.z, c0 = blockIdx.x * cols;
+  constexpr int across = cols / 4;
+  const int tid = threadIdx.x, tx = tid & (across - 1), row0 = tid / across, q0 = row0 * 8, c = c0 + tx * 4;
   extern __shared__ __align__(16) float rot_s[];
   float* u_s = rot_s;               // [m][mp], zeros behind column m
-  float* x_s = u_s + m * mp;        // [m][kRotCols]
+  float* x_s = u_s + m * mp;        // [m][cols]
   const bool vec = (C & 3) == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15) == 0;
   for (int e = tid; e < m * mp; e += kRotThreads) {
     const int i = e / mp, q = e - i * mp;
     u_s[e] = q < m ? U[(static_cast<size_t>(G) * m + i) * m + q] : 0.f;
   }
-  for (int i = tid >> 4; i < m; i += kRotThreads / 16) {
+  for (int i = row0; i < m; i += kRotThreads / across) {
     const float* src = X + static_cast<size_t>(seg_pos(G, i, g, d, fold) + im) * C + c;
     float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
     if (vec) { if (c < C) x = *reinterpret_cast<const float4*>(src); }
@@ -59,14 +63,14 @@ __global__ void __launch_bounds__(kRotThreads) rorope_apply_kernel(const float* 
       if (c + 2 < C) x.z = src[2];
       if (c + 3 < C) x.w = src[3];
     }
-    *reinterpret_cast<float4*>(x_s + i * kRotCols + tx * 4) = x;
+    *reinterpret_cast<float4*>(x_s + i * cols + tx * 4) = x;
   }
   __syncthreads();
   if (q0 >= m) return;
   float acc[8][4] = {};
 #pragma unroll 4
   for (int i = 0; i < m; ++i) {
-    const float4 x = *reinterpret_cast<const float4*>(x_s + i * kRotCols + tx * 4);
+    const float4 x = *reinterpret_cast<const float4*>(x_s + i * cols + tx * 4);
     const float4 ua = *reinterpret_cast<const float4*>(u_s + i * mp + q0), ub = *reinterpret_cast<const float4*>(u_s + i * mp + q0 + 4);
     const float u[8] = {ua.x, ua.y, ua.z, ua.w, ub.x, ub.y, ub.z, ub.w};
 #pragma unroll
@@ -91,12 +95,21 @@ __global__ void __launch_bounds__(kRotThreads) rorope_apply_kernel(const float* 
 cudaError_t rorope_apply(const float* X, int C, const float* U, int g, int d, int fold, float* Y, cudaStream_t stream) {
   const int m = g * fold, mp = (m + 7) & ~7, groups = d / 2 / fold;
   if (m > kRotMax) return cudaErrorInvalidValue;
-  const size_t smem = static_cast<size_t>(m) * (mp + kRotCols) * sizeof(float);
-  static PerDeviceFlag smem_set;
-  if (cudaError_t e = ensure_dynamic_smem(rorope_apply_kernel, kRotMax * (kRotMax + kRotCols) * 4, smem_set); e != cudaSuccess) return e;
-  dim3 grid((C + kRotCols - 1) / kRotCols, groups, 2);
-  rorope_apply_kernel<<<grid, kRotThreads, smem, stream>>>(X, C, U, g, d, fold, Y);
-  return cudaGetLastError();
+  auto launch = [&](auto kernel, int cols) {
+    const size_t smem = static_cast<size_t>(m) * (mp + cols) * sizeof(float);
+    kernel<<<dim3((C + cols - 1) / cols, groups, 2), kRotThreads, smem, stream>>>(X, C, U, g, d, fold, Y);
+    return cudaGetLastError();
+  };
+  if (m <= 8) return launch(rorope_apply_kernel<1024>, 1024);
+  if (m <= 16) return launch(rorope_apply_kernel<512>, 512);
+  if (m <= 32) return launch(rorope_apply_kernel<256>, 256);
+  static PerDeviceFlag smem_set[2];  // above the default limit
+  if (m <= 64) {
+    if (cudaError_t e = ensure_dynamic_smem(rorope_apply_kernel<128>, 64 * (64 + 128) * 4, smem_set[0]); e != cudaSuccess) return e;
+    return launch(rorope_apply_kernel<128>, 128);
+  }
+  if (cudaError_t e = ensure_dynamic_smem(rorope_apply_kernel<64>, kRotMax * (kRotMax + 64) * 4, smem_set[1]); e != cudaSuccess) return e;
+  return launch(rorope_apply_kernel<64>, 64);
 }
 
 // ------------------------------------------------------------------------------------------------ Eq. 19

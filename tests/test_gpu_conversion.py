@@ -205,7 +205,8 @@ def test_rorope_apply_matches_the_oracle_and_keeps_the_rope_inner_product(fold):
             assert abs(got_ip - want_ip) < 1e-4 * max(1.0, abs(want_ip))
 
 
-@pytest.mark.parametrize('g,d,fold,C', [(32, 128, 4, 192), (3, 16, 4, 68), (5, 4, 2, 65), (1, 2, 1, 3)])
+@pytest.mark.parametrize('g,d,fold,C', [(32, 128, 4, 192), (3, 16, 4, 68), (5, 4, 2, 65), (1, 2, 1, 3), (8, 8, 1, 1028),
+                                        (9, 4, 1, 515), (16, 8, 2, 260), (33, 4, 1, 129), (65, 2, 1, 66)])
 def test_rorope_apply_at_the_edges_of_its_tiles(g, d, fold, C):
     # the largest order, orders off the 8 values of a thread, columns off the tile of 64 and off the 4 of a thread
     gu.ensure_built()
