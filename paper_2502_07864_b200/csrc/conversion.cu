@@ -194,6 +194,8 @@ cudaError_t balance_concat(const float* k_nope, int n, int mk, const float* v, i
 // the next round's angles: two barriers a round.  Index pairs advance by one a round, so no thread divides.
 // 16 matrices of order 128: 9.15 ms with columns and rows of A in passes of their own, 1.6 to 2.7 ms (by sweeps needed) in
 // this form, and eigenvalues ten times closer because the angles' own 2 x 2 blocks are set to their exact form.
+// A warp for every pair of V's columns and two for the angles, 32 at most: a small order then leaves room for several matrices
+// on an SM.  512 matrices of order 16: 127 us before, 206 with 32 warps whatever the order, now 103.
 constexpr int kEigMax = 128, kEigSweeps = 30, kEigThreads = 1024;
 constexpr int kEigBlocks = (kEigMax / 2) * (kEigMax / 2 - 1) / 2;                  // pairs of index pairs
 constexpr int kEigOwn = (kEigBlocks + kEigThreads - 1) / kEigThreads;             // of one thread
@@ -205,7 +207,7 @@ __device__ __forceinline__ float eig_block_sum(float x, float* red) {
   __syncthreads();  // the readers of the call before are done
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
   __syncthreads();
-  x = red[threadIdx.x & 31];
+  x = (threadIdx.x & 31) < blockDim.x / 32 ? red[threadIdx.x & 31] : 0.f;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   return x;
@@ -222,9 +224,9 @@ __global__ void __launch_bounds__(kEigThreads) jacobi_eigh_kernel(const float* a
   __shared__ float2 cs[2][kEigMax / 2];  // cosine and sine of each pair, this round's and the next one's
   __shared__ float red[kEigThreads / 32];
   __shared__ int order[kEigMax];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, threads = blockDim.x, warps = threads >> 5;
   const float* src = a_in + static_cast<size_t>(blockIdx.x) * m * m;
-  for (int e = tid; e < mm * mm; e += kEigThreads) {
+  for (int e = tid; e < mm * mm; e += threads) {
     const int i = e / mm, j = e % mm;
     A[i * ld + j] = i < m && j < m ? 0.5f * (src[i * m + j] + src[j * m + i]) : 0.f;  // exactly symmetric whatever rounding the input carries
     V[i * ld + j] = i == j ? 1.f : 0.f;
@@ -233,7 +235,7 @@ __global__ void __launch_bounds__(kEigThreads) jacobi_eigh_kernel(const float* a
   int own_k[kEigOwn], own_l[kEigOwn];
 #pragma unroll
   for (int u = 0; u < kEigOwn; ++u) {
-    const int e = tid + u * kEigThreads;
+    const int e = tid + u * threads;
     own_k[u] = -1;
     own_l[u] = 0;
     if (half < 2) continue;
@@ -267,7 +269,7 @@ __global__ void __launch_bounds__(kEigThreads) jacobi_eigh_kernel(const float* a
   for (int sweep = 0; sweep < kEigSweeps; ++sweep) {
     // convergence: off-diagonal sum of squares against the whole
     float off = 0.f, diag = 0.f;
-    for (int i = warp; i < m; i += kEigThreads / 32)
+    for (int i = warp; i < m; i += warps)
       for (int j = lane; j < m; j += 32) {
         const float x = A[i * ld + j];
         if (i == j) diag += x * x; else off += x * x;
@@ -296,7 +298,7 @@ __global__ void __launch_bounds__(kEigThreads) jacobi_eigh_kernel(const float* a
       if (warp < 2) {
         if (rd + 1 < ring) find_angles(rd + 1);
       } else {
-        for (int k = warp - 2; k < half; k += kEigThreads / 32 - 2) {  // V <- V J, a pair of columns a warp
+        for (int k = warp - 2; k < half; k += warps - 2) {  // V <- V J, a pair of columns a warp
           const float2 r = rot[k];
           float* vp = V + first_of(k, rd) + lane * ld;
           float* vq = V + second_of(k, rd) + lane * ld;
@@ -326,8 +328,8 @@ __global__ void __launch_bounds__(kEigThreads) jacobi_eigh_kernel(const float* a
   __syncthreads();
   float* w = eigvals + static_cast<size_t>(blockIdx.x) * m;
   float* vec = eigvecs + static_cast<size_t>(blockIdx.x) * m * m;
-  for (int q = tid; q < m; q += kEigThreads) w[q] = A[order[q] * ld + order[q]];
-  for (int e = tid; e < m * m; e += kEigThreads) { const int i = e / m, q = e % m; vec[e] = V[i * ld + order[q]]; }
+  for (int q = tid; q < m; q += threads) w[q] = A[order[q] * ld + order[q]];
+  for (int e = tid; e < m * m; e += threads) { const int i = e / m, q = e % m; vec[e] = V[i * ld + order[q]]; }
 }
 
 cudaError_t sym_eig(float* a, int batch, int m, float* eigvals, float* eigvecs, int32_t* dev_status, cudaStream_t stream) {
@@ -336,7 +338,8 @@ cudaError_t sym_eig(float* a, int batch, int m, float* eigvals, float* eigvecs, 
   if (cudaError_t e = cudaFuncSetAttribute(jacobi_eigh_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
       e != cudaSuccess)
     return e;
-  jacobi_eigh_kernel<<<batch, kEigThreads, smem, stream>>>(a, m, eigvals, eigvecs, dev_status);
+  const int pairs = (m + 1) / 2, warps = pairs + 2 < kEigThreads / 32 ? pairs + 2 : kEigThreads / 32;
+  jacobi_eigh_kernel<<<batch, warps * 32, smem, stream>>>(a, m, eigvals, eigvecs, dev_status);
   return cudaGetLastError();
 }
 }  // namespace conv

@@ -163,9 +163,9 @@ def test_symmetric_eigendecomposition(m, batch):
             assert abs(cv.captured_energy(a[b], v[b][:, :keep]) - want[:keep].sum()) < 1e-4 * top
 
 
-@pytest.mark.parametrize('m,batch', [(3, 2), (66, 2), (97, 1), (127, 2)])
+@pytest.mark.parametrize('m,batch', [(3, 2), (66, 2), (97, 1), (127, 2), (1, 2), (2, 3), (5, 400), (16, 300), (59, 3)])
 def test_symmetric_eigendecomposition_of_odd_orders(m, batch):
-    # odd orders get an index of zeros, and odd numbers of pairs split the triangle of blocks unevenly
+    # odd orders get an index of zeros, odd numbers of pairs split the triangle of blocks unevenly, small orders take fewer warps
     gu.ensure_built()
     rng = np.random.default_rng(130 + m)
     x = rng.standard_normal((batch, 3 * m + 2, m)) * (np.arange(1, m + 1) ** -0.7)
