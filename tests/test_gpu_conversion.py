@@ -235,6 +235,17 @@ def test_alpha_and_balanced_concatenation():
     assert _rel(z[:, :mk], k.astype(np.float64) / float(alpha.item())) < 1e-6 and np.array_equal(z[:, mk:], v.astype(np.float64))
 
 
+@pytest.mark.parametrize('n,mk,mv', [(1, 1, 1), (700, 4, 8), (5000, 16, 16), (333, 5, 2), (3, 3968, 4096), (129, 1001, 24)])
+def test_concatenation_of_short_and_long_rows(n, mk, mv):
+    # from one thread a row to a block a row, rows that are and are not whole 16 bytes
+    gu.ensure_built()
+    k, v = torch.randn(n, mk, device='cuda'), torch.randn(n, mv, device='cuda')
+    alpha = torch.tensor([1.7], device='cuda')
+    z = torch.full((n, mk + mv), float('nan'), device='cuda')
+    binding.transmla_conv_balance_concat(k, v, alpha, z)
+    assert torch.equal(z, torch.cat([k * (1.0 / alpha), v], dim=1))
+
+
 @pytest.mark.parametrize('m,r', [(96, 24), (300, 64), (333, 33), (40, 1), (200, 129), (1100, 1024)])
 def test_top_subspace_captures_what_the_leading_eigenvectors_capture(m, r):
     gu.ensure_built()
