@@ -330,8 +330,10 @@ cholesky_kernel(double* G, double* X, int r, float* X32, int diagonal, int32_t* 
 #pragma unroll
       for (int j = 0; j < NB; ++j) { a[j] = D[lane * kPitch + j]; x[j] = j == lane ? 1.0 : 0.0; }
       double pivot = a[0];
+      const int left = r - p * NB;  // what is behind is an identity's already
 #pragma unroll
       for (int k = 0; k < NB; ++k) {
+        if (k % 8 == 0 && k >= left) break;
         double d = __shfl_sync(0xffffffffu, pivot, k);
         if (!(d > 0.0)) { bad = true; d = 1.0; }
         const double inv = rsqrt(d);
