@@ -270,7 +270,7 @@ transmla_status_t transmla_decode_step_host(const transmla_params_t* params, con
  *
  * Limits and rules:
  *   - transmla_workspace_layout(params).total_bytes must not exceed the capacity (with num_partitions == 0
- *     the call tries half the library's own partition count before it gives up), otherwise the call
+ *     the call tries as many as there are SMs to blocks of 32 query rows before it gives up), otherwise the call
  *     returns TRANSMLA_ERR_WORKSPACE and launches nothing.  The size grows with
  *     (num_partitions + B - 1) * S * H * r * 4 bytes; pass a smaller params->num_partitions to fit.
  *   - The first call on each device looks up the array's device address (with that device current)

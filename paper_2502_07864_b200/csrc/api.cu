@@ -106,19 +106,7 @@ transmla_status_t transmla_workspace_layout(const transmla_params_t* p, transmla
   transmla_status_t st = check_shape(p, false);
   if (st != TRANSMLA_OK) return st;
   int G = p->num_partitions;
-  if (G == 0) {
-    int sms = 0;
-    st = check_device(&sms);
-    if (st != TRANSMLA_OK) return st;
-    const int rows = decode_row_block(*p);
-    const int row_blocks = (p->q_len * p->num_heads + rows - 1) / rows;
-    G = sms / row_blocks;
-    // Small problems: no more partitions than a quarter of the pages the batch can hold, so that a partition
-    // keeps at least about four pages and a sequence is not cut into dozens of one-page partials.
-    const long long cap = (static_cast<long long>(p->batch) * p->max_pages_per_seq + 3) / 4;
-    if (G > cap) G = static_cast<int>(cap);
-    if (G < 1) G = 1;
-  }
+  if (G == 0 && (st = library_partitions(*p, decode_row_block(*p), &G)) != TRANSMLA_OK) return st;
   const size_t B = p->batch, SH = static_cast<size_t>(p->q_len) * p->num_heads;
   const size_t K = p->kv_lora_rank + p->qk_rope_dim;
   const size_t slots = static_cast<size_t>(G) + B - 1;
@@ -169,6 +157,19 @@ static transmla_status_t check_decode_args(const transmla_params_t* p, const voi
 // Host-side checks of a whole decode step, for callers inside the library that launch other kernels first.
 extern "C++" {
 namespace transmla {
+transmla_status_t library_partitions(const transmla_params_t& p, int rows, int* partitions) {
+  int sms = 0;
+  const transmla_status_t st = check_device(&sms);
+  if (st != TRANSMLA_OK) return st;
+  const int row_blocks = (p.q_len * p.num_heads + rows - 1) / rows;
+  int G = sms / row_blocks;
+  // Small problems: no more partitions than a quarter of the pages the batch can hold, so that a partition
+  // keeps at least about four pages and a sequence is not cut into dozens of one-page partials.
+  const long long cap = (static_cast<long long>(p.batch) * p.max_pages_per_seq + 3) / 4;
+  if (G > cap) G = static_cast<int>(cap);
+  *partitions = G < 1 ? 1 : G;
+  return TRANSMLA_OK;
+}
 transmla_status_t validate_step_args(const transmla_params_t* p, const void* x, const void* q_nope, const void* q_pe,
                                      const void* w_dkv_kr, const void* w_uk, const void* w_uv, const void* cache,
                                      const int32_t* page_table, const int32_t* seqlens, void* workspace,

@@ -189,6 +189,9 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// The partition count the library chooses for a kernel that takes `rows` query rows a CTA.
+transmla_status_t library_partitions(const transmla_params_t& p, int rows, int* partitions);
+
 // Every host-side check of transmla_decode_step, without launching anything.
 transmla_status_t validate_step_args(const transmla_params_t* p, const void* x, const void* q_nope, const void* q_pe,
                                      const void* w_dkv_kr, const void* w_uk, const void* w_uv, const void* cache,

@@ -53,8 +53,10 @@ transmla_status_t transmla_mla_attention_static(const transmla_params_t* params,
   if (st != TRANSMLA_OK) return st;
   transmla_params_t fitted = *params;
   if (lay.total_bytes > kStaticWorkspaceBytes && params->num_partitions == 0) {
-    // The library's own partition count is chosen for speed; half as many partitions need about half the partials.
-    fitted.num_partitions = (lay.num_partitions + 1) / 2;
+    // The library's own partition count is chosen for speed, as many as a kernel with 64 query rows a CTA has use for.  The
+    // count for 32 rows needs half the partials or fewer.
+    st = transmla::library_partitions(*params, transmla::kRowBlock, &fitted.num_partitions);
+    if (st != TRANSMLA_OK) return st;
     st = transmla_workspace_layout(&fitted, &lay);
     if (st != TRANSMLA_OK) return st;
     params = &fitted;

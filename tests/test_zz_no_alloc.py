@@ -52,6 +52,26 @@ def test_two_calls_in_a_row_match_the_workspace_path():
         gu.assert_lse_close(lifts.f64(lse), want_lse, 'lse vs oracle')
 
 
+def test_many_query_rows_that_fit_with_fewer_partitions():
+    # 1024 query rows: the library's own count (64 rows a CTA, 9) and half of it do not fit the array, that for 32 rows (4) does
+    gu.ensure_built()
+    shape = synth.MLAShape(H=256, dn=128, dR=64, dv=128, r=512, D=4096, S=4)
+    seqlens = [300, 4, 65]
+    case = synth.make_decode_case(shape, seqlens, 43)
+    pad = torch.full((3, 32 - case['page_table'].shape[1]), -1, dtype=torch.int32)
+    case['page_table'] = torch.cat([case['page_table'], pad], dim=1)
+    case, scale = gu.to_dev(case), gu.mla_scale(shape)
+    params = binding.make_params(shape, 3, case['cache'].shape[0], 32, scale)
+    assert binding.transmla_workspace_layout(params).total_bytes > binding.transmla_static_workspace_capacity()
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    out = torch.full((3, shape.S, shape.H, shape.dv), float('nan'), dtype=torch.bfloat16, device='cuda')
+    binding.transmla_mla_attention_static(params, case['q_nope'], case['q_pe'], case['w_uk'], case['w_uv'], case['cache'],
+                                          case['page_table'], case['seqlens'], out, None, status)
+    ref, _, ref_status, _, _ = gu.gpu_decode(shape, case, scale)
+    assert int(status.item()) == 0 and ref_status == 0
+    gu.assert_close(lifts.f64(out), lifts.f64(ref), 'static workspace vs caller workspace')
+
+
 def test_problem_larger_than_the_builtin_array_is_refused():
     gu.ensure_built()
     shape = synth.LLAMA2_7B
