@@ -84,7 +84,8 @@ typedef struct {
   int32_t batch;             /* B */
   int32_t num_partitions;    /* G: how many pieces the batch's pages are split into; 0 = library chooses
                                 (SMs / row blocks of 32 query rows, 64 where S*H > 32
-                                and r = 512; at most batch * max_pages_per_seq / 4).  With an explicit G
+                                and r = 512; at most batch * max_pages_per_seq / 4, of which
+                                the device leaves some empty when the batch holds few pages).  With an explicit G
                                 every partition handles exactly the page range of the plan and a rerun gives
                                 the same bits.  With 0, r = 512, dR = 64 and at least 8 partitions per
                                 sequence, the CTAs that share a sequence take its pages from a counter as they
@@ -116,7 +117,7 @@ typedef struct {
  *   partial_lse fp32  [G+B-1, S*H]      natural-log softmax denominator of the segment (-inf = empty)
  * Row index inside a slot is s*H + h. */
 typedef struct {
-  int32_t num_partitions;  /* the G actually used */
+  int32_t num_partitions;  /* the G that the workspace is laid out for, and that an explicit G means; 0 may plan for fewer */
   int32_t num_slots;       /* G + B - 1 */
   size_t q_hat_offset;
   size_t cum_pages_offset;

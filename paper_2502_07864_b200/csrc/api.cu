@@ -213,7 +213,7 @@ transmla_status_t transmla_mla_decode(const transmla_params_t* p, const void* q_
   if (st != TRANSMLA_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
-  if (launch_absorb_plan(*p, lay.num_partitions, static_cast<const __nv_bfloat16*>(q_nope),
+  if (launch_absorb_plan(*p, decode_partitioning(*p, lay.num_partitions), static_cast<const __nv_bfloat16*>(q_nope),
                          static_cast<const __nv_bfloat16*>(q_pe), static_cast<const __nv_bfloat16*>(w_uk),
                          reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset), seqlens,
                          reinterpret_cast<int32_t*>(ws + lay.cum_pages_offset),
@@ -236,6 +236,7 @@ transmla_status_t transmla_mla_combine(const transmla_params_t* p, const void* w
   if (st != TRANSMLA_OK) return st;
   const char* ws = static_cast<const char*>(workspace);
   cudaError_t e = launch_combine(*p, lay.num_partitions, reinterpret_cast<const int32_t*>(ws + lay.cum_pages_offset),
+                                 reinterpret_cast<const int32_t*>(ws + lay.plan_offset),
                                  reinterpret_cast<const float*>(ws + lay.partial_o_offset),
                                  reinterpret_cast<const float*>(ws + lay.partial_lse_offset),
                                  static_cast<const __nv_bfloat16*>(w_uv), static_cast<__nv_bfloat16*>(out), lse_out,
@@ -274,7 +275,8 @@ transmla_status_t transmla_mla_decode_fp8(const transmla_params_t* p, const void
   if (!decode_fp8_supported(*p)) return TRANSMLA_ERR_SHAPE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
-  if (launch_absorb_plan(*p, lay.num_partitions, static_cast<const __nv_bfloat16*>(q_nope),
+  const Partitioning parts = decode_fp8_partitioning(*p, lay.num_partitions);
+  if (launch_absorb_plan(*p, parts, static_cast<const __nv_bfloat16*>(q_nope),
                          static_cast<const __nv_bfloat16*>(q_pe), static_cast<const __nv_bfloat16*>(w_uk),
                          reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset), seqlens,
                          reinterpret_cast<int32_t*>(ws + lay.cum_pages_offset),
@@ -283,7 +285,7 @@ transmla_status_t transmla_mla_decode_fp8(const transmla_params_t* p, const void
   cudaEvent_t ev0 = tl_prof_start, ev1 = tl_prof_stop;
   tl_prof_start = tl_prof_stop = nullptr;
   if (ev0 != nullptr && cudaEventRecord(ev0, s) != cudaSuccess) return TRANSMLA_ERR_CUDA;
-  if (launch_decode_fp8(*p, lay.num_partitions, reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset), cache_fp8, page_table,
+  if (launch_decode_fp8(*p, parts.most, reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset), cache_fp8, page_table,
                         seqlens, reinterpret_cast<int32_t*>(ws + lay.cum_pages_offset),
                         reinterpret_cast<int32_t*>(ws + lay.plan_offset), reinterpret_cast<float*>(ws + lay.partial_o_offset),
                         reinterpret_cast<float*>(ws + lay.partial_lse_offset), dev_status, s) != cudaSuccess)
@@ -353,7 +355,7 @@ transmla_status_t transmla_decode_step(const transmla_params_t* p, const void* x
   if (st != TRANSMLA_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
-  if (launch_prologue(*p, lay.num_partitions, static_cast<const __nv_bfloat16*>(x),
+  if (launch_prologue(*p, decode_partitioning(*p, lay.num_partitions), static_cast<const __nv_bfloat16*>(x),
                       static_cast<const __nv_bfloat16*>(w_dkv_kr), page_table, static_cast<__nv_bfloat16*>(cache),
                       static_cast<const __nv_bfloat16*>(q_nope), static_cast<const __nv_bfloat16*>(q_pe),
                       static_cast<const __nv_bfloat16*>(w_uk), reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset),

@@ -198,13 +198,27 @@ transmla_status_t validate_step_args(const transmla_params_t* p, const void* x, 
                                      const int32_t* page_table, const int32_t* seqlens, void* workspace,
                                      size_t workspace_bytes, const void* out, int32_t* dev_status);
 
+// How many partitions a batch is planned for.  With per_sequence = 0 `most`.  Otherwise (the library chooses) at most that, and
+// as many as leave a partition about four of the pages that the batch holds, but per_sequence a sequence if it has the pages.
+struct Partitioning {
+  int most, per_sequence;
+  // What the batch holds counts, not what its page table has room for, and only the device knows that: planned for the room
+  // (128K tokens a sequence) a step over one sequence of 777 tokens took 35.6 us and now takes 22.4, of 8192 43.8 and 28.8,
+  // with 64 query rows 37.0 and 24.0, 45.3 and 30.0.  Up to 16 partitions a sequence: 8 sequences of 100 to 5000 tokens 28.7 us
+  // without that, 26.9 with it, 16 of 512 24.3 and 23.0; 8 with 64 query rows a CTA: 8 of 100 to 5000 31.4, 32.3 with 16.
+  __device__ __forceinline__ int count(int pages, int sequences) const {
+    if (per_sequence == 0) return most;
+    return min(most, max(max((pages + 3) / 4, min(per_sequence * sequences, pages)), 1));
+  }
+};
+
 // Launchers (host).  Each enqueues on `stream` and returns the launch error, if any.
 bool dynamic_claims(const transmla_params_t& p, int G);  // whether the split-KV kernel hands pages out at run time
-cudaError_t launch_absorb_plan(const transmla_params_t& p, int G, const __nv_bfloat16* q_nope,
+cudaError_t launch_absorb_plan(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* q_nope,
                                const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                                const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
                                cudaStream_t stream);
-cudaError_t launch_prologue(const transmla_params_t& p, int G, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
+cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
                             const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope,
                             const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                             const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
@@ -218,6 +232,8 @@ cudaError_t launch_decode_generic(const transmla_params_t& p, int G, const __nv_
                                   int32_t* dev_status, cudaStream_t stream);
 bool decode_sm100_supported(const transmla_params_t& p);
 int decode_row_block(const transmla_params_t& p);  // query rows one split-KV CTA works on: 32, or 64
+Partitioning decode_partitioning(const transmla_params_t& p, int G);      // G: the workspace's count
+Partitioning decode_fp8_partitioning(const transmla_params_t& p, int G);  // G: the workspace's count
 cudaError_t launch_decode_rows64(const transmla_params_t& p, int G, const __nv_bfloat16* q_hat, const __nv_bfloat16* cache,
                                  const int32_t* page_table, const int32_t* seqlens, const int32_t* cum, const int32_t* plan,
                                  float* partial_o, float* partial_lse, int32_t* dev_status, cudaStream_t stream);
@@ -234,7 +250,7 @@ cudaError_t launch_append_fp8(const transmla_params_t& p, const __nv_bfloat16* x
                               cudaStream_t stream);
 cudaError_t launch_stream_probe(const transmla_params_t& p, int G, const __nv_bfloat16* cache, const int32_t* page_table,
                                 const int32_t* cum, const int32_t* plan, int32_t* dev_status, cudaStream_t stream);
-cudaError_t launch_combine(const transmla_params_t& p, int G, const int32_t* cum, const float* partial_o,
+cudaError_t launch_combine(const transmla_params_t& p, int G, const int32_t* cum, const int32_t* plan, const float* partial_o,
                            const float* partial_lse, const __nv_bfloat16* w_uv, __nv_bfloat16* out, float* lse_out,
                            int32_t* dev_status, cudaStream_t stream);
 

@@ -155,7 +155,7 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
                     const int32_t* page_table, const int32_t* seqlens,
                     const int32_t* cum, const int32_t* plan, float* partial_o,
                     float* partial_lse, int32_t* dev_status, int S, int H, int num_pages, int max_pages,
-                    float scale_log2, int B, int dynamic, int32_t* next, int G, int merge) {
+                    float scale_log2, int B, int dynamic, int32_t* next) {
   extern __shared__ unsigned char smem_unaligned[];
   const uint32_t raw = smem_u32(smem_unaligned);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -203,8 +203,9 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
   tc_fence_after();
   const uint32_t tmem = *tmem_base_s;
   pdl_wait();  // the plan, the absorbed queries and the appended cache rows come from the kernel before this one
-  const int part = blockIdx.x * merge, parts = min(merge, G - part);
-  const bool has_home = reinterpret_cast<const int4*>(plan)[part + parts - 1].y > reinterpret_cast<const int4*>(plan)[part].x;
+  const int part = blockIdx.x;
+  const int4 pl = reinterpret_cast<const int4*>(plan)[part];
+  const bool has_home = pl.y > pl.x;
 
   if (has_home) {
     if (warp == 4) {
@@ -254,9 +255,9 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
         __syncwarp();
         ++g;
       };
-      const PartitionWalk walk = {page_table, seqlens, cum, next + static_cast<size_t>(rb) * B, partial_lse, part, parts,
-                                  rb * kRowBlock, kRowBlock, SH, max_pages, dynamic};
-      walk_partition(walk, lane < parts ? reinterpret_cast<const int4*>(plan)[part + lane] : make_int4(0, 0, -1, -1), lane, issue_queries, issue_page);
+      const PartitionWalk walk = {page_table, seqlens, cum, next + static_cast<size_t>(rb) * B, partial_lse, part, rb * kRowBlock,
+                                  kRowBlock, SH, max_pages, dynamic};
+      walk_partition(walk, pl, lane, issue_queries, issue_page);
       {  // closing item
         const uint32_t stage = acquire(g);
         if (elect_one()) {
@@ -694,6 +695,14 @@ bool decode_fp8_supported(const transmla_params_t& p) {
   return p.kv_lora_rank == fp8::R && p.qk_rope_dim == fp8::DR && p.q_len * p.num_heads <= 1024;
 }
 
+// The workspace's own partition count suits the bf16 kernels, which may take 64 query rows a CTA; here a CTA takes 32, and the
+// batch is planned for as many partitions as bring the grid to one wave (two waves measured 290 us a step instead of 267 at
+// B=30, S=2, 11K to 20K tokens).
+Partitioning decode_fp8_partitioning(const transmla_params_t& p, int G) {
+  if (p.num_partitions == 0 && library_partitions(p, kRowBlock, &G) != TRANSMLA_OK) G = 1;
+  return {G, p.num_partitions == 0 ? 16 : 0};
+}
+
 cudaError_t launch_decode_fp8(const transmla_params_t& p, int G, const __nv_bfloat16* q_hat, const void* cache_fp8,
                               const int32_t* page_table, const int32_t* seqlens, const int32_t* cum, const int32_t* plan,
                               float* partial_o, float* partial_lse, int32_t* dev_status, cudaStream_t stream) {
@@ -709,16 +718,11 @@ cudaError_t launch_decode_fp8(const transmla_params_t& p, int G, const __nv_bflo
     return cudaErrorInvalidValue;
   static PerDeviceFlag smem_set;
   if (cudaError_t e = ensure_dynamic_smem(decode_fp8_kernel, kSmemBytes, smem_set); e != cudaSuccess) return e;
-  // The library's own partition count suits the bf16 kernels, which take 64 query rows a CTA from 33 rows on; here a CTA
-  // takes 32, so that each works on as many partitions as bring the grid back to one wave (two waves measured
-  // 290 us a step instead of 267 at B=30, S=2, 11K to 20K tokens).
-  const int blocks = (SH + kRowBlock - 1) / kRowBlock, bf16_blocks = (SH + decode_row_block(p) - 1) / decode_row_block(p);
-  const int merge = p.num_partitions == 0 && G > 1 ? (blocks + bf16_blocks - 1) / bf16_blocks : 1;
-  dim3 grid((G + merge - 1) / merge, blocks);
+  dim3 grid(G, (SH + kRowBlock - 1) / kRowBlock);
   int32_t* next = const_cast<int32_t*>(cum) + 3 * p.batch + 1;  // page counters, zeroed by the plan
   return launch_pdl(decode_fp8_kernel, grid, dim3(kThreads), static_cast<size_t>(kSmemBytes), stream, map, smap, qmap,
                     static_cast<const unsigned char*>(cache_fp8), page_table, seqlens, cum, plan, partial_o, partial_lse, dev_status, p.q_len, p.num_heads,
-                    p.num_pages, p.max_pages_per_seq, p.softmax_scale * kLog2e, p.batch, dynamic_claims(p, G) ? 1 : 0, next, G, merge);
+                    p.num_pages, p.max_pages_per_seq, p.softmax_scale * kLog2e, p.batch, dynamic_claims(p, G) ? 1 : 0, next);
 }
 
 }  // namespace transmla

@@ -162,9 +162,9 @@ decode_rows64_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid
         __syncwarp();
         ++g; ++n;
       };
-      const PartitionWalk walk = {page_table, seqlens, cum, next + static_cast<size_t>(rb) * B, partial_lse, part, 1,
-                                  rb * kRows, kRows, SH, max_pages, dynamic};
-      walk_partition(walk, lane < 1 ? pl : make_int4(0, 0, -1, -1), lane, issue_queries, issue_page);
+      const PartitionWalk walk = {page_table, seqlens, cum, next + static_cast<size_t>(rb) * B, partial_lse, part, rb * kRows,
+                                  kRows, SH, max_pages, dynamic};
+      walk_partition(walk, pl, lane, issue_queries, issue_page);
       {  // closing item
         const int stage = acquire();
         if (elect_one()) {

@@ -152,9 +152,9 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
         __syncwarp();
         ++g;
       };
-      const PartitionWalk walk = {page_table, seqlens, cum, next + static_cast<size_t>(rb) * B, partial_lse, part, 1,
-                                  rb * kRowBlock, kRowBlock, SH, max_pages, dynamic};
-      walk_partition(walk, lane < 1 ? pl : make_int4(0, 0, -1, -1), lane, issue_queries, issue_page);
+      const PartitionWalk walk = {page_table, seqlens, cum, next + static_cast<size_t>(rb) * B, partial_lse, part, rb * kRowBlock,
+                                  kRowBlock, SH, max_pages, dynamic};
+      walk_partition(walk, pl, lane, issue_queries, issue_page);
       {  // closing item
         const uint32_t stage = acquire(g);
         if (elect_one()) {
@@ -454,13 +454,19 @@ bool decode_sm100_supported(const transmla_params_t& p) { return p.kv_lora_rank 
 // us, 32 heads S=2 B=32 x 4K-8K 101 -> 75 us) - unless the batch is so small that a 32-row CTA handles no more than about
 // 16 pages (12 with more than two row blocks) anyway: then the shorter start and end of the 32-row kernel count (32 heads
 // S=2 B=4 x 4K-8K: 34.1 us against 37.3, B=8 39.8 against 41.3; 64 heads S=2 B=4 x 1K-2K 30.4 against 32.4, x 2K-4K 34.3
-// against 34.9, x 4K-8K 42.1 against 40.5).  Like the partition count the rule goes by the page table's capacity.
+// against 34.9, x 4K-8K 42.1 against 40.5).  The rule goes by the page table's capacity: a table with room for much more than a
+// small batch holds costs up to 3 us a step (4 x 8192 tokens, 32 heads S=2: 35 against 32).  One kernel with both forms, chosen
+// on the device, cost 2 to 4 us in either.
 int decode_row_block(const transmla_params_t& p) {
   constexpr int kSms = 148;
   if (!decode_sm100_supported(p) || p.q_len * p.num_heads <= kRowBlock) return kRowBlock;
   const long long blocks = (p.q_len * p.num_heads + kRowBlock - 1) / kRowBlock;
   const long long ctas = (static_cast<long long>(p.batch) * p.max_pages_per_seq + 3) / 4 * blocks;  // of four pages each
   return ctas <= (blocks <= 2 ? 4 : 3) * kSms ? kRowBlock : 64;
+}
+
+Partitioning decode_partitioning(const transmla_params_t& p, int G) {
+  return {G, p.num_partitions != 0 ? 0 : decode_row_block(p) == 64 ? 8 : 16};
 }
 
 // Pages are handed out at run time only when the library chose the partition count itself (a caller who fixes the

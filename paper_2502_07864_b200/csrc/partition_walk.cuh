@@ -11,24 +11,17 @@ struct PartitionWalk {
   const int32_t* cum;
   int32_t* counters;      // page counters of this block of query rows, one per sequence (run-time claims)
   float* partial_lse;
-  int part, parts;        // the CTA's partitions: `parts` consecutive ones (at most 32) from `part` on
+  int part;               // the CTA's partition
   int row0, rows;         // first query row and row count of the block
   int SH, max_pages, dynamic;
 };
 
 // Calls queries(b, slot, L) at the start of every segment (the part of sequence b that this CTA works on; its partial
 // goes to `slot`) and page(b, page number within the sequence, first of the segment, last of the segment) for each of
-// its pages.  All lanes of the warp call it together; lane i hands in the plan row of partition `part` + i (empty from
-// `parts` on).  Several partitions are walked as one range: a sequence's pages in them form one segment, whose partial
-// goes to the slot of the first of them that holds any; the others' slots get an empty partial.
+// its pages.  All lanes of the warp call it together, with the partition's row of the plan.
 template <class Queries, class Page>
-__device__ __forceinline__ void walk_partition(const PartitionWalk& w, int4 mine, int lane, Queries&& queries, Page&& page) {
+__device__ __forceinline__ void walk_partition(const PartitionWalk& w, int4 pl, int lane, Queries&& queries, Page&& page) {
   constexpr uint32_t kAll = 0xffffffffu;
-  const uint32_t owners = __ballot_sync(kAll, mine.y > mine.x);
-  if (owners == 0) return;
-  const int lo_lane = __ffs(owners) - 1, hi_lane = 31 - __clz(owners);
-  const int4 pl = make_int4(__shfl_sync(kAll, mine.x, lo_lane), __shfl_sync(kAll, mine.y, hi_lane),
-                            __shfl_sync(kAll, mine.z, lo_lane), __shfl_sync(kAll, mine.w, hi_lane));
   auto empty_partial = [&](int slot) {
     for (int i = lane; i < w.rows && w.row0 + i < w.SH; i += 32)
       w.partial_lse[static_cast<size_t>(slot) * w.SH + w.row0 + i] = -INFINITY;
@@ -54,12 +47,7 @@ __device__ __forceinline__ void walk_partition(const PartitionWalk& w, int4 mine
     const int c0s = cb + kSegCost;  // slot of page 0 of sequence b
     const int pg_lo = max(pl.x, c0s) - c0s, pg_hi = min(pl.y, cb1) - c0s;
     if (pg_hi <= pg_lo) continue;
-    int slot = w.part + b;
-    if (w.parts > 1) {
-      uint32_t have = __ballot_sync(kAll, min(mine.y, cb1) > max(mine.x, c0s));  // partitions with pages of b
-      slot += __ffs(have) - 1;
-      for (have &= have - 1; have != 0; have &= have - 1) empty_partial(w.part + __ffs(have) - 1 + b);
-    }
+    const int slot = w.part + b;
     if (!w.dynamic) {  // exactly the plan's range
       prefetch_table(b, pg_lo, pg_hi);
       queries(b, slot, L);

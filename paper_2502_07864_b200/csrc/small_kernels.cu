@@ -24,7 +24,7 @@ __device__ __forceinline__ int kperm(int p) { return ((p & 7) >> 1) * 8 + (p >> 
 // ------------------------------------------------------------------------------------------------
 // Split plan.  Every non-empty sequence owns ceil(L_b/P) page slots preceded by kSegCost virtual slots (the
 // price of opening a sequence); cum[b] = slots before sequence b; partition i owns slots
-// [floor(i*T/G), floor((i+1)*T/G)); plan row = (begin, end, sequence of first slot, of last slot).
+// [floor(i*T/G), floor((i+1)*T/G)), of the G that are planned (see plan_block); plan row = (begin, end, sequence of first slot, of last slot).
 // One block of 256 threads; the scan runs in chunks of 256 sequences; the prefix sums are kept in
 // shared memory (when they fit) for the binary searches.
 // ------------------------------------------------------------------------------------------------
@@ -40,13 +40,14 @@ __device__ __forceinline__ int seq_of_page(const int32_t* cum, int B, int x) {
   return lo - 1;
 }
 
-__device__ void plan_block(const int32_t* seqlens, int B, int G, int RB, int max_pages, int32_t* cum, int32_t* plan,
+__device__ void plan_block(const int32_t* seqlens, int B, Partitioning parts, int RB, int max_pages, int32_t* cum, int32_t* plan,
                            int32_t* dev_status, unsigned char* smem_raw) {
   __shared__ int warp_sums[8];
   __shared__ int carry;
   int32_t* cum_s = reinterpret_cast<int32_t*>(smem_raw);  // [B+1] when B < kPlanSmemSeqs
   const bool in_smem = B < kPlanSmemSeqs;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int sequences = 0;  // that are not empty
   pdl_wait();
   if (tid == 0) { carry = 0; cum[0] = 0; if (in_smem) cum_s[0] = 0; }
   __syncthreads();
@@ -63,12 +64,14 @@ __device__ void plan_block(const int32_t* seqlens, int B, int G, int RB, int max
     for (int w = 0; w < warp; ++w) before += warp_sums[w];
     const int incl = v + before;
     if (b < B) { cum[b + 1] = incl; if (in_smem) cum_s[b + 1] = incl; }
-    __syncthreads();
+    sequences += __syncthreads_count(n > 0);
     if (tid == 255) carry = incl;
     __syncthreads();
   }
   const int32_t* cs = in_smem ? cum_s : cum;
   const long long T = cs[B];
+  const int G = parts.count(static_cast<int>(T) - kSegCost * sequences, sequences);
+  for (int i = G + tid; i < parts.most; i += 256) reinterpret_cast<int4*>(plan)[i] = make_int4(0, 0, -1, -1);
   for (int i = tid; i < G; i += 256) {
     const int p0 = static_cast<int>((static_cast<long long>(i) * T) / G);
     const int p1 = static_cast<int>((static_cast<long long>(i + 1) * T) / G);
@@ -232,7 +235,7 @@ __global__ void __launch_bounds__(256) absorb_plan_kernel(const __nv_bfloat16* q
                                                           __nv_bfloat16* q_hat,
                                                           const int32_t* seqlens, int32_t* cum,
                                                           int32_t* plan, int32_t* dev_status, int B, int S, int H,
-                                                          int dn, int dR, int r, int G, int max_pages, int nt) {
+                                                          int dn, int dR, int r, Partitioning parts, int max_pages, int nt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
   const int per_head = (r + 127) / 128 / nt;  // absorb blocks per head, nt tiles each
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(256) absorb_plan_kernel(const __nv_bfloat16* q
   if (static_cast<int>(blockIdx.x) < n_absorb) {
     absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, blockIdx.x / per_head, blockIdx.x % per_head * nt, nt, smem_raw);
   } else {
-    plan_block(seqlens, B, G, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
+    plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
   }
 }
 
@@ -251,14 +254,14 @@ __global__ void __launch_bounds__(256) prologue_kernel(
     const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope,
     const __nv_bfloat16* q_pe, const __nv_bfloat16* __restrict__ w_uk, __nv_bfloat16* q_hat,
     const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status, int B, int S, int H, int D,
-    int dn, int dR, int r, int num_pages, int max_pages, float theta, int G, int t_splits, int wide, int nt) {
+    int dn, int dR, int r, int num_pages, int max_pages, float theta, Partitioning parts, int t_splits, int wide, int nt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
   const int n_append = (r + dR) / (wide ? 32 : 8) * t_splits;
   const int per_head = (r + 127) / 128 / nt;  // absorb blocks per head, nt tiles each
   const int bid = static_cast<int>(blockIdx.x) - 1;
   if (bid < 0) {
-    plan_block(seqlens, B, G, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
+    plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
   } else if (bid < n_append) {
     if (wide)
       append_block<1, 4>(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages,
@@ -297,7 +300,7 @@ cudaError_t launch_append(const transmla_params_t& p, const __nv_bfloat16* x, co
                     p.max_pages_per_seq, p.rope_theta, ts, wide);
 }
 
-cudaError_t launch_absorb_plan(const transmla_params_t& p, int G, const __nv_bfloat16* q_nope,
+cudaError_t launch_absorb_plan(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* q_nope,
                                const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                                const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
                                cudaStream_t stream) {
@@ -308,11 +311,11 @@ cudaError_t launch_absorb_plan(const transmla_params_t& p, int G, const __nv_bfl
   if (cudaError_t e = ensure_dynamic_smem(absorb_plan_kernel, kPrologueMaxSmem, smem_set); e != cudaSuccess) return e;
   const int blocks = p.num_heads * ((p.kv_lora_rank + 127) / 128 / nt) + 1;
   return launch_pdl(absorb_plan_kernel, dim3(blocks), dim3(256), smem, stream, q_nope, q_pe, w_uk, q_hat, seqlens, cum,
-                    plan, dev_status, p.batch, p.q_len, p.num_heads, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, G,
+                    plan, dev_status, p.batch, p.q_len, p.num_heads, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, parts,
                     p.max_pages_per_seq, nt);
 }
 
-cudaError_t launch_prologue(const transmla_params_t& p, int G, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
+cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
                             const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope,
                             const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                             const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
@@ -328,7 +331,7 @@ cudaError_t launch_prologue(const transmla_params_t& p, int G, const __nv_bfloat
   const int blocks = 1 + n_append + p.num_heads * ((p.kv_lora_rank + 127) / 128 / nt);
   return launch_pdl(prologue_kernel, dim3(blocks), dim3(256), smem, stream, x, w_dkv_kr, page_table, cache, q_nope, q_pe,
                     w_uk, q_hat, seqlens, cum, plan, dev_status, p.batch, p.q_len, p.num_heads, p.hidden_dim,
-                    p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, p.num_pages, p.max_pages_per_seq, p.rope_theta, G, ts, wide, nt);
+                    p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, p.num_pages, p.max_pages_per_seq, p.rope_theta, parts, ts, wide, nt);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -347,6 +350,7 @@ constexpr int kCombineRows = 16;
 // matters); otherwise load weights window by window and keep the register count low enough for two blocks per SM.
 template <bool kPrefetch>
 __global__ void __launch_bounds__(256, kPrefetch ? 1 : 2) combine_kernel(const int32_t* cum,
+                                                      const int32_t* plan,
                                                       const float* partial_o,
                                                       const float* partial_lse,
                                                       const __nv_bfloat16* __restrict__ w_uv,
@@ -386,16 +390,17 @@ __global__ void __launch_bounds__(256, kPrefetch ? 1 : 2) combine_kernel(const i
       const int b = bs / S, s = bs % S, row = s * H + h;
       const int32_t* seq_parts = cum + B + 1;  // only 4-byte aligned: B + 1 may be odd
       const int i_first = seq_parts[2 * b], nseg = seq_parts[2 * b + 1] - i_first + 1;
-      const bool dense = T >= G;  // then every partition owns at least one slot
+      const bool dense = T >= G;  // then every partition owns at least one slot (of G at most)
       if (nseg > 0) {
         auto seg_lse = [&](int j) -> float {  // lse of the j-th candidate partition, -inf if it is empty or absent
           if (j >= nseg) return -INFINITY;
           const int pi = i_first + j;
+          const float l = partial_lse[static_cast<size_t>(pi + b) * SH + row];
           if (!dense) {
-            const long long p0 = (static_cast<long long>(pi) * T) / G, p1 = (static_cast<long long>(pi + 1) * T) / G;
-            if (p1 <= p0) return -INFINITY;
+            const int2 range = *reinterpret_cast<const int2*>(plan + 4 * pi);
+            if (range.y <= range.x) return -INFINITY;
           }
-          return partial_lse[static_cast<size_t>(pi + b) * SH + row];
+          return l;
         };
         float m = -INFINITY;
         for (int base = 0; base < nseg; base += 32) m = fmaxf(m, seg_lse(base + lane));
@@ -496,7 +501,7 @@ __global__ void __launch_bounds__(256, kPrefetch ? 1 : 2) combine_kernel(const i
   }
 }
 
-cudaError_t launch_combine(const transmla_params_t& p, int G, const int32_t* cum, const float* partial_o,
+cudaError_t launch_combine(const transmla_params_t& p, int G, const int32_t* cum, const int32_t* plan, const float* partial_o,
                            const float* partial_lse, const __nv_bfloat16* w_uv, __nv_bfloat16* out, float* lse_out,
                            int32_t* dev_status, cudaStream_t stream) {
   (void)dev_status;
@@ -508,9 +513,9 @@ cudaError_t launch_combine(const transmla_params_t& p, int G, const int32_t* cum
   dim3 grid(p.num_heads, (BS + rows - 1) / rows, zsplit);
   const size_t smem = 2 * kCombineRows * (p.kv_lora_rank + 8) * sizeof(__nv_bfloat16);
   if (BS <= 32)
-    return launch_pdl(combine_kernel<true>, grid, dim3(256), smem, stream, cum, partial_o, partial_lse, w_uv, out, lse_out,
+    return launch_pdl(combine_kernel<true>, grid, dim3(256), smem, stream, cum, plan, partial_o, partial_lse, w_uv, out, lse_out,
                       p.batch, p.q_len, p.num_heads, p.kv_lora_rank, p.v_dim, G, rows);
-  return launch_pdl(combine_kernel<false>, grid, dim3(256), smem, stream, cum, partial_o, partial_lse, w_uv, out, lse_out,
+  return launch_pdl(combine_kernel<false>, grid, dim3(256), smem, stream, cum, plan, partial_o, partial_lse, w_uv, out, lse_out,
                     p.batch, p.q_len, p.num_heads, p.kv_lora_rank, p.v_dim, G, rows);
 }
 

@@ -133,10 +133,9 @@ def test_fp8_small_rows_beside_zero_rows(octave):
 
 
 @pytest.mark.parametrize('seqlens,columns', [([64 * 40 + 5, 1, 700, 0, 333], 600), ([2900], 1200)])
-def test_fp8_two_partitions_a_cta(seqlens, columns):
-    # 64 query rows and a page table with room for many pages: the library picks its partition count for 64 rows a CTA,
-    # and a CTA of this kernel (32 rows) takes two of them, as one segment per sequence (planned ranges, and with one
-    # sequence pages claimed at run time)
+def test_fp8_more_than_32_query_rows(seqlens, columns):
+    # 64 query rows and a page table with room for many pages: the workspace is laid out for 64 rows a CTA, and this kernel
+    # (32 rows) plans the batch for half as many partitions (planned ranges, and with one sequence pages claimed at run time)
     gu.ensure_built()
     shape = synth.MLAShape(H=32, dn=128, dR=64, dv=128, r=512, D=4096, S=2)
     scale = gu.mla_scale(shape)
@@ -148,8 +147,8 @@ def test_fp8_two_partitions_a_cta(seqlens, columns):
     only = [(b, s, h) for b in range(len(seqlens)) for s in range(2) for h in (0, 15, 31)]
     want, want_lse = oracle_fp8(shape, case, scale, only=only)
     idx = tuple(np.array(only).T)
-    gu.assert_close(lifts.f64(out)[idx], want[idx], 'two partitions a CTA')
-    gu.assert_lse_close(lifts.f64(lse)[idx], want_lse[idx], 'two partitions a CTA, lse')
+    gu.assert_close(lifts.f64(out)[idx], want[idx], 'more than 32 rows')
+    gu.assert_lse_close(lifts.f64(lse)[idx], want_lse[idx], 'more than 32 rows, lse')
 
 
 def test_fp8_append_writes_the_quantised_row():

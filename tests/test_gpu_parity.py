@@ -134,6 +134,29 @@ def test_row_blocks_of_64(H, S, G):
     gu.assert_lse_close(lifts.f64(lse)[idx], want_lse[idx], 'lse')
 
 
+@pytest.mark.parametrize('shape', [synth.LLAMA2_7B, synth.MLAShape(H=64, dn=128, dR=64, dv=128, r=512, D=4096), synth.TINY])
+@pytest.mark.parametrize('seqlens', [[1], [300, 64, 0, 1], [8192], [777] * 3, [640] * 70, [0, 0]])
+def test_partitions_follow_the_batch_not_the_page_table(shape, seqlens):
+    # a table with room for 128K tokens a sequence: the library plans for about four of the pages that the batch holds a
+    # partition, or 16 (8) partitions a sequence, up to what the table's room lets it have; the rest of the plan is empty, and
+    # no slot of it is read
+    case = synth.make_decode_case(shape, seqlens, 19, nan_tails=True)
+    _widen_table(case, 2048)
+    scale = gu.mla_scale(shape)
+    out, lse, status, views, lay = gu.gpu_decode(shape, gu.to_dev(case), scale, want_views=True)
+    assert status == 0
+    pages = sum((L + 63) // 64 for L in seqlens)
+    slots = pages + 2 * sum(L > 0 for L in seqlens)
+    per_sequence = 8 if shape.r == 512 and shape.S * shape.H > 32 else 16
+    G = min(lay.num_partitions, max((pages + 3) // 4, min(per_sequence * sum(L > 0 for L in seqlens), pages), 1))
+    plan = views['plan'].cpu().numpy()
+    assert [tuple(r[:2]) for r in plan[:G]] == [(i * slots // G, (i + 1) * slots // G) for i in range(G)]
+    assert all(r[1] <= r[0] for r in plan[G:])
+    want, want_lse = gu.oracle_decode(shape, case, scale)
+    gu.assert_close(lifts.f64(out), want, f'{G} partitions')
+    gu.assert_lse_close(lifts.f64(lse), want_lse, 'lse')
+
+
 def test_wide_heads_and_many_sequences():
     # dn = dv = 256 (largest supported head dims) on the small latent; 5000 one-page sequences make the plan
     # block take its global-memory path (more sequences than its shared-memory buffer holds)
