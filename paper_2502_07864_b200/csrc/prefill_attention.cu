@@ -1,7 +1,7 @@
 // Causal attention of a chunk of query positions over the decompressed keys and values (Eq. 9 left): prefill in
 // the MHA form, per head  z = q_nope . k^C + q_pe . k^R,  softmax,  sum p v.
 //
-// One CTA = two tiles of 128 query positions x one head x one sequence.  Per 64-token page and tile
+// One CTA = two tiles of 128 query positions (or one, see the launch) x one head x one sequence.  Per 64-token page and tile
 //   S [128 x 64]  = Q x [k^C | k^R]^T, K = 192 (a third of Q from tensor memory, the rest and the page from shared memory)
 //   O [128 x 128] += P (tensor memory, bf16) x V (shared memory, MN-major)
 // What bounds it: the products need 640 cycles a tile and page, 780 with two thirds of Q from shared memory, and the
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 prefill_attention_kernel(const __grid_constant__ CUtensorMap qn_map, const __grid_constant__ CUtensorMap qr_map,
                          const __grid_constant__ CUtensorMap kv_map, const __grid_constant__ CUtensorMap cache_map,
                          const int32_t* page_table, const int32_t* seqlens, __nv_bfloat16* out, float* lse_out,
-                         int32_t* dev_status, int S, int H, int num_pages, int max_pages, float scale_log2) {
+                         int32_t* dev_status, int S, int H, int num_pages, int max_pages, float scale_log2, int cta_tiles) {
   extern __shared__ __align__(1024) unsigned char smem_aligned[];  // no room to align by hand
   unsigned char* sm = smem_aligned;
   const uint32_t base = smem_u32(sm);
@@ -89,8 +89,8 @@ prefill_attention_kernel(const __grid_constant__ CUtensorMap qn_map, const __gri
   const int L = clamped_len(seqlens[b], max_pages, (tid == 0 && blockIdx.x == 0 && h == 0) ? dev_status : nullptr);
   // Query position s of the chunk sees tokens [0, L - (S - 1 - s)); a tile's last position sees the most.
   auto tile_pages = [&](int t) -> int {  // pages that tile t of this CTA looks at (0: nothing to see, or no rows)
-    const int s_first = (qt * kTiles + t) * kQRows;
-    if (s_first >= S) return 0;
+    const int s_first = (qt * cta_tiles + t) * kQRows;
+    if (t >= cta_tiles || s_first >= S) return 0;
     return (max(0, L - (S - 1 - (min(S, s_first + kQRows) - 1))) + kPage - 1) / kPage;
   };
   const int nt0 = tile_pages(0), nt1 = tile_pages(1), n_pages = max(nt0, nt1);  // block-uniform
@@ -99,10 +99,10 @@ prefill_attention_kernel(const __grid_constant__ CUtensorMap qn_map, const __gri
     // ======================================================================== TMA producer
     // Page n uses stage (n + 1) % 4; the first use of stage 0 is q_nope's.
     if (elect_one()) {
-      const int tiles = (qt * kTiles + 1) * kQRows < S ? 2 : 1;
+      const int tiles = cta_tiles == 2 && (qt * 2 + 1) * kQRows < S ? 2 : 1;
       mbar_arrive_expect_tx(bar(A_KV_FULL), tiles * 3 * kQSub);
       for (int t = 0; t < tiles; ++t) {
-        const int row0 = b * S + (qt * kTiles + t) * kQRows;
+        const int row0 = b * S + (qt * cta_tiles + t) * kQRows;
         tma_load_2d(base + kOffKv + t * kQSub, &qn_map, h * DN_, row0, bar(A_KV_FULL));
         tma_load_2d(base + kOffQ + 2 * t * kQSub, &qn_map, h * DN_ + 64, row0, bar(A_KV_FULL));
         tma_load_2d(base + kOffQ + (2 * t + 1) * kQSub, &qr_map, h * DR_, row0, bar(A_KV_FULL));
@@ -180,8 +180,8 @@ prefill_attention_kernel(const __grid_constant__ CUtensorMap qn_map, const __gri
     // ======================================================================== softmax + write-out
     const int tile = warp >> 3, half = (warp >> 2) & 1, quad = warp & 3;
     const uint32_t lane_base = static_cast<uint32_t>(quad * 32) << 16;
-    const int row = quad * 32 + lane, s = (qt * kTiles + tile) * kQRows + row;
-    const bool in_chunk = s < S;
+    const int row = quad * 32 + lane, s = (qt * cta_tiles + tile) * kQRows + row;
+    const bool in_chunk = s < S && tile < cta_tiles;
     const int nt = tile ? nt1 : nt0;
     if (n_pages > 0) {
       // a quarter of this row of q_nope: shared memory (swizzled sub-tile of 128 rows x 128 bytes) -> tensor memory
@@ -343,9 +343,16 @@ cudaError_t launch_prefill_attention(const transmla_params_t& p, const __nv_bflo
     return cudaErrorInvalidValue;
   static PerDeviceFlag smem_set;
   if (cudaError_t e = ensure_dynamic_smem(prefill_attention_kernel, kAttnSmem, smem_set); e != cudaSuccess) return e;
-  dim3 grid((p.q_len + kTiles * kQRows - 1) / (kTiles * kQRows), p.num_heads, p.batch);
+  // Two tiles a CTA take about 1.3 times as long as one, so that one is better where the device then needs no more waves than
+  // 1.3 times those of CTAs with two (32 heads over 8192 tokens: 1 x 256 positions 100 us with one, 126 with two; 3 x 300 over
+  // 16384 397 and 464; 4 x 256 200 and 155, 6 x 256 306 and 268).
+  constexpr long long kSms = 148;
+  const long long heads = static_cast<long long>(p.num_heads) * p.batch;
+  auto waves = [&](int tiles) { return ((p.q_len + tiles * kQRows - 1) / (tiles * kQRows) * heads + kSms - 1) / kSms; };
+  const int cta_tiles = 10 * waves(1) < 13 * waves(2) ? 1 : 2;
+  dim3 grid((p.q_len + cta_tiles * kQRows - 1) / (cta_tiles * kQRows), p.num_heads, p.batch);
   return launch_pdl(prefill_attention_kernel, grid, dim3(kAttnThreads), static_cast<size_t>(kAttnSmem), stream, qn, qr, kv, cm, page_table,
                     seqlens, out, lse, dev_status, p.q_len, p.num_heads, p.num_pages, p.max_pages_per_seq,
-                    p.softmax_scale * kLog2e);
+                    p.softmax_scale * kLog2e, cta_tiles);
 }
 }  // namespace transmla

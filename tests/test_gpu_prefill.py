@@ -58,7 +58,7 @@ def test_decompressed_store_matches_the_oracle_row_by_row():
                                        (129, [129, 700]), (256, [256, 300]), (257, [100, 260, 130]), (385, [200, 390])])
 def test_prefill_all_outputs_small_head_count(S, seqlens):
     # every output and lse; S = 130 and 300 leave the last 128-row tile ragged, L = S is a pure prefill,
-    # (a CTA takes two tiles: 129 .. 257 and 385 leave one of them short, empty or without anything to see)
+    # (with so few heads every tile has a CTA of its own)
     # L = 64 < S = 130 leaves the first positions with nothing to see (zeros, lse = -inf)
     gu.ensure_built()
     shape = synth.MLAShape(H=2, dn=128, dR=64, dv=128, r=512, D=4096, S=S)
@@ -72,6 +72,27 @@ def test_prefill_all_outputs_small_head_count(S, seqlens):
         for s in range(S):
             if orc.visible_tokens(L, S, s) == 0:
                 assert torch.all(out[b, s] == 0) and torch.all(torch.isneginf(lse[b, s]))
+
+
+@pytest.mark.parametrize('S,seqlens', [(130, [130, 257, 64, 1000]), (129, [129, 700]), (256, [256, 300]), (257, [100, 260, 130]),
+                                       (300, [320, 1100]), (385, [200, 390])])
+def test_prefill_two_tiles_a_cta(S, seqlens):
+    # enough heads that a CTA takes two tiles of 128 positions: one of them short, empty or without anything to see
+    gu.ensure_built()
+    B, tiles = len(seqlens), (S + 127) // 128
+    H = 80 // B + 1 if tiles == 2 else 72 // B
+    assert 10 * -(-tiles * H * B // 148) >= 13 * -(-((tiles + 1) // 2) * H * B // 148)
+    shape = synth.MLAShape(H=H, dn=128, dR=64, dv=128, r=512, D=4096, S=S)
+    case = synth.make_decode_case(shape, seqlens, seed=132 + S, nan_tails=True)
+    out, lse, status, _ = _prefill(shape, gu.to_dev(case), gu.mla_scale(shape))
+    assert status == 0
+    at = sorted({s for e in range(0, S, 128) for s in (e - 1, e, e + 1, e + 63, e + 64)} & set(range(S)) | {S - 1})
+    only = [(b, s, h) for b in range(B) for s in at for h in (0, 1, H - 1)]
+    want, want_lse = gu.oracle_decode(shape, case, gu.mla_scale(shape), only=only)
+    idx = tuple(np.array(only).T)
+    gu.assert_close(lifts.f64(out)[idx], want[idx], 'two tiles a CTA')
+    gu.assert_lse_close(lse.cpu().numpy()[idx], want_lse[idx], 'two tiles a CTA, lse')
+    assert bool(torch.isfinite(out).all())
 
 
 def test_prefill_llama_heads_sampled_outputs():
