@@ -76,6 +76,9 @@ class ClockSampler:
                                           '-i', str(index), '-lms', '20'], stdout=subprocess.PIPE, text=True)
             self.thread = threading.Thread(target=self._read, daemon=True)
             self.thread.start()
+            give_up = time.perf_counter() + 3.0   # nvidia-smi takes longer to start than a short row runs
+            while not self.rows and time.perf_counter() < give_up:
+                time.sleep(0.01)
         except Exception:
             self.proc = None
 
@@ -185,7 +188,7 @@ def kernel_source_hash(fp8=False):
     """Hash of the sources the split-KV kernel is compiled from; ties an ncu capture to the code it was taken on."""
     import hashlib
     h = hashlib.sha256()
-    for f in ('decode_fp8.cu' if fp8 else 'decode_sm100.cu', 'common.cuh', 'sm100_ptx.cuh'):
+    for f in ('decode_fp8.cu' if fp8 else 'decode_sm100.cu', 'partition_walk.cuh', 'common.cuh', 'sm100_ptx.cuh'):
         h.update(open(os.path.join(ROOT, 'paper_2502_07864_b200', 'csrc', f), 'rb').read())
     return h.hexdigest()[:16]
 
@@ -270,11 +273,11 @@ def measure_prefill(args, name, shape, seqlens, seed, rank, world, local):
         binding.transmla_mla_prefill(params, case['q_nope'], case['q_pe'], case['w_uk'], case['w_uv'], caches[i % n_copies],
                                      case['page_table'], case['seqlens'], scratch, out, lse, status, stream)
 
+    sampler = ClockSampler(local) if rank == 0 else None   # before the warm-up: it waits until samples come
     for i in range(3):
         step(i)
     replicas.barrier('cuda')
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    sampler = ClockSampler(local) if rank == 0 else None
     t0 = time.perf_counter()
     e0.record(stream)
     for i in range(steps):
@@ -376,11 +379,11 @@ def measure_conversion(args, name, shape, seqlens, seed, rank, world, local):
         binding.transmla_conv_gemm(Q, w_dkv, out_dkv, ta=True); mark('rewrite')
 
     steps = max(2, min(args.steps, 3))
+    sampler = ClockSampler(local) if rank == 0 else None   # before the warm-up: it waits until samples come
     for _ in range(3):
         step()
     torch.cuda.synchronize()
     ev.clear()
-    sampler = ClockSampler(local) if rank == 0 else None
     t0 = time.perf_counter()
     for _ in range(steps):
         step()
@@ -413,8 +416,8 @@ def measure_conversion(args, name, shape, seqlens, seed, rank, world, local):
                      'peak': peak, 'unit': 'TFLOP/s', 'frac': f_sm / part_ms['second_moment'] / 1e9 / peak,
                      'peak_kind': f'{tpeak_kind} bf16 GEMM / 6 products x 2 for the mirrored half', 'traffic': None, 'flops_per_launch': f_sm,
                      'sm_mhz_sampled': sm_mhz},
-        # gemm 6, gather 1, Jacobi 1, rotation 1, norms 3, concat 1, and (iters + 3) Cholesky QRs of four launches each
-        'gpu_launches': (13 + iters + 4 * (iters + 3)) * steps, 'clocks': clocks,
+        # gemm 6, gather 1, Jacobi 1, rotation 1, norms 3, concat 1, and (iters + 3) Cholesky QRs of four launches each, the last with one more
+        'gpu_launches': (13 + iters + 4 * (iters + 3) + 1) * steps, 'clocks': clocks,
     }
 
 
@@ -474,6 +477,7 @@ def measure(args, name, shape, seqlens, seed, rank, world, local, full):
     def barrier():
         replicas.barrier('cuda')
 
+    sampler = ClockSampler(local) if rank == 0 else None   # before the warm-up: it waits until samples come
     for i in range(max(args.warmup, 3)):
         step(i)
     barrier()
@@ -485,7 +489,6 @@ def measure(args, name, shape, seqlens, seed, rank, world, local, full):
     for a, b_ in kev.values():       # create the underlying CUDA events before handing them to the library
         a.record(stream); b_.record(stream)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    sampler = ClockSampler(local) if rank == 0 else None
     barrier()
     t0 = time.perf_counter()
     e0.record(stream)
