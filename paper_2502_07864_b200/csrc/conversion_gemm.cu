@@ -65,7 +65,8 @@ __device__ __forceinline__ void mbar_arrive_first(uint32_t bar) {
                ::"r"(bar) : "memory");
 }
 
-// The same without a release: for an arrival that hands over tensor memory (the reads have completed), nothing in memory.
+// The same without a release: for an arrival that hands over tensor memory and nothing in memory (tcgen05.wait::ld has completed
+// the reads before it is issued).
 __device__ __forceinline__ void mbar_arrive_first_relaxed(uint32_t bar) {
   asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, 0;\nmbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [a];\n}"
                ::"r"(bar) : "memory");

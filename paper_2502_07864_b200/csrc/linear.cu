@@ -112,7 +112,8 @@ transmla_status_t transmla_layer_decode_step(const transmla_params_t* p, const t
   // tokens meet three short maps in a row: their blocks start beside those of the kernel before and have their weights on the
   // way to L2 by then, which is all that counts there.  Full step, mma.sync / tcgen05: 33 M weights (LLaMA-2-7B, rank 1536)
   // 49.0 / 50.6 us at 1 token, 51.7 / 52.8 at 8, 58.4 / 54.2 at 16; 99 M (Qwen2.5-72B) 102 / 75 at 3; full rank, two longer
-  // maps, 42 M: 49.3 / 47.8 at 1, 53.0 / 50.0 at 8.
+  // maps, 42 M: 49.3 / 47.8 at 1, 53.0 / 50.0 at 8.  (No low-rank layer between 33 M and 99 M was measured: the line is drawn
+  // near the smaller one, and between 8 and 16 tokens likewise.)
   const size_t map_weights = static_cast<size_t>(rq) * D + static_cast<size_t>(H) * (p->qk_nope_dim + p->qk_rope_dim) * Kq + static_cast<size_t>(D) * Ko;
   const bool short_maps = low_rank && M <= 8 && map_weights <= (size_t(40) << 20);
   auto on_sm100 = [&](const LinearArgs& la) { return !short_maps && linear_sm100_supported(la); };

@@ -13,13 +13,13 @@
 // memory (the ring is free by then), and after a cluster barrier every CTA adds the slices of its share of the
 // tokens in slice order, reading the others' shared memory directly, applies RoPE where asked and writes bf16 (no
 // float atomics: reruns give the same bits).
-// What bounds it: the 31 bytes a cycle that an SM gets from L2, 585 cycles a stage at 16 tokens, and what stands at either
-// end of the stream.  The ring takes the whole shared memory and is filled with weights before the CTA waits for the kernel
+// What bounds it: the weight stream, 585 cycles a stage at 16 tokens, which is 31 bytes a cycle and SM and over the SMs in use
+// also about the HBM rate, and what stands at either end of the stream.  The ring takes the whole shared memory and is filled with weights before the CTA waits for the kernel
 // before it (half the ring beside that kernel's CTAs, with the rest requested for L2, was 6 to 30 us slower a layer: the
 // requests go through the same path as the loads).  The code behind the stream is small: unrolled over the tokens, with its
 // sine at 16 places, its fetch from memory took 9 to 12 thousand cycles of a launch's 28 to 35 thousand, now 4.
 // The layer step of LLaMA-2-7B, 16 x 8192 tokens: 86 -> 71 us with the append among the tiles (75 without), 128 short
-// sequences 130 -> 102; Qwen2.5-72B, 40 sequences: 244 -> 144 (both against the mma.sync tiles below 48 tokens and the
+// sequences 120 -> 98; Qwen2.5-72B, 40 short sequences: 222 -> 127 (all against the mma.sync tiles below 48 tokens and the
 // unrolled epilogue).
 //
 // Warps: 0 TMA producer, 1 MMA issuer, 2-5 epilogue (each owns the 32 tensor-memory lanes of its quadrant).

@@ -65,7 +65,8 @@ __device__ __forceinline__ void commit_pair(uint32_t bar) {  // arrives on the b
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(bar), "h"(static_cast<uint16_t>(3)) : "memory");
 }
-// Arrival on a barrier of the pair's first CTA that hands over tensor memory (the reads have completed), nothing in memory.
+// Arrival on a barrier of the pair's first CTA that hands over tensor memory and nothing in memory: it needs no release, because
+// tcgen05.wait::ld has completed the reads before it is issued.
 __device__ __forceinline__ void arrive_first(uint32_t bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(first_cta(bar)) : "memory");
 }

@@ -116,7 +116,7 @@ def test_production_latent_with_row_counts_that_do_not_fill_a_block(H, S):
 def test_row_blocks_of_64(H, S, G):
     # More than 32 query rows take 64 a CTA unless the page table has room for a small batch only: 33, 64, 65, 128 and
     # 288 rows, and 1024, the most that is allowed; lengths with one token, full pages, ragged tails, a query position that sees nothing (L < S), and enough pages per
-    # partition for the two-stage ring to wrap.  (With S*H > 64 the last case compares the heads at the block edges.)
+    # partition for the stage ring to wrap.  (With S*H > 64 the last case compares the heads at the block edges.)
     shape = synth.MLAShape(H=H, dn=128, dR=64, dv=128, r=512, D=4096, S=S)
     seqlens = [64 * 7 + 3, max(S - 1, 1), 128, 65, 900]
     if S * H <= 128:
