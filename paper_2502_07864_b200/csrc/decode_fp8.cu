@@ -569,9 +569,11 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
           // Lazy rescale: the reference maximum only moves when some row's new maximum exceeds it by 2^8.  Every
           // warp holds all 32 rows, so the four warps take the same decision without talking to each other.
           float alpha = 1.f;
-          bool rescale = !first && __any_sync(0xffffffffu, rowmax > m_used + 8.f);
+          // (Not after a give-up: what the warps then see may differ, and there are barriers below.)
+          // (a segment's first page moves it from -infinity)
+          bool rescale = __any_sync(0xffffffffu, rowmax > m_used + 8.f) && !aborted;
           uint32_t zero_rows = 0;
-          if (first || rescale) {
+          if (rescale) {
             const unsigned char* page_s = sm + kOffStage + stage * kStageBytes;
             zero_rows = find_zero_rows(page_s, warp, lane);
             int again;
@@ -585,12 +587,13 @@ decode_fp8_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_co
               asm volatile("bar.sync 1, 128;" ::: "memory");
               rowmax = fmaxf(fmaxf(pmax_s[(buf * 4 + 0) * 32 + lane], pmax_s[(buf * 4 + 1) * 32 + lane]),
                              fmaxf(pmax_s[(buf * 4 + 2) * 32 + lane], pmax_s[(buf * 4 + 3) * 32 + lane]));
-              rescale = !first && __any_sync(0xffffffffu, rowmax > m_used + 8.f);
+              rescale = __any_sync(0xffffffffu, rowmax > m_used + 8.f);
             }
           }
           if (tid == 0) mbar_arrive(bar(BAR_KV_EMPTY + stage));  // scales (and codes) have been read: the softmax warps' share
           if (first) {
             m_used = rowmax;
+            rescale = false;
           } else {
             if (rescale) {
               const float m_new = fmaxf(m_used, rowmax);

@@ -332,7 +332,8 @@ decode_sm100_kernel(const __grid_constant__ CUtensorMap cache_map, const __grid_
           if (first) {
             m_used = rowmax;
           } else {
-            rescale = __any_sync(0xffffffffu, rowmax > m_used + 8.f);
+            // (not after a give-up: what the warps then see may differ, and the rescale has a barrier)
+            rescale = __any_sync(0xffffffffu, rowmax > m_used + 8.f) && !aborted;
             if (rescale) {
               const float m_new = fmaxf(m_used, rowmax);
               alpha = (m_new == -INFINITY) ? 1.f : exp2f(m_used - m_new);
