@@ -12,17 +12,19 @@
 // up as well.
 //
 // A CTA pair (cta_group::2) works on a 256 x 256 tile of C, or a single CTA on a 128 x 128 one; either way a CTA converts
-// 128 rows of op(A) and 128 columns of op(B) a chunk.  Two groups of eight worker warps take the chunks in turn: they read
-// fp32 (whole 128-byte lines whatever the storage order) a chunk ahead, split, and write the terms to a four-stage ring in
-// shared memory - K-major where K is contiguous in memory (64-byte swizzle), MN-major where it is not (128-byte swizzle,
-// 64-wide pieces).  All sixteen drain the accumulators (two, in tensor memory) in between.  One warp of the pair's first
-// CTA issues the products.
-// Rates (fp32 products): 8192 x 4096 x 4096 185 TFLOP/s, X^T X of 8192 x 8064 303 (half of it mirrored), 8064 x 512 x 8064
-// 161; the fp32 multiply-add kernel this one replaced reached 48, 50 and 42.  What bounds it: a chunk takes about 3000
-// cycles, 1540 of them the tensor pipe's, in a ring of waits: sums drained (650) and reported to the issuer, products,
-// stages freed, pieces converted (900).  (With arrivals that release to the other CTA in every worker, which wait for the
-// thread's loads in flight, it took 4400; with the jobs split over converting and adding warps and the fp32 pieces fetched
-// through shared memory 2900 at more shared-memory traffic and no gain.)
+// 128 rows of op(A) and 128 columns of op(B) a chunk.  Eight converting warps read fp32 (whole 128-byte lines whatever the
+// storage order) a chunk ahead, split, and write the terms to a four-stage ring in shared memory - K-major where K is
+// contiguous in memory (64-byte swizzle), MN-major where it is not (128-byte swizzle, 64-wide pieces).  Eight adding warps
+// drain the accumulators (two, in tensor memory), 128 sums a thread.  One warp of the pair's first CTA issues the products.
+// Why two kinds of warps: an accumulator has to be drained while the product behind it runs (1540 cycles).  With all sixteen
+// warps doing both, a finished accumulator waited for the conversion its warp was in, and a chunk took 2730 cycles; now about
+// 1800, of which the converters wait 1100 for a free stage.  What bounds it is the tensor pipe under the power limit: 6 x 240
+// TFLOP/s of bf16 products, which is the rate cuBLAS sustains for seconds, at 1.45 GHz.
+// Rates (fp32 products), before -> now: 8192 x 4096 x 4096 218 -> 241 TFLOP/s, X^T X of 8192 x 8064 370 -> 436 (half of it
+// mirrored), 8064 x 512 x 8064 196 -> 228; the fp32 multiply-add kernel before those reached 48, 50 and 42.
+// (Arrivals that release to the other CTA wait for the thread's loads in flight: none in the converters.  fp32 pieces fetched
+// through shared memory: more of its traffic, no gain.  Two fp16 terms and three products a value: 311, 512 and 240 TFLOP/s,
+// but errors 5 to 25 % larger, and no range.)
 #include "conversion.cuh"
 #include "sm100_ptx.cuh"
 
@@ -35,14 +37,14 @@ namespace {
 
 constexpr int kRows = 128, kKc = 32;           // rows of op(A) and columns of op(B) a CTA converts; K per chunk
 constexpr int kStages = 4;
-constexpr int kWorkers = 512, kThreads = kWorkers + 128;   // the last warpgroup has one warp at work: issuer or messenger
+constexpr int kConverters = 256, kAdders = 256, kThreads = kConverters + kAdders + 128;  // the last warpgroup has one warp at work: issuer or messenger
 constexpr int kPlane = kRows * kKc * 2;        // 8192 bytes: one term of one operand's chunk
 constexpr int kStageBytes = 6 * kPlane;
 constexpr int kOffBar = kStages * kStageBytes;
 constexpr int kSmemBytes = kOffBar + 256 + 1024;
-constexpr int kLaunchRegs = 96, kWorkerRegs = 112, kIssuerRegs = 24;
+constexpr int kLaunchRegs = 96, kConverterRegs = 72, kAdderRegs = 152, kIssuerRegs = 24;
 static_assert(kSmemBytes <= 232448, "shared memory budget");
-static_assert(kThreads * kLaunchRegs <= 65536 && kWorkers * kWorkerRegs + 128 * kIssuerRegs <= kThreads * kLaunchRegs, "register split");
+static_assert(kThreads * kLaunchRegs <= 65536 && kConverters * kConverterRegs + kAdders * kAdderRegs + 128 * kIssuerRegs <= kThreads * kLaunchRegs, "register split");
 enum { BAR_FULL = 0, BAR_EMPTY = kStages, BAR_D_FULL = 2 * kStages, BAR_D_FREE = BAR_D_FULL + 2,
        BAR_FULL2 = BAR_D_FREE + 2, BAR_D_FREE2 = BAR_FULL2 + kStages, BAR_LAST = BAR_D_FREE2 + 2, BAR_COUNT };  // ..2: the second CTA's word
 static_assert(BAR_COUNT <= 24, "barrier block");
@@ -92,6 +94,12 @@ __device__ __forceinline__ void wait_for(uint32_t bar, uint32_t parity, volatile
   while (!try_wait<kCluster>(bar, parity)) {
     if (*abort_flag || clock64() - t0 > kLimit) { *abort_flag = 1; return; }
   }
+}
+
+__device__ __forceinline__ float2 add2(float2 s, uint32_t x, uint32_t y) {
+  asm("{\n.reg .b64 a, b;\nmov.b64 a, {%0, %1};\nmov.b64 b, {%2, %3};\nadd.rn.f32x2 a, a, b;\nmov.b64 {%0, %1}, a;\n}"
+      : "+f"(s.x), "+f"(s.y) : "r"(x), "r"(y));
+  return s;
 }
 
 struct GemmArgs {
@@ -192,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
 
   if (tid == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(bar(BAR_FULL + i), 8); mbar_init(bar(BAR_EMPTY + i), 1); mbar_init(bar(BAR_FULL2 + i), 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(bar(BAR_D_FULL + i), 1); mbar_init(bar(BAR_D_FREE + i), 16); mbar_init(bar(BAR_D_FREE2 + i), 16); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar(BAR_D_FULL + i), 1); mbar_init(bar(BAR_D_FREE + i), 8); mbar_init(bar(BAR_D_FREE2 + i), 8); }
     mbar_init(bar(BAR_LAST), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -214,10 +222,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
   auto wait = [&](uint32_t b, uint32_t parity) { wait_for<false, kLimit>(b, parity, abort_flag); };
   auto wait_cluster = [&](uint32_t b, uint32_t parity) { wait_for<true, kLimit>(b, parity, abort_flag); };
 
-  if (warp >= kWorkers / 32) {
+  if (warp >= (kConverters + kAdders) / 32) {
     // ========================================================================== MMA issuer
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssuerRegs));
-    if (warp == kWorkers / 32 && rank == 0) {
+    if (warp == (kConverters + kAdders) / 32 && rank == 0) {
       constexpr uint32_t idesc = instr_desc(kTile, !kAContig, kTile) | (kBContig ? 0u : 1u << 16);
       for (int c = 0; c < chunks; ++c) {
         const int stage = c % kStages, buf = c & 1;
@@ -252,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
       if (elect_one()) { if (kCtas == 2) tc_commit2(bar(BAR_LAST)); else tc_commit(bar(BAR_LAST)); }
       __syncwarp();
       for (const long long t0 = clock64(); !mbar_try_wait(bar(BAR_LAST), 0) && clock64() - t0 < kWaitCycles;) {}
-    } else if (rank == 1 && warp == kWorkers / 32) {
+    } else if (warp == (kConverters + kAdders) / 32) {
       // The second CTA's messenger tells the issuer of written stages: an arrival that releases to the other CTA waits for
       // everything its thread has in flight, which the workers must not.
       for (int c = 0; c < chunks; ++c) {
@@ -262,42 +270,19 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
         __syncwarp();
       }
     }
-  } else {
-    // ========================================================================== workers
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kWorkerRegs));
+  } else if (warp < kConverters / 32) {
+    // ========================================================================== converters
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConverterRegs));
     const bool vec_a = (args.lda & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
     const bool vec_b = (args.ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
-    constexpr int kCols = kTile / 4;                    // columns of the tile a thread sums: those of its warp's quarter
-    const int quad = warp & 3, quarter = warp >> 2;
-    const uint32_t d_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + quarter * kCols;
-    float acc[kCols];
-#pragma unroll
-    for (int j = 0; j < kCols; ++j) acc[j] = 0.f;
-    auto drain = [&](int d) {
-      const int buf = d & 1;
-      wait(bar(BAR_D_FULL + buf), (d >> 1) & 1);
-      tc_fence_after();
-#pragma unroll
-      for (int j0 = 0; j0 < kCols; j0 += 16) {
-        uint32_t v[16];
-        tmem_ld16(d_addr + buf * kTile + j0, v);
-        tc_wait_ld();
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j0 + j] += __uint_as_float(v[j]);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) { if (rank == 0) mbar_arrive(bar(BAR_D_FREE + buf)); else mbar_arrive_first_relaxed(bar(BAR_D_FREE2 + buf)); }
-    };
-    const int gtid = tid & 255;                         // thread of its group: two pieces of A and two of B a chunk
     const int nb0 = n0 + rank * kRows;                  // this CTA's columns of op(B)
-    float xa[2][8], xb[2][8];
+    float xa[2][8], xb[2][8];                           // two pieces of A and two of B a thread and chunk
     // Away from the edges a thread's pieces sit at fixed distances from one address per operand.
     const bool inside = vec_a && vec_b && m0 + kRows <= M && nb0 + kRows <= N;
-    const float* next_a = A + (kAContig ? static_cast<size_t>(m0 + (gtid >> 2)) * args.lda + (gtid & 3) * 8
-                                        : static_cast<size_t>(gtid >> 3) * args.lda + m0 + (gtid & 7) * 8);
-    const float* next_b = B + (kBContig ? static_cast<size_t>(nb0 + (gtid >> 2)) * args.ldb + (gtid & 3) * 8
-                                        : static_cast<size_t>(gtid >> 3) * args.ldb + nb0 + (gtid & 7) * 8);
+    const float* next_a = A + (kAContig ? static_cast<size_t>(m0 + (tid >> 2)) * args.lda + (tid & 3) * 8
+                                        : static_cast<size_t>(tid >> 3) * args.lda + m0 + (tid & 7) * 8);
+    const float* next_b = B + (kBContig ? static_cast<size_t>(nb0 + (tid >> 2)) * args.ldb + (tid & 3) * 8
+                                        : static_cast<size_t>(tid >> 3) * args.ldb + nb0 + (tid & 7) * 8);
     auto load8 = [](float (&x)[8], const float* src) {
       const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
       x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
@@ -314,35 +299,57 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        load_group<kAContig>(xa[u], A, vec_a, args.lda, m0, M, c * kKc, K, gtid + u * 256);
-        load_group<kBContig>(xb[u], B, vec_b, args.ldb, nb0, N, c * kKc, K, gtid + u * 256);
+        load_group<kAContig>(xa[u], A, vec_a, args.lda, m0, M, c * kKc, K, tid + u * 256);
+        load_group<kBContig>(xb[u], B, vec_b, args.ldb, nb0, N, c * kKc, K, tid + u * 256);
       }
     };
-    const int group = warp >> 3;
-    int drained = 0;
-    if (group < chunks) load(group);
-    for (int c = group; c < chunks; c += 2) {
+    load(0);
+    for (int c = 0; c < chunks; ++c) {
       const int stage = c % kStages;
       if (c >= kStages) wait(bar(BAR_EMPTY + stage), (c / kStages - 1) & 1);
       unsigned char* st = sm + stage * kStageBytes;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        store_group<kAContig>(xa[u], st, kPlane, gtid + u * 256);
-        store_group<kBContig>(xb[u], st + 3 * kPlane, kPlane, gtid + u * 256);
+        store_group<kAContig>(xa[u], st, kPlane, tid + u * 256);
+        store_group<kBContig>(xb[u], st + 3 * kPlane, kPlane, tid + u * 256);
       }
       fence_proxy_async();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(BAR_FULL + stage));
-      if (c + 2 < chunks) load(c + 2);
-      while (drained + 2 <= c) drain(drained++);
+      if (c + 1 < chunks) load(c + 1);
     }
-    while (drained < chunks) drain(drained++);
+  } else {
+    // ========================================================================== adders
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kAdderRegs));
+    constexpr int kCols = kTile / 2;                    // columns of the tile a thread sums: those of its warp's half
+    const int adder = warp - kConverters / 32, quad = warp & 3, half = adder >> 2;
+    const uint32_t d_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * kCols;
+    float2 acc2[kCols / 2];
+    float* const acc = reinterpret_cast<float*>(acc2);
+#pragma unroll
+    for (int j = 0; j < kCols / 2; ++j) acc2[j] = make_float2(0.f, 0.f);
+    for (int d = 0; d < chunks; ++d) {
+      const int buf = d & 1;
+      wait(bar(BAR_D_FULL + buf), (d >> 1) & 1);
+      tc_fence_after();
+#pragma unroll
+      for (int j0 = 0; j0 < kCols; j0 += 16) {
+        uint32_t v[16];
+        tmem_ld16(d_addr + buf * kTile + j0, v);
+        tc_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 16; j += 2) acc2[(j0 + j) / 2] = add2(acc2[(j0 + j) / 2], v[j], v[j + 1]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) { if (rank == 0) mbar_arrive(bar(BAR_D_FREE + buf)); else mbar_arrive_first_relaxed(bar(BAR_D_FREE2 + buf)); }
+    }
 
     // (After a give-up other warps may still be writing terms over these sums' staging place: NaN goes straight to C.)
     const bool bad = __any_sync(0xffffffffu, *abort_flag != 0);
     // ---- write-out through shared memory (every product has completed), in whole lines
     constexpr int kPitch = kCols + 4;
-    float* mine = reinterpret_cast<float*>(sm) + warp * 32 * kPitch;
+    float* mine = reinterpret_cast<float*>(sm) + adder * 32 * kPitch;
 #pragma unroll
     for (int j = 0; j < kCols; j += 4)
       *reinterpret_cast<float4*>(mine + lane * kPitch + j) =
@@ -358,14 +365,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
     if (small || __any_sync(0xffffffffu, !(all < INFINITY))) {
 #pragma unroll 1
       for (int j = 0; j < kCols; ++j) {
-        const int m = m0 + quad * 32 + lane, n = n0 + quarter * kCols + j;
+        const int m = m0 + quad * 32 + lane, n = n0 + half * kCols + j;
         if (m < M && n < N && (small || !isfinite(mine[lane * kPitch + j])))
           mine[lane * kPitch + j] = args.alpha * plain_sum<kAContig, kBContig>(args, m, n);
       }
     }
     __syncwarp();
     float* C = args.C + args.stride_c * blockIdx.y;
-    const int mw = m0 + quad * 32, nw = n0 + quarter * kCols;
+    const int mw = m0 + quad * 32, nw = n0 + half * kCols;
     const bool whole = !bad && !args.symmetric && n0 + kTile <= N && (args.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
     if (whole) {  // 16 bytes a lane
       constexpr int kLanes = kCols / 4, kAtOnce = 32 / kLanes;   // of a row; rows
