@@ -335,169 +335,224 @@ cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& part
 }
 
 // ------------------------------------------------------------------------------------------------
-// Combine + up-projection (Eq. 9 right, last line before W_O).  Block = one head x 8 or 16 query rows
+// Combine + up-projection (Eq. 9 right, last line before W_O).  Block = one head x kRows query rows
 // x (optionally) one half of the dv output columns.
-// Phase 1: each warp merges the split partials of its rows by their lse (segments of sequence b live
-// in slots i + b for the partitions i that overlap its pages) into shared memory as a bf16 hi/lo
+// Phase 1: each warp merges the split partials of its rows (or of half a row's latents) by their lse (segments of sequence b
+// live in slots i + b for the partitions i that overlap its pages) into shared memory as a bf16 hi/lo
 // pair, so that the tensor-core product of phase 2 carries fp32-like precision of o_hat.  The merged
-// row is stored in kperm order.
-// Phase 2: out[rows, h, :] = o_hat W_UV_h^T with W_UV_h read straight from global memory, 16 bytes per
-// lane and all loads of a tile in flight together.
+// rows are stored in kperm order.
+// Phase 2: out[rows, h, :]^T = W_UV_h o_hat^T with W_UV_h read straight from global memory, 16 bytes per lane: 16 output
+// columns a warp are the M of its products, 8 query rows the N.
+// What bounds it is a chain of round trips to L2 (look-ups of the row's partitions, their lse, the partials, the weights; a
+// partial's is 2000 to 3000 cycles with all blocks asking), then the mma.sync products, 16 cycles each on an SM's quarter:
+// with the rows as M, 16 of which 4 to 8 were there, and one accumulator for all, they took 3000 to 6400 cycles a tile.
 // ------------------------------------------------------------------------------------------------
-constexpr int kCombineRows = 16;
-
-// kPrefetch: hold the first weight tile in registers from before the dependency wait (few blocks, latency
-// matters); otherwise load weights window by window and keep the register count low enough for two blocks per SM.
-template <bool kPrefetch>
+// kPrefetch: hold the weights in registers from before the dependency wait, one block per SM; otherwise load them
+// between the phases and keep the register count low enough for two blocks per SM.
+template <int kRows, int kHalves, bool kPrefetch>
 __global__ void __launch_bounds__(256, kPrefetch ? 1 : 2) combine_kernel(const int32_t* cum,
                                                       const int32_t* plan,
                                                       const float* partial_o,
                                                       const float* partial_lse,
                                                       const __nv_bfloat16* __restrict__ w_uv,
                                                       __nv_bfloat16* out, float* lse_out,
-                                                      int B, int S, int H, int r, int dv, int G, int rows_per_block) {
+                                                      int B, int S, int H, int r, int dv, int G) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int kWarpsPerRow = kRows < 8 ? 8 / kRows : 1;
+  constexpr int kAtOnce = kRows > 8 ? 2 : 1;                    // rows a warp merges side by side
+  constexpr int kChunks = 4 / kWarpsPerRow;                     // 128-latent chunks of a row a warp merges
+  constexpr int kSegs = (kPrefetch ? 20 : 16) / (kAtOnce * kChunks);  // partials of each row in flight
+  constexpr int kWin = kPrefetch ? 16 : 16 / kHalves;           // windows of 32 latents whose weights are in registers at once
+  constexpr int kRowTiles = (kRows + 7) / 8;
   const int pitch = r + 8;
-  __nv_bfloat16* o_hi = reinterpret_cast<__nv_bfloat16*>(smem_raw);  // [16][pitch]
-  __nv_bfloat16* o_lo = o_hi + kCombineRows * pitch;                 // [16][pitch]
+  __nv_bfloat16* o_hi = reinterpret_cast<__nv_bfloat16*>(smem_raw);                 // [kRows, 8 at least][pitch]
+  __nv_bfloat16* o_lo = o_hi + (kRows < 8 ? 8 : kRows) * pitch;
   pdl_trigger();
-  const int h = blockIdx.x, bs0 = blockIdx.y * rows_per_block;
+  const int h = blockIdx.x, bs0 = blockIdx.y * kRows;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int SH = S * H, BS = B * S;
   const int g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
+  // kHalves = 2: tiles of 16 output columns, the block has all of them; 1: of 8 (M is half empty), it has half of them.
   const int tiles = dv / 8, tiles_per_z = (tiles + gridDim.z - 1) / gridDim.z;
   const int nt_lo = blockIdx.z * tiles_per_z, nt_hi = min(tiles, nt_lo + tiles_per_z);
-  // The weights do not depend on the merge: the first tile's 16-byte loads are issued now and land while
-  // the partials are merged.
-  constexpr int kWin = kPrefetch ? 16 : 4;  // windows of 32 columns held in registers per round
-  uint4 wv[kWin];
-  if (kPrefetch) {
-    const int nt = nt_lo + warp;
-    const __nv_bfloat16* wrow = w_uv + (static_cast<size_t>(h) * dv + min(nt, tiles - 1) * 8 + g) * r + t4 * 8;
+  uint4 wv[kHalves][kWin];
+  auto load_weights = [&](int nt, int w0) {
 #pragma unroll
-    for (int u = 0; u < kWin; ++u) wv[u] = (nt < nt_hi && u * 32 < r) ? ld_u128(wrow + u * 32) : make_uint4(0, 0, 0, 0);
-  }
+    for (int j = 0; j < kHalves; ++j) {
+      const __nv_bfloat16* wrow = w_uv + (static_cast<size_t>(h) * dv + min(nt + j, tiles - 1) * 8 + g) * r + t4 * 8;
+#pragma unroll
+      for (int u = 0; u < kWin; ++u)
+        wv[j][u] = (nt + j < nt_hi && w0 + u * 32 < r) ? ld_u128(wrow + w0 + u * 32) : make_uint4(0, 0, 0, 0);
+    }
+  };
+  const int nt_first = nt_lo + warp * kHalves;
+  // The weights do not depend on the merge: they are asked for now and land while the partials are merged.
+  if (kPrefetch) load_weights(nt_first, 0);
   pdl_wait();  // the partials and the prefix sums come from the kernels before this one
   const long long T = cum[B];
+  const bool dense = T >= G;  // then every partition owns at least one slot (of G at most)
+  const int32_t* seq_parts = cum + B + 1;  // only 4-byte aligned: B + 1 may be odd
 
-  for (int rr = warp; rr < kCombineRows; rr += 8) {
-    const int bs = bs0 + rr;
-    float acc[4][4];
+#pragma unroll 1
+  for (int r0 = warp / kWarpsPerRow; r0 < kRows; r0 += 8 * kAtOnce) {
+    const int c0 = kWarpsPerRow > 1 ? warp % kWarpsPerRow * (kChunks * 128) + lane * 4 : lane * 4;  // the lane's first latent
+    int nseg[kAtOnce], i_first[kAtOnce], batch[kAtOnce], row[kAtOnce];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.f;
-    float lse = -INFINITY, inv = 0.f;
-    if (rr < rows_per_block && bs < BS) {
-      const int b = bs / S, s = bs % S, row = s * H + h;
-      const int32_t* seq_parts = cum + B + 1;  // only 4-byte aligned: B + 1 may be odd
-      const int i_first = seq_parts[2 * b], nseg = seq_parts[2 * b + 1] - i_first + 1;
-      const bool dense = T >= G;  // then every partition owns at least one slot (of G at most)
-      if (nseg > 0) {
-        auto seg_lse = [&](int j) -> float {  // lse of the j-th candidate partition, -inf if it is empty or absent
-          if (j >= nseg) return -INFINITY;
-          const int pi = i_first + j;
-          const float l = partial_lse[static_cast<size_t>(pi + b) * SH + row];
-          if (!dense) {
-            const int2 range = *reinterpret_cast<const int2*>(plan + 4 * pi);
-            if (range.y <= range.x) return -INFINITY;
-          }
-          return l;
-        };
-        float m = -INFINITY;
-        for (int base = 0; base < nseg; base += 32) m = fmaxf(m, seg_lse(base + lane));
+    for (int u = 0; u < kAtOnce; ++u) {
+      const int bs = bs0 + r0 + 8 * u;
+      batch[u] = bs / S;
+      row[u] = bs % S * H + h;
+      i_first[u] = nseg[u] = 0;
+      if (bs < BS) {
+        i_first[u] = seq_parts[2 * batch[u]];
+        nseg[u] = seq_parts[2 * batch[u] + 1] - i_first[u] + 1;
+      }
+    }
+    auto seg_lse = [&](int u, int j) -> float {  // lse of the j-th candidate partition, -inf if it is empty or absent
+      if (j >= nseg[u]) return -INFINITY;
+      const int pi = i_first[u] + j;
+      const float l = partial_lse[static_cast<size_t>(pi + batch[u]) * SH + row[u]];
+      if (!dense) {
+        const int2 range = *reinterpret_cast<const int2*>(plan + 4 * pi);
+        if (range.y <= range.x) return -INFINITY;
+      }
+      return l;
+    };
+    float l_first[kAtOnce], m[kAtOnce], den[kAtOnce], acc[kAtOnce][kChunks][4];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (m > -INFINITY) {
-          float den = 0.f;
-          for (int base = 0; base < nseg; base += 32) {
-            const float l = seg_lse(base + lane);
-            const float wgt = l > -INFINITY ? __expf(l - m) : 0.f;
-            den += wgt;
-            const int cnt = min(32, nseg - base);
-            const float* po0 = partial_o + (static_cast<size_t>(i_first + base + b) * SH + row) * r + lane * 4;
-            const size_t seg_stride = static_cast<size_t>(SH) * r;
-            // four segments per round so that their loads overlap; a zero weight skips the (unwritten) slot
-            for (int j0 = 0; j0 < cnt; j0 += 4) {
-              float wj[4];
-              float4 v[4][4];
+    for (int u = 0; u < kAtOnce; ++u) l_first[u] = seg_lse(u, lane);
+    int most = 0;
 #pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                wj[u] = (j0 + u < cnt) ? __shfl_sync(0xffffffffu, wgt, (j0 + u) & 31) : 0.f;
+    for (int u = 0; u < kAtOnce; ++u) {
+      m[u] = l_first[u];
+      for (int base = 32; base < nseg[u]; base += 32) m[u] = fmaxf(m[u], seg_lse(u, base + lane));
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                  v[u][c] = make_float4(0.f, 0.f, 0.f, 0.f);
-                  if (wj[u] != 0.f && c * 128 + lane * 4 < r)
-                    v[u][c] = *reinterpret_cast<const float4*>(po0 + (j0 + u) * seg_stride + c * 128);
-                }
-              }
+      for (int o = 16; o > 0; o >>= 1) m[u] = fmaxf(m[u], __shfl_xor_sync(0xffffffffu, m[u], o));
+      if (m[u] == -INFINITY) nseg[u] = 0;  // nothing to merge
+      most = max(most, nseg[u]);
+      den[u] = 0.f;
 #pragma unroll
-              for (int u = 0; u < 4; ++u)
+      for (int c = 0; c < kChunks; ++c) acc[u][c][0] = acc[u][c][1] = acc[u][c][2] = acc[u][c][3] = 0.f;
+    }
+    const size_t seg_stride = static_cast<size_t>(SH) * r;
+#pragma unroll 1
+    for (int base = 0; base < most; base += 32) {
+      float wgt[kAtOnce];
+      const float* po[kAtOnce];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                  acc[c][0] = fmaf(wj[u], v[u][c].x, acc[c][0]); acc[c][1] = fmaf(wj[u], v[u][c].y, acc[c][1]);
-                  acc[c][2] = fmaf(wj[u], v[u][c].z, acc[c][2]); acc[c][3] = fmaf(wj[u], v[u][c].w, acc[c][3]);
-                }
+      for (int u = 0; u < kAtOnce; ++u) {
+        const float l = base == 0 ? l_first[u] : seg_lse(u, base + lane);
+        wgt[u] = nseg[u] > 0 && l > -INFINITY ? __expf(l - m[u]) : 0.f;
+        den[u] += wgt[u];
+        po[u] = partial_o + (static_cast<size_t>(i_first[u] + base + batch[u]) * SH + row[u]) * r + c0;
+      }
+      const int cnt = min(32, most - base);
+      // the loads of a round overlap; a zero weight skips the (unwritten) slot
+#pragma unroll 1
+      for (int j0 = 0; j0 < cnt; j0 += kSegs) {
+        float wj[kAtOnce][kSegs];
+        float4 v[kAtOnce][kSegs][kChunks];
+#pragma unroll
+        for (int u = 0; u < kAtOnce; ++u)
+#pragma unroll
+          for (int q = 0; q < kSegs; ++q) {
+            wj[u][q] = (j0 + q < cnt) ? __shfl_sync(0xffffffffu, wgt[u], (j0 + q) & 31) : 0.f;
+#pragma unroll
+            for (int c = 0; c < kChunks; ++c) {
+              v[u][q][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+              if (wj[u][q] != 0.f && c * 128 + c0 < r)
+                v[u][q][c] = *reinterpret_cast<const float4*>(po[u] + (j0 + q) * seg_stride + c * 128);
             }
           }
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
-          inv = 1.f / den;
-          lse = m + __logf(den);
-        }
+        for (int u = 0; u < kAtOnce; ++u)
+#pragma unroll
+          for (int q = 0; q < kSegs; ++q)
+#pragma unroll
+            for (int c = 0; c < kChunks; ++c) {
+              acc[u][c][0] = fmaf(wj[u][q], v[u][q][c].x, acc[u][c][0]); acc[u][c][1] = fmaf(wj[u][q], v[u][q][c].y, acc[u][c][1]);
+              acc[u][c][2] = fmaf(wj[u][q], v[u][q][c].z, acc[u][c][2]); acc[u][c][3] = fmaf(wj[u][q], v[u][q][c].w, acc[u][c][3]);
+            }
       }
-      if (lse_out != nullptr && lane == 0 && blockIdx.z == 0) lse_out[(static_cast<size_t>(b) * S + s) * H + h] = lse;
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int k = c * 128 + lane * 4;
-      if (k < r) {
-        float v[4], lo[4];
+    for (int u = 0; u < kAtOnce; ++u) {
+      float inv = 0.f, lse = -INFINITY;
+      if (nseg[u] > 0) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          v[e] = acc[c][e] * inv;
-          lo[e] = v[e] - __bfloat162float(__float2bfloat16_rn(v[e]));
+        for (int o = 16; o > 0; o >>= 1) den[u] += __shfl_xor_sync(0xffffffffu, den[u], o);
+        inv = 1.f / den[u];
+        lse = m[u] + __logf(den[u]);
+      }
+      const int rr = r0 + 8 * u;
+      if (lse_out != nullptr && lane == 0 && warp % kWarpsPerRow == 0 && blockIdx.z == 0 && bs0 + rr < BS)
+        lse_out[static_cast<size_t>(bs0 + rr) * H + h] = lse;
+#pragma unroll
+      for (int c = 0; c < kChunks; ++c) {
+        const int k = c * 128 + c0;
+        if (k < r) {
+          float v[4], lo[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            v[e] = acc[u][c][e] * inv;
+            lo[e] = v[e] - __bfloat162float(__float2bfloat16_rn(v[e]));
+          }
+          const int win = k & ~31, p = k & 31;  // elements p..p+3 of the window: two pairs, each stays adjacent
+          const int q0 = win + kperm(p), q1 = win + kperm(p + 2);
+          *reinterpret_cast<uint32_t*>(o_hi + rr * pitch + q0) = pack_bf16(v[0], v[1]);
+          *reinterpret_cast<uint32_t*>(o_hi + rr * pitch + q1) = pack_bf16(v[2], v[3]);
+          *reinterpret_cast<uint32_t*>(o_lo + rr * pitch + q0) = pack_bf16(lo[0], lo[1]);
+          *reinterpret_cast<uint32_t*>(o_lo + rr * pitch + q1) = pack_bf16(lo[2], lo[3]);
         }
-        const int win = k & ~31, p = k & 31;  // elements p..p+3 of the window: two pairs, each stays adjacent
-        const int q0 = win + kperm(p), q1 = win + kperm(p + 2);
-        *reinterpret_cast<uint32_t*>(o_hi + rr * pitch + q0) = pack_bf16(v[0], v[1]);
-        *reinterpret_cast<uint32_t*>(o_hi + rr * pitch + q1) = pack_bf16(v[2], v[3]);
-        *reinterpret_cast<uint32_t*>(o_lo + rr * pitch + q0) = pack_bf16(lo[0], lo[1]);
-        *reinterpret_cast<uint32_t*>(o_lo + rr * pitch + q1) = pack_bf16(lo[2], lo[3]);
       }
     }
   }
+  if (!kPrefetch) load_weights(nt_first, 0);
   __syncthreads();
 
-  for (int nt = nt_lo + warp; nt < nt_hi; nt += 8) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    const __nv_bfloat16* wrow = w_uv + (static_cast<size_t>(h) * dv + nt * 8 + g) * r + t4 * 8;
-    for (int w0 = 0; w0 < r; w0 += kWin * 32) {  // kWin windows per round, all their loads in flight together
-      if (!kPrefetch || nt != nt_lo + warp || w0 != 0) {
+  // (Rows 4 to 7 of a block that has 4 are whatever is there: nothing of them is stored, and a product's rows do not mix.)
+  for (int nt = nt_first; nt < nt_hi; nt += 8 * kHalves) {
+    float acc[kRowTiles][2][4];  // high and low part apart: two chains
 #pragma unroll
-        for (int u = 0; u < kWin; ++u)
-          wv[u] = (w0 + u * 32 < r) ? ld_u128(wrow + w0 + u * 32) : make_uint4(0, 0, 0, 0);
-      }
+    for (int n = 0; n < kRowTiles; ++n)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[n][e >> 2][e & 3] = 0.f;
+#pragma unroll 1
+    for (int w0 = 0; w0 < r; w0 += kWin * 32) {
+      if (nt != nt_first || w0 != 0) load_weights(nt, w0);
 #pragma unroll
       for (int u = 0; u < kWin; ++u) {
         if (w0 + u * 32 < r) {
-          uint32_t ah[4], al[4];
-          const int off = ((mi & 1) * 8 + (lane & 7)) * pitch + w0 + u * 32 + (mi >> 1) * 8;
-          ldmatrix_x4(ah, o_hi + off);
-          ldmatrix_x4(al, o_lo + off);
-          mma_bf16_16816(acc, ah, wv[u].x, wv[u].y);
-          mma_bf16_16816(acc, al, wv[u].x, wv[u].y);
-          ldmatrix_x4(ah, o_hi + off + 16);
-          ldmatrix_x4(al, o_lo + off + 16);
-          mma_bf16_16816(acc, ah, wv[u].z, wv[u].w);
-          mma_bf16_16816(acc, al, wv[u].z, wv[u].w);
+          const uint4 wa = wv[0][u], wb = kHalves == 2 ? wv[kHalves - 1][u] : make_uint4(0, 0, 0, 0);
+          const uint32_t a0[4] = {wa.x, wb.x, wa.y, wb.y}, a1[4] = {wa.z, wb.z, wa.w, wb.w};
+#pragma unroll
+          for (int n = 0; n < kRowTiles; ++n) {
+            uint32_t hi[4], lo[4];
+            const int off = (n * 8 + (lane & 7)) * pitch + w0 + u * 32 + mi * 8;
+            ldmatrix_x4(hi, o_hi + off);
+            ldmatrix_x4(lo, o_lo + off);
+            mma_bf16_16816(acc[n][0], a0, hi[0], hi[1]);
+            mma_bf16_16816(acc[n][1], a0, lo[0], lo[1]);
+            mma_bf16_16816(acc[n][0], a1, hi[2], hi[3]);
+            mma_bf16_16816(acc[n][1], a1, lo[2], lo[3]);
+          }
         }
       }
     }
-    const int col = nt * 8 + t4 * 2;
-    const int bs_a = bs0 + g, bs_b = bs0 + g + 8;
-    if (g < rows_per_block && bs_a < BS)
-      *reinterpret_cast<uint32_t*>(out + (static_cast<size_t>(bs_a) * H + h) * dv + col) = pack_bf16(acc[0], acc[1]);
-    if (g + 8 < rows_per_block && bs_b < BS)
-      *reinterpret_cast<uint32_t*>(out + (static_cast<size_t>(bs_b) * H + h) * dv + col) = pack_bf16(acc[2], acc[3]);
+    // A lane has columns g and (second half) g + 8 of rows 2 t4 and 2 t4 + 1: neighbouring columns meet by an exchange.
+#pragma unroll
+    for (int n = 0; n < kRowTiles; ++n) {
+#pragma unroll
+      for (int j = 0; j < kHalves; ++j) {
+        const float v0 = acc[n][0][2 * j] + acc[n][1][2 * j], v1 = acc[n][0][2 * j + 1] + acc[n][1][2 * j + 1];
+        // even g keeps row 2 t4, odd g row 2 t4 + 1, each of columns g & ~1 and g | 1
+        const float got = __shfl_xor_sync(0xffffffffu, g & 1 ? v0 : v1, 4);
+        const int rr = n * 8 + 2 * t4 + (g & 1), col = (nt + j) * 8 + (g & ~1);
+        if (nt + j < nt_hi && rr < kRows && bs0 + rr < BS)
+          *reinterpret_cast<uint32_t*>(out + (static_cast<size_t>(bs0 + rr) * H + h) * dv + col) =
+              g & 1 ? pack_bf16(got, v1) : pack_bf16(v0, got);
+      }
+    }
   }
 }
 
@@ -505,18 +560,22 @@ cudaError_t launch_combine(const transmla_params_t& p, int G, const int32_t* cum
                            const float* partial_lse, const __nv_bfloat16* w_uv, __nv_bfloat16* out, float* lse_out,
                            int32_t* dev_status, cudaStream_t stream) {
   (void)dev_status;
-  const int BS = p.batch * p.q_len;
-  // 8 rows per block while the register-prefetching variant runs (few query rows, more parallelism), 16 beyond:
-  // at 64 query rows that is 256 blocks, one wave at two blocks per SM, instead of 512
-  const int rows = BS <= 32 ? 8 : 16;
-  const int zsplit = (BS <= 64 && p.v_dim >= 128) ? 2 : 1;
-  dim3 grid(p.num_heads, (BS + rows - 1) / rows, zsplit);
-  const size_t smem = 2 * kCombineRows * (p.kv_lora_rank + 8) * sizeof(__nv_bfloat16);
-  if (BS <= 32)
-    return launch_pdl(combine_kernel<true>, grid, dim3(256), smem, stream, cum, plan, partial_o, partial_lse, w_uv, out, lse_out,
-                      p.batch, p.q_len, p.num_heads, p.kv_lora_rank, p.v_dim, G, rows);
-  return launch_pdl(combine_kernel<false>, grid, dim3(256), smem, stream, cum, plan, partial_o, partial_lse, w_uv, out, lse_out,
-                    p.batch, p.q_len, p.num_heads, p.kv_lora_rank, p.v_dim, G, rows);
+  const int BS = p.batch * p.q_len, H = p.num_heads;
+  constexpr int kSms = 148;
+  auto blocks = [&](int rows) { return static_cast<long long>(H) * ((BS + rows - 1) / rows); };
+  auto launch = [&](auto kernel, int rows, int halves) {
+    const size_t smem = 2 * (rows < 8 ? 8 : rows) * (p.kv_lora_rank + 8) * sizeof(__nv_bfloat16);
+    return launch_pdl(kernel, dim3(H, (BS + rows - 1) / rows, halves), dim3(256), smem, stream, cum, plan, partial_o, partial_lse, w_uv,
+                      out, lse_out, p.batch, p.q_len, H, p.kv_lora_rank, p.v_dim, G);
+  };
+  if (p.v_dim >= 128 && 2 * blocks(4) <= kSms) return launch(combine_kernel<4, 1, true>, 4, 2);
+  if (blocks(4) <= kSms) return launch(combine_kernel<4, 2, true>, 4, 1);
+  if (blocks(8) <= kSms) return launch(combine_kernel<8, 2, true>, 8, 1);
+  if (blocks(8) <= 2 * kSms) return launch(combine_kernel<8, 2, false>, 8, 1);
+  if (blocks(16) <= 2 * kSms) return launch(combine_kernel<16, 2, false>, 16, 1);
+  static PerDeviceFlag smem_set;
+  if (cudaError_t e = ensure_dynamic_smem(combine_kernel<32, 2, false>, 2 * 32 * (512 + 8) * 2, smem_set); e != cudaSuccess) return e;
+  return launch(combine_kernel<32, 2, false>, 32, 1);
 }
 
 }  // namespace transmla

@@ -3,6 +3,7 @@
 Tolerances (bf16 storage, fp32 accumulation): max-abs 2e-2 and relative L2 5e-3 on outputs;
 index paths (split plan, page slots, untouched cache bytes) bit-exact.
 """
+import dataclasses
 import math
 
 import numpy as np
@@ -172,6 +173,14 @@ def test_wide_heads_and_many_sequences():
     want, want_lse = gu.oracle_decode(synth.TINY, case, gu.mla_scale(synth.TINY), only=only)
     idx = tuple(np.array(only).T)
     gu.assert_close(lifts.f64(out)[idx], want[idx], 'many sequences')
+
+
+@pytest.mark.parametrize('B,S', [(8, 1), (9, 1), (16, 1), (17, 1), (33, 1), (73, 1), (74, 2), (149, 1)])
+def test_combine_forms(B, S):
+    # 32 heads: the launch changes its rows per block, halves of dv and weight prefetch at 8, 16, 32, 72 and 144 query rows;
+    # lengths that make a row of one partial, of several, and of none (a query position that sees nothing)
+    lens = [(7 * i) % 90 + 1 for i in range(B - 1)] + [64 * 40 + 5]
+    _run_and_compare(dataclasses.replace(synth.LLAMA2_7B, S=S), lens, seed=61)
 
 
 def test_qwen_shape_two_query_positions():
