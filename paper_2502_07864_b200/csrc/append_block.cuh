@@ -38,6 +38,38 @@ __device__ void append_block(const __nv_bfloat16* x, const __nv_bfloat16* __rest
   });
 }
 
+// The same by a cluster (see slice_gemm_tile); cluster c = (token tile, feature tile).
+template <int kTok>
+__device__ __forceinline__ void append_cluster(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w, const int32_t* pos_base,
+                                               int pos_shift, const int32_t* page_table, __nv_bfloat16* cache, int32_t* dev_status, int B,
+                                               int S, int D, int r, int dR, int num_pages, int max_pages, float theta, int cluster,
+                                               int rank, unsigned char* smem_raw) {
+  const int K = r + dR, f_tiles = (K + kSliceFeatures - 1) / kSliceFeatures, T = B * S;
+  struct Slot { int pos; __nv_bfloat16* row; };
+  slice_gemm_tile<kTok>(
+      x, w, D, K, cluster % f_tiles * kSliceFeatures, cluster / f_tiles * kTok, T, rank, smem_raw,
+      [&](int t) -> Slot {
+        if (t < 0) return {0, nullptr};
+        const int b = t / S, pos = pos_base[b] + pos_shift + t % S, pj = pos / kPage;
+        int page = -1;
+        if (pos >= 0 && pj < max_pages) page = page_table[static_cast<size_t>(b) * max_pages + pj];
+        if (page < 0 || page >= num_pages) {
+          set_status(dev_status, TRANSMLA_DEV_BAD_PAGE);
+          return {0, nullptr};
+        }
+        return {pos, cache + (static_cast<size_t>(page) * kPage + pos % kPage) * K};
+      },
+      [&](int, int f, float re, float im, Slot slot) {
+        if (slot.row == nullptr) return;
+        if (f >= r) rope_pair(re, im, slot.pos, (f - r) >> 1, dR, theta);  // RoPE pair l of the decoupled key (Eq. 1)
+        *reinterpret_cast<uint32_t*>(slot.row + f) = pack_bf16(re, im);
+      });
+}
+inline int append_clusters(const transmla_params_t& p) {
+  const int tok = slice_gemm_tokens(p.batch * p.q_len);
+  return (p.kv_lora_rank + p.qk_rope_dim + kSliceFeatures - 1) / kSliceFeatures * ((p.batch * p.q_len + tok - 1) / tok);
+}
+
 // Shared memory an append block needs, and how the host cuts the append into blocks.
 constexpr size_t kAppendBlockSmem = kAppendSmem;
 bool append_wide(const transmla_params_t& p);        // 32 features x 16 tokens per block instead of 8 x 64

@@ -8,25 +8,22 @@
 
 namespace transmla {
 
-// y[t, :] = [W_DKV; W_KR] x_t with RoPE on y[r:], fp32, into scratch [T, r + dR].  Block = 8 NT features x a share of the
-// tokens.  Bound by what an SM gets from L2: a block reads its features' weights and its tokens' activations.  64 tokens of
-// D = 4096: 72 blocks of 8 features and all tokens read 576 KB each, 144 of 16 features and 16 tokens 256 KB:
-// 19 -> 10.8 us.  The whole step at 64 tokens 106.5 -> 103 us, at 100 142.5 -> 122.7, at 128 shorter sequences 138 -> 108.
-// A value is the same sum in the same order in every form.
-template <int MAXMT, int NT>
-__global__ void __launch_bounds__(256) append_rows_f32_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w,
-                                                              const int32_t* positions, float* rows, int B, int S, int D, int r,
-                                                              int dR, float theta, int t_splits) {
+// y[t, :] = [W_DKV; W_KR] x_t with RoPE on y[r:], fp32, into scratch [T, r + dR] (r + dR = 576: whole tiles of 64 features).
+// 64 tokens of D = 4096: 9.5 us behind the kernel before it where one block per 16 features x 16 tokens took 20.
+template <int kTok>
+__global__ void __launch_bounds__(256, 2) append_rows_f32_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w,
+                                                                 const int32_t* positions, float* rows, int T, int S, int D, int r,
+                                                                 int dR, float theta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
-  const int K = r + dR, f_tiles = K / (8 * NT), f0 = (blockIdx.x % f_tiles) * 8 * NT;
-  const int t_chunk = (((B * S + t_splits - 1) / t_splits) + 15) & ~15;
-  const int t_begin = (blockIdx.x / f_tiles) * t_chunk, t_end = min(B * S, t_begin + t_chunk);
-  skinny_gemm_tile<MAXMT, NT>(x, w, D, f0, t_begin, t_end, smem_raw, [&](int t, int pr, float re, float im) {
-    const int f = f0 + pr * 2;
-    if (f >= r) rope_pair(re, im, positions[t / S] + t % S, (f - r) >> 1, dR, theta);  // RoPE pair l of the decoupled key (Eq. 1)
-    *reinterpret_cast<float2*>(rows + static_cast<size_t>(t) * K + f) = make_float2(re, im);
-  });
+  const int K = r + dR, f_tiles = K / kSliceFeatures, cluster = blockIdx.x / kSliceCtas;
+  slice_gemm_tile<kTok>(
+      x, w, D, K, cluster % f_tiles * kSliceFeatures, cluster / f_tiles * kTok, T, blockIdx.x % kSliceCtas, smem_raw,
+      [&](int t) { return t < 0 ? 0 : positions[t / S] + t % S; },
+      [&](int t, int f, float re, float im, int pos) {
+        if (f >= r) rope_pair(re, im, pos, (f - r) >> 1, dR, theta);  // RoPE pair l of the decoupled key (Eq. 1)
+        *reinterpret_cast<float2*>(rows + static_cast<size_t>(t) * K + f) = make_float2(re, im);
+      });
 }
 
 // One warp per token: scale = max|c| / 448 (1 for an all-zero row), codes = e4m3(c / scale), k^R / scale as bf16,
@@ -76,16 +73,14 @@ cudaError_t launch_append_fp8(const transmla_params_t& p, const __nv_bfloat16* x
                               const int32_t* page_table, void* cache_fp8, float* scratch, int32_t* dev_status,
                               cudaStream_t stream) {
   const int K = p.kv_lora_rank + p.qk_rope_dim, T = p.batch * p.q_len;
-  // Up to 48 tokens 8 features a block (the whole step at 33 tokens: 74.9 us, 77.1 in the next form), up to 64 tokens 16
-  // features x 16 tokens, beyond that 32 x 16: about as many blocks as SMs (r + dR = 576 is a multiple of 32).
-  const int ts = T <= 48 ? 1 : (T + 15) / 16 > 32 ? 32 : (T + 15) / 16;
-  auto rows = [&](auto kernel, int features) {
-    return launch_pdl(kernel, dim3(K / features * ts), dim3(256), kAppendSmem, stream, x, w, positions, scratch, p.batch, p.q_len,
-                      p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.rope_theta, ts);
+  const int tok = slice_gemm_tokens(T), clusters = K / kSliceFeatures * ((T + tok - 1) / tok);
+  static PerDeviceFlag smem_set[3];
+  auto rows = [&](auto kernel) -> cudaError_t {
+    if (cudaError_t e = ensure_dynamic_smem(kernel, static_cast<int>(slice_gemm_smem(tok)), smem_set[tok / 32]); e != cudaSuccess) return e;
+    return launch_slices(kernel, clusters * kSliceCtas, slice_gemm_smem(tok), stream, x, w, positions, scratch, T, p.q_len,
+                         p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.rope_theta);
   };
-  static_assert(skinny_gemm_smem(1, 4) <= kAppendSmem && skinny_gemm_smem(1, 2) <= kAppendSmem, "shared memory of the wide forms");
-  cudaError_t e = T <= 48 ? rows(append_rows_f32_kernel<kAppendMaxMT, 1>, 8)
-                          : T <= 64 ? rows(append_rows_f32_kernel<1, 2>, 16) : rows(append_rows_f32_kernel<1, 4>, 32);
+  const cudaError_t e = tok == 16 ? rows(append_rows_f32_kernel<16>) : tok == 32 ? rows(append_rows_f32_kernel<32>) : rows(append_rows_f32_kernel<64>);
   if (e != cudaSuccess) return e;
   return launch_pdl(quantize_rows_kernel, dim3((T + 3) / 4), dim3(128), static_cast<size_t>(0), stream,
                     static_cast<const float*>(scratch), positions, page_table, static_cast<unsigned char*>(cache_fp8), dev_status,

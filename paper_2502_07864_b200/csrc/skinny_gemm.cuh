@@ -126,4 +126,154 @@ __device__ __forceinline__ void skinny_gemm_tile(const __nv_bfloat16* x, const _
   }
 }
 
+// ------------------------------------------------------------------------------------------------
+// The append's form: a cluster of kSliceCtas CTAs owns 64 features x kTok tokens, each CTA a slice of the contracted
+// dimension, which it takes through shared memory 128 wide (asynchronous copies, three pieces in flight, the weights of the
+// first three from before the dependency wait).  Its warps take 32 of a piece's 128 each and half of the tokens (of the
+// features where there are few tokens), meet in shared memory, and the CTAs' sums meet through distributed shared memory: CTA
+// i finishes the i-th share of the tokens, adding the slices in order.  A value is the same sum in the same order whatever kTok.
+// What bounds the append is what an SM gets from L2 (30 bytes a cycle) and round trips: a block of 32 features x 16 tokens read
+// 384 KB at 128 tokens of D = 4096, one of 64 x 64 x D/8 reads 128, as many blocks.
+// ------------------------------------------------------------------------------------------------
+constexpr int kSliceCtas = 8, kSliceFeatures = 64, kSliceK = 128, kSliceStages = 3;
+constexpr int kSlicePitch = kSliceFeatures + 8;  // of the sums, floats (conflict-free fragments)
+constexpr int kSliceRow = kSliceK + 8;           // of the operands, bf16 (conflict-free ldmatrix)
+constexpr size_t slice_gemm_smem(int tokens) {
+  const size_t ring = static_cast<size_t>(kSliceStages) * (kSliceFeatures + tokens) * kSliceRow * sizeof(__nv_bfloat16);
+  const size_t sums = static_cast<size_t>(4) * tokens * kSlicePitch * sizeof(float);
+  return ring > sums ? ring : sums;
+}
+inline int slice_gemm_tokens(int T) { return T <= 16 ? 16 : T <= 32 ? 32 : 64; }
+
+__device__ __forceinline__ void slice_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// x [*, K] row-major, w [n_features, K] row-major, K a multiple of 256; features f0 .. f0 + 63 (those below n_features), tokens
+// t_begin .. t_begin + kTok - 1 (those below t_end).  rank: of the CTA in its cluster.  Each (token, pair of features) belongs
+// to one thread of the cluster: it calls prep(token) when the kernels before this one have finished, and
+// epi(token, f, value of f, value of f + 1, what prep gave) with the sums.
+template <int kTok, class Prep, class Epi>
+__device__ __forceinline__ void slice_gemm_tile(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w, int K, int n_features,
+                                                int f0, int t_begin, int t_end, int rank, unsigned char* smem_raw, Prep prep, Epi epi) {
+  constexpr int kWarpsT = kTok == 64 ? 2 : 1, kWarpsF = 2 / kWarpsT, kWarpsK = 4;
+  constexpr int MT = kTok / kWarpsT / 16, NT = kSliceFeatures / kWarpsF / 8;
+  constexpr int kStage = (kSliceFeatures + kTok) * kSliceRow;                   // bf16
+  __nv_bfloat16* ring = reinterpret_cast<__nv_bfloat16*>(smem_raw);             // stages of [features | tokens][kSliceRow]
+  float* red = reinterpret_cast<float*>(smem_raw);                              // later: [kWarpsK][kTok][kSlicePitch]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
+  const int wk = warp & 3, wt = kWarpsT == 2 ? warp >> 2 : 0, wf = kWarpsF == 2 ? warp >> 2 : 0;
+  const int k_lo = rank * (K / kSliceCtas), k_hi = k_lo + K / kSliceCtas, pieces = (K / kSliceCtas + kSliceK - 1) / kSliceK;
+  auto copy = [&](int piece, const __nv_bfloat16* src, int row0, int rows_end, int rows, int at) {  // 16 bytes a thread and turn
+    __nv_bfloat16* dst = ring + piece % kSliceStages * kStage + at * kSliceRow;
+#pragma unroll
+    for (int i = tid; i < rows * (kSliceK / 8); i += 256) {
+      const int rr = i / (kSliceK / 8), c = i % (kSliceK / 8) * 8, k = k_lo + piece * kSliceK + c;
+      const bool in = row0 + rr < rows_end && k < k_hi;  // the rest is filled with zeros
+      cp_async16(dst + rr * kSliceRow + c, src + (in ? static_cast<size_t>(row0 + rr) * K + k : 0), in ? 16 : 0);
+    }
+  };
+#pragma unroll
+  for (int p = 0; p < kSliceStages; ++p)
+    if (p < pieces) copy(p, w, f0, n_features, kSliceFeatures, 0);
+  cp_async_commit();
+  pdl_wait();  // activations and everything the epilogue touches may belong to kernels still in flight; weights may not
+#pragma unroll
+  for (int p = 0; p < kSliceStages; ++p) {
+    if (p < pieces) copy(p, x, t_begin, t_end, kTok, kSliceFeatures);
+    cp_async_commit();
+  }
+  const int my_t = t_begin + rank * (kTok / kSliceCtas) + (tid >> 5);
+  const bool mine = tid < kTok / kSliceCtas * 32 && my_t < t_end && f0 + 2 * lane < n_features;
+  auto prepared = prep(mine ? my_t : -1);
+  float acc[MT][NT][4];
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) acc[mt][nt][0] = acc[mt][nt][1] = acc[mt][nt][2] = acc[mt][nt][3] = 0.f;
+#pragma unroll 1
+  for (int p = 0; p < pieces; ++p) {
+    if (p == 0) cp_async_wait<kSliceStages - 1>(); else cp_async_wait<kSliceStages - 2>();
+    __syncthreads();  // the piece is there for all, and all have finished the one before
+    if (p > 0) {
+      const int q = p + kSliceStages - 1;
+      if (q < pieces) {
+        copy(q, w, f0, n_features, kSliceFeatures, 0);
+        copy(q, x, t_begin, t_end, kTok, kSliceFeatures);
+      }
+      cp_async_commit();
+    }
+    const __nv_bfloat16* ws = ring + p % kSliceStages * kStage + wf * NT * 8 * kSliceRow + wk * 32;
+    const __nv_bfloat16* xs = ring + p % kSliceStages * kStage + (kSliceFeatures + wt * MT * 16) * kSliceRow + wk * 32;
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+      uint32_t a[MT][4], b[NT / 2][4];
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) ldmatrix_x4(a[mt], xs + (mt * 16 + (mi & 1) * 8 + (lane & 7)) * kSliceRow + ks * 16 + (mi >> 1) * 8);
+#pragma unroll
+      for (int n2 = 0; n2 < NT / 2; ++n2) ldmatrix_x4(b[n2], ws + (n2 * 16 + (mi >> 1) * 8 + (lane & 7)) * kSliceRow + ks * 16 + (mi & 1) * 8);
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc[mt][nt], a[mt], b[nt / 2][nt % 2 * 2], b[nt / 2][nt % 2 * 2 + 1]);
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      float* d = red + (wk * kTok + (wt * MT + mt) * 16 + g) * kSlicePitch + (wf * NT + nt) * 8 + t4 * 2;
+      *reinterpret_cast<float2*>(d) = make_float2(acc[mt][nt][0], acc[mt][nt][1]);
+      *reinterpret_cast<float2*>(d + 8 * kSlicePitch) = make_float2(acc[mt][nt][2], acc[mt][nt][3]);
+    }
+  __syncthreads();
+#pragma unroll
+  for (int i = tid; i < kTok * 16; i += 256) {  // the CTA's sum takes the place of its first warp's
+    float4* d = reinterpret_cast<float4*>(red + (i >> 4) * kSlicePitch + (i & 15) * 4);
+    float4 sum = *d;
+#pragma unroll
+    for (int wv = 1; wv < kWarpsK; ++wv) {
+      const float4 v = *reinterpret_cast<const float4*>(red + (wv * kTok + (i >> 4)) * kSlicePitch + (i & 15) * 4);
+      sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+    }
+    *d = sum;
+  }
+  slice_cluster_sync();
+  if (mine) {
+    const uint32_t local = smem_u32(red + (my_t - t_begin) * kSlicePitch + 2 * lane);
+    float2 v[kSliceCtas];
+#pragma unroll
+    for (int c = 0; c < kSliceCtas; ++c) {
+      uint32_t remote;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(c));
+      asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v[c].x), "=f"(v[c].y) : "r"(remote) : "memory");
+    }
+    float re = v[0].x, im = v[0].y;
+#pragma unroll
+    for (int c = 1; c < kSliceCtas; ++c) { re += v[c].x; im += v[c].y; }
+    epi(my_t, f0 + 2 * lane, re, im, prepared);
+  }
+  slice_cluster_sync();  // nobody leaves while its memory may still be read
+}
+
+// Launch with programmatic dependent launch in clusters of kSliceCtas.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_slices(void (*kernel)(KArgs...), int blocks, size_t smem, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = kSliceCtas;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 }  // namespace transmla

@@ -100,22 +100,22 @@ __device__ void plan_block(const int32_t* seqlens, int B, Partitioning parts, in
 
 // ------------------------------------------------------------------------------------------------
 // Absorb (Eq. 9 right, first line): q_hat[bs,h,:r] = W_UK_h^T q_nope[bs,h,:], q_hat[bs,h,r:] = q_pe[bs,h,:].
-// A block owns nt consecutive 128-column tiles of one head's latent columns (nt = 1, or 2 when that brings the
-// launch down to one wave): it stages W_UK_h[:, tiles] and the head's query rows (128 at a time) in shared
-// memory with asynchronous 16-byte copies, all in flight together, and walks the rows in 16-row tiles, so W_UK
-// is read once.  The block that owns a head's first tile also copies the rope part of the rows.
+// A block owns 128 of one head's latent columns: it stages W_UK_h[:, columns] and the head's query rows (128 at a time) in
+// shared memory with asynchronous 16-byte copies, all in flight together, and walks the rows in 16-row tiles, so W_UK
+// is read once.  The block that owns a head's first columns also copies the rope part of the rows.
 // ------------------------------------------------------------------------------------------------
 constexpr int kAbsorbRows = 128;  // query rows staged per pass
 
 __device__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q_pe,
                              const __nv_bfloat16* __restrict__ w_uk, __nv_bfloat16* q_hat, int BS, int H,
-                             int dn, int dR, int r, int h, int rt0, int nt, unsigned char* smem_raw) {
-  const int apitch = dn + 8, wpitch = nt * 128 + 8;
+                             int dn, int dR, int r, int h, int rt0, unsigned char* smem_raw) {
+  constexpr int vec_per_row = 16, wpitch = 128 + 8;
+  const int apitch = dn + 8;
   __nv_bfloat16* w_s = reinterpret_cast<__nv_bfloat16*>(smem_raw);  // [dn][wpitch]
   __nv_bfloat16* a_s = w_s + dn * wpitch;                            // [kAbsorbRows][dn + 8]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
-  const int n0 = rt0 * 128, K = r + dR, vec_per_row = nt * 16;
+  const int n0 = rt0 * 128, K = r + dR;
   for (int i = tid; i < dn * vec_per_row; i += 256) {  // columns beyond r are zero-filled
     const int k = i / vec_per_row, c = i % vec_per_row;
     const bool in = n0 + c * 8 < r;
@@ -164,7 +164,8 @@ __device__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q
     cp_async_wait<0>();
     __syncthreads();
     for (int m0 = 0; m0 < rows16; m0 += 16) {
-      for (int wc = warp * 16 * nt; wc < (warp + 1) * 16 * nt; wc += 16) {  // this warp's 16-column steps
+      {
+        const int wc = warp * 16;  // this warp's columns
         float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll 4
         for (int ks = 0; ks < dn / 16; ++ks) {
@@ -188,44 +189,18 @@ __device__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q
   }
 }
 
-static size_t absorb_smem(int dn, int nt) {
-  return (static_cast<size_t>(dn) * (nt * 128 + 8) + static_cast<size_t>(kAbsorbRows) * (dn + 8)) * sizeof(__nv_bfloat16);
+static size_t absorb_smem(int dn) {
+  return (static_cast<size_t>(dn) * (128 + 8) + static_cast<size_t>(kAbsorbRows) * (dn + 8)) * sizeof(__nv_bfloat16);
 }
 
-// Tiles per absorb block: two when the prologue launch would otherwise not fit the device in one wave of one block
-// per SM (the append's accumulators allow no more), the tile count is even and the pair's weights fit.
-static int absorb_tiles_per_block(const transmla_params_t& p, int other_blocks) {
-  static PerDeviceFlag sms_of;  // SM count per device, asked once
-  const int slot = current_device_slot();
-  int sms = slot >= 0 ? sms_of.value[slot].load(std::memory_order_acquire) : 0;
-  if (sms == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-      cudaGetLastError();
-      return 1;
-    }
-    if (slot >= 0) sms_of.value[slot].store(sms, std::memory_order_release);
-  }
-  const int r_tiles = (p.kv_lora_rank + 127) / 128;
-  const bool fits_one = other_blocks + p.num_heads * r_tiles <= sms;
-  return (!fits_one && r_tiles % 2 == 0 && p.qk_nope_dim <= 128) ? 2 : 1;
-}
-
-__global__ void __launch_bounds__(256) append_kernel(const __nv_bfloat16* x,
-                                                     const __nv_bfloat16* __restrict__ w,
-                                                     const int32_t* positions,
-                                                     const int32_t* page_table,
-                                                     __nv_bfloat16* cache, int32_t* dev_status, int B,
-                                                     int S, int D, int r, int dR, int num_pages, int max_pages,
-                                                     float theta, int t_splits, int wide) {
+template <int kTok>
+__global__ void __launch_bounds__(256, 2) append_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w, const int32_t* positions,
+                                                        const int32_t* page_table, __nv_bfloat16* cache, int32_t* dev_status, int B,
+                                                        int S, int D, int r, int dR, int num_pages, int max_pages, float theta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
-  if (wide)
-    append_block<1, 4>(x, w, positions, 0, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
-                       blockIdx.x, t_splits, smem_raw);
-  else
-    append_block<kAppendMaxMT, 1>(x, w, positions, 0, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages,
-                                  theta, blockIdx.x, t_splits, smem_raw);
+  append_cluster<kTok>(x, w, positions, 0, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
+                       blockIdx.x / kSliceCtas, blockIdx.x % kSliceCtas, smem_raw);
 }
 
 // Absorb blocks followed by one plan block: everything transmla_mla_decode needs before the split-KV kernel.
@@ -235,49 +210,44 @@ __global__ void __launch_bounds__(256) absorb_plan_kernel(const __nv_bfloat16* q
                                                           __nv_bfloat16* q_hat,
                                                           const int32_t* seqlens, int32_t* cum,
                                                           int32_t* plan, int32_t* dev_status, int B, int S, int H,
-                                                          int dn, int dR, int r, Partitioning parts, int max_pages, int nt) {
+                                                          int dn, int dR, int r, Partitioning parts, int max_pages) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
-  const int per_head = (r + 127) / 128 / nt;  // absorb blocks per head, nt tiles each
+  const int per_head = (r + 127) / 128;  // absorb blocks per head
   const int n_absorb = H * per_head;
   if (static_cast<int>(blockIdx.x) < n_absorb) {
-    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, blockIdx.x / per_head, blockIdx.x % per_head * nt, nt, smem_raw);
+    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, blockIdx.x / per_head, blockIdx.x % per_head, smem_raw);
   } else {
     plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
   }
 }
 
-// The whole prologue of a decode step in one launch: plan block, append blocks, absorb blocks.
+// The whole prologue of a decode step in one launch: append clusters, plan block, absorb blocks.
 // The appended token of sequence b sits at seqlens[b] - S + s.
-__global__ void __launch_bounds__(256) prologue_kernel(
+template <int kTok>
+__global__ void __launch_bounds__(256, 2) prologue_kernel(
     const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w_dkv_kr,
     const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope,
     const __nv_bfloat16* q_pe, const __nv_bfloat16* __restrict__ w_uk, __nv_bfloat16* q_hat,
     const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status, int B, int S, int H, int D,
-    int dn, int dR, int r, int num_pages, int max_pages, float theta, Partitioning parts, int t_splits, int wide, int nt) {
+    int dn, int dR, int r, int num_pages, int max_pages, float theta, Partitioning parts, int n_append) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
-  const int n_append = (r + dR) / (wide ? 32 : 8) * t_splits;
-  const int per_head = (r + 127) / 128 / nt;  // absorb blocks per head, nt tiles each
-  const int bid = static_cast<int>(blockIdx.x) - 1;
+  const int per_head = (r + 127) / 128;  // absorb blocks per head
+  const int bid = static_cast<int>(blockIdx.x) - n_append * kSliceCtas;
   if (bid < 0) {
+    append_cluster<kTok>(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
+                         blockIdx.x / kSliceCtas, blockIdx.x % kSliceCtas, smem_raw);
+  } else if (bid == 0) {
     plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
-  } else if (bid < n_append) {
-    if (wide)
-      append_block<1, 4>(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages,
-                         theta, bid, t_splits, smem_raw);
-    else
-      append_block<kAppendMaxMT, 1>(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages,
-                                    max_pages, theta, bid, t_splits, smem_raw);
-  } else {
-    const int a = bid - n_append;
-    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, a / per_head, a % per_head * nt, nt, smem_raw);
+  } else if (bid <= H * per_head) {  // (the grid is whole clusters: a few blocks at its end have nothing to do)
+    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, (bid - 1) / per_head, (bid - 1) % per_head, smem_raw);
   }
 }
 
 constexpr int kPrologueMaxSmem = 144 * 1024;
 
-// Token splits of the append: one per 64 new tokens, at most 4.
+// The append as blocks of linear.cu's launch.  Token splits: one per 64 new tokens, at most 4.
 // With many new tokens a block takes 32 output features and 16 tokens (activations re-read a quarter as often
 // per feature, weights four times as often per token: 384 KB per block instead of 576 KB at 128 tokens).
 bool append_wide(const transmla_params_t& p) {
@@ -292,27 +262,29 @@ int append_token_splits(const transmla_params_t& p) {
 cudaError_t launch_append(const transmla_params_t& p, const __nv_bfloat16* x, const __nv_bfloat16* w,
                           const int32_t* positions, const int32_t* page_table, __nv_bfloat16* cache,
                           int32_t* dev_status, cudaStream_t stream) {
-  const int K = p.kv_lora_rank + p.qk_rope_dim;
-  const int ts = append_token_splits(p);
-  const int wide = append_wide(p) ? 1 : 0;
-  return launch_pdl(append_kernel, dim3(K / (wide ? 32 : 8) * ts), dim3(256), kAppendSmem, stream, x, w, positions, page_table,
-                    cache, dev_status, p.batch, p.q_len, p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.num_pages,
-                    p.max_pages_per_seq, p.rope_theta, ts, wide);
+  static PerDeviceFlag smem_set[3];
+  const int tok = slice_gemm_tokens(p.batch * p.q_len);
+  auto launch = [&](auto kernel) -> cudaError_t {
+    if (cudaError_t e = ensure_dynamic_smem(kernel, static_cast<int>(slice_gemm_smem(tok)), smem_set[tok / 32]); e != cudaSuccess) return e;
+    return launch_slices(kernel, append_clusters(p) * kSliceCtas, slice_gemm_smem(tok), stream, x, w, positions, page_table, cache,
+                         dev_status, p.batch, p.q_len, p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.num_pages,
+                         p.max_pages_per_seq, p.rope_theta);
+  };
+  return tok == 16 ? launch(append_kernel<16>) : tok == 32 ? launch(append_kernel<32>) : launch(append_kernel<64>);
 }
 
 cudaError_t launch_absorb_plan(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* q_nope,
                                const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                                const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
                                cudaStream_t stream) {
-  const int nt = absorb_tiles_per_block(p, 1);
-  size_t smem = absorb_smem(p.qk_nope_dim, nt);
+  size_t smem = absorb_smem(p.qk_nope_dim);
   if (smem < kPlanSmemSeqs * sizeof(int32_t)) smem = kPlanSmemSeqs * sizeof(int32_t);
   static PerDeviceFlag smem_set;  // zero-initialised; one slot per device
   if (cudaError_t e = ensure_dynamic_smem(absorb_plan_kernel, kPrologueMaxSmem, smem_set); e != cudaSuccess) return e;
-  const int blocks = p.num_heads * ((p.kv_lora_rank + 127) / 128 / nt) + 1;
+  const int blocks = p.num_heads * ((p.kv_lora_rank + 127) / 128) + 1;
   return launch_pdl(absorb_plan_kernel, dim3(blocks), dim3(256), smem, stream, q_nope, q_pe, w_uk, q_hat, seqlens, cum,
                     plan, dev_status, p.batch, p.q_len, p.num_heads, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, parts,
-                    p.max_pages_per_seq, nt);
+                    p.max_pages_per_seq);
 }
 
 cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
@@ -320,18 +292,19 @@ cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& part
                             const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                             const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
                             cudaStream_t stream) {
-  const int ts = append_token_splits(p);
-  const int wide = append_wide(p) ? 1 : 0;
-  const int n_append = (p.kv_lora_rank + p.qk_rope_dim) / (wide ? 32 : 8) * ts;
-  const int nt = absorb_tiles_per_block(p, 1 + n_append);
-  size_t smem = absorb_smem(p.qk_nope_dim, nt);
-  if (smem < kAppendSmem) smem = kAppendSmem;
-  static PerDeviceFlag smem_set;  // zero-initialised; one slot per device
-  if (cudaError_t e = ensure_dynamic_smem(prologue_kernel, kPrologueMaxSmem, smem_set); e != cudaSuccess) return e;
-  const int blocks = 1 + n_append + p.num_heads * ((p.kv_lora_rank + 127) / 128 / nt);
-  return launch_pdl(prologue_kernel, dim3(blocks), dim3(256), smem, stream, x, w_dkv_kr, page_table, cache, q_nope, q_pe,
-                    w_uk, q_hat, seqlens, cum, plan, dev_status, p.batch, p.q_len, p.num_heads, p.hidden_dim,
-                    p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, p.num_pages, p.max_pages_per_seq, p.rope_theta, parts, ts, wide, nt);
+  const int tok = slice_gemm_tokens(p.batch * p.q_len), n_append = append_clusters(p);
+  size_t smem = absorb_smem(p.qk_nope_dim);
+  if (smem < slice_gemm_smem(tok)) smem = slice_gemm_smem(tok);
+  const int others = 1 + p.num_heads * ((p.kv_lora_rank + 127) / 128);
+  const int blocks = (n_append + (others + kSliceCtas - 1) / kSliceCtas) * kSliceCtas;
+  static PerDeviceFlag smem_set[3];
+  auto launch = [&](auto kernel) -> cudaError_t {
+    if (cudaError_t e = ensure_dynamic_smem(kernel, kPrologueMaxSmem, smem_set[tok / 32]); e != cudaSuccess) return e;
+    return launch_slices(kernel, blocks, smem, stream, x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan,
+                         dev_status, p.batch, p.q_len, p.num_heads, p.hidden_dim, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank,
+                         p.num_pages, p.max_pages_per_seq, p.rope_theta, parts, n_append);
+  };
+  return tok == 16 ? launch(prologue_kernel<16>) : tok == 32 ? launch(prologue_kernel<32>) : launch(prologue_kernel<64>);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -388,6 +361,10 @@ __global__ void __launch_bounds__(256, kPrefetch ? 1 : 2) combine_kernel(const i
   const int nt_first = nt_lo + warp * kHalves;
   // The weights do not depend on the merge: they are asked for now and land while the partials are merged.
   if (kPrefetch) load_weights(nt_first, 0);
+  else {
+    const __nv_bfloat16* w = w_uv + (static_cast<size_t>(h) * dv + nt_lo * 8) * r;
+    for (int i = tid * 64; i < (nt_hi - nt_lo) * 8 * r; i += 256 * 64) prefetch_l2(w + i);
+  }
   pdl_wait();  // the partials and the prefix sums come from the kernels before this one
   const long long T = cum[B];
   const bool dense = T >= G;  // then every partition owns at least one slot (of G at most)

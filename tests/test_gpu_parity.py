@@ -337,6 +337,30 @@ def test_append_values_slots_and_untouched_bytes(shape, positions):
 
 
 # ------------------------------------------------------------------ whole step from host buffers
+@pytest.mark.parametrize('shape', [synth.LLAMA2_7B, synth.TINY])
+@pytest.mark.parametrize('B', [17, 32, 33, 65])
+def test_append_of_many_tokens_writes_the_bytes_of_few(shape, B):
+    # a cluster takes 16, 32 or 64 tokens, whichever the count asks for; a value's sum and its order do not change
+    positions = [3 + 5 * (i % 40) for i in range(B)]
+    ac = gu.to_dev(synth.make_append_case(shape, positions, 46))
+    pos = torch.tensor(positions, dtype=torch.int32, device='cuda')
+    cols = max(positions) // 64 + 1
+    table = torch.arange(B * cols, dtype=torch.int32, device='cuda').reshape(B, cols)
+    caches = []
+    for chunk in (B, 16):
+        cache = torch.zeros(B * cols, 64, shape.row, dtype=torch.bfloat16, device='cuda')
+        status = torch.zeros(1, dtype=torch.int32, device='cuda')
+        for i in range(0, B, chunk):
+            n = min(chunk, B - i)
+            params = binding.make_params(shape, n, B * cols, cols, 1.0)
+            binding.transmla_latent_append(params, ac['x'][i:i + n].contiguous(), ac['w_dkv_kr'], pos[i:i + n].contiguous(),
+                                           table[i:i + n].contiguous(), cache, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        caches.append(cache)
+    assert torch.equal(caches[0], caches[1])
+
+
 @pytest.mark.parametrize('pinned', [True, False])
 def test_decode_step_from_host_buffers(pinned):
     shape = synth.LLAMA2_7B
