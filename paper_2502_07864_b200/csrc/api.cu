@@ -203,10 +203,11 @@ static transmla_status_t launch_split_kv(const transmla_params_t* p, const trans
   return TRANSMLA_OK;
 }
 
-transmla_status_t transmla_mla_decode(const transmla_params_t* p, const void* q_nope, const void* q_pe,
-                                      const void* w_uk, const void* cache, const int32_t* page_table,
-                                      const int32_t* seqlens, void* workspace, size_t workspace_bytes,
-                                      int32_t* dev_status, void* stream) {
+extern "C++" {
+namespace transmla {
+transmla_status_t mla_decode(const transmla_params_t* p, const void* q_nope, const void* q_pe, const void* w_uk, const void* cache,
+                             const int32_t* page_table, const int32_t* seqlens, void* workspace, size_t workspace_bytes,
+                             int32_t* dev_status, bool behind_maps, void* stream) {
   transmla_workspace_layout_t lay;
   transmla_status_t st = check_decode_args(p, q_nope, q_pe, w_uk, cache, page_table, seqlens, workspace,
                                            workspace_bytes, dev_status, &lay);
@@ -217,9 +218,18 @@ transmla_status_t transmla_mla_decode(const transmla_params_t* p, const void* q_
                          static_cast<const __nv_bfloat16*>(q_pe), static_cast<const __nv_bfloat16*>(w_uk),
                          reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset), seqlens,
                          reinterpret_cast<int32_t*>(ws + lay.cum_pages_offset),
-                         reinterpret_cast<int32_t*>(ws + lay.plan_offset), dev_status, s) != cudaSuccess)
+                         reinterpret_cast<int32_t*>(ws + lay.plan_offset), dev_status, behind_maps, s) != cudaSuccess)
     return TRANSMLA_ERR_CUDA;
   return launch_split_kv(p, lay, cache, page_table, seqlens, ws, dev_status, s);
+}
+}  // namespace transmla
+}  // extern "C++"
+
+transmla_status_t transmla_mla_decode(const transmla_params_t* p, const void* q_nope, const void* q_pe,
+                                      const void* w_uk, const void* cache, const int32_t* page_table,
+                                      const int32_t* seqlens, void* workspace, size_t workspace_bytes,
+                                      int32_t* dev_status, void* stream) {
+  return mla_decode(p, q_nope, q_pe, w_uk, cache, page_table, seqlens, workspace, workspace_bytes, dev_status, false, stream);
 }
 
 transmla_status_t transmla_mla_combine(const transmla_params_t* p, const void* workspace, size_t workspace_bytes,
@@ -280,7 +290,7 @@ transmla_status_t transmla_mla_decode_fp8(const transmla_params_t* p, const void
                          static_cast<const __nv_bfloat16*>(q_pe), static_cast<const __nv_bfloat16*>(w_uk),
                          reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset), seqlens,
                          reinterpret_cast<int32_t*>(ws + lay.cum_pages_offset),
-                         reinterpret_cast<int32_t*>(ws + lay.plan_offset), dev_status, s) != cudaSuccess)
+                         reinterpret_cast<int32_t*>(ws + lay.plan_offset), dev_status, false, s) != cudaSuccess)
     return TRANSMLA_ERR_CUDA;
   cudaEvent_t ev0 = tl_prof_start, ev1 = tl_prof_stop;
   tl_prof_start = tl_prof_stop = nullptr;

@@ -39,15 +39,14 @@ __device__ void append_block(const __nv_bfloat16* x, const __nv_bfloat16* __rest
 }
 
 // The same by a cluster (see slice_gemm_tile); cluster c = (token tile, feature tile).
-template <int kTok>
 __device__ __forceinline__ void append_cluster(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w, const int32_t* pos_base,
                                                int pos_shift, const int32_t* page_table, __nv_bfloat16* cache, int32_t* dev_status, int B,
                                                int S, int D, int r, int dR, int num_pages, int max_pages, float theta, int cluster,
                                                int rank, unsigned char* smem_raw) {
   const int K = r + dR, f_tiles = (K + kSliceFeatures - 1) / kSliceFeatures, T = B * S;
   struct Slot { int pos; __nv_bfloat16* row; };
-  slice_gemm_tile<kTok>(
-      x, w, D, K, cluster % f_tiles * kSliceFeatures, cluster / f_tiles * kTok, T, rank, smem_raw,
+  slice_gemm_tile(
+      x, w, D, K, cluster % f_tiles * kSliceFeatures, cluster / f_tiles * kSliceTokens, T, rank, smem_raw,
       [&](int t) -> Slot {
         if (t < 0) return {0, nullptr};
         const int b = t / S, pos = pos_base[b] + pos_shift + t % S, pj = pos / kPage;
@@ -66,9 +65,17 @@ __device__ __forceinline__ void append_cluster(const __nv_bfloat16* x, const __n
       });
 }
 inline int append_clusters(const transmla_params_t& p) {
-  const int tok = slice_gemm_tokens(p.batch * p.q_len);
-  return (p.kv_lora_rank + p.qk_rope_dim + kSliceFeatures - 1) / kSliceFeatures * ((p.batch * p.q_len + tok - 1) / tok);
+  return (p.kv_lora_rank + p.qk_rope_dim + kSliceFeatures - 1) / kSliceFeatures * ((p.batch * p.q_len + kSliceTokens - 1) / kSliceTokens);
 }
+
+// The append, and the whole prologue, on the Blackwell tensor path (prologue_sm100.cu).
+bool prologue_sm100_supported(const transmla_params_t& p);
+cudaError_t launch_append_sm100(const transmla_params_t& p, const __nv_bfloat16* x, const __nv_bfloat16* w, const int32_t* positions,
+                                const int32_t* page_table, __nv_bfloat16* cache, float* rows_f32, int32_t* dev_status, cudaStream_t stream);
+cudaError_t launch_absorb_sm100(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
+                                const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope, const __nv_bfloat16* q_pe,
+                                const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat, const int32_t* seqlens, int32_t* cum, int32_t* plan,
+                                int32_t* dev_status, cudaStream_t stream);  // x null: without the append
 
 // Shared memory an append block needs, and how the host cuts the append into blocks.
 constexpr size_t kAppendBlockSmem = kAppendSmem;

@@ -4,27 +4,9 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
-#include "skinny_gemm.cuh"
+#include "append_block.cuh"
 
 namespace transmla {
-
-// y[t, :] = [W_DKV; W_KR] x_t with RoPE on y[r:], fp32, into scratch [T, r + dR] (r + dR = 576: whole tiles of 64 features).
-// 64 tokens of D = 4096: 9.5 us behind the kernel before it where one block per 16 features x 16 tokens took 20.
-template <int kTok>
-__global__ void __launch_bounds__(256, 2) append_rows_f32_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w,
-                                                                 const int32_t* positions, float* rows, int T, int S, int D, int r,
-                                                                 int dR, float theta) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_trigger();
-  const int K = r + dR, f_tiles = K / kSliceFeatures, cluster = blockIdx.x / kSliceCtas;
-  slice_gemm_tile<kTok>(
-      x, w, D, K, cluster % f_tiles * kSliceFeatures, cluster / f_tiles * kTok, T, blockIdx.x % kSliceCtas, smem_raw,
-      [&](int t) { return t < 0 ? 0 : positions[t / S] + t % S; },
-      [&](int t, int f, float re, float im, int pos) {
-        if (f >= r) rope_pair(re, im, pos, (f - r) >> 1, dR, theta);  // RoPE pair l of the decoupled key (Eq. 1)
-        *reinterpret_cast<float2*>(rows + static_cast<size_t>(t) * K + f) = make_float2(re, im);
-      });
-}
 
 // One warp per token: scale = max|c| / 448 (1 for an all-zero row), codes = e4m3(c / scale), k^R / scale as bf16,
 // written to the token's 656-byte row.  r = 512, dR = 64.
@@ -72,16 +54,9 @@ __global__ void __launch_bounds__(128) quantize_rows_kernel(const float* rows, c
 cudaError_t launch_append_fp8(const transmla_params_t& p, const __nv_bfloat16* x, const __nv_bfloat16* w, const int32_t* positions,
                               const int32_t* page_table, void* cache_fp8, float* scratch, int32_t* dev_status,
                               cudaStream_t stream) {
-  const int K = p.kv_lora_rank + p.qk_rope_dim, T = p.batch * p.q_len;
-  const int tok = slice_gemm_tokens(T), clusters = K / kSliceFeatures * ((T + tok - 1) / tok);
-  static PerDeviceFlag smem_set[3];
-  auto rows = [&](auto kernel) -> cudaError_t {
-    if (cudaError_t e = ensure_dynamic_smem(kernel, static_cast<int>(slice_gemm_smem(tok)), smem_set[tok / 32]); e != cudaSuccess) return e;
-    return launch_slices(kernel, clusters * kSliceCtas, slice_gemm_smem(tok), stream, x, w, positions, scratch, T, p.q_len,
-                         p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.rope_theta);
-  };
-  const cudaError_t e = tok == 16 ? rows(append_rows_f32_kernel<16>) : tok == 32 ? rows(append_rows_f32_kernel<32>) : rows(append_rows_f32_kernel<64>);
-  if (e != cudaSuccess) return e;
+  const int T = p.batch * p.q_len;
+  // (the FP8 cache has the shape that kernel takes: r = 512, dR = 64; it is not asked for dn, which the append does not have)
+  if (cudaError_t e = launch_append_sm100(p, x, w, positions, page_table, nullptr, scratch, dev_status, stream); e != cudaSuccess) return e;
   return launch_pdl(quantize_rows_kernel, dim3((T + 3) / 4), dim3(128), static_cast<size_t>(0), stream,
                     static_cast<const float*>(scratch), positions, page_table, static_cast<unsigned char*>(cache_fp8), dev_status,
                     p.batch, p.q_len, p.num_pages, p.max_pages_per_seq);

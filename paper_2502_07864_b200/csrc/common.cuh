@@ -192,6 +192,11 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 // The partition count the library chooses for a kernel that takes `rows` query rows a CTA.
 transmla_status_t library_partitions(const transmla_params_t& p, int rows, int* partitions);
 
+// transmla_mla_decode; behind_maps: the launch before it is one of linear maps.
+transmla_status_t mla_decode(const transmla_params_t* p, const void* q_nope, const void* q_pe, const void* w_uk, const void* cache,
+                             const int32_t* page_table, const int32_t* seqlens, void* workspace, size_t workspace_bytes,
+                             int32_t* dev_status, bool behind_maps, void* stream);
+
 // Every host-side check of transmla_decode_step, without launching anything.
 transmla_status_t validate_step_args(const transmla_params_t* p, const void* x, const void* q_nope, const void* q_pe,
                                      const void* w_dkv_kr, const void* w_uk, const void* w_uv, const void* cache,
@@ -217,7 +222,7 @@ bool dynamic_claims(const transmla_params_t& p, int G);  // whether the split-KV
 cudaError_t launch_absorb_plan(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* q_nope,
                                const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                                const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
-                               cudaStream_t stream);
+                               bool behind_maps, cudaStream_t stream);
 cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
                             const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope,
                             const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,

@@ -156,7 +156,7 @@ transmla_status_t transmla_layer_decode_step(const transmla_params_t* p, const t
   a.append = AppendJob{};
 
   if (appended) {  // the new tokens' rows are in the cache (or on their way, earlier in the stream): attention only
-    st = transmla_mla_decode(p, q_nope, q_pe, w->w_uk, cache, page_table, seqlens, workspace, workspace_bytes, dev_status, stream);
+    st = mla_decode(p, q_nope, q_pe, w->w_uk, cache, page_table, seqlens, workspace, workspace_bytes, dev_status, true, stream);
     if (st == TRANSMLA_OK)
       st = transmla_mla_combine(p, workspace, workspace_bytes, w->w_uv, attn, nullptr, dev_status, stream);
   } else {

@@ -14,11 +14,14 @@ __device__ __forceinline__ uint4 ld_u128(const __nv_bfloat16* p) { return *reint
 // RoPE of Eq. 1 on the pair (re, im) = elements (2l, 2l+1) of a d-vector at position pos.  The angle is formed
 // and reduced to [-pi, pi] in fp64 so that positions of 10^5 keep their phase; sine and cosine are fp32.
 __device__ __forceinline__ double rope_freq(int l, int d, float theta) { return exp2(-2.0 * l / d * log2(static_cast<double>(theta))); }
-__device__ __forceinline__ void rope_pair_at(float& re, float& im, int pos, double freq) {
+__device__ __forceinline__ void rope_angle(int pos, double freq, float& cs, float& sn) {
   const double ang = static_cast<double>(pos) * freq;
   const double red_ang = ang - 6.283185307179586476925 * rint(ang * 0.15915494309189533577);
-  float sn, cs;
   sincosf(static_cast<float>(red_ang), &sn, &cs);
+}
+__device__ __forceinline__ void rope_pair_at(float& re, float& im, int pos, double freq) {
+  float sn, cs;
+  rope_angle(pos, freq, cs, sn);
   const float nre = re * cs - im * sn, nim = im * cs + re * sn;
   re = nre;
   im = nim;
@@ -127,41 +130,36 @@ __device__ __forceinline__ void skinny_gemm_tile(const __nv_bfloat16* x, const _
 }
 
 // ------------------------------------------------------------------------------------------------
-// The append's form: a cluster of kSliceCtas CTAs owns 64 features x kTok tokens, each CTA a slice of the contracted
-// dimension, which it takes through shared memory 128 wide (asynchronous copies, three pieces in flight, the weights of the
-// first three from before the dependency wait).  Its warps take 32 of a piece's 128 each and half of the tokens (of the
-// features where there are few tokens), meet in shared memory, and the CTAs' sums meet through distributed shared memory: CTA
-// i finishes the i-th share of the tokens, adding the slices in order.  A value is the same sum in the same order whatever kTok.
-// What bounds the append is what an SM gets from L2 (30 bytes a cycle) and round trips: a block of 32 features x 16 tokens read
+// The append's form for latents and rope keys of any size (r = 512, dR = 64 has prologue_sm100.cu): a cluster of kSliceCtas
+// CTAs owns 64 features x 64 tokens, each CTA a slice of the contracted dimension, which it takes through shared memory 128
+// wide (asynchronous copies, three pieces in flight, the weights of the first three from before the dependency wait).  Its
+// warps take 32 of a piece's 128 each and half of the tokens, meet in shared memory, and the CTAs' sums meet through
+// distributed shared memory: CTA i finishes the i-th share of the tokens, adding the slices in order.
+// What bounds it is what an SM gets from L2 (30 bytes a cycle) and round trips: a block of 32 features x 16 tokens read
 // 384 KB at 128 tokens of D = 4096, one of 64 x 64 x D/8 reads 128, as many blocks.
 // ------------------------------------------------------------------------------------------------
-constexpr int kSliceCtas = 8, kSliceFeatures = 64, kSliceK = 128, kSliceStages = 3;
+constexpr int kSliceCtas = 8, kSliceFeatures = 64, kSliceTokens = 64, kSliceK = 128, kSliceStages = 3;
 constexpr int kSlicePitch = kSliceFeatures + 8;  // of the sums, floats (conflict-free fragments)
 constexpr int kSliceRow = kSliceK + 8;           // of the operands, bf16 (conflict-free ldmatrix)
-constexpr size_t slice_gemm_smem(int tokens) {
-  const size_t ring = static_cast<size_t>(kSliceStages) * (kSliceFeatures + tokens) * kSliceRow * sizeof(__nv_bfloat16);
-  const size_t sums = static_cast<size_t>(4) * tokens * kSlicePitch * sizeof(float);
-  return ring > sums ? ring : sums;
-}
-inline int slice_gemm_tokens(int T) { return T <= 16 ? 16 : T <= 32 ? 32 : 64; }
+constexpr size_t kSliceSmem = static_cast<size_t>(kSliceStages) * (kSliceFeatures + kSliceTokens) * kSliceRow * sizeof(__nv_bfloat16);
+static_assert(4 * kSliceTokens * kSlicePitch * sizeof(float) <= kSliceSmem, "the warps' sums take the ring's place");
 
 __device__ __forceinline__ void slice_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // x [*, K] row-major, w [n_features, K] row-major, K a multiple of 256; features f0 .. f0 + 63 (those below n_features), tokens
-// t_begin .. t_begin + kTok - 1 (those below t_end).  rank: of the CTA in its cluster.  Each (token, pair of features) belongs
+// t_begin .. t_begin + 63 (those below t_end).  rank: of the CTA in its cluster.  Each (token, pair of features) belongs
 // to one thread of the cluster: it calls prep(token) when the kernels before this one have finished, and
 // epi(token, f, value of f, value of f + 1, what prep gave) with the sums.
-template <int kTok, class Prep, class Epi>
+template <class Prep, class Epi>
 __device__ __forceinline__ void slice_gemm_tile(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w, int K, int n_features,
                                                 int f0, int t_begin, int t_end, int rank, unsigned char* smem_raw, Prep prep, Epi epi) {
-  constexpr int kWarpsT = kTok == 64 ? 2 : 1, kWarpsF = 2 / kWarpsT, kWarpsK = 4;
-  constexpr int MT = kTok / kWarpsT / 16, NT = kSliceFeatures / kWarpsF / 8;
+  constexpr int kTok = kSliceTokens, kWarpsK = 4, MT = kTok / 2 / 16, NT = kSliceFeatures / 8;
   constexpr int kStage = (kSliceFeatures + kTok) * kSliceRow;                   // bf16
   __nv_bfloat16* ring = reinterpret_cast<__nv_bfloat16*>(smem_raw);             // stages of [features | tokens][kSliceRow]
   float* red = reinterpret_cast<float*>(smem_raw);                              // later: [kWarpsK][kTok][kSlicePitch]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
-  const int wk = warp & 3, wt = kWarpsT == 2 ? warp >> 2 : 0, wf = kWarpsF == 2 ? warp >> 2 : 0;
+  const int wk = warp & 3, wt = warp >> 2;
   const int k_lo = rank * (K / kSliceCtas), k_hi = k_lo + K / kSliceCtas, pieces = (K / kSliceCtas + kSliceK - 1) / kSliceK;
   auto copy = [&](int piece, const __nv_bfloat16* src, int row0, int rows_end, int rows, int at) {  // 16 bytes a thread and turn
     __nv_bfloat16* dst = ring + piece % kSliceStages * kStage + at * kSliceRow;
@@ -202,7 +200,7 @@ __device__ __forceinline__ void slice_gemm_tile(const __nv_bfloat16* x, const __
       }
       cp_async_commit();
     }
-    const __nv_bfloat16* ws = ring + p % kSliceStages * kStage + wf * NT * 8 * kSliceRow + wk * 32;
+    const __nv_bfloat16* ws = ring + p % kSliceStages * kStage + wk * 32;
     const __nv_bfloat16* xs = ring + p % kSliceStages * kStage + (kSliceFeatures + wt * MT * 16) * kSliceRow + wk * 32;
 #pragma unroll
     for (int ks = 0; ks < 2; ++ks) {
@@ -223,7 +221,7 @@ __device__ __forceinline__ void slice_gemm_tile(const __nv_bfloat16* x, const __
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
-      float* d = red + (wk * kTok + (wt * MT + mt) * 16 + g) * kSlicePitch + (wf * NT + nt) * 8 + t4 * 2;
+      float* d = red + (wk * kTok + (wt * MT + mt) * 16 + g) * kSlicePitch + nt * 8 + t4 * 2;
       *reinterpret_cast<float2*>(d) = make_float2(acc[mt][nt][0], acc[mt][nt][1]);
       *reinterpret_cast<float2*>(d + 8 * kSlicePitch) = make_float2(acc[mt][nt][2], acc[mt][nt][3]);
     }

@@ -13,6 +13,7 @@
 // is stored there in the matching order (kperm below).
 #include "append_block.cuh"
 #include "common.cuh"
+#include "plan_block.cuh"
 #include "skinny_gemm.cuh"
 
 namespace transmla {
@@ -20,83 +21,6 @@ namespace transmla {
 // Position, inside its 32-wide window, at which element p must sit in shared memory so that ldmatrix
 // hands out the fragment that pairs with a uint4 global load of the other operand.
 __device__ __forceinline__ int kperm(int p) { return ((p & 7) >> 1) * 8 + (p >> 3) * 2 + (p & 1); }
-
-// ------------------------------------------------------------------------------------------------
-// Split plan.  Every non-empty sequence owns ceil(L_b/P) page slots preceded by kSegCost virtual slots (the
-// price of opening a sequence); cum[b] = slots before sequence b; partition i owns slots
-// [floor(i*T/G), floor((i+1)*T/G)), of the G that are planned (see plan_block); plan row = (begin, end, sequence of first slot, of last slot).
-// One block of 256 threads; the scan runs in chunks of 256 sequences; the prefix sums are kept in
-// shared memory (when they fit) for the binary searches.
-// ------------------------------------------------------------------------------------------------
-constexpr int kPlanSmemSeqs = 4096;
-
-__device__ __forceinline__ int seq_of_page(const int32_t* cum, int B, int x) {
-  // the b in [0, B) with cum[b] <= x < cum[b+1]  ==  (first index with cum > x) - 1
-  int lo = 0, hi = B + 1;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (cum[mid] > x) hi = mid; else lo = mid + 1;
-  }
-  return lo - 1;
-}
-
-__device__ void plan_block(const int32_t* seqlens, int B, Partitioning parts, int RB, int max_pages, int32_t* cum, int32_t* plan,
-                           int32_t* dev_status, unsigned char* smem_raw) {
-  __shared__ int warp_sums[8];
-  __shared__ int carry;
-  int32_t* cum_s = reinterpret_cast<int32_t*>(smem_raw);  // [B+1] when B < kPlanSmemSeqs
-  const bool in_smem = B < kPlanSmemSeqs;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int sequences = 0;  // that are not empty
-  pdl_wait();
-  if (tid == 0) { carry = 0; cum[0] = 0; if (in_smem) cum_s[0] = 0; }
-  __syncthreads();
-  for (int base = 0; base < B; base += 256) {
-    const int b = base + tid;
-    int n = 0;
-    if (b < B) { const int L = clamped_len(seqlens[b], max_pages, dev_status); n = L > 0 ? (L + kPage - 1) / kPage + kSegCost : 0; }
-    int v = n;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { int t = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += t; }
-    if (lane == 31) warp_sums[warp] = v;
-    __syncthreads();
-    int before = carry;
-    for (int w = 0; w < warp; ++w) before += warp_sums[w];
-    const int incl = v + before;
-    if (b < B) { cum[b + 1] = incl; if (in_smem) cum_s[b + 1] = incl; }
-    sequences += __syncthreads_count(n > 0);
-    if (tid == 255) carry = incl;
-    __syncthreads();
-  }
-  const int32_t* cs = in_smem ? cum_s : cum;
-  const long long T = cs[B];
-  const int G = parts.count(static_cast<int>(T) - kSegCost * sequences, sequences);
-  for (int i = G + tid; i < parts.most; i += 256) reinterpret_cast<int4*>(plan)[i] = make_int4(0, 0, -1, -1);
-  for (int i = tid; i < G; i += 256) {
-    const int p0 = static_cast<int>((static_cast<long long>(i) * T) / G);
-    const int p1 = static_cast<int>((static_cast<long long>(i + 1) * T) / G);
-    int b0 = -1, b1 = -1;
-    if (p1 > p0) { b0 = seq_of_page(cs, B, p0); b1 = seq_of_page(cs, B, p1 - 1); }
-    reinterpret_cast<int4*>(plan)[i] = make_int4(p0, p1, b0, b1);
-  }
-  // Partitions that hold pages of sequence b: first and last index (0, -1 for an empty sequence), stored behind
-  // the prefix sums so that the combine does not repeat the 64-bit divisions for every row and head.
-  int32_t* seq_parts = cum + B + 1;
-  for (int b = tid; b < B; b += 256) {
-    const long long c0 = static_cast<long long>(cs[b]) + kSegCost, c1 = cs[b + 1];
-    int i_first = 0, i_last = -1;
-    if (c1 > c0) {
-      i_first = static_cast<int>(((c0 + 1) * G - 1) / T);
-      i_last = static_cast<int>((c1 * G - 1) / T);
-    }
-    seq_parts[2 * b] = i_first;
-    seq_parts[2 * b + 1] = i_last;
-  }
-  // The page counters of the split-KV kernel start at zero.  Every earlier kernel of the stream has completed
-  // here (the dependency wait above), so nobody is still counting.
-  int32_t* next = cum + 3 * B + 1;
-  for (int i = tid; i < RB * B; i += 256) next[i] = 0;
-}
 
 // ------------------------------------------------------------------------------------------------
 // Absorb (Eq. 9 right, first line): q_hat[bs,h,:r] = W_UK_h^T q_nope[bs,h,:], q_hat[bs,h,r:] = q_pe[bs,h,:].
@@ -193,13 +117,12 @@ static size_t absorb_smem(int dn) {
   return (static_cast<size_t>(dn) * (128 + 8) + static_cast<size_t>(kAbsorbRows) * (dn + 8)) * sizeof(__nv_bfloat16);
 }
 
-template <int kTok>
 __global__ void __launch_bounds__(256, 2) append_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w, const int32_t* positions,
                                                         const int32_t* page_table, __nv_bfloat16* cache, int32_t* dev_status, int B,
                                                         int S, int D, int r, int dR, int num_pages, int max_pages, float theta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
-  append_cluster<kTok>(x, w, positions, 0, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
+  append_cluster(x, w, positions, 0, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
                        blockIdx.x / kSliceCtas, blockIdx.x % kSliceCtas, smem_raw);
 }
 
@@ -224,7 +147,6 @@ __global__ void __launch_bounds__(256) absorb_plan_kernel(const __nv_bfloat16* q
 
 // The whole prologue of a decode step in one launch: append clusters, plan block, absorb blocks.
 // The appended token of sequence b sits at seqlens[b] - S + s.
-template <int kTok>
 __global__ void __launch_bounds__(256, 2) prologue_kernel(
     const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w_dkv_kr,
     const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope,
@@ -236,7 +158,7 @@ __global__ void __launch_bounds__(256, 2) prologue_kernel(
   const int per_head = (r + 127) / 128;  // absorb blocks per head
   const int bid = static_cast<int>(blockIdx.x) - n_append * kSliceCtas;
   if (bid < 0) {
-    append_cluster<kTok>(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
+    append_cluster(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
                          blockIdx.x / kSliceCtas, blockIdx.x % kSliceCtas, smem_raw);
   } else if (bid == 0) {
     plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
@@ -262,21 +184,23 @@ int append_token_splits(const transmla_params_t& p) {
 cudaError_t launch_append(const transmla_params_t& p, const __nv_bfloat16* x, const __nv_bfloat16* w,
                           const int32_t* positions, const int32_t* page_table, __nv_bfloat16* cache,
                           int32_t* dev_status, cudaStream_t stream) {
-  static PerDeviceFlag smem_set[3];
-  const int tok = slice_gemm_tokens(p.batch * p.q_len);
-  auto launch = [&](auto kernel) -> cudaError_t {
-    if (cudaError_t e = ensure_dynamic_smem(kernel, static_cast<int>(slice_gemm_smem(tok)), smem_set[tok / 32]); e != cudaSuccess) return e;
-    return launch_slices(kernel, append_clusters(p) * kSliceCtas, slice_gemm_smem(tok), stream, x, w, positions, page_table, cache,
-                         dev_status, p.batch, p.q_len, p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.num_pages,
-                         p.max_pages_per_seq, p.rope_theta);
-  };
-  return tok == 16 ? launch(append_kernel<16>) : tok == 32 ? launch(append_kernel<32>) : launch(append_kernel<64>);
+  if (prologue_sm100_supported(p)) return launch_append_sm100(p, x, w, positions, page_table, cache, nullptr, dev_status, stream);
+  static PerDeviceFlag smem_set;
+  if (cudaError_t e = ensure_dynamic_smem(append_kernel, static_cast<int>(kSliceSmem), smem_set); e != cudaSuccess) return e;
+  return launch_slices(append_kernel, append_clusters(p) * kSliceCtas, kSliceSmem, stream, x, w, positions, page_table, cache,
+                       dev_status, p.batch, p.q_len, p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.num_pages,
+                       p.max_pages_per_seq, p.rope_theta);
 }
 
 cudaError_t launch_absorb_plan(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* q_nope,
                                const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                                const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
-                               cudaStream_t stream) {
+                               bool behind_maps, cudaStream_t stream) {
+  // Few rows behind a launch of linear maps: the maps' CTAs leave some SMs free, where more and shorter blocks end sooner
+  // (layer step, mma.sync / tcgen05: 1 token 47.1 / 47.6 us, 16 70.5 / 71.9, 32 75.6 / 76.0, 48 91.1 / 90.1, 64 91.0 / 85.1; 64
+  // heads: 8 99.6 / 101.3, 32 118.2 / 118.5, 64 145.4 / 143.2; behind the FP8 append: 4 35.7 / 35.6, 16 55.2 / 52.0).
+  if (prologue_sm100_supported(p) && !(behind_maps && p.batch * p.q_len <= 32))
+    return launch_absorb_sm100(p, parts, nullptr, nullptr, nullptr, nullptr, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan, dev_status, stream);
   size_t smem = absorb_smem(p.qk_nope_dim);
   if (smem < kPlanSmemSeqs * sizeof(int32_t)) smem = kPlanSmemSeqs * sizeof(int32_t);
   static PerDeviceFlag smem_set;  // zero-initialised; one slot per device
@@ -292,19 +216,18 @@ cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& part
                             const __nv_bfloat16* q_pe, const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat,
                             const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status,
                             cudaStream_t stream) {
-  const int tok = slice_gemm_tokens(p.batch * p.q_len), n_append = append_clusters(p);
+  if (prologue_sm100_supported(p))
+    return launch_absorb_sm100(p, parts, x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan, dev_status, stream);
+  const int n_append = append_clusters(p);
   size_t smem = absorb_smem(p.qk_nope_dim);
-  if (smem < slice_gemm_smem(tok)) smem = slice_gemm_smem(tok);
+  if (smem < kSliceSmem) smem = kSliceSmem;
   const int others = 1 + p.num_heads * ((p.kv_lora_rank + 127) / 128);
   const int blocks = (n_append + (others + kSliceCtas - 1) / kSliceCtas) * kSliceCtas;
-  static PerDeviceFlag smem_set[3];
-  auto launch = [&](auto kernel) -> cudaError_t {
-    if (cudaError_t e = ensure_dynamic_smem(kernel, kPrologueMaxSmem, smem_set[tok / 32]); e != cudaSuccess) return e;
-    return launch_slices(kernel, blocks, smem, stream, x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan,
-                         dev_status, p.batch, p.q_len, p.num_heads, p.hidden_dim, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank,
-                         p.num_pages, p.max_pages_per_seq, p.rope_theta, parts, n_append);
-  };
-  return tok == 16 ? launch(prologue_kernel<16>) : tok == 32 ? launch(prologue_kernel<32>) : launch(prologue_kernel<64>);
+  static PerDeviceFlag smem_set;
+  if (cudaError_t e = ensure_dynamic_smem(prologue_kernel, kPrologueMaxSmem, smem_set); e != cudaSuccess) return e;
+  return launch_slices(prologue_kernel, blocks, smem, stream, x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan,
+                       dev_status, p.batch, p.q_len, p.num_heads, p.hidden_dim, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank,
+                       p.num_pages, p.max_pages_per_seq, p.rope_theta, parts, n_append);
 }
 
 // ------------------------------------------------------------------------------------------------
