@@ -4,9 +4,11 @@
 // cholesky_kernel   L^-T in fp64 by one cluster of CTAs, rounded to fp32
 // gemm_f32          Q = Y L^-T, with the products exact to fp32 (conversion_gemm.cu)
 // For a basis of 512 columns of length 8064: 0.24 + 1.86 + 0.74 ms in the form this one replaced (whole G, one block for the
-// factor, a triangular solve per row), now 0.13 + 0.22 + 0.03.
-#include "conversion.cuh"
+// factor, a triangular solve per row), now 0.13 + 0.14 + 0.03.
+#include <type_traits>
+
 #include "common.cuh"
+#include "conversion.cuh"
 
 namespace transmla {
 namespace conv {
@@ -120,264 +122,339 @@ __global__ void sum_slices_kernel(const double* part, int r, int slices, double*
 // ------------------------------------------------------------------------------------------------ Cholesky factor
 // Right-looking blocked factorisation in blocks of 32, with the rows of an identity carried along below G: what the
 // factorisation does to them makes them X = L^-T (X L^T = I).  One cluster; per panel p, with P(.,p) the finished columns
-//   all CTAs   D = G(p,p) - P(p,p-1) P(p,p-1)^T, factored and inverted by warp 0 of each (the same bits everywhere, which
-//              saves a meeting), while warps 1-7 apply panel p-1 to the rest: first to this CTA's blocks of column p, then to
+//   all CTAs   D = G(p,p) - P(p,p-1) P(p,p-1)^T, factored by warp 0 of each and inverted by warp 4 (the same bits everywhere, which
+//              saves a meeting), while the others apply panel p-1 to the rest: first to this CTA's blocks of column p, then to
 //              its share of the blocks behind column p
 //   each CTA   P(R,p) = B(R,p) L(p,p)^-T for its blocks R of column p: G rows below p, and X rows up to p
-// and one cluster barrier.  What bounds it is the chain of r square roots and the updates between them, about 300 cycles
-// each, with the fp64 units beside it: a block's product takes one SM's units 1000 cycles, and a panel has about 100 of them.
+// and one cluster barrier.  What bounds it is the chain of r square roots with the steps between them, and a panel's round trips to
+// L2: D's operands, the barrier.  The products are fp64 tensor instructions (at the fp64 units' rate, with a sixth of the
+// instructions), a block's operands are asked for at the start of the panel, and the factor takes four columns a step.
 // (A device that cannot hold 16 such CTAs in a cluster gets 8, 4, .. of them: what it holds at once is asked.)
-// At r = 512: 359 us by 8 CTAs with the own blocks one a warp, 221 us by 16 (the cluster's size limit with the opt-in), four
-// rows of a block a warp and whole lines moved.  Rows and columns beyond r behave as an identity.
-constexpr int NB = 32, kCluster = kOrthCluster, kCholThreads = 256, kPitch = NB + 1, kBlock = NB * kPitch;
-constexpr int kMaxBlocks = 1024 / NB, kMaxOwn = kMaxBlocks / kCluster;
-// doubles: D, W, P(p,p-1), col[2][32], the CTA's blocks of column p, two operands for each of warps 1-7
-constexpr int kCholSmem = (3 * kBlock + 2 * NB + kMaxOwn * kBlock + 14 * kBlock) * 8;
+// Rows and columns beyond r behave as an identity.
+// At r = 512, cycles a panel: 26 000 with one column a step (12 000 in the factor, beside multiply-adds of 16 000 in warps of the same
+// quarter of the SM), now 15 500 (D 1900, factor 8900, P 1500, barrier 2000 and more); 218 -> 136 us.
+constexpr int NB = 32, kCluster = kOrthCluster, kCholThreads = 384, kPitch = NB + 4, kBlock = NB * kPitch;  // (conflict-free fragments)
+constexpr int kMaxBlocks = 1024 / NB, kMaxOwn = kMaxBlocks / kCluster, kStep = 16 + 4 * NB, kExchange = 16 + NB / 4 * kStep;
+// Warps with a part in the products: not those of the factor's quarter of the SM, which has its fp64 units alone.  The first
+// kFormers form a block of column p and come last where the blocks behind it are shared out.
+constexpr int kWorkers = 9, kFormers = 4;
+// doubles: D, W, P(p,p-1), the factor's exchange, the CTA's blocks of column p, two operands for each worker
+constexpr int kCholSmem = (3 * kBlock + kExchange + kMaxOwn * kBlock + 2 * kWorkers * kBlock) * 8;
 static_assert(kCholSmem <= 232448, "shared memory budget");
 
 struct CholView {
   double* G;   // [r, r], lower
   double* X;   // [r, r], upper
   int r, n;    // n block rows of each
-  bool even;   // pairs of elements are aligned
-  __device__ __forceinline__ bool next(int c, int j) const { return c * NB + j + 1 < r; }
+  bool even;   // pairs of elements are aligned, and both inside or both outside
   // element (i, j) of block (R, c): R < n rows of G, otherwise rows of X
   __device__ __forceinline__ double* at(int R, int c, int i, int j, bool& in) const {
     const int row = (R < n ? R : R - n) * NB + i, col = c * NB + j;
     in = row < r && col < r;
     return (R < n ? G : X) + static_cast<size_t>(row) * r + col;
   }
-};
-// A warp copies block (R, c) to shared memory (pitch 33).
-__device__ __forceinline__ void load_block(const CholView& v, int R, int c, double* dst, int lane) {
-  double x[NB];  // all on their way before the first is stored
-#pragma unroll
-  for (int i = 0; i < NB; ++i) {
+  __device__ __forceinline__ double load(int R, int c, int i, int j) const {
     bool in;
-    const double* p = v.at(R, c, i, lane, in);
-    x[i] = in ? __ldcg(p) : 0.0;
+    const double* p = at(R, c, i, j, in);
+    return in ? __ldcg(p) : 0.0;
   }
-#pragma unroll
-  for (int i = 0; i < NB; ++i) dst[i * kPitch + lane] = x[i];
+  // elements (i, j) and (i, j + 1), j even
+  __device__ __forceinline__ double2 load2(int R, int c, int i, int j) const {
+    bool in;
+    const double* p = at(R, c, i, j, in);
+    double2 e = make_double2(0.0, 0.0);
+    if (in && even) e = __ldcg(reinterpret_cast<const double2*>(p));
+    else if (in) { e.x = __ldcg(p); if (c * NB + j + 1 < r) e.y = __ldcg(p + 1); }
+    return e;
+  }
+  __device__ __forceinline__ void store2(int R, int c, int i, int j, double2 e) const {
+    bool in;
+    double* p = at(R, c, i, j, in);
+    if (in && even) __stcg(reinterpret_cast<double2*>(p), e);
+    else if (in) { __stcg(p, e.x); if (c * NB + j + 1 < r) __stcg(p + 1, e.y); }
+  }
+};
+// c += a b for 8 x 8 x 4: lane l has a(l/4, l%4), b(l%4, l/4) and c(l/4, 2 (l%4) + {0, 1}).
+__device__ __forceinline__ void mma_f64(double2& c, double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c.x), "+d"(c.y) : "d"(a), "d"(b));
 }
-// A lane's elements of a product: rows l/8 + 4i for i from `from`, columns 2 (l%8) + {0, 1} + 16h: eight lanes move one line.
-template <int kRows>
-__device__ __forceinline__ void load_elements(const CholView& v, int R, int c, int from, double (&x)[kRows][4], int lane) {
+// A warp asks for block (R, c) in shared memory; the caller waits (cp_async_wait, __syncwarp).
+__device__ __forceinline__ void fetch_block(const CholView& v, int R, int c, double* dst, int lane) {
+  if (v.even) {
 #pragma unroll
-  for (int i = 0; i < kRows; ++i) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int u = 0; u < NB / 2; ++u) {  // 16 lanes a row
+      const int i = 2 * u + (lane >> 4), j = 2 * (lane & 15);
       bool in;
-      const double* p = v.at(R, c, (lane >> 3) + 4 * (from + i), 2 * (lane & 7) + 16 * h, in);
-      double2 e = make_double2(0.0, 0.0);
-      if (in && v.even) e = __ldcg(reinterpret_cast<const double2*>(p));  // an even order has both or neither
-      else if (in) { e.x = __ldcg(p); if (v.next(c, 2 * (lane & 7) + 16 * h)) e.y = __ldcg(p + 1); }
-      x[i][2 * h] = e.x;
-      x[i][2 * h + 1] = e.y;
+      const double* p = v.at(R, c, i, j, in);
+      cp_async16(dst + i * kPitch + j, in ? p : v.G, in ? 16 : 0);
     }
+    cp_async_commit();
+  } else {
+#pragma unroll 8
+    for (int i = 0; i < NB; ++i) dst[i * kPitch + lane] = v.load(R, c, i, lane);
   }
 }
-template <int kRows>
-__device__ __forceinline__ void store_elements(const CholView& v, int R, int c, const double (&x)[kRows][4], int lane) {
+// 1 / sqrt(d): the approximation of PTX (about 2^-20 off), then one step of Householder's method of third order, y + y e (1/2 +
+// 3/8 e) with e = 1 - d y^2: what is left is of the order of e^3.  No branches, so that the steps around it overlap.
+__device__ __forceinline__ double inverse_root(double d, bool& bad) {
+  if (!(d > 0.0)) { bad = true; d = 1.0; }
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-d * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+// Two warps: D = L L^T and W = L^-T, four columns a step.  Lane i of the first holds row i of D; it factors each step's 4 x 4
+// block (every lane, redundantly), hands the finished columns over and goes on, waiting for nobody.  Lane i of the second holds row i
+// of the identity and follows a step behind.  A step's share of the exchange: l10 l20 l30 l21 l31 l32 of its block and the
+// inverse roots of its diagonal, then the finished columns [32][4].
+// left: rows that are there, what is behind is an identity's already.
+__device__ __forceinline__ void step_done(int step) { asm volatile("bar.arrive %0, 64;" ::"r"(1 + step) : "memory"); }
+__device__ __forceinline__ void step_wait(int step) { asm volatile("bar.sync %0, 64;" ::"r"(1 + step) : "memory"); }
+// v, one row, times the inverse of the block's L^T
+template <int k>
+__device__ __forceinline__ void solve_row(double (&v)[NB], const double (&l)[6], const double (&inv)[4]) {
+  v[k] *= inv[0];
+  v[k + 1] = fma(-v[k], l[0], v[k + 1]) * inv[1];
+  v[k + 2] = fma(-v[k + 1], l[3], fma(-v[k], l[1], v[k + 2])) * inv[2];
+  v[k + 3] = fma(-v[k + 2], l[5], fma(-v[k + 1], l[4], fma(-v[k], l[2], v[k + 3]))) * inv[3];
+}
+template <int k>
+__device__ __forceinline__ void update_row(double (&v)[NB], const double* done) {
 #pragma unroll
-  for (int i = 0; i < kRows; ++i) {
+  for (int j = k + 4; j < NB; ++j) {
+    const double2 u = *reinterpret_cast<const double2*>(done + j * 4), w = *reinterpret_cast<const double2*>(done + j * 4 + 2);
+    v[j] = fma(-v[k + 3], w.y, fma(-v[k + 2], w.x, fma(-v[k + 1], u.y, fma(-v[k], u.x, v[j]))));
+  }
+}
+template <class Columns>
+__device__ __forceinline__ void all_steps(Columns columns, int left) {
+  columns(std::integral_constant<int, 0>());
+  columns(std::integral_constant<int, 4>());
+  if (left <= 8) return;
+  columns(std::integral_constant<int, 8>());
+  columns(std::integral_constant<int, 12>());
+  if (left <= 16) return;
+  columns(std::integral_constant<int, 16>());
+  columns(std::integral_constant<int, 20>());
+  if (left <= 24) return;
+  columns(std::integral_constant<int, 24>());
+  columns(std::integral_constant<int, 28>());
+}
+__device__ __forceinline__ void factor_block(const double* D, double* diag, double* exchange, int left, bool& bad) {
+  const int lane = threadIdx.x & 31;
+  double a[NB];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      bool in;
-      double* p = v.at(R, c, (lane >> 3) + 4 * i, 2 * (lane & 7) + 16 * h, in);
-      if (in && v.even) __stcg(reinterpret_cast<double2*>(p), make_double2(x[i][2 * h], x[i][2 * h + 1]));
-      else if (in) { __stcg(p, x[i][2 * h]); if (v.next(c, 2 * (lane & 7) + 16 * h)) __stcg(p + 1, x[i][2 * h + 1]); }
+  for (int j = 0; j < NB; ++j) a[j] = D[lane * kPitch + j];
+  all_steps([&](auto first) {
+    constexpr int k = decltype(first)::value;
+    double* out = exchange + k / 4 * kStep;
+    if (lane >= k && lane < k + 4) {
+      double2* d = reinterpret_cast<double2*>(diag + (lane - k) * 4);
+      d[0] = make_double2(a[k], a[k + 1]);
+      d[1] = make_double2(a[k + 2], a[k + 3]);
     }
-  }
+    __syncwarp();
+    double l[6], inv[4];
+    inv[0] = inverse_root(diag[0], bad);
+    l[0] = diag[4] * inv[0]; l[1] = diag[8] * inv[0]; l[2] = diag[12] * inv[0];
+    inv[1] = inverse_root(fma(-l[0], l[0], diag[5]), bad);
+    l[3] = fma(-l[1], l[0], diag[9]) * inv[1]; l[4] = fma(-l[2], l[0], diag[13]) * inv[1];
+    inv[2] = inverse_root(fma(-l[3], l[3], fma(-l[1], l[1], diag[10])), bad);
+    l[5] = fma(-l[4], l[3], fma(-l[2], l[1], diag[14])) * inv[2];
+    inv[3] = inverse_root(fma(-l[5], l[5], fma(-l[4], l[4], fma(-l[2], l[2], diag[15]))), bad);
+    solve_row<k>(a, l, inv);
+    double2* mine = reinterpret_cast<double2*>(out + 16 + lane * 4);
+    mine[0] = make_double2(a[k], a[k + 1]);
+    mine[1] = make_double2(a[k + 2], a[k + 3]);
+    if (lane == 0) {
+#pragma unroll
+      for (int i = 0; i < 6; ++i) out[i] = l[i];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) out[6 + i] = inv[i];
+    }
+    __syncwarp();
+    step_done(k / 4);
+    update_row<k>(a, out + 16);
+  }, left);
 }
-// acc -= A B^T at the lane's elements; A's first row is that of acc's
-template <int kRows>
-__device__ __forceinline__ void warp_product(double (&acc)[kRows][4], const double* A, const double* B, int lane) {
-  const double* ar = A + (lane >> 3) * kPitch;
-  const double* br = B + 2 * (lane & 7) * kPitch;
-#pragma unroll 4
-  for (int k = 0; k < NB; ++k) {
-    double a[kRows], b[4];
+__device__ __forceinline__ void inverse_block(double* W, const double* exchange, int left) {
+  const int lane = threadIdx.x & 31;
+  double x[NB];
 #pragma unroll
-    for (int i = 0; i < kRows; ++i) a[i] = ar[4 * i * kPitch + k];
+  for (int j = 0; j < NB; ++j) x[j] = j == lane ? 1.0 : 0.0;
+  all_steps([&](auto first) {
+    constexpr int k = decltype(first)::value;
+    const double* in = exchange + k / 4 * kStep;
+    step_wait(k / 4);
+    double l[6], inv[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = br[((j & 1) + 16 * (j >> 1)) * kPitch + k];
+    for (int i = 0; i < 6; ++i) l[i] = in[i];
 #pragma unroll
-    for (int i = 0; i < kRows; ++i)
+    for (int i = 0; i < 4; ++i) inv[i] = in[6 + i];
+    solve_row<k>(x, l, inv);
+    update_row<k>(x, in + 16);
+  }, left);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = fma(-a[i], b[j], acc[i][j]);
-  }
+  for (int j = 0; j < NB; ++j) W[lane * kPitch + j] = x[j];
 }
+
 __global__ void __launch_bounds__(kCholThreads, 1)
 cholesky_kernel(double* G, double* X, int r, float* X32, int diagonal, int32_t* dev_status) {
   extern __shared__ __align__(16) double cs[];
   double* D = cs;                     // the panel's diagonal block
   double* W = D + kBlock;             // L(p,p)^-T
   double* Pp = W + kBlock;            // P(p,p-1)
-  double* col = Pp + kBlock;          // [2][32]
-  double* Bs = col + 2 * NB;          // [kMaxOwn] blocks of column p
-  double* ops = Bs + kMaxOwn * kBlock;  // [7][2]
+  double* exchange = Pp + kBlock;
+  double* Bs = exchange + kExchange;  // [kMaxOwn] blocks of column p
+  double* ops = Bs + kMaxOwn * kBlock;  // [kWorkers][2]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = blockIdx.x, ctas = gridDim.x;
+  const int lr = lane >> 2, lc = lane & 3;
   const CholView v = {G, X, r, (r + NB - 1) / NB, (r & 1) == 0};
   const int n = v.n;
-  double* opA = ops + (warp - 1) * 2 * kBlock;  // warps 1-7
+  const int worker = (warp & 3) == 0 ? -1 : (warp >> 2) * 3 + (warp & 3) - 1;  // -1: warps 0, 4 and (without work) 8
+  double* opA = ops + worker * 2 * kBlock;
   double* opB = opA + kBlock;
   bool bad = false;
 
   // The blocks of column p of this CTA: list entry e is G row p + 1 + e, then X rows 0 .. p.  At most kMaxOwn at a time,
-  // entries `first`, first + ctas ..: formed in Bs by warps 1-7, four rows a warp, then multiplied by W by all.
+  // entries `first`, first + ctas ..: formed in Bs by the workers, eight rows a warp, then multiplied by W by all.
+  auto entry = [&](int p, int e) { return e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p); };
   auto form_blocks = [&](int p, int first) {
-    for (int own = 0, e = first; own < kMaxOwn && e < n; e += ctas, ++own) {
-      const int R = e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p), q = R - n;  // (q < 0 for G rows)
-      double* B = Bs + own * kBlock;
-      for (int slab = warp - 1; slab < NB / 4; slab += 7) {
-        double acc[1][4] = {{0.0, 0.0, 0.0, 0.0}};
-        const int row = 4 * slab + (lane >> 3);
-        if (q == p) {  // nothing stored yet in X rows p - 1 (zeros) and p (the identity's block)
+    for (int item = worker; item < kMaxOwn * 4; item += kWorkers) {
+      const int own = item >> 2, row = (item & 3) * 8 + lr, e = first + own * ctas;
+      if (e >= n) break;
+      const int R = entry(p, e), q = R - n;  // (q < 0 for G rows)
+      double2 acc[4];
+      double a[8];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[0][j] = row == 2 * (lane & 7) + (j & 1) + 16 * (j >> 1) ? 1.0 : 0.0;
-        } else {
-          if (R < n || q < p - 1) load_elements(v, R, p, slab, acc, lane);
-          if (p > 0) {
-            double x[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              bool in;
-              const double* g = v.at(R, p - 1, 4 * slab + i, lane, in);
-              x[i] = in ? __ldcg(g) : 0.0;
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) opA[i * kPitch + lane] = x[i];
-            __syncwarp();
-            warp_product(acc, opA, Pp, lane);
-            __syncwarp();
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) B[row * kPitch + 2 * (lane & 7) + (j & 1) + 16 * (j >> 1)] = acc[0][j];
+      for (int t = 0; t < 4; ++t) {
+        const int j = 8 * t + 2 * lc;
+        acc[t] = make_double2(0.0, 0.0);  // nothing stored yet in X rows p - 1 (zeros) and p (the identity's block)
+        if (q == p) acc[t] = make_double2(row == j ? 1.0 : 0.0, row == j + 1 ? 1.0 : 0.0);
+        else if (R < n || q < p - 1) acc[t] = v.load2(R, p, row, j);
       }
+      if (p > 0 && q != p) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) a[k] = -v.load(R, p - 1, row, 4 * k + lc);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) mma_f64(acc[t], a[k], Pp[(8 * t + lr) * kPitch + 4 * k + lc]);
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) *reinterpret_cast<double2*>(Bs + own * kBlock + row * kPitch + 8 * t + 2 * lc) = acc[t];
     }
   };
-  // P(R,p) = B W.  W is an upper triangle: a warp's four columns need only the rows of W up to the last of them
+  // P(R,p) = B W, two 8 x 8 tiles a warp
+  const int tr = (warp & 3) * 8, tc = (warp >> 2) * 16;  // (D's tiles of a warp too; of warps 0-7)
   auto finish_blocks = [&](int p, int first) {
-    const int lo = tid & 15, up = tid >> 4;
-    for (int own = 0, e = first; own < kMaxOwn && e < n; e += ctas, ++own) {
-      const int R = e < n - 1 - p ? p + 1 + e : n + e - (n - 1 - p);
+    for (int own = 0, e = first; own < kMaxOwn && e < n && warp < 8; e += ctas, ++own) {
+      const int R = entry(p, e);
       const double* B = Bs + own * kBlock;
-      const double* b = B + lo * kPitch;
-      const double* w = W + 2 * up;
-      double o[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll 4
-      for (int k = 0; k < 4 * warp + 4; ++k) {
-        const double b0 = b[k], b1 = b[16 * kPitch + k], w0 = w[k * kPitch], w1 = w[k * kPitch + 1];
-        o[0][0] = fma(b0, w0, o[0][0]); o[0][1] = fma(b0, w1, o[0][1]);
-        o[1][0] = fma(b1, w0, o[1][0]); o[1][1] = fma(b1, w1, o[1][1]);
+      double2 o[2] = {};
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const double b = B[(tr + lr) * kPitch + 4 * k + lc];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) mma_f64(o[t], b, W[(4 * k + lc) * kPitch + tc + 8 * t + lr]);
       }
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          bool in;
-          double* g = v.at(R, p, lo + 16 * i, 2 * up + j, in);
-          if (in) __stcg(g, o[i][j]);
-        }
+      for (int t = 0; t < 2; ++t) v.store2(R, p, tr + lr, tc + 8 * t + 2 * lc, o[t]);
     }
   };
 
   for (int p = 0; p < n; ++p) {
-    // ---- D, by all warps: 4 elements a thread
-    const int lo = tid & 15, up = tid >> 4;  // rows and columns lo, lo + 16, up, up + 16 of a block
-    {
-      double d[2][2];
+    // ---- the warp's first block behind column p: column j takes G rows j .. n-1 and X rows 0 .. p-1
+    int t = (worker >= kFormers ? worker - kFormers : worker + kWorkers - kFormers) * ctas + cta, j = p + 1, R = 0;
+    auto settle = [&] {  // t, counted from column j's first block on, to a block of a column
+      for (; j < n; ++j) {
+        const int count = n - j + p;
+        if (t < count) { R = t < n - j ? j + t : n + t - (n - j); return true; }
+        t -= count;
+      }
+      return false;
+    };
+    double2 acc[4][4];
+    auto ask = [&] {
+      fetch_block(v, R, p - 1, opA, lane);
+      fetch_block(v, j, p - 1, opB, lane);
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int a = up + 16 * i, b = lo + 16 * j;
+        for (int u = 0; u < 4; ++u) acc[i][u] = R != n + p - 1 ? v.load2(R, j, 8 * i + lr, 8 * u + 2 * lc) : make_double2(0.0, 0.0);
+    };
+    // ---- D: two 8 x 8 tiles a warp
+    double2 d[2] = {};
+    if (warp < 8) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int a = tr + lr;
+        auto element = [&](int b) {
           bool in;
           const double* g = v.at(p, p, max(a, b), min(a, b), in);
-          d[i][j] = in ? __ldcg(g) : (a == b ? 1.0 : 0.0);
-        }
+          return in ? __ldcg(g) : (a == b ? 1.0 : 0.0);
+        };
+        d[u] = make_double2(element(tc + 8 * u + 2 * lc), element(tc + 8 * u + 2 * lc + 1));
+      }
       if (p > 0) {
         double x[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          bool in;
-          const double* g = v.at(p, p - 1, warp * 4 + i, lane, in);
-          x[i] = in ? __ldcg(g) : 0.0;
-        }
+        for (int i = 0; i < 4; ++i) x[i] = v.load(p, p - 1, warp * 4 + i, lane);
 #pragma unroll
         for (int i = 0; i < 4; ++i) Pp[(warp * 4 + i) * kPitch + lane] = x[i];
-        __syncthreads();
-        const double* a = Pp + up * kPitch;
-        const double* b = Pp + lo * kPitch;
-#pragma unroll 8
-        for (int k = 0; k < NB; ++k) {
-          const double a0 = a[k], a1 = a[16 * kPitch + k], b0 = b[k], b1 = b[16 * kPitch + k];
-          d[0][0] = fma(-a0, b0, d[0][0]); d[0][1] = fma(-a0, b1, d[0][1]);
-          d[1][0] = fma(-a1, b0, d[1][0]); d[1][1] = fma(-a1, b1, d[1][1]);
+      }
+    }
+    __syncthreads();
+    if (warp < 8) {
+      if (p > 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const double a = -Pp[(tr + lr) * kPitch + 4 * k + lc];
+#pragma unroll
+          for (int u = 0; u < 2; ++u) mma_f64(d[u], a, Pp[(tc + 8 * u + lr) * kPitch + 4 * k + lc]);
         }
       }
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) D[(up + 16 * i) * kPitch + lo + 16 * j] = d[i][j];
+      for (int u = 0; u < 2; ++u) *reinterpret_cast<double2*>(D + (tr + lr) * kPitch + tc + 8 * u + 2 * lc) = d[u];
     }
     __syncthreads();
     if (warp == 0) {
-      // ---- lane i holds row i of D and of the identity
-      double a[NB], x[NB];
-#pragma unroll
-      for (int j = 0; j < NB; ++j) { a[j] = D[lane * kPitch + j]; x[j] = j == lane ? 1.0 : 0.0; }
-      double pivot = a[0];
-      const int left = r - p * NB;  // what is behind is an identity's already
-#pragma unroll
-      for (int k = 0; k < NB; ++k) {
-        if (k % 8 == 0 && k >= left) break;
-        double d = __shfl_sync(0xffffffffu, pivot, k);
-        if (!(d > 0.0)) { bad = true; d = 1.0; }
-        const double inv = rsqrt(d);
-        const double l = a[k] * inv;
-        if (k + 1 < NB) pivot = fma(-l, l, a[k + 1]);  // in lane k + 1: the next step need not wait for the exchange
-        x[k] *= inv;
-        col[(k & 1) * NB + lane] = l;
+      factor_block(D, exchange, exchange + 16, r - p * NB, bad);
+    } else if (warp == 4) {
+      inverse_block(W, exchange + 16, r - p * NB);
+    } else if (worker >= 0) {
+      bool more = p > 0 && settle();
+      if (more) ask();
+      form_blocks(p, cta);
+      // ---- panel p - 1 on the blocks behind column p
+      while (more) {
+        cp_async_wait<0>();
         __syncwarp();
 #pragma unroll
-        for (int j = k + 1; j < NB; ++j) {
-          const double lj = col[(k & 1) * NB + j];
-          a[j] = fma(-l, lj, a[j]);
-          x[j] = fma(-x[k], lj, x[j]);
-        }
-      }
+        for (int k = 0; k < 8; ++k) {
+          double a[4], b[4];
 #pragma unroll
-      for (int j = 0; j < NB; ++j) W[lane * kPitch + j] = x[j];
-    } else {
-      form_blocks(p, cta);
-      // ---- panel p - 1 on the blocks behind column p: column j takes G rows j .. n-1 and X rows 0 .. p-1
-      if (p > 0) {
-        int t = cta * 7 + warp - 1;
-        for (int j = p + 1; j < n; ++j) {
-          const int count = n - j + p;
-          for (; t < count; t += ctas * 7) {
-            const int R = t < n - j ? j + t : n + t - (n - j);
-            double acc[8][4] = {};
-            if (R != n + p - 1) load_elements(v, R, j, 0, acc, lane);
-            load_block(v, R, p - 1, opA, lane);
-            load_block(v, j, p - 1, opB, lane);
-            __syncwarp();
-            warp_product(acc, opA, opB, lane);
-            store_elements(v, R, j, acc, lane);
-            __syncwarp();
-          }
-          t -= count;
+          for (int i = 0; i < 4; ++i) { a[i] = -opA[(8 * i + lr) * kPitch + 4 * k + lc]; b[i] = opB[(8 * i + lr) * kPitch + 4 * k + lc]; }
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) mma_f64(acc[i][u], a[i], b[u]);
         }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v.store2(R, j, 8 * i + lr, 8 * u + 2 * lc, acc[i][u]);
+        __syncwarp();
+        t += ctas * kWorkers;
+        more = settle();
+        if (more) ask();
       }
     }
     __syncthreads();
     finish_blocks(p, cta);
     for (int first = cta + kMaxOwn * ctas; first < n; first += kMaxOwn * ctas) {  // (a cluster below its full size)
       __syncthreads();
-      if (warp > 0) form_blocks(p, first);
+      if (worker >= 0) form_blocks(p, first);
       __syncthreads();
       finish_blocks(p, first);
     }
