@@ -4,7 +4,7 @@
 // cholesky_kernel   L^-T in fp64 by one cluster of CTAs, rounded to fp32
 // gemm_f32          Q = Y L^-T, with the products exact to fp32 (conversion_gemm.cu)
 // For a basis of 512 columns of length 8064: 0.24 + 1.86 + 0.74 ms in the form this one replaced (whole G, one block for the
-// factor, a triangular solve per row), now 0.13 + 0.14 + 0.03.
+// factor, a triangular solve per row), now 0.10 + 0.14 + 0.03.
 #include <type_traits>
 
 #include "common.cuh"
@@ -15,11 +15,17 @@ namespace conv {
 
 namespace {
 
+// c += a b for 8 x 8 x 4: lane l has a(l/4, l%4), b(l%4, l/4) and c(l/4, 2 (l%4) + {0, 1}).
+__device__ __forceinline__ void mma_f64(double2& c, double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c.x), "+d"(c.y) : "d"(a), "d"(b));
+}
+
 // ------------------------------------------------------------------------------------------------ Gram matrix
-// 128 x 128 tile, 256 threads x (8 x 8) fp64 sums, 16 rows of Y a step through two shared-memory buffers, converted to fp64
-// on the way in.  Bound by the fp64 units: 64 multiply-adds a thread and step against eight 16-byte reads.
-constexpr int GT = 128, GK = 16;
-constexpr int kGramSmem = 2 * 2 * GK * GT * 8;
+// 128 x 128 tile, eight warps with 64 x 32 fp64 sums each, 16 rows of Y a step through two shared-memory buffers, converted to
+// fp64 on the way in.  Bound by the fp64 units: tensor instructions run at their rate (64 multiply-adds a cycle and SM) and leave
+// the issue slots to the loads and conversions, which multiply-adds of single threads compete with.  8064 x 512: 124 -> 100 us.
+constexpr int GT = 128, GK = 16, GP = GT + 4;  // pitch: conflict-free fragments
+constexpr int kGramSmem = 2 * 2 * GK * GP * 8;
 
 struct GramRegs { float4 v[2]; };
 __device__ __forceinline__ void gram_fetch(GramRegs& t, const float* Y, bool vec, int r, int c0, int k0, int k_end, int tid) {
@@ -42,7 +48,7 @@ __device__ __forceinline__ void gram_stash(const GramRegs& t, double* S, int tid
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int f = tid + 256 * u;
-    double2* d = reinterpret_cast<double2*>(S + (f / 32) * GT + (f % 32) * 4);
+    double2* d = reinterpret_cast<double2*>(S + (f / 32) * GP + (f % 32) * 4);
     d[0] = make_double2(t.v[u].x, t.v[u].y);
     d[1] = make_double2(t.v[u].z, t.v[u].w);
   }
@@ -50,26 +56,27 @@ __device__ __forceinline__ void gram_stash(const GramRegs& t, double* S, int tid
 
 __global__ void __launch_bounds__(256) gram_kernel(const float* Y, int m, int r, int ks, double* partial) {
   extern __shared__ __align__(16) unsigned char gram_smem[];
-  double* As = reinterpret_cast<double*>(gram_smem);   // [2][GK][GT]
-  double* Bs = As + 2 * GK * GT;
+  double* As = reinterpret_cast<double*>(gram_smem);   // [2][GK][GP]
+  double* Bs = As + 2 * GK * GP;
   int ti = 0, tj = blockIdx.x;
   while (tj > ti) tj -= ++ti;
-  const int i0 = ti * GT, j0 = tj * GT, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int i0 = ti * GT, j0 = tj * GT, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, lr = lane >> 2, lc = lane & 3;
+  const int mi = (warp >> 2) * 64, nj = (warp & 3) * 32;  // the warp's rows and columns of the tile
   const bool diag = ti == tj, vec = (r & 3) == 0 && (reinterpret_cast<uintptr_t>(Y) & 15) == 0;
   const int k_lo = blockIdx.y * ks, k_hi = min(m, k_lo + ks);
-  double acc[8][8];
+  double2 acc[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_double2(0.0, 0.0);
   GramRegs ra, rb;
   auto fetch = [&](int k) {
     gram_fetch(ra, Y, vec, r, i0, k, k_hi, tid);
     if (!diag) gram_fetch(rb, Y, vec, r, j0, k, k_hi, tid);
   };
   auto stash = [&](int buf) {
-    gram_stash(ra, As + buf * GK * GT, tid);
-    if (!diag) gram_stash(rb, Bs + buf * GK * GT, tid);
+    gram_stash(ra, As + buf * GK * GP, tid);
+    if (!diag) gram_stash(rb, Bs + buf * GK * GP, tid);
   };
   fetch(k_lo);
   stash(0);
@@ -78,22 +85,19 @@ __global__ void __launch_bounds__(256) gram_kernel(const float* Y, int m, int r,
   for (int k = k_lo; k < k_hi; k += GK, buf ^= 1) {
     const bool more = k + GK < k_hi;
     if (more) fetch(k + GK);
-    const double* a_s = As + buf * GK * GT;
-    const double* b_s = diag ? a_s : Bs + buf * GK * GT;
-#pragma unroll 4
-    for (int kk = 0; kk < GK; ++kk) {
-      double a[8], b[8];
+    const double* a_s = As + buf * GK * GP + mi + lr;
+    const double* b_s = (diag ? As : Bs) + buf * GK * GP + nj + lr;
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {  // pairs of columns, 32 apart: consecutive lanes read consecutive pairs
-        const double2 a2 = *reinterpret_cast<const double2*>(a_s + kk * GT + h * 32 + ty * 2);
-        const double2 b2 = *reinterpret_cast<const double2*>(b_s + kk * GT + h * 32 + tx * 2);
-        a[2 * h] = a2.x; a[2 * h + 1] = a2.y;
-        b[2 * h] = b2.x; b[2 * h + 1] = b2.y;
-      }
+    for (int k4 = 0; k4 < GK; k4 += 4) {
+      double a[8], b[4];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) a[i] = a_s[(k4 + lc) * GP + 8 * i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = b_s[(k4 + lc) * GP + 8 * j];
 #pragma unroll
       for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) mma_f64(acc[i][j], a[i], b[j]);
     }
     if (more) stash(buf ^ 1);
     __syncthreads();
@@ -101,11 +105,12 @@ __global__ void __launch_bounds__(256) gram_kernel(const float* Y, int m, int r,
   double* out = partial + static_cast<size_t>(blockIdx.y) * r * r;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const int row = i0 + ty * 2 + (i & 1) + (i >> 1) * 32;
+    const int row = i0 + mi + 8 * i + lr;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int col = j0 + tx * 2 + (j & 1) + (j >> 1) * 32;
-      if (row < r && col <= row) out[static_cast<size_t>(row) * r + col] = acc[i][j];
+    for (int j = 0; j < 4; ++j) {
+      const int col = j0 + nj + 8 * j + 2 * lc;
+      if (row < r && col <= row) out[static_cast<size_t>(row) * r + col] = acc[i][j].x;
+      if (row < r && col + 1 <= row) out[static_cast<size_t>(row) * r + col + 1] = acc[i][j].y;
     }
   }
 }
@@ -174,10 +179,6 @@ struct CholView {
     else if (in) { __stcg(p, e.x); if (c * NB + j + 1 < r) __stcg(p + 1, e.y); }
   }
 };
-// c += a b for 8 x 8 x 4: lane l has a(l/4, l%4), b(l%4, l/4) and c(l/4, 2 (l%4) + {0, 1}).
-__device__ __forceinline__ void mma_f64(double2& c, double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c.x), "+d"(c.y) : "d"(a), "d"(b));
-}
 // A warp asks for block (R, c) in shared memory; the caller waits (cp_async_wait, __syncwarp).
 __device__ __forceinline__ void fetch_block(const CholView& v, int R, int c, double* dst, int lane) {
   if (v.even) {
