@@ -42,9 +42,16 @@ constexpr int kPlane = kRows * kKc * 2;        // 8192 bytes: one term of one op
 constexpr int kStageBytes = 6 * kPlane;
 constexpr int kOffBar = kStages * kStageBytes;
 constexpr int kSmemBytes = kOffBar + 256 + 1024;
-constexpr int kLaunchRegs = 96, kConverterRegs = 72, kAdderRegs = 152, kIssuerRegs = 24;
+constexpr int kLaunchRegs = 96, kIssuerRegs = 32;
+// A single CTA's adders have half the sums, its converters a second chunk on its way (a pair's wait for stages instead): 16 products of
+// 128 x 128 x 16384 464 us, 509 without (one kind of warp for both jobs: 406, 512 x 4096 x 8064 227 against 239 here).
+template <int kCtas>
+struct RegisterSplit {
+  static constexpr int kConverter = kCtas == 2 ? 72 : 104, kAdder = kCtas == 2 ? 152 : 120;
+  static_assert(kConverters * kConverter + kAdders * kAdder + 128 * kIssuerRegs <= kThreads * kLaunchRegs, "register split");
+};
 static_assert(kSmemBytes <= 232448, "shared memory budget");
-static_assert(kThreads * kLaunchRegs <= 65536 && kConverters * kConverterRegs + kAdders * kAdderRegs + 128 * kIssuerRegs <= kThreads * kLaunchRegs, "register split");
+static_assert(kThreads * kLaunchRegs <= 65536, "registers at launch");
 enum { BAR_FULL = 0, BAR_EMPTY = kStages, BAR_D_FULL = 2 * kStages, BAR_D_FREE = BAR_D_FULL + 2,
        BAR_FULL2 = BAR_D_FREE + 2, BAR_D_FREE2 = BAR_FULL2 + kStages, BAR_LAST = BAR_D_FREE2 + 2, BAR_COUNT };  // ..2: the second CTA's word
 static_assert(BAR_COUNT <= 24, "barrier block");
@@ -272,11 +279,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
     }
   } else if (warp < kConverters / 32) {
     // ========================================================================== converters
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConverterRegs));
+    constexpr int kRegs = RegisterSplit<kCtas>::kConverter;
+    if constexpr (kRegs < kLaunchRegs) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs));
+    else asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
     const bool vec_a = (args.lda & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
     const bool vec_b = (args.ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
     const int nb0 = n0 + rank * kRows;                  // this CTA's columns of op(B)
-    float xa[2][8], xb[2][8];                           // two pieces of A and two of B a thread and chunk
+    constexpr int kAhead = kCtas == 2 ? 1 : 2;          // chunks on their way
+    float xa[kAhead][2][8], xb[kAhead][2][8];           // two pieces of A and two of B a thread and chunk
     // Away from the edges a thread's pieces sit at fixed distances from one address per operand.
     const bool inside = vec_a && vec_b && m0 + kRows <= M && nb0 + kRows <= N;
     const float* next_a = A + (kAContig ? static_cast<size_t>(m0 + (tid >> 2)) * args.lda + (tid & 3) * 8
@@ -287,40 +297,48 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
       const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
       x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
     };
-    auto load = [&](int c) {
+    auto load = [&](int c, float (&ya)[2][8], float (&yb)[2][8]) {
       if (inside && (c + 1) * kKc <= K) {
         const float* a = next_a + (kAContig ? static_cast<size_t>(c) * kKc : static_cast<size_t>(c) * kKc * args.lda);
         const float* b = next_b + (kBContig ? static_cast<size_t>(c) * kKc : static_cast<size_t>(c) * kKc * args.ldb);
-        load8(xa[0], a);
-        load8(xa[1], a + (kAContig ? static_cast<size_t>(64) * args.lda : 64));
-        load8(xb[0], b);
-        load8(xb[1], b + (kBContig ? static_cast<size_t>(64) * args.ldb : 64));
+        load8(ya[0], a);
+        load8(ya[1], a + (kAContig ? static_cast<size_t>(64) * args.lda : 64));
+        load8(yb[0], b);
+        load8(yb[1], b + (kBContig ? static_cast<size_t>(64) * args.ldb : 64));
         return;
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        load_group<kAContig>(xa[u], A, vec_a, args.lda, m0, M, c * kKc, K, tid + u * 256);
-        load_group<kBContig>(xb[u], B, vec_b, args.ldb, nb0, N, c * kKc, K, tid + u * 256);
+        load_group<kAContig>(ya[u], A, vec_a, args.lda, m0, M, c * kKc, K, tid + u * 256);
+        load_group<kBContig>(yb[u], B, vec_b, args.ldb, nb0, N, c * kKc, K, tid + u * 256);
       }
     };
-    load(0);
-    for (int c = 0; c < chunks; ++c) {
-      const int stage = c % kStages;
-      if (c >= kStages) wait(bar(BAR_EMPTY + stage), (c / kStages - 1) & 1);
-      unsigned char* st = sm + stage * kStageBytes;
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        store_group<kAContig>(xa[u], st, kPlane, tid + u * 256);
-        store_group<kBContig>(xb[u], st + 3 * kPlane, kPlane, tid + u * 256);
+    for (int s = 0; s < kAhead; ++s)
+      if (s < chunks) load(s, xa[s], xb[s]);
+    for (int c0 = 0; c0 < chunks; c0 += kAhead) {
+#pragma unroll
+      for (int s = 0; s < kAhead; ++s) {
+        const int c = c0 + s, stage = c % kStages;
+        if (c >= chunks) break;
+        if (c >= kStages) wait(bar(BAR_EMPTY + stage), (c / kStages - 1) & 1);
+        unsigned char* st = sm + stage * kStageBytes;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          store_group<kAContig>(xa[s][u], st, kPlane, tid + u * 256);
+          store_group<kBContig>(xb[s][u], st + 3 * kPlane, kPlane, tid + u * 256);
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(BAR_FULL + stage));
+        if (c + kAhead < chunks) load(c + kAhead, xa[s], xb[s]);
       }
-      fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(BAR_FULL + stage));
-      if (c + 1 < chunks) load(c + 1);
     }
   } else {
     // ========================================================================== adders
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kAdderRegs));
+    constexpr int kRegs = RegisterSplit<kCtas>::kAdder;
+    static_assert(kRegs >= kLaunchRegs, "adders only gain");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
     constexpr int kCols = kTile / 2;                    // columns of the tile a thread sums: those of its warp's half
     const int adder = warp - kConverters / 32, quad = warp & 3, half = adder >> 2;
     const uint32_t d_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * kCols;
