@@ -1,5 +1,5 @@
-// The append's block routine, shared by the kernels that hold append blocks (the prologue launches and, in the
-// layer step, the launch of the query maps).
+// The append's routines: a block's, for the launch of the layer's mma.sync maps, a cluster's, for the prologue and the append of sizes
+// that prologue_sm100.cu does not take, and the entries of that file.
 #pragma once
 #include "common.cuh"
 #include "skinny_gemm.cuh"

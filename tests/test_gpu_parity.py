@@ -337,6 +337,12 @@ def test_append_values_slots_and_untouched_bytes(shape, positions):
 
 
 # ------------------------------------------------------------------ whole step from host buffers
+@pytest.mark.parametrize('D', [256, 768, 1280, 4352])
+def test_append_with_pieces_of_the_hidden_dimension_that_are_not_whole(D):
+    # a cluster's CTA takes D / 8 in pieces of 128, four or three at a time: part of one, of a second, of a ring that wraps
+    test_append_values_slots_and_untouched_bytes(dataclasses.replace(synth.LLAMA2_7B, D=D), [5, 64, 130] + list(range(200, 240)))
+
+
 @pytest.mark.parametrize('shape', [synth.LLAMA2_7B, synth.TINY])
 @pytest.mark.parametrize('B', [17, 32, 33, 65])
 def test_append_of_many_tokens_writes_the_bytes_of_few(shape, B):
