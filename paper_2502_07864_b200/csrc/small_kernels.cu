@@ -25,22 +25,22 @@ __device__ __forceinline__ int kperm(int p) { return ((p & 7) >> 1) * 8 + (p >> 
 
 // ------------------------------------------------------------------------------------------------
 // Absorb (Eq. 9 right, first line): q_hat[bs,h,:r] = W_UK_h^T q_nope[bs,h,:], q_hat[bs,h,r:] = q_pe[bs,h,:].
-// A block owns 128 of one head's latent columns: it stages W_UK_h[:, columns] and the head's query rows (128 at a time) in
-// shared memory with asynchronous 16-byte copies, all in flight together, and walks the rows in 16-row tiles, so W_UK
-// is read once.  The block that owns a head's first columns also copies the rope part of the rows.
+// A block owns nt consecutive 128-column tiles of one head's latent columns (nt = 1, or 2 when that brings the
+// launch down to one wave): it stages W_UK_h[:, tiles] and the head's query rows (128 at a time) in shared
+// memory with asynchronous 16-byte copies, all in flight together, and walks the rows in 16-row tiles, so W_UK
+// is read once.  The block that owns a head's first tile also copies the rope part of the rows.
 // ------------------------------------------------------------------------------------------------
 constexpr int kAbsorbRows = 128;  // query rows staged per pass
 
 __device__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q_pe,
                              const __nv_bfloat16* __restrict__ w_uk, __nv_bfloat16* q_hat, int BS, int H,
-                             int dn, int dR, int r, int h, int rt0, unsigned char* smem_raw) {
-  constexpr int vec_per_row = 16, wpitch = 128 + 8;
-  const int apitch = dn + 8;
+                             int dn, int dR, int r, int h, int rt0, int nt, unsigned char* smem_raw) {
+  const int apitch = dn + 8, wpitch = nt * 128 + 8;
   __nv_bfloat16* w_s = reinterpret_cast<__nv_bfloat16*>(smem_raw);  // [dn][wpitch]
   __nv_bfloat16* a_s = w_s + dn * wpitch;                            // [kAbsorbRows][dn + 8]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
-  const int n0 = rt0 * 128, K = r + dR;
+  const int n0 = rt0 * 128, K = r + dR, vec_per_row = nt * 16;
   for (int i = tid; i < dn * vec_per_row; i += 256) {  // columns beyond r are zero-filled
     const int k = i / vec_per_row, c = i % vec_per_row;
     const bool in = n0 + c * 8 < r;
@@ -89,8 +89,7 @@ __device__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q
     cp_async_wait<0>();
     __syncthreads();
     for (int m0 = 0; m0 < rows16; m0 += 16) {
-      {
-        const int wc = warp * 16;  // this warp's columns
+      for (int wc = warp * 16 * nt; wc < (warp + 1) * 16 * nt; wc += 16) {  // this warp's 16-column steps
         float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll 4
         for (int ks = 0; ks < dn / 16; ++ks) {
@@ -114,17 +113,54 @@ __device__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q
   }
 }
 
-static size_t absorb_smem(int dn) {
-  return (static_cast<size_t>(dn) * (128 + 8) + static_cast<size_t>(kAbsorbRows) * (dn + 8)) * sizeof(__nv_bfloat16);
+static size_t absorb_smem(int dn, int nt) {
+  return (static_cast<size_t>(dn) * (nt * 128 + 8) + static_cast<size_t>(kAbsorbRows) * (dn + 8)) * sizeof(__nv_bfloat16);
 }
 
-__global__ void __launch_bounds__(256, 2) append_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w, const int32_t* positions,
-                                                        const int32_t* page_table, __nv_bfloat16* cache, int32_t* dev_status, int B,
-                                                        int S, int D, int r, int dR, int num_pages, int max_pages, float theta) {
+// Tiles per absorb block: two when the prologue launch would otherwise not fit the device in one wave of one block
+// per SM (the append's accumulators allow no more), the tile count is even and the pair's weights fit.
+static int absorb_tiles_per_block(const transmla_params_t& p, int other_blocks) {
+  static PerDeviceFlag sms_of;  // SM count per device, asked once
+  const int slot = current_device_slot();
+  int sms = slot >= 0 ? sms_of.value[slot].load(std::memory_order_acquire) : 0;
+  if (sms == 0) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return 1;
+    }
+    if (slot >= 0) sms_of.value[slot].store(sms, std::memory_order_release);
+  }
+  const int r_tiles = (p.kv_lora_rank + 127) / 128;
+  const bool fits_one = other_blocks + p.num_heads * r_tiles <= sms;
+  return (!fits_one && r_tiles % 2 == 0 && p.qk_nope_dim <= 128) ? 2 : 1;
+}
+
+// The append of sizes that prologue_sm100.cu does not take goes by clusters (see slice_gemm_tile) or by blocks.
+__global__ void __launch_bounds__(256, 2) append_cluster_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w,
+                                                                const int32_t* positions, const int32_t* page_table,
+                                                                __nv_bfloat16* cache, int32_t* dev_status, int B, int S, int D,
+                                                                int r, int dR, int num_pages, int max_pages, float theta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
   append_cluster(x, w, positions, 0, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
-                       blockIdx.x / kSliceCtas, blockIdx.x % kSliceCtas, smem_raw);
+                 blockIdx.x / kSliceCtas, blockIdx.x % kSliceCtas, smem_raw);
+}
+__global__ void __launch_bounds__(256) append_kernel(const __nv_bfloat16* x,
+                                                     const __nv_bfloat16* __restrict__ w,
+                                                     const int32_t* positions,
+                                                     const int32_t* page_table,
+                                                     __nv_bfloat16* cache, int32_t* dev_status, int B,
+                                                     int S, int D, int r, int dR, int num_pages, int max_pages,
+                                                     float theta, int t_splits, int wide) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_trigger();
+  if (wide)
+    append_block<1, 4>(x, w, positions, 0, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
+                       blockIdx.x, t_splits, smem_raw);
+  else
+    append_block<kAppendMaxMT, 1>(x, w, positions, 0, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages,
+                                  theta, blockIdx.x, t_splits, smem_raw);
 }
 
 // Absorb blocks followed by one plan block: everything transmla_mla_decode needs before the split-KV kernel.
@@ -134,45 +170,53 @@ __global__ void __launch_bounds__(256) absorb_plan_kernel(const __nv_bfloat16* q
                                                           __nv_bfloat16* q_hat,
                                                           const int32_t* seqlens, int32_t* cum,
                                                           int32_t* plan, int32_t* dev_status, int B, int S, int H,
-                                                          int dn, int dR, int r, Partitioning parts, int max_pages) {
+                                                          int dn, int dR, int r, Partitioning parts, int max_pages, int nt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
-  const int per_head = (r + 127) / 128;  // absorb blocks per head
+  const int per_head = (r + 127) / 128 / nt;  // absorb blocks per head, nt tiles each
   const int n_absorb = H * per_head;
   if (static_cast<int>(blockIdx.x) < n_absorb) {
-    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, blockIdx.x / per_head, blockIdx.x % per_head, smem_raw);
+    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, blockIdx.x / per_head, blockIdx.x % per_head * nt, nt, smem_raw);
   } else {
     plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
   }
 }
 
-// The whole prologue of a decode step in one launch: append clusters, plan block, absorb blocks.
-// The appended token of sequence b sits at seqlens[b] - S + s.
-__global__ void __launch_bounds__(256, 2) prologue_kernel(
+// The whole prologue of a decode step in one launch: append clusters or blocks, plan block, absorb blocks.
+// The appended token of sequence b sits at seqlens[b] - S + s.  n_append: clusters, or blocks of t_splits token splits.
+template <bool kClusters>
+__global__ void __launch_bounds__(256, kClusters ? 2 : 1) prologue_kernel(
     const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w_dkv_kr,
     const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope,
     const __nv_bfloat16* q_pe, const __nv_bfloat16* __restrict__ w_uk, __nv_bfloat16* q_hat,
     const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status, int B, int S, int H, int D,
-    int dn, int dR, int r, int num_pages, int max_pages, float theta, Partitioning parts, int n_append) {
+    int dn, int dR, int r, int num_pages, int max_pages, float theta, Partitioning parts, int n_append, int t_splits, int wide, int nt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
-  const int per_head = (r + 127) / 128;  // absorb blocks per head
-  const int bid = static_cast<int>(blockIdx.x) - n_append * kSliceCtas;
+  const int per_head = (r + 127) / 128 / nt;  // absorb blocks per head, nt tiles each
+  const int bid = static_cast<int>(blockIdx.x) - n_append * (kClusters ? kSliceCtas : 1);
   if (bid < 0) {
-    append_cluster(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
-                         blockIdx.x / kSliceCtas, blockIdx.x % kSliceCtas, smem_raw);
+    if (kClusters)
+      append_cluster(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages, theta,
+                     blockIdx.x / kSliceCtas, blockIdx.x % kSliceCtas, smem_raw);
+    else if (wide)
+      append_block<1, 4>(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages, max_pages,
+                         theta, blockIdx.x, t_splits, smem_raw);
+    else
+      append_block<kAppendMaxMT, 1>(x, w_dkv_kr, seqlens, -S, page_table, cache, dev_status, B, S, D, r, dR, num_pages,
+                                    max_pages, theta, blockIdx.x, t_splits, smem_raw);
   } else if (bid == 0) {
     plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
-  } else if (bid <= H * per_head) {  // (the grid is whole clusters: a few blocks at its end have nothing to do)
-    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, (bid - 1) / per_head, (bid - 1) % per_head, smem_raw);
+  } else if (bid <= H * per_head) {  // (a grid of clusters is whole: a few blocks at its end have nothing to do)
+    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, (bid - 1) / per_head, (bid - 1) % per_head * nt, nt, smem_raw);
   }
 }
 
 constexpr int kPrologueMaxSmem = 144 * 1024;
 
-// The append as blocks of linear.cu's launch.  Token splits: one per 64 new tokens, at most 4.
-// With many new tokens a block takes 32 output features and 16 tokens (activations re-read a quarter as often
-// per feature, weights four times as often per token: 384 KB per block instead of 576 KB at 128 tokens).
+// Token splits of the append's blocks.  With many new tokens a block takes 32 output features and 16 tokens (activations re-read
+// a quarter as often per feature, weights four times as often per token: 384 KB per block instead of 576 KB at 128 tokens).
+// Otherwise 8 features: one split per 64 tokens, at most 4.
 bool append_wide(const transmla_params_t& p) {
   return p.batch * p.q_len > 32 && (p.kv_lora_rank + p.qk_rope_dim) % 32 == 0 && p.kv_lora_rank % 2 == 0;
 }
@@ -181,16 +225,33 @@ int append_token_splits(const transmla_params_t& p) {
   if (append_wide(p)) return (T + 15) / 16 > 32 ? 32 : (T + 15) / 16;
   return T <= 64 ? 1 : (T + 63) / 64 > 4 ? 4 : (T + 63) / 64;
 }
+// Clusters read the operands a quarter as often but take 2 to 3 us more to start and to meet.  The decode step, blocks / clusters:
+// r = 64, dR = 16, D = 256 1 sequence 14.0 / 15.2 us, 16 (64 heads) 16.6 / 19.0, 64 18.0 to 23.2 / 19.3 to 25.3; the same with D = 4096 16
+// 20.6 / 21.9, 64 27.7 / 21.2; r = 512, dR = 64, dn = 64 1 20.6 / 22.2, 16 22.2 / 24.6, 160 46.1 / 39.5 and (64 heads) 75.4 / 69.8.  With
+// r = 128, dR = 0 blocks of 32 features x 16 tokens are as many as clusters have CTAs: 16 19.1 / 22.2, 64 22.5 / 22.9, 160 23.8 / 26.3.
+// (The two forms add a value's products in other orders, both in fp32.)
+static bool append_in_clusters(const transmla_params_t& p) {
+  return p.batch * p.q_len > 32 && (p.kv_lora_rank + p.qk_rope_dim) % 128 != 0;
+}
 
 cudaError_t launch_append(const transmla_params_t& p, const __nv_bfloat16* x, const __nv_bfloat16* w,
                           const int32_t* positions, const int32_t* page_table, __nv_bfloat16* cache,
                           int32_t* dev_status, cudaStream_t stream) {
-  if (prologue_sm100_supported(p)) return launch_append_sm100(p, x, w, positions, page_table, cache, nullptr, dev_status, stream);
-  static PerDeviceFlag smem_set;
-  if (cudaError_t e = ensure_dynamic_smem(append_kernel, static_cast<int>(kSliceSmem), smem_set); e != cudaSuccess) return e;
-  return launch_slices(append_kernel, append_clusters(p) * kSliceCtas, kSliceSmem, stream, x, w, positions, page_table, cache,
-                       dev_status, p.batch, p.q_len, p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.num_pages,
-                       p.max_pages_per_seq, p.rope_theta);
+  const int K = p.kv_lora_rank + p.qk_rope_dim;
+  if (prologue_sm100_supported(p))
+    return launch_append_sm100(p, x, w, positions, page_table, cache, nullptr, dev_status, stream);
+  if (append_in_clusters(p)) {
+    static PerDeviceFlag smem_set;
+    if (cudaError_t e = ensure_dynamic_smem(append_cluster_kernel, static_cast<int>(kSliceSmem), smem_set); e != cudaSuccess) return e;
+    return launch_slices(append_cluster_kernel, append_clusters(p) * kSliceCtas, kSliceSmem, stream, x, w, positions, page_table, cache,
+                         dev_status, p.batch, p.q_len, p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.num_pages,
+                         p.max_pages_per_seq, p.rope_theta);
+  }
+  const int ts = append_token_splits(p);
+  const int wide = append_wide(p) ? 1 : 0;
+  return launch_pdl(append_kernel, dim3(K / (wide ? 32 : 8) * ts), dim3(256), kAppendSmem, stream, x, w, positions, page_table,
+                    cache, dev_status, p.batch, p.q_len, p.hidden_dim, p.kv_lora_rank, p.qk_rope_dim, p.num_pages,
+                    p.max_pages_per_seq, p.rope_theta, ts, wide);
 }
 
 cudaError_t launch_absorb_plan(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* q_nope,
@@ -200,16 +261,18 @@ cudaError_t launch_absorb_plan(const transmla_params_t& p, const Partitioning& p
   // Few rows behind a launch of linear maps: the maps' CTAs leave some SMs free, where more and shorter blocks end sooner
   // (layer step, mma.sync / tcgen05: 1 token 47.1 / 47.6 us, 16 70.5 / 71.9, 32 75.6 / 76.0, 48 91.1 / 90.1, 64 91.0 / 85.1; 64
   // heads: 8 99.6 / 101.3, 32 118.2 / 118.5, 64 145.4 / 143.2; behind the FP8 append: 4 35.7 / 35.6, 16 55.2 / 52.0).
-  if (prologue_sm100_supported(p) && !(behind_maps && p.batch * p.q_len <= 32))
+  const bool sm100 = prologue_sm100_supported(p);
+  if (sm100 && !(behind_maps && p.batch * p.q_len <= 32))
     return launch_absorb_sm100(p, parts, nullptr, nullptr, nullptr, nullptr, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan, dev_status, stream);
-  size_t smem = absorb_smem(p.qk_nope_dim);
+  const int nt = sm100 ? 1 : absorb_tiles_per_block(p, 1);
+  size_t smem = absorb_smem(p.qk_nope_dim, nt);
   if (smem < kPlanSmemSeqs * sizeof(int32_t)) smem = kPlanSmemSeqs * sizeof(int32_t);
   static PerDeviceFlag smem_set;  // zero-initialised; one slot per device
   if (cudaError_t e = ensure_dynamic_smem(absorb_plan_kernel, kPrologueMaxSmem, smem_set); e != cudaSuccess) return e;
-  const int blocks = p.num_heads * ((p.kv_lora_rank + 127) / 128) + 1;
+  const int blocks = p.num_heads * ((p.kv_lora_rank + 127) / 128 / nt) + 1;
   return launch_pdl(absorb_plan_kernel, dim3(blocks), dim3(256), smem, stream, q_nope, q_pe, w_uk, q_hat, seqlens, cum,
                     plan, dev_status, p.batch, p.q_len, p.num_heads, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, parts,
-                    p.max_pages_per_seq);
+                    p.max_pages_per_seq, nt);
 }
 
 cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
@@ -219,16 +282,26 @@ cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& part
                             cudaStream_t stream) {
   if (prologue_sm100_supported(p))
     return launch_absorb_sm100(p, parts, x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan, dev_status, stream);
-  const int n_append = append_clusters(p);
-  size_t smem = absorb_smem(p.qk_nope_dim);
-  if (smem < kSliceSmem) smem = kSliceSmem;
-  const int others = 1 + p.num_heads * ((p.kv_lora_rank + 127) / 128);
-  const int blocks = (n_append + (others + kSliceCtas - 1) / kSliceCtas) * kSliceCtas;
-  static PerDeviceFlag smem_set;
-  if (cudaError_t e = ensure_dynamic_smem(prologue_kernel, kPrologueMaxSmem, smem_set); e != cudaSuccess) return e;
-  return launch_slices(prologue_kernel, blocks, smem, stream, x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan,
-                       dev_status, p.batch, p.q_len, p.num_heads, p.hidden_dim, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank,
-                       p.num_pages, p.max_pages_per_seq, p.rope_theta, parts, n_append);
+  const bool clusters = append_in_clusters(p);
+  const int ts = append_token_splits(p), wide = append_wide(p) ? 1 : 0;
+  const int n_append = clusters ? append_clusters(p) : (p.kv_lora_rank + p.qk_rope_dim) / (wide ? 32 : 8) * ts;
+  const int nt = clusters ? 1 : absorb_tiles_per_block(p, 1 + n_append);
+  const int others = 1 + p.num_heads * ((p.kv_lora_rank + 127) / 128 / nt);
+  const size_t smem_append = clusters ? kSliceSmem : kAppendSmem;
+  size_t smem = absorb_smem(p.qk_nope_dim, nt);
+  if (smem < smem_append) smem = smem_append;
+  static PerDeviceFlag smem_set[2];  // zero-initialised; one slot per device
+  if (cudaError_t e = ensure_dynamic_smem(clusters ? prologue_kernel<true> : prologue_kernel<false>, kPrologueMaxSmem, smem_set[clusters]); e != cudaSuccess) return e;
+  auto with_args = [&](auto launch) {
+    return launch(x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan, dev_status, p.batch, p.q_len,
+                  p.num_heads, p.hidden_dim, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, p.num_pages, p.max_pages_per_seq,
+                  p.rope_theta, parts, n_append, ts, wide, nt);
+  };
+  if (clusters)
+    return with_args([&](auto... a) {
+      return launch_slices(prologue_kernel<true>, (n_append + (others + kSliceCtas - 1) / kSliceCtas) * kSliceCtas, smem, stream, a...);
+    });
+  return with_args([&](auto... a) { return launch_pdl(prologue_kernel<false>, dim3(n_append + others), dim3(256), smem, stream, a...); });
 }
 
 // ------------------------------------------------------------------------------------------------

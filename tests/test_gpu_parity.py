@@ -367,6 +367,96 @@ def test_append_of_many_tokens_writes_the_bytes_of_few(shape, B):
     assert torch.equal(caches[0], caches[1])
 
 
+def _seqlens(n):
+    return [3 + (37 * i) % 150 for i in range(n - 1)] + [64 * 9 + 5]
+
+
+@pytest.mark.parametrize('shape,B', [
+    # one and several tiles of 64 new tokens ahead of the plan and the absorb, a ring of four pieces and of three; 64 heads, two
+    # positions, more than 128 query rows
+    (synth.LLAMA2_7B, 1), (synth.LLAMA2_7B, 33), (synth.LLAMA2_7B, 65), (synth.LLAMA2_7B, 130), (synth.QWEN25_72B, 3),
+    (synth.QWEN25_72B, 70), (dataclasses.replace(synth.LLAMA2_7B, D=1280), 17), (dataclasses.replace(synth.LLAMA2_7B, D=4352), 40),
+    # other shapes: append blocks up to 32 new tokens, then clusters (r + dR a multiple of 128: blocks), whose CTAs take D / 8 in
+    # pieces of 128; one and two tiles of 128 latents an absorb block
+    (synth.TINY, 3), (synth.TINY, 33), (synth.MLAShape(H=16, dn=64, dR=0, dv=64, r=128, D=768), 20),
+    (synth.MLAShape(H=16, dn=64, dR=0, dv=64, r=128, D=768), 70), (dataclasses.replace(synth.LLAMA2_7B, dn=64), 32),
+    (dataclasses.replace(synth.LLAMA2_7B, dn=64, D=768), 33), (dataclasses.replace(synth.LLAMA2_7B, dn=64, D=1280, S=2), 35),
+    (dataclasses.replace(synth.LLAMA2_7B, dn=192, D=4352), 65), (synth.MLAShape(H=8, dn=32, dR=16, dv=32, r=64, D=4352), 49)])
+def test_decode_step_in_one_call(shape, B):
+    """Cache rows, absorbed queries and results of the fused step against the oracle, and against append, decode and combine by
+    themselves."""
+    S, seqlens, scale = shape.S, _seqlens(B), gu.mla_scale(shape)
+    dc = synth.make_decode_case(shape, seqlens, 71)
+    ac = synth.make_append_case(shape, [L - S for L in seqlens], 72)
+    dev, w = gu.to_dev(dc), ac['w_dkv_kr'].cuda()
+    params = binding.make_params(shape, B, dc['cache'].shape[0], dc['page_table'].shape[1], scale)
+    results = []
+    for fused in (True, False):
+        ws, lay = binding.alloc_workspace(params)
+        ws.fill_(0xff)
+        status = torch.zeros(1, dtype=torch.int32, device='cuda')
+        out = torch.full((B, S, shape.H, shape.dv), float('nan'), dtype=torch.bfloat16, device='cuda')
+        lse = torch.full((B, S, shape.H), float('nan'), device='cuda')
+        cache, q_pe, x = dc['cache'].cuda(), dev['q_pe'] if shape.dR else None, ac['x'].cuda()
+        if fused:
+            binding.transmla_decode_step(params, x, dev['q_nope'], q_pe, dev['page_table'], dev['seqlens'], w, dev['w_uk'],
+                                         dev['w_uv'], cache, ws, out, lse, status)
+        else:
+            binding.transmla_latent_append(params, x, w, ac['positions'].cuda(), dev['page_table'], cache, status)
+            binding.transmla_mla_decode(params, dev['q_nope'], q_pe, dev['w_uk'], cache, dev['page_table'], dev['seqlens'], ws, status)
+            binding.transmla_mla_combine(params, ws, dev['w_uv'], out, lse, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        results.append((cache.cpu(), lifts.f64(binding.workspace_views(params, ws, lay)['q_hat']), lifts.f64(out), lifts.f64(lse)))
+    want = lifts.f64(dc['cache'])
+    touched = np.zeros(want.shape[:2], bool)
+    for s in range(S):
+        pos = [L - S + s for L in seqlens]
+        orc.latent_append(lifts.f64(ac['x'][:, s]), lifts.f64(ac['w_dkv_kr']), pos, dc['page_table'].numpy(), want, shape.r)
+        for b in range(B):
+            touched[orc.append_slot(dc['page_table'][b].numpy(), pos[b], 64)] = True
+    case = dict(dc, cache=torch.tensor(want).to(torch.bfloat16))
+    heads = sorted({0, shape.H // 2, shape.H - 1})
+    only = [(b, s, h) for b in sorted({0, B // 2, 63 % B, 64 % B, 128 % B, B - 1}) for s in range(S) for h in heads]
+    idx = tuple(np.array(only).T)
+    want_out, want_lse = gu.oracle_decode(shape, case, scale, only=only)
+    c = lifts.case_f64(dc)
+    want_q = orc.absorb(c['q_nope'], c['q_pe'], c['w_uk'])
+    for cache, q_hat, out, lse in results:
+        got = lifts.f64(cache)
+        assert np.all(np.abs(got[touched] - want[touched]) <= 2.0 ** -7 * np.abs(want[touched]) + 1e-3)
+        t = torch.tensor(touched)
+        assert torch.equal(cache.view(torch.int16)[~t], dc['cache'].view(torch.int16)[~t])
+        assert np.all(np.abs(q_hat - want_q) <= 2.0 ** -7 * np.abs(want_q) + 1e-3)
+        assert np.all(np.isfinite(out)) and np.all(np.isfinite(lse))
+        gu.assert_close(out[idx], want_out[idx], 'step')
+        gu.assert_lse_close(lse[idx], want_lse[idx], 'step lse')
+    # the same sums in another order at most: a bf16 step of a cache row or query, and what that moves the results by
+    one, two = lifts.f64(results[0][0]), lifts.f64(results[1][0])
+    assert np.all(np.abs(one - two) <= 2.0 ** -7 * np.abs(two) + 1e-3)
+    gu.assert_close(results[0][2], results[1][2], 'fused against separate')
+
+
+@pytest.mark.parametrize('shape,B', [(dataclasses.replace(synth.LLAMA2_7B, dn=64, D=768), 40), (synth.LLAMA2_7B, 40), (synth.TINY, 5)])
+def test_append_leaves_alone_what_has_no_page(shape, B):
+    # a position beyond the page table and a page beyond the pool: reported, nothing written for those tokens, the others are
+    positions = [3 + 5 * i for i in range(B)]
+    ac = gu.to_dev(synth.make_append_case(shape, positions, 73))
+    cols = max(positions) // 64 + 1
+    table = torch.arange(B * cols, dtype=torch.int32, device='cuda').reshape(B, cols)
+    table[1] = B * cols                                # outside the pool
+    pos = torch.tensor(positions, dtype=torch.int32, device='cuda')
+    pos[2] = cols * 64                                 # outside the table
+    cache = torch.zeros(B * cols, 64, shape.row, dtype=torch.bfloat16, device='cuda')
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    params = binding.make_params(shape, B, B * cols, cols, 1.0)
+    binding.transmla_latent_append(params, ac['x'], ac['w_dkv_kr'], pos, table, cache, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) != 0
+    rows = (cache != 0).any(-1).sum(1).view(B, cols).sum(1)
+    assert rows.tolist() == [0 if b in (1, 2) else 1 for b in range(B)]
+
+
 @pytest.mark.parametrize('pinned', [True, False])
 def test_decode_step_from_host_buffers(pinned):
     shape = synth.LLAMA2_7B
