@@ -542,11 +542,22 @@ cudaError_t launch_combine(const transmla_params_t& p, int G, const int32_t* cum
     return launch_pdl(kernel, dim3(H, (BS + rows - 1) / rows, halves), dim3(256), smem, stream, cum, plan, partial_o, partial_lse, w_uv,
                       out, lse_out, p.batch, p.q_len, H, p.kv_lora_rank, p.v_dim, G);
   };
+  // Up to one wave of blocks.  Two halves of dv a row where that leaves room: a block then reads half of W_UV_h, which is what
+  // is left to wait for where the merge is short.  Four rows a block merge sooner than eight while two halves of them fit;
+  // beyond that eight rows and halves instead of four rows and all of dv.  The step of 32 heads, dv = 128, at 9 / 12 / 16
+  // sequences of 1000: 25.6 / 26.2 / 24.6 us -> 22.6 / 22.8 / 23.7; of 300: 25.0 / 25.6 / 27.3 -> 24.4 / 25.3 / 26.1; of 8192: 32.8 / 36.7 /
+  // 42.0 -> 33.5 / 36.6 / 42.1; 64 heads at 6 of 300 and 8192: 26.0 and 34.4 -> 24.6 and 34.3.  With dv <= 64 a warp has one tile of columns
+  // as it is, and few rows leave more SMs to the launches either side: dv = 64, append + decode + combine of 4 sequences of
+  // 100 27.8 us (4 rows, all of dv), 26.7 (halves), 25.2.
   if (p.v_dim >= 128 && 2 * blocks(4) <= kSms) return launch(combine_kernel<4, 1, true>, 4, 2);
+  if (p.v_dim <= 64 && BS <= 32 && blocks(8) <= kSms) return launch(combine_kernel<8, 1, true>, 8, 1);
+  if (2 * blocks(8) <= kSms) return launch(combine_kernel<8, 1, true>, 8, 2);
   if (blocks(4) <= kSms) return launch(combine_kernel<4, 2, true>, 4, 1);
   if (blocks(8) <= kSms) return launch(combine_kernel<8, 2, true>, 8, 1);
   if (combine_sm100_supported(p)) return launch_combine_sm100(p, G, cum, plan, partial_o, partial_lse, w_uv, out, lse_out, dev_status, stream);
-  return launch(combine_kernel<16, 2, false>, 16, 1);
+  // (8 warps x 16 columns are 128 of dv: while a wave of two blocks an SM has room, dv = 256 goes in halves.  32 heads x 64 rows, the
+  // step of 300 and 4000 cached tokens: 40.4 and 79.6 us -> 32.4 and 72.6; with more blocks it costs: x 128 rows 17.3 -> 21.1 alone.)
+  return launch(combine_kernel<16, 2, false>, 16, p.v_dim > 128 && blocks(16) <= kSms ? 2 : 1);
 }
 
 }  // namespace transmla

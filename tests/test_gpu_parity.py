@@ -175,12 +175,23 @@ def test_wide_heads_and_many_sequences():
     gu.assert_close(lifts.f64(out)[idx], want[idx], 'many sequences')
 
 
-@pytest.mark.parametrize('B,S', [(8, 1), (9, 1), (16, 1), (17, 1), (33, 1), (73, 1), (74, 2), (149, 1)])
+@pytest.mark.parametrize('B,S', [(8, 1), (9, 1), (16, 1), (17, 1), (32, 1), (33, 1), (64, 1), (65, 1), (73, 1), (128, 1), (129, 1),
+                                 (74, 2), (149, 1)])
 def test_combine_forms(B, S):
-    # 32 heads: the launch changes its rows per block, halves of dv and weight prefetch at 8, 16, 32, 72 and 144 query rows;
-    # lengths that make a row of one partial, of several, and of none (a query position that sees nothing)
+    # 32 heads: the launch changes its rows per block, halves of dv, weight prefetch and instructions behind 8, 16, 32, 64 and 128
+    # query rows; lengths that make a row of one partial, of several, and of none (a query position that sees nothing)
     lens = [(7 * i) % 90 + 1 for i in range(B - 1)] + [64 * 40 + 5]
     _run_and_compare(dataclasses.replace(synth.LLAMA2_7B, S=S), lens, seed=61)
+
+
+@pytest.mark.parametrize('H,dv,B', [(128, 128, 1), (128, 128, 4), (8, 128, 36), (8, 128, 37), (160, 128, 1),
+                                    (32, 64, 1), (32, 64, 32), (8, 64, 33), (32, 64, 33), (160, 64, 9), (32, 256, 1), (32, 256, 16),
+                                    (32, 256, 64), (32, 256, 73), (8, 200, 9), (40, 96, 9), (40, 96, 17), (16, 24, 9), (8, 8, 3)])
+def test_combine_forms_of_other_head_counts_and_widths(H, dv, B):
+    # more heads than half a wave takes with 4 or 8 rows a block, dv below and above what the warps of a block take at once, halves
+    # of an odd number of 8-column tiles
+    lens = [(7 * i) % 90 + 1 for i in range(B - 1)] + [64 * 11 + 5]
+    _run_and_compare(dataclasses.replace(synth.LLAMA2_7B, H=H, dv=dv), lens, seed=62)
 
 
 def test_qwen_shape_two_query_positions():
