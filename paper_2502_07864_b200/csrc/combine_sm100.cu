@@ -163,11 +163,14 @@ cudaError_t launch_combine_sm100(const transmla_params_t& p, int G, const int32_
     return launch_pdl(kernel, dim3(H, (BS + rows - 1) / rows), dim3(kCbThreads), static_cast<size_t>(bytes), stream, cum, plan, partial_o,
                       partial_lse, w_uv, out, lse_out, dev_status, p.batch, p.q_len, H, G);
   };
-  // One wave of blocks, one an SM, with as few rows a block as that allows.
+  // One wave of blocks, one an SM, with as few rows a block as that allows; beyond a wave as many rows a block as there are, up
+  // to 64: W_UV_h is then read less often.  16 / 32 / 64 rows a block, alone: 160 heads x 16 rows 10.8 / 11.9 / 15.1 us, x 32 16.4 / 13.1 / 16.2;
+  // 512 x 32 47.0 / 34.6 / 41.7; 1.7 waves of 64 (64 x 256) 39.5 / 26.6 / 20.2 (mma.sync, 16 rows 37.2), 2.2 (32 x 300) 26.7 / 18.9 / 18.5 (26.7),
+  // just over one (64 x 129) 22.0 / 17.8 / 16.9 (21.0).
   constexpr int kSms = 148;
   auto blocks = [&](int rows) { return static_cast<long long>(H) * ((BS + rows - 1) / rows); };
-  if (blocks(16) <= kSms) return launch(combine_sm100_kernel<16>, 16, CombineMap<16>::kBytes, smem_set[0]);
-  if (blocks(32) <= kSms) return launch(combine_sm100_kernel<32>, 32, CombineMap<32>::kBytes, smem_set[1]);
+  if (blocks(16) <= kSms || BS <= 16) return launch(combine_sm100_kernel<16>, 16, CombineMap<16>::kBytes, smem_set[0]);
+  if (blocks(32) <= kSms || BS <= 32) return launch(combine_sm100_kernel<32>, 32, CombineMap<32>::kBytes, smem_set[1]);
   return launch(combine_sm100_kernel<64>, 64, CombineMap<64>::kBytes, smem_set[2]);
 }
 

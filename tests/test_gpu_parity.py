@@ -184,9 +184,11 @@ def test_combine_forms(B, S):
     _run_and_compare(dataclasses.replace(synth.LLAMA2_7B, S=S), lens, seed=61)
 
 
-@pytest.mark.parametrize('H,dv,B', [(128, 128, 1), (128, 128, 4), (8, 128, 36), (8, 128, 37), (160, 128, 1),
+@pytest.mark.parametrize('H,dv,B', [(128, 128, 1), (128, 128, 4), (8, 128, 36), (8, 128, 37),
                                     (32, 64, 1), (32, 64, 32), (8, 64, 33), (32, 64, 33), (160, 64, 9), (32, 256, 1), (32, 256, 16),
-                                    (32, 256, 64), (32, 256, 73), (8, 200, 9), (40, 96, 9), (40, 96, 17), (16, 24, 9), (8, 8, 3)])
+                                    (32, 256, 64), (32, 256, 73), (8, 200, 9), (40, 96, 9), (40, 96, 17), (16, 24, 9), (8, 8, 3),
+                                    # more than a wave of blocks whatever their rows: 16, 32 or 64 of them
+                                    (160, 128, 1), (160, 128, 16), (160, 128, 17), (160, 128, 32), (160, 128, 33)])
 def test_combine_forms_of_other_head_counts_and_widths(H, dv, B):
     # more heads than half a wave takes with 4 or 8 rows a block, dv below and above what the warps of a block take at once, halves
     # of an odd number of 8-column tiles
