@@ -63,11 +63,14 @@ typedef enum {
 /* page-equivalents charged to a partition for every sequence it opens (split plan) */
 #define TRANSMLA_SEGMENT_COST_PAGES 2
 
-/* bits of the device status word; when TRANSMLA_DEV_TIMEOUT is set, bits 8 and up tell which of the kernel's
- * internal waits were still pending (diagnostic only, no stable meaning) */
+/* bits of the device status word; when TRANSMLA_DEV_TIMEOUT is set, TRANSMLA_DEV_IN_PROLOGUE and TRANSMLA_DEV_IN_COMBINE tell
+ * that a wait gave up in the launch before or behind the split-KV kernel (whose results are then NaN), and bits 8 and up
+ * which internal waits of the other kernels were still pending (diagnostic only, no stable meaning) */
 #define TRANSMLA_DEV_BAD_PAGE 1
 #define TRANSMLA_DEV_TIMEOUT 2
 #define TRANSMLA_DEV_BAD_LEN 4
+#define TRANSMLA_DEV_IN_PROLOGUE 64
+#define TRANSMLA_DEV_IN_COMBINE 128
 #define TRANSMLA_DEV_NUMERIC 8 /* conversion calls: an eigen-iteration did not converge, or a Gram matrix was singular */
 
 typedef struct {
@@ -302,6 +305,16 @@ transmla_status_t transmla_selftest_bounded_wait(int32_t* dev_status, long long*
  * and NaN in C [M,N]. */
 transmla_status_t transmla_selftest_conv_gemm(int pairs, int M, int N, int K, const float* A, const float* B, float* C,
                                               int32_t* dev_status, void* stream);
+
+/* Diagnostic: the tcgen05 kernels either side of the split-KV kernel, as transmla_decode_step launches them (the combine's also
+ * for few query rows), with barrier waits that give up at once: the prologue (append, plan, absorb), then the combine of
+ * the partials that an earlier step has left in the workspace.  Shows what that leaves behind: TRANSMLA_DEV_TIMEOUT and both
+ * bits of these kernels in *dev_status (required) and NaN in the new cache rows, the absorbed queries and out.  Needs
+ * r = 512, dR = 64, dn = dv = 128. */
+transmla_status_t transmla_selftest_step_gives_up(const transmla_params_t* params /* host */, const void* x, const void* q_nope,
+                                                  const void* q_pe, const int32_t* page_table, const int32_t* seqlens,
+                                                  const void* w_dkv_kr, const void* w_uk, const void* w_uv, void* cache,
+                                                  void* workspace, size_t workspace_bytes, void* out, int32_t* dev_status, void* stream);
 
 /* Diagnostic: transmla_conv_top_subspace with the cluster of its Cholesky factor limited to most_ctas CTAs (1, 2, 4, 8 or
  * 16), as on a device or partition that holds no larger one. */

@@ -15,7 +15,7 @@ EXPORTS = ('transmla_workspace_layout', 'transmla_latent_append', 'transmla_mla_
            'transmla_validate_tables', 'transmla_step_staging_bytes', 'transmla_decode_step_host',
            'transmla_decode_step', 'transmla_profile_decode_kernel', 'transmla_status_string',
            'transmla_static_workspace_capacity', 'transmla_mla_attention_static', 'transmla_selftest_bounded_wait',
-           'transmla_selftest_conv_gemm', 'transmla_selftest_conv_subspace',
+           'transmla_selftest_conv_gemm', 'transmla_selftest_conv_subspace', 'transmla_selftest_step_gives_up',
            'transmla_layer_scratch_bytes', 'transmla_layer_decode_step', 'transmla_stream_probe', 'transmla_page_claims_at_run_time', 'transmla_latent_append_fp8',
            'transmla_mla_decode_fp8', 'transmla_prefill_scratch_bytes', 'transmla_prefill_decompress',
            'transmla_prefill_attention', 'transmla_mla_prefill', 'transmla_conv_gemm',
@@ -78,6 +78,7 @@ def lib():
         L.transmla_static_workspace_capacity.restype = sz
         L.transmla_mla_attention_static.argtypes = [pp, vp, vp, vp, vp, vp, i32p, i32p, vp, vp, i32p, vp]
         L.transmla_selftest_bounded_wait.argtypes = [i32p, vp, vp]
+        L.transmla_selftest_step_gives_up.argtypes = [pp, vp, vp, vp, i32p, i32p, vp, vp, vp, vp, vp, sz, vp, i32p, vp]
         L.transmla_stream_probe.argtypes = [pp, vp, i32p, vp, sz, i32p, vp]
         L.transmla_page_claims_at_run_time.argtypes = [pp]
         L.transmla_latent_append_fp8.argtypes = [pp, vp, vp, i32p, i32p, vp, vp, sz, i32p, vp]
@@ -200,6 +201,14 @@ def transmla_decode_step(params, x, q_nope, q_pe, page_table, seqlens, w_dkv_kr,
         _ptr(w_uk), _ptr(w_uv), _ptr(cache), _ptr(workspace),
         workspace.numel() * workspace.element_size(), _ptr(out), _ptr(lse_out), _ptr(dev_status), _stream(stream)),
         'transmla_decode_step')
+
+
+def transmla_selftest_step_gives_up(params, x, q_nope, q_pe, page_table, seqlens, w_dkv_kr, w_uk, w_uv, cache, workspace, out,
+                                    dev_status, stream=None):
+    _check(lib().transmla_selftest_step_gives_up(
+        ctypes.byref(params), _ptr(x), _ptr(q_nope), _ptr(q_pe), _ptr(page_table), _ptr(seqlens), _ptr(w_dkv_kr), _ptr(w_uk),
+        _ptr(w_uv), _ptr(cache), _ptr(workspace), workspace.numel() * workspace.element_size(), _ptr(out), _ptr(dev_status),
+        _stream(stream)), 'transmla_selftest_step_gives_up')
 
 
 def transmla_static_workspace_capacity():

@@ -4,6 +4,8 @@
 #include <unordered_set>
 #include <vector>
 
+#include "append_block.cuh"
+#include "combine.cuh"
 #include "common.cuh"
 
 using namespace transmla;
@@ -375,6 +377,33 @@ transmla_status_t transmla_decode_step(const transmla_params_t* p, const void* x
   st = launch_split_kv(p, lay, cache, page_table, seqlens, ws, dev_status, s);
   if (st != TRANSMLA_OK) return st;
   return transmla_mla_combine(p, workspace, workspace_bytes, w_uv, out, lse_out, dev_status, stream);
+}
+
+transmla_status_t transmla_selftest_step_gives_up(const transmla_params_t* p, const void* x, const void* q_nope, const void* q_pe,
+                                                  const int32_t* page_table, const int32_t* seqlens, const void* w_dkv_kr,
+                                                  const void* w_uk, const void* w_uv, void* cache, void* workspace,
+                                                  size_t workspace_bytes, void* out, int32_t* dev_status, void* stream) {
+  transmla_status_t st = validate_step_args(p, x, q_nope, q_pe, w_dkv_kr, w_uk, w_uv, cache, page_table, seqlens, workspace,
+                                            workspace_bytes, out, dev_status);
+  if (st != TRANSMLA_OK) return st;
+  if (!prologue_sm100_supported(*p) || !combine_sm100_supported(*p)) return TRANSMLA_ERR_SHAPE;
+  if (!dev_status) return TRANSMLA_ERR_NULL;
+  transmla_workspace_layout_t lay;
+  if ((st = transmla_workspace_layout(p, &lay)) != TRANSMLA_OK) return st;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  char* ws = static_cast<char*>(workspace);
+  auto* cum = reinterpret_cast<int32_t*>(ws + lay.cum_pages_offset);
+  auto* plan = reinterpret_cast<int32_t*>(ws + lay.plan_offset);
+  if (launch_absorb_sm100(*p, decode_partitioning(*p, lay.num_partitions), static_cast<const __nv_bfloat16*>(x),
+                          static_cast<const __nv_bfloat16*>(w_dkv_kr), page_table, static_cast<__nv_bfloat16*>(cache),
+                          static_cast<const __nv_bfloat16*>(q_nope), static_cast<const __nv_bfloat16*>(q_pe),
+                          static_cast<const __nv_bfloat16*>(w_uk), reinterpret_cast<__nv_bfloat16*>(ws + lay.q_hat_offset), seqlens,
+                          cum, plan, dev_status, s, true) != cudaSuccess)
+    return TRANSMLA_ERR_CUDA;
+  return launch_combine_sm100(*p, lay.num_partitions, cum, plan, reinterpret_cast<const float*>(ws + lay.partial_o_offset),
+                              reinterpret_cast<const float*>(ws + lay.partial_lse_offset), static_cast<const __nv_bfloat16*>(w_uv),
+                              static_cast<__nv_bfloat16*>(out), nullptr, dev_status, s, true) == cudaSuccess
+             ? TRANSMLA_OK : TRANSMLA_ERR_CUDA;
 }
 
 size_t transmla_step_staging_bytes(const transmla_params_t* p) {

@@ -75,7 +75,8 @@ cudaError_t launch_append_sm100(const transmla_params_t& p, const __nv_bfloat16*
 cudaError_t launch_absorb_sm100(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
                                 const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope, const __nv_bfloat16* q_pe,
                                 const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat, const int32_t* seqlens, int32_t* cum, int32_t* plan,
-                                int32_t* dev_status, cudaStream_t stream);  // x null: without the append
+                                int32_t* dev_status, cudaStream_t stream, bool give_up = false);  // x null: without the append
+// (give_up, here and in launch_combine_sm100: with waits that give up at once, for a test.)
 
 // Shared memory an append block needs, and how the host cuts the append into blocks.
 constexpr size_t kAppendBlockSmem = kAppendSmem;

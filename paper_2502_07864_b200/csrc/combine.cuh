@@ -123,6 +123,6 @@ __device__ __forceinline__ void merge_rows(const MergeArgs& a, int h, int bs_fir
 bool combine_sm100_supported(const transmla_params_t& p);
 cudaError_t launch_combine_sm100(const transmla_params_t& p, int G, const int32_t* cum, const int32_t* plan, const float* partial_o,
                                  const float* partial_lse, const __nv_bfloat16* w_uv, __nv_bfloat16* out, float* lse_out,
-                                 int32_t* dev_status, cudaStream_t stream);
+                                 int32_t* dev_status, cudaStream_t stream, bool give_up = false);
 
 }  // namespace transmla

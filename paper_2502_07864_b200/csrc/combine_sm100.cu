@@ -2,6 +2,7 @@
 // Block = one head x kRows query rows: sixteen warps merge the split partials into shared memory as a bf16 high/low pair, then
 // out [rows x 128] = (o_hi + o_lo) W_UV_h^T as weight-stationary products of 32 or 64 rows; W_UV_h comes by asynchronous copies
 // from before the dependency wait.
+// A barrier wait that gives up (which no launch should see) is reported, and the block's part of out becomes NaN.
 // What bounds it: the partials (30 bytes a cycle and SM from L2) and the look-ups before them.  The mma.sync form (small_kernels.cu)
 // spends 16 cycles of an SM's quarter on each 16 x 8 x 16 product: 9 us of the launch with 64 heads x 128 rows, 5 with 32 x 128,
 // 3 with 32 x 64.  Fewer rows than that (one wave of blocks of 8) stay there: its products take 1 to 2 us, and its
@@ -24,7 +25,7 @@ struct CombineMap {
   static_assert(kBytes <= 232448 && kMisc % 256 == 0, "shared memory budget");
 };
 
-template <int kRows>
+template <int kRows, long long kLimit>
 __global__ void __launch_bounds__(kCbThreads, 1)
 combine_sm100_kernel(const int32_t* cum, const int32_t* plan, const float* partial_o, const float* partial_lse,
                      const __nv_bfloat16* __restrict__ w_uv, __nv_bfloat16* out, float* lse_out, int32_t* dev_status, int B, int S, int H, int G) {
@@ -35,6 +36,7 @@ combine_sm100_kernel(const int32_t* cum, const int32_t* plan, const float* parti
   unsigned char* sm = smem_unaligned + (base - raw);
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(sm + Map::kMisc + 128);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_s + 1);
+  constexpr int kWhere = TRANSMLA_DEV_IN_COMBINE;
   auto bar = [&](int i) -> uint32_t { return base + Map::kMisc + 8 * i; };  // 0: all products; 1, 2: those with pieces 0 and 1
   pdl_trigger();
   const int h = blockIdx.x, bs0 = blockIdx.y * kRows, BS = B * S;
@@ -111,8 +113,7 @@ combine_sm100_kernel(const int32_t* cum, const int32_t* plan, const float* parti
   }
   if (Map::kSlots < 8) {  // the last pieces take the places of the first
     for (int piece = Map::kSlots; piece < 8; ++piece) {
-      mbar_wait(bar(1 + piece - Map::kSlots), 0, abort_flag, dev_status);
-      copy_weights(piece);
+      if (mbar_wait<kLimit, kWhere>(bar(1 + piece - Map::kSlots), 0, abort_flag, dev_status)) copy_weights(piece);
     }
     cp_async_commit();
     cp_async_wait<0>();
@@ -126,7 +127,9 @@ combine_sm100_kernel(const int32_t* cum, const int32_t* plan, const float* parti
       __syncwarp();
     }
   }
-  mbar_wait(bar(0), 0, abort_flag, dev_status);
+  const bool done = mbar_wait<kLimit, kWhere>(bar(0), 0, abort_flag, dev_status);
+  const bool bad = __any_sync(0xffffffffu, !done || *abort_flag != 0);
+  if (bad) mbar_retire(bar(0), 0);
   tc_fence_after();
   // 32 rows: quadrant q has columns 32 q ..; 64 rows: row i of columns 0-63 in lane i, of 64-127 in lane 64 + i.  16 columns a warp.
   const int quad = warp & 3, part = warp >> 2;
@@ -136,7 +139,7 @@ combine_sm100_kernel(const int32_t* cum, const int32_t* plan, const float* parti
     tmem_ld16(tmem + (static_cast<uint32_t>(quad * 32) << 16) + part * 16, v);
     tc_wait_ld();
     if (rr < kRows && bs0 + rr < BS) {
-      auto two = [&](int i) { return pack_bf16(__uint_as_float(v[i]), __uint_as_float(v[i + 1])); };
+      auto two = [&](int i) { return bad ? 0x7fff7fffu : pack_bf16(__uint_as_float(v[i]), __uint_as_float(v[i + 1])); };
       uint4* dst = reinterpret_cast<uint4*>(out + (static_cast<size_t>(bs0 + rr) * H + h) * kCbDv + n0);
       dst[0] = make_uint4(two(0), two(2), two(4), two(6));
       dst[1] = make_uint4(two(8), two(10), two(12), two(14));
@@ -152,9 +155,10 @@ combine_sm100_kernel(const int32_t* cum, const int32_t* plan, const float* parti
 
 bool combine_sm100_supported(const transmla_params_t& p) { return p.kv_lora_rank == sm100::kCbR && p.v_dim == sm100::kCbDv; }
 
-cudaError_t launch_combine_sm100(const transmla_params_t& p, int G, const int32_t* cum, const int32_t* plan, const float* partial_o,
-                                 const float* partial_lse, const __nv_bfloat16* w_uv, __nv_bfloat16* out, float* lse_out,
-                                 int32_t* dev_status, cudaStream_t stream) {
+template <long long kLimit>
+static cudaError_t launch_rows(const transmla_params_t& p, int G, const int32_t* cum, const int32_t* plan, const float* partial_o,
+                               const float* partial_lse, const __nv_bfloat16* w_uv, __nv_bfloat16* out, float* lse_out,
+                               int32_t* dev_status, cudaStream_t stream) {
   using namespace sm100;
   const int BS = p.batch * p.q_len, H = p.num_heads;
   static PerDeviceFlag smem_set[3];
@@ -169,9 +173,15 @@ cudaError_t launch_combine_sm100(const transmla_params_t& p, int G, const int32_
   // just over one (64 x 129) 22.0 / 17.8 / 16.9 (21.0).
   constexpr int kSms = 148;
   auto blocks = [&](int rows) { return static_cast<long long>(H) * ((BS + rows - 1) / rows); };
-  if (blocks(16) <= kSms || BS <= 16) return launch(combine_sm100_kernel<16>, 16, CombineMap<16>::kBytes, smem_set[0]);
-  if (blocks(32) <= kSms || BS <= 32) return launch(combine_sm100_kernel<32>, 32, CombineMap<32>::kBytes, smem_set[1]);
-  return launch(combine_sm100_kernel<64>, 64, CombineMap<64>::kBytes, smem_set[2]);
+  if (blocks(16) <= kSms || BS <= 16) return launch(combine_sm100_kernel<16, kLimit>, 16, CombineMap<16>::kBytes, smem_set[0]);
+  if (blocks(32) <= kSms || BS <= 32) return launch(combine_sm100_kernel<32, kLimit>, 32, CombineMap<32>::kBytes, smem_set[1]);
+  return launch(combine_sm100_kernel<64, kLimit>, 64, CombineMap<64>::kBytes, smem_set[2]);
+}
+
+cudaError_t launch_combine_sm100(const transmla_params_t& p, int G, const int32_t* cum, const int32_t* plan, const float* partial_o,
+                                 const float* partial_lse, const __nv_bfloat16* w_uv, __nv_bfloat16* out, float* lse_out,
+                                 int32_t* dev_status, cudaStream_t stream, bool give_up) {
+  return (give_up ? launch_rows<0> : launch_rows<kWaitCycles>)(p, G, cum, plan, partial_o, partial_lse, w_uv, out, lse_out, dev_status, stream);
 }
 
 }  // namespace transmla

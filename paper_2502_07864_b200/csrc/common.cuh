@@ -109,22 +109,29 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait.  Returns at once when the phase is complete or the CTA has already given up.  For diagnosis, bit 8 + i of the status word
-// is set for every barrier slot i (position within its 256-byte block) on which a wait was still pending when the
-// CTA gave up; the first of them is the one whose limit expired.
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* dev_status) {
-  if (mbar_test(bar, parity)) return;
-  if (*abort_flag) return;
-  if (mbar_try_wait(bar, parity)) return;
+// Bounded wait.  Returns at once when the phase is complete or the CTA has already given up: true where it is complete.  For
+// diagnosis the status word gets kWhere, or (0) bit 8 + i for every barrier slot i (position within its 256-byte block) on which a
+// wait was still pending when the CTA gave up; the first of them is the one whose limit expired.  A limit of 0 (for a
+// test): whatever is not there at the first look.
+template <long long kLimit = kWaitCycles, int kWhere = 0>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* dev_status) {
+  if (mbar_test(bar, parity)) return true;
+  if (*abort_flag) return false;
+  if (kLimit > 0 && mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    const bool expired = clock64() - t0 > kWaitCycles;
+  while (kLimit == 0 || !mbar_try_wait(bar, parity)) {
+    const bool expired = kLimit == 0 || clock64() - t0 > kLimit;
     if (expired || *abort_flag) {
       *abort_flag = 1;
-      set_status(dev_status, TRANSMLA_DEV_TIMEOUT | (1 << (8 + ((bar & 255u) >> 3))));
-      return;
+      set_status(dev_status, TRANSMLA_DEV_TIMEOUT | (kWhere != 0 ? kWhere : 1 << (8 + ((bar & 255u) >> 3))));
+      return false;
     }
   }
+  return true;
+}
+// After a wait gave up: until what the barrier stands for has retired, so that its shared and tensor memory can be used again.
+__device__ __forceinline__ void mbar_retire(uint32_t bar, uint32_t parity) {
+  for (const long long t0 = clock64(); !mbar_try_wait(bar, parity) && clock64() - t0 < kWaitCycles;) {}
 }
 // True in exactly one lane of a converged warp.  Code around it stays warp-uniform, so descriptors and
 // addresses can live in uniform registers instead of being moved there for every instruction.

@@ -9,6 +9,7 @@
 //   absorb   (Eq. 9 right, first line) a block a head and 256 latents: q_hat [rows x 256] = q_nope [rows x 128] W_UK_h, 128 rows a
 //            time as weight-stationary products of 64 rows (82 cycles for 64 x 256 x 16; the plain form takes 286 for 128);
 //            the block with a head's first latents copies the rope part
+// A barrier wait that gives up (which no launch should see) is reported, and what the block had still to write becomes NaN.
 // What bounds it: chains of round trips (look-ups and operands, sums of the other CTAs, stores), 3 to 5 us.  The mma.sync tiles
 // of small_kernels.cu, 16 cycles each on a quarter of an SM, made that 6 us at 16 tokens, 15 at 128 and 22 with 64 heads, where
 // their registers also allowed two blocks an SM of twice as many.
@@ -66,6 +67,10 @@ __device__ __forceinline__ void tmem_free(uint32_t tmem, uint32_t cols) {
 // 16-byte chunk c of row rr of a 128-byte-swizzled tile whose rows are 64 bf16
 __device__ __forceinline__ uint32_t swizzled(int rr, int c) { return rr * 128 + ((c ^ (rr & 7)) << 4); }
 
+constexpr int kPrWhere = TRANSMLA_DEV_IN_PROLOGUE;
+constexpr uint32_t kPrNan = 0x7fffffffu;
+
+template <long long kLimit>
 __device__ __forceinline__ void append_role(const PrologueArgs& a, unsigned char* sm, uint32_t base, uint32_t* tmem_base_s,
                                             volatile int* abort_flag) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -89,7 +94,7 @@ __device__ __forceinline__ void append_role(const PrologueArgs& a, unsigned char
   for (int p = 0; p < ring && p < pieces; ++p) copy(p, w, 64, 0, kPrSub);
   cp_async_commit();
   if (tid == 0) {
-    for (int i = 0; i < 4; ++i) mbar_init(bar(i), 1);
+    for (int i = 0; i < 5; ++i) mbar_init(bar(i), 1);  // 4: the last product
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -139,21 +144,24 @@ __device__ __forceinline__ void append_role(const PrologueArgs& a, unsigned char
         for (int kk = 0; kk < 8; ++kk) {
           mma_ws_ss(tmem, desc_advance(w0, (kk >> 2) * kPrSub + (kk & 3) * 32), desc_advance(x0, (kk >> 2) * x_sub + (kk & 3) * 32), instr_desc(kPrTok, false, 64), (p | kk) != 0);
         }
-        tc_commit(bar(p % ring));
+        tc_commit(bar(p + 1 < pieces ? p % ring : 4));
       }
       __syncwarp();
     }
     if (p > 0) {
       const int q = p + ring - 1;
       if (q < pieces) {
-        mbar_wait(bar((p - 1) % ring), ((p - 1) / ring) & 1, abort_flag, a.dev_status);
-        copy(q, w, 64, 0, kPrSub);
-        copy(q, x, rows, 2 * kPrSub, x_sub);
+        if (mbar_wait<kLimit, kPrWhere>(bar((p - 1) % ring), ((p - 1) / ring) & 1, abort_flag, a.dev_status)) {
+          copy(q, w, 64, 0, kPrSub);
+          copy(q, x, rows, 2 * kPrSub, x_sub);
+        }
       }
       cp_async_commit();
     }
   }
-  mbar_wait(bar((pieces - 1) % ring), ((pieces - 1) / ring) & 1, abort_flag, a.dev_status);
+  const bool done = mbar_wait<kLimit, kPrWhere>(bar(4), 0, abort_flag, a.dev_status);
+  const bool bad = __any_sync(0xffffffffu, !done || *abort_flag != 0);
+  if (bad) mbar_retire(bar(4), 0);
   tc_fence_after();
   const uint32_t tmem = *tmem_base_s;
   float* sums = reinterpret_cast<float*>(sm);  // [token][kPrSums]: every product has completed
@@ -164,7 +172,7 @@ __device__ __forceinline__ void append_role(const PrologueArgs& a, unsigned char
     tmem_ld16(tmem + (static_cast<uint32_t>(quad * 32) << 16) + hf * 16, v);
     tc_wait_ld();
 #pragma unroll
-    for (int j = 0; j < 16; ++j) sums[(tok + j) * kPrSums + feature] = __uint_as_float(v[j]);
+    for (int j = 0; j < 16; ++j) sums[(tok + j) * kPrSums + feature] = __uint_as_float(bad ? kPrNan : v[j]);
   }
   tc_fence_before();
   slice_cluster_sync();
@@ -190,6 +198,7 @@ __device__ __forceinline__ void append_role(const PrologueArgs& a, unsigned char
   if (warp == 0) tmem_free(tmem, 32);
 }
 
+template <long long kLimit>
 __device__ __forceinline__ void absorb_role(const PrologueArgs& a, int h, int half, unsigned char* sm, uint32_t base,
                                             uint32_t* tmem_base_s, volatile int* abort_flag) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, BS = a.B * a.S, H = a.H;
@@ -253,7 +262,9 @@ __device__ __forceinline__ void absorb_role(const PrologueArgs& a, int h, int ha
       }
       __syncwarp();
     }
-    mbar_wait(bar, tile & 1, abort_flag, a.dev_status);
+    const bool done = mbar_wait<kLimit, kPrWhere>(bar, tile & 1, abort_flag, a.dev_status);
+    const bool bad = __any_sync(0xffffffffu, !done || *abort_flag != 0);
+    if (bad) mbar_retire(bar, tile & 1);
     tc_fence_after();
     // Write-out: 32 rows x 64 latents a warp (rows i of latents 0-127 in lane i, of 128-255 in lane 64 + i), through the warp's own
     // 4 KB of the queries' place, whole lines.
@@ -267,6 +278,10 @@ __device__ __forceinline__ void absorb_role(const PrologueArgs& a, int h, int ha
       tmem_ld32(addr, v);
       tmem_ld32(addr + 32, v + 32);
       tc_wait_ld();
+      if (bad) {
+#pragma unroll
+        for (int e = 0; e < 64; ++e) v[e] = kPrNan;
+      }
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const uint32_t* e = v + 8 * c;
@@ -290,6 +305,7 @@ __device__ __forceinline__ void absorb_role(const PrologueArgs& a, int h, int ha
   if (warp == 0) tmem_free(*tmem_base_s, 256);
 }
 
+template <long long kLimit>
 __global__ void __launch_bounds__(256, 2) prologue_sm100_kernel(const __grid_constant__ PrologueArgs a) {
   extern __shared__ unsigned char smem_unaligned[];
   const uint32_t raw = smem_u32(smem_unaligned), base = (raw + 1023u) & ~1023u;
@@ -298,10 +314,10 @@ __global__ void __launch_bounds__(256, 2) prologue_sm100_kernel(const __grid_con
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_base_s + 1);
   pdl_trigger();
   const int bid = static_cast<int>(blockIdx.x) - a.n_append * kSliceCtas;
-  if (bid < 0) append_role(a, sm, base, tmem_base_s, abort_flag);
+  if (bid < 0) append_role<kLimit>(a, sm, base, tmem_base_s, abort_flag);
   else if (bid >= a.others) return;  // the grid is whole clusters
   else if (bid == 0) plan_block(a.seqlens, a.B, a.parts, (a.S * a.H + kRowBlock - 1) / kRowBlock, a.max_pages, a.cum, a.plan, a.dev_status, sm);
-  else absorb_role(a, (bid - 1) >> 1, (bid - 1) & 1, sm, base, tmem_base_s, abort_flag);
+  else absorb_role<kLimit>(a, (bid - 1) >> 1, (bid - 1) & 1, sm, base, tmem_base_s, abort_flag);
 }
 
 }  // namespace sm100
@@ -310,16 +326,18 @@ bool prologue_sm100_supported(const transmla_params_t& p) {
   return p.kv_lora_rank == sm100::kPrR && p.qk_rope_dim == sm100::kPrDR && p.qk_nope_dim == sm100::kPrDn;
 }
 
+template <long long kLimit = kWaitCycles>
 static cudaError_t launch_prologue_sm100(const transmla_params_t& p, sm100::PrologueArgs& a, bool append, bool absorb, cudaStream_t stream) {
+  auto kernel = sm100::prologue_sm100_kernel<kLimit>;
   a.B = p.batch; a.S = p.q_len; a.H = p.num_heads; a.D = p.hidden_dim;
   a.num_pages = p.num_pages; a.max_pages = p.max_pages_per_seq; a.theta = p.rope_theta;
   a.n_append = append ? sm100::kPrRow / 64 * ((p.batch * p.q_len + sm100::kPrTok - 1) / sm100::kPrTok) : 0;
   a.others = absorb ? 1 + 2 * p.num_heads : 0;
   static PerDeviceFlag smem_set;
-  if (cudaError_t e = ensure_dynamic_smem(sm100::prologue_sm100_kernel, sm100::kPrSmem, smem_set); e != cudaSuccess) return e;
+  if (cudaError_t e = ensure_dynamic_smem(kernel, sm100::kPrSmem, smem_set); e != cudaSuccess) return e;
   if (!append)  // small blocks that need not find room in eights beside the kernel before them
-    return launch_pdl(sm100::prologue_sm100_kernel, dim3(a.others), dim3(256), static_cast<size_t>(sm100::kPrSmem), stream, a);
-  return launch_slices(sm100::prologue_sm100_kernel, (a.n_append + (a.others + kSliceCtas - 1) / kSliceCtas) * kSliceCtas,
+    return launch_pdl(kernel, dim3(a.others), dim3(256), static_cast<size_t>(sm100::kPrSmem), stream, a);
+  return launch_slices(kernel, (a.n_append + (a.others + kSliceCtas - 1) / kSliceCtas) * kSliceCtas,
                        static_cast<size_t>(sm100::kPrSmem), stream, a);
 }
 
@@ -334,12 +352,12 @@ cudaError_t launch_append_sm100(const transmla_params_t& p, const __nv_bfloat16*
 cudaError_t launch_absorb_sm100(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
                                 const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope, const __nv_bfloat16* q_pe,
                                 const __nv_bfloat16* w_uk, __nv_bfloat16* q_hat, const int32_t* seqlens, int32_t* cum, int32_t* plan,
-                                int32_t* dev_status, cudaStream_t stream) {
+                                int32_t* dev_status, cudaStream_t stream, bool give_up) {
   sm100::PrologueArgs a = {};
   a.x = x; a.w_dkv_kr = w_dkv_kr; a.pos_base = seqlens; a.pos_shift = -p.q_len; a.page_table = page_table; a.cache = cache;
   a.q_nope = q_nope; a.q_pe = q_pe; a.w_uk = w_uk; a.q_hat = q_hat; a.seqlens = seqlens; a.cum = cum; a.plan = plan;
   a.parts = parts; a.dev_status = dev_status;
-  return launch_prologue_sm100(p, a, x != nullptr, true, stream);
+  return give_up ? launch_prologue_sm100<0>(p, a, x != nullptr, true, stream) : launch_prologue_sm100(p, a, x != nullptr, true, stream);
 }
 
 }  // namespace transmla

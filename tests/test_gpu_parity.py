@@ -314,6 +314,44 @@ def test_a_wait_that_nothing_satisfies_ends_by_itself_and_leaves_the_context_usa
     _run_and_compare(synth.TINY, [17, 64], seed=1, G=2)   # and ordinary work still runs afterwards
 
 
+@pytest.mark.parametrize('shape,B', [(synth.LLAMA2_7B, 5), (synth.LLAMA2_7B, 70), (synth.LLAMA2_7B, 130), (synth.QWEN25_72B, 3),
+                                     (dataclasses.replace(synth.LLAMA2_7B, D=8192), 40)])
+def test_waits_that_give_up_around_the_attention_leave_no_unfinished_values(shape, B):
+    # rings of four and of three pieces that do and do not wrap, one and two tiles of queries, 16, 32 and 64 rows a combine block;
+    # the launches end normally, and a step behind them gives what it gave before
+    S, seqlens = shape.S, [3 + (37 * i) % 150 for i in range(B)]
+    dc = gu.to_dev(synth.make_decode_case(shape, seqlens, 81))
+    ac = gu.to_dev(synth.make_append_case(shape, [L - S for L in seqlens], 82))
+    params = binding.make_params(shape, B, dc['cache'].shape[0], dc['page_table'].shape[1], gu.mla_scale(shape))
+    params.num_partitions = binding.transmla_workspace_layout(params).num_partitions
+    ws, lay = binding.alloc_workspace(params)
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    before = dc['cache'].clone()
+    q_hat = binding.workspace_views(params, ws, lay)['q_hat']
+
+    def run(step, out, *more):
+        step(params, ac['x'], dc['q_nope'], dc['q_pe'], dc['page_table'], dc['seqlens'], ac['w_dkv_kr'], dc['w_uk'], dc['w_uv'],
+             dc['cache'], ws, out, *more, status)
+        torch.cuda.synchronize()
+        return dc['cache'].clone(), out.clone(), q_hat.clone()
+
+    out = torch.zeros(B, S, shape.H, shape.dv, dtype=torch.bfloat16, device='cuda')
+    first = run(binding.transmla_decode_step, out, None)
+    assert int(status.item()) == 0
+    new = (first[0] != before).any(-1)
+    assert int(new.sum()) == B * S
+    for _ in range(20):
+        out.zero_(); status.zero_()
+        cache, got, q = run(binding.transmla_selftest_step_gives_up, out)
+        assert int(status.item()) == 2 | 64 | 128      # TRANSMLA_DEV_TIMEOUT, _IN_PROLOGUE, _IN_COMBINE
+        assert bool(torch.isnan(cache[new]).all()) and torch.equal(cache[~new], before[~new])
+        assert bool(torch.isnan(q[..., :shape.r]).all()) and torch.equal(q[..., shape.r:], first[2][..., shape.r:])
+        assert bool(torch.isnan(got).all())
+    status.zero_()
+    again = run(binding.transmla_decode_step, out, None)
+    assert int(status.item()) == 0 and all(torch.equal(a, b) for a, b in zip(first, again))
+
+
 # ------------------------------------------------------------------ append
 @pytest.mark.parametrize('shape,positions', [(synth.TINY, [16, 63, 64, 0]), (synth.LLAMA2_7B, [8191, 0, 77, 131071]),
                                              (synth.QWEN25_72B, [126, 63, 4000]),
