@@ -373,18 +373,24 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
       *reinterpret_cast<float4*>(mine + lane * kPitch + j) =
           make_float4(acc[j] * args.alpha, acc[j + 1] * args.alpha, acc[j + 2] * args.alpha, acc[j + 3] * args.alpha);
     // Where the split does not hold the sum is taken once more, by fp32 multiply-adds: an infinite or too large operand value
-    // has no exact terms and made its sums NaN, and operands so small that all of the warp's sums stay below 2^-63 may have
-    // lost their last terms.
-    float size[4] = {0.f, 0.f, 0.f, 0.f};
+    // has no exact terms and made its sums NaN, and operands so small that all sums of a region (32 rows x a quarter of the
+    // tile's columns) stay below 2^-63 may have lost their last terms.
+    constexpr int kRegion = kTile / 4;
+    uint32_t small = 0, odd = 0;                        // bits of the warp's regions
 #pragma unroll
-    for (int j = 0; j < kCols; ++j) size[j & 3] += fabsf(acc[j]);
-    const float all = (size[0] + size[1]) + (size[2] + size[3]);
-    const bool small = __all_sync(0xffffffffu, all < 0x1p-63f) && __any_sync(0xffffffffu, all > 0.f);
-    if (small || __any_sync(0xffffffffu, !(all < INFINITY))) {
+    for (int g = 0; g < kCols / kRegion; ++g) {
+      float size[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int j = 0; j < kRegion; ++j) size[j & 3] += fabsf(acc[g * kRegion + j]);
+      const float all = (size[0] + size[1]) + (size[2] + size[3]);
+      if (__all_sync(0xffffffffu, all < 0x1p-63f) && __any_sync(0xffffffffu, all > 0.f)) small |= 1u << g;
+      if (__any_sync(0xffffffffu, !(all < INFINITY))) odd |= 1u << g;
+    }
+    if ((small | odd) != 0) {
 #pragma unroll 1
       for (int j = 0; j < kCols; ++j) {
         const int m = m0 + quad * 32 + lane, n = n0 + half * kCols + j;
-        if (m < M && n < N && (small || !isfinite(mine[lane * kPitch + j])))
+        if (m < M && n < N && ((small >> (j / kRegion) & 1u) || !isfinite(mine[lane * kPitch + j])))
           mine[lane * kPitch + j] = args.alpha * plain_sum<kAContig, kBContig>(args, m, n);
       }
     }

@@ -93,6 +93,27 @@ def test_gemm_of_infinities_and_of_values_at_the_ends_of_fp32(M, N, K, ta, tb):
         assert float(rel) < K * 2.0 ** -24, scale
 
 
+@pytest.mark.parametrize('M,N,K,ta,tb,cols', [(200, 150, 100, 0, 0, 32), (200, 150, 100, 1, 1, 32), (6000, 5000, 40, 0, 1, 64),
+                                              (5001, 5003, 40, 1, 0, 64)])
+@pytest.mark.parametrize('scale', [2.0 ** -112, 2.0 ** -120])
+def test_gemm_of_tiny_columns_beside_ordinary_ones(M, N, K, ta, tb, cols, scale):
+    # whether tiny operands' sums are taken again is decided for a quarter of a tile's columns (32 of one CTA's, 64 of a
+    # pair's): every other quarter tiny, each column's error against its own norm, K 2^-24 at most as a chain of fp32
+    # multiply-adds keeps
+    gu.ensure_built()
+    gen = torch.Generator(device='cuda'); gen.manual_seed(M + cols)
+    a = torch.randn((K, M) if ta else (M, K), generator=gen, device='cuda')
+    b = torch.randn((N, K) if tb else (K, N), generator=gen, device='cuda')
+    op_a, op_b = (a.T if ta else a), (b.T if tb else b)
+    tiny = torch.arange(N, device='cuda') // cols % 2 == 0
+    op_b[:, tiny] *= scale
+    c = torch.empty(M, N, device='cuda')
+    binding.transmla_conv_gemm(a, b, c, ta=bool(ta), tb=bool(tb))
+    want = op_a.double() @ op_b.double()
+    rel = (c.double() - want).norm(dim=0) / want.norm(dim=0)
+    assert float(rel.max()) < K * 2.0 ** -24, (float(rel[tiny].max()), float(rel[~tiny].max()))
+
+
 @pytest.mark.parametrize('pairs,M,N,K', [(0, 100, 90, 500), (0, 300, 1000, 40), (1, 100, 90, 500), (1, 1000, 700, 300)])
 def test_gemm_that_gives_up_leaves_no_unfinished_sums(pairs, M, N, K):
     # one CTA a tile and CTA pairs, with waits that expire in every CTA; the launch ends normally
