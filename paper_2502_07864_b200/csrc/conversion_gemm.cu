@@ -12,14 +12,18 @@
 // up as well.
 //
 // A CTA pair (cta_group::2) works on a 256 x 256 tile of C, or a single CTA on a 128 x 128 one; either way a CTA converts
-// 128 rows of op(A) and 128 columns of op(B) a chunk.  Eight converting warps read fp32 (whole 128-byte lines whatever the
-// storage order) a chunk ahead, split, and write the terms to a four-stage ring in shared memory - K-major where K is
-// contiguous in memory (64-byte swizzle), MN-major where it is not (128-byte swizzle, 64-wide pieces).  Eight adding warps
-// drain the accumulators (two, in tensor memory), 128 sums a thread.  One warp of the pair's first CTA issues the products.
-// Why two kinds of warps: an accumulator has to be drained while the product behind it runs (1540 cycles).  With all sixteen
-// warps doing both, a finished accumulator waited for the conversion its warp was in, and a chunk took 2730 cycles; now about
-// 1800, of which the converters wait 1100 for a free stage.  What bounds it is the tensor pipe under the power limit: 6 x 240
-// TFLOP/s of bf16 products, which is the rate cuBLAS sustains for seconds, at 1.45 GHz.
+// 128 rows of op(A) and 128 columns of op(B) a chunk.  Converting warps read fp32 (whole 128-byte lines whatever the storage
+// order) ahead, split, and write the terms to a four-stage ring in shared memory - K-major where K is contiguous in memory
+// (64-byte swizzle), MN-major where it is not (128-byte swizzle, 64-wide pieces).  Adding warps drain the accumulators (two, in
+// tensor memory).  One warp of the pair's first CTA issues the products.
+// A pair has eight warps of either kind, 128 sums a thread, a chunk ahead: an accumulator has to be drained while the product
+// behind it runs (1540 cycles), and with all sixteen warps doing both it waited for the conversion its warp was in, 2730 cycles
+// a chunk; now about 1800, of which the converters wait 1100 for a free stage.  What bounds it is the tensor pipe under the
+// power limit: 6 x 240 TFLOP/s of bf16 products, which is the rate cuBLAS sustains for seconds, at 1.45 GHz.
+// A single CTA's product is a quarter of that, and converting bounds its chunks.  Where A's K is not contiguous all sixteen
+// warps do both, two groups of eight taking the chunks in turn, 32 sums a thread; otherwise eight and eight, 64 sums a thread, two
+// chunks ahead.  One kind / two kinds, a single CTA a tile: covariance of 16 x 128 x 128 x 16384 (ta) 564 / 613 us, 512 x 4096 x 8064 (ta) 241 /
+// 250, 128 x 128 x 4096 (ta) 114.7 / 114.7, (tb) 112.6 / 106.5; 1024 x 1024 x 4096 (tb) 114.7 / 109.3; 4096 x 512 x 4096 (tb) 114.7 / 116.7.
 // Rates (fp32 products), before -> now: 8192 x 4096 x 4096 218 -> 241 TFLOP/s, X^T X of 8192 x 8064 370 -> 436 (half of it
 // mirrored), 8064 x 512 x 8064 196 -> 228; the fp32 multiply-add kernel before those reached 48, 50 and 42.
 // (Arrivals that release to the other CTA wait for the thread's loads in flight: none in the converters.  fp32 pieces fetched
@@ -42,14 +46,14 @@ constexpr int kPlane = kRows * kKc * 2;        // 8192 bytes: one term of one op
 constexpr int kStageBytes = 6 * kPlane;
 constexpr int kOffBar = kStages * kStageBytes;
 constexpr int kSmemBytes = kOffBar + 256 + 1024;
-constexpr int kLaunchRegs = 96, kIssuerRegs = 32;
-// A single CTA's adders have half the sums, its converters a second chunk on its way (a pair's wait for stages instead): 16 products of
-// 128 x 128 x 16384 464 us, 509 without (one kind of warp for both jobs: 406, 512 x 4096 x 8064 227 against 239 here).
+constexpr int kLaunchRegs = 96, kIssuerRegs = 32, kBothRegs = 112;
+// A single CTA's converters have a second chunk on its way (a pair's wait for stages instead).
 template <int kCtas>
 struct RegisterSplit {
   static constexpr int kConverter = kCtas == 2 ? 72 : 104, kAdder = kCtas == 2 ? 152 : 120;
   static_assert(kConverters * kConverter + kAdders * kAdder + 128 * kIssuerRegs <= kThreads * kLaunchRegs, "register split");
 };
+static_assert((kConverters + kAdders) * kBothRegs + 128 * kIssuerRegs <= kThreads * kLaunchRegs, "register split, one kind of warp");
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 static_assert(kThreads * kLaunchRegs <= 65536, "registers at launch");
 enum { BAR_FULL = 0, BAR_EMPTY = kStages, BAR_D_FULL = 2 * kStages, BAR_D_FREE = BAR_D_FULL + 2,
@@ -179,6 +183,7 @@ template <int kCtas, bool kAContig, bool kBContig, long long kLimit>
 __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_constant__ GemmArgs args) {
   extern __shared__ unsigned char smem_unaligned[];
   constexpr int kTile = kRows * kCtas;   // tile of C, both ways
+  constexpr bool kOneKind = kCtas == 1 && !kAContig;  // of warps: all sixteen convert and add
   const uint32_t raw = smem_u32(smem_unaligned);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* sm = smem_unaligned + (base - raw);
@@ -207,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
 
   if (tid == 0) {
     for (int i = 0; i < kStages; ++i) { mbar_init(bar(BAR_FULL + i), 8); mbar_init(bar(BAR_EMPTY + i), 1); mbar_init(bar(BAR_FULL2 + i), 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(bar(BAR_D_FULL + i), 1); mbar_init(bar(BAR_D_FREE + i), 8); mbar_init(bar(BAR_D_FREE2 + i), 8); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar(BAR_D_FULL + i), 1); mbar_init(bar(BAR_D_FREE + i), kOneKind ? 16 : 8); mbar_init(bar(BAR_D_FREE2 + i), 8); }
     mbar_init(bar(BAR_LAST), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -277,76 +282,58 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
         __syncwarp();
       }
     }
-  } else if (warp < kConverters / 32) {
-    // ========================================================================== converters
-    constexpr int kRegs = RegisterSplit<kCtas>::kConverter;
-    if constexpr (kRegs < kLaunchRegs) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs));
-    else asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
+  } else {
+    // ========================================================================== converting and adding
     const bool vec_a = (args.lda & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
     const bool vec_b = (args.ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
     const int nb0 = n0 + rank * kRows;                  // this CTA's columns of op(B)
-    constexpr int kAhead = kCtas == 2 ? 1 : 2;          // chunks on their way
-    float xa[kAhead][2][8], xb[kAhead][2][8];           // two pieces of A and two of B a thread and chunk
+    const int ctid = tid & 255;                         // thread of its group of converting warps: two pieces of A and two of B a chunk
+    constexpr int kAhead = kCtas == 2 || kOneKind ? 1 : 2;  // chunks on their way, of a group
+    float xa[kAhead][2][8], xb[kAhead][2][8];
     // Away from the edges a thread's pieces sit at fixed distances from one address per operand.
     const bool inside = vec_a && vec_b && m0 + kRows <= M && nb0 + kRows <= N;
-    const float* next_a = A + (kAContig ? static_cast<size_t>(m0 + (tid >> 2)) * args.lda + (tid & 3) * 8
-                                        : static_cast<size_t>(tid >> 3) * args.lda + m0 + (tid & 7) * 8);
-    const float* next_b = B + (kBContig ? static_cast<size_t>(nb0 + (tid >> 2)) * args.ldb + (tid & 3) * 8
-                                        : static_cast<size_t>(tid >> 3) * args.ldb + nb0 + (tid & 7) * 8);
+    const float* next_a = A + (kAContig ? static_cast<size_t>(m0 + (ctid >> 2)) * args.lda + (ctid & 3) * 8
+                                        : static_cast<size_t>(ctid >> 3) * args.lda + m0 + (ctid & 7) * 8);
+    const float* next_b = B + (kBContig ? static_cast<size_t>(nb0 + (ctid >> 2)) * args.ldb + (ctid & 3) * 8
+                                        : static_cast<size_t>(ctid >> 3) * args.ldb + nb0 + (ctid & 7) * 8);
     auto load8 = [](float (&x)[8], const float* src) {
       const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
       x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
     };
-    auto load = [&](int c, float (&ya)[2][8], float (&yb)[2][8]) {
+    auto load = [&](int c, int s = 0) {
       if (inside && (c + 1) * kKc <= K) {
         const float* a = next_a + (kAContig ? static_cast<size_t>(c) * kKc : static_cast<size_t>(c) * kKc * args.lda);
         const float* b = next_b + (kBContig ? static_cast<size_t>(c) * kKc : static_cast<size_t>(c) * kKc * args.ldb);
-        load8(ya[0], a);
-        load8(ya[1], a + (kAContig ? static_cast<size_t>(64) * args.lda : 64));
-        load8(yb[0], b);
-        load8(yb[1], b + (kBContig ? static_cast<size_t>(64) * args.ldb : 64));
+        load8(xa[s][0], a);
+        load8(xa[s][1], a + (kAContig ? static_cast<size_t>(64) * args.lda : 64));
+        load8(xb[s][0], b);
+        load8(xb[s][1], b + (kBContig ? static_cast<size_t>(64) * args.ldb : 64));
         return;
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        load_group<kAContig>(ya[u], A, vec_a, args.lda, m0, M, c * kKc, K, tid + u * 256);
-        load_group<kBContig>(yb[u], B, vec_b, args.ldb, nb0, N, c * kKc, K, tid + u * 256);
+        load_group<kAContig>(xa[s][u], A, vec_a, args.lda, m0, M, c * kKc, K, ctid + u * 256);
+        load_group<kBContig>(xb[s][u], B, vec_b, args.ldb, nb0, N, c * kKc, K, ctid + u * 256);
       }
     };
+    auto convert = [&](int c, int s = 0) {
+      const int stage = c % kStages;
+      if (c >= kStages) wait(bar(BAR_EMPTY + stage), (c / kStages - 1) & 1);
+      unsigned char* st = sm + stage * kStageBytes;
 #pragma unroll
-    for (int s = 0; s < kAhead; ++s)
-      if (s < chunks) load(s, xa[s], xb[s]);
-    for (int c0 = 0; c0 < chunks; c0 += kAhead) {
-#pragma unroll
-      for (int s = 0; s < kAhead; ++s) {
-        const int c = c0 + s, stage = c % kStages;
-        if (c >= chunks) break;
-        if (c >= kStages) wait(bar(BAR_EMPTY + stage), (c / kStages - 1) & 1);
-        unsigned char* st = sm + stage * kStageBytes;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          store_group<kAContig>(xa[s][u], st, kPlane, tid + u * 256);
-          store_group<kBContig>(xb[s][u], st + 3 * kPlane, kPlane, tid + u * 256);
-        }
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(BAR_FULL + stage));
-        if (c + kAhead < chunks) load(c + kAhead, xa[s], xb[s]);
+      for (int u = 0; u < 2; ++u) {
+        store_group<kAContig>(xa[s][u], st, kPlane, ctid + u * 256);
+        store_group<kBContig>(xb[s][u], st + 3 * kPlane, kPlane, ctid + u * 256);
       }
-    }
-  } else {
-    // ========================================================================== adders
-    constexpr int kRegs = RegisterSplit<kCtas>::kAdder;
-    static_assert(kRegs >= kLaunchRegs, "adders only gain");
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
-    constexpr int kCols = kTile / 2;                    // columns of the tile a thread sums: those of its warp's half
-    const int adder = warp - kConverters / 32, quad = warp & 3, half = adder >> 2;
-    const uint32_t d_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * kCols;
-    float2 acc2[kCols / 2];
-    float* const acc = reinterpret_cast<float*>(acc2);
-#pragma unroll
-    for (int j = 0; j < kCols / 2; ++j) acc2[j] = make_float2(0.f, 0.f);
-    for (int d = 0; d < chunks; ++d) {
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(BAR_FULL + stage));
+    };
+    // Columns of the tile a thread sums: those of its warp's half (of eight warps) or quarter (of sixteen).
+    constexpr int kCols = kTile / (kOneKind ? 4 : 2);
+    const int index = kOneKind ? warp : warp - kConverters / 32, quad = warp & 3, part = index >> 2;
+    const uint32_t d_addr = tmem + (static_cast<uint32_t>(quad * 32) << 16) + part * kCols;
+    auto drain = [&](int d, float (&acc)[kCols]) {
       const int buf = d & 1;
       wait(bar(BAR_D_FULL + buf), (d >> 1) & 1);
       tc_fence_after();
@@ -356,70 +343,122 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
         tmem_ld16(d_addr + buf * kTile + j0, v);
         tc_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 16; j += 2) acc2[(j0 + j) / 2] = add2(acc2[(j0 + j) / 2], v[j], v[j + 1]);
+        for (int j = 0; j < 16; j += 2) {
+          if constexpr (kOneKind) {  // (two at a time there: 2 to 6 % slower)
+            acc[j0 + j] += __uint_as_float(v[j]);
+            acc[j0 + j + 1] += __uint_as_float(v[j + 1]);
+          } else {
+            const float2 sum = add2(make_float2(acc[j0 + j], acc[j0 + j + 1]), v[j], v[j + 1]);
+            acc[j0 + j] = sum.x;
+            acc[j0 + j + 1] = sum.y;
+          }
+        }
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) { if (rank == 0) mbar_arrive(bar(BAR_D_FREE + buf)); else mbar_arrive_first_relaxed(bar(BAR_D_FREE2 + buf)); }
-    }
-
-    // (After a give-up other warps may still be writing terms over these sums' staging place: NaN goes straight to C.)
-    const bool bad = __any_sync(0xffffffffu, *abort_flag != 0);
-    // ---- write-out through shared memory (every product has completed), in whole lines
-    constexpr int kPitch = kCols + 4;
-    float* mine = reinterpret_cast<float*>(sm) + adder * 32 * kPitch;
+    };
+    auto write_out = [&](float (&acc)[kCols]) {
+      // (After a give-up other warps may still be writing terms over these sums' staging place: NaN goes straight to C.)
+      const bool bad = __any_sync(0xffffffffu, *abort_flag != 0);
+      // ---- write-out through shared memory (every product has completed), in whole lines
+      constexpr int kPitch = kCols + 4;
+      float* mine = reinterpret_cast<float*>(sm) + index * 32 * kPitch;
 #pragma unroll
-    for (int j = 0; j < kCols; j += 4)
-      *reinterpret_cast<float4*>(mine + lane * kPitch + j) =
-          make_float4(acc[j] * args.alpha, acc[j + 1] * args.alpha, acc[j + 2] * args.alpha, acc[j + 3] * args.alpha);
-    // Where the split does not hold the sum is taken once more, by fp32 multiply-adds: an infinite or too large operand value
-    // has no exact terms and made its sums NaN, and operands so small that all sums of a region (32 rows x a quarter of the
-    // tile's columns) stay below 2^-63 may have lost their last terms.
-    constexpr int kRegion = kTile / 4;
-    uint32_t small = 0, odd = 0;                        // bits of the warp's regions
+      for (int j = 0; j < kCols; j += 4)
+        *reinterpret_cast<float4*>(mine + lane * kPitch + j) =
+            make_float4(acc[j] * args.alpha, acc[j + 1] * args.alpha, acc[j + 2] * args.alpha, acc[j + 3] * args.alpha);
+      // Where the split does not hold the sum is taken once more, by fp32 multiply-adds: an infinite or too large operand value
+      // has no exact terms and made its sums NaN, and operands so small that all sums of a region (32 rows x a quarter of the
+      // tile's columns) stay below 2^-63 may have lost their last terms.
+      constexpr int kRegion = kTile / 4;
+      constexpr int kRegions = kCols / kRegion;
+      float size[kRegions][4 / kRegions] = {}, all = 0.f;
 #pragma unroll
-    for (int g = 0; g < kCols / kRegion; ++g) {
-      float size[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int j = 0; j < kCols; ++j) size[j / kRegion][j % (4 / kRegions)] += fabsf(acc[j]);
+      uint32_t small = 0;                               // bits of the warp's regions
 #pragma unroll
-      for (int j = 0; j < kRegion; ++j) size[j & 3] += fabsf(acc[g * kRegion + j]);
-      const float all = (size[0] + size[1]) + (size[2] + size[3]);
-      if (__all_sync(0xffffffffu, all < 0x1p-63f) && __any_sync(0xffffffffu, all > 0.f)) small |= 1u << g;
-      if (__any_sync(0xffffffffu, !(all < INFINITY))) odd |= 1u << g;
-    }
-    if ((small | odd) != 0) {
+      for (int g = 0; g < kRegions; ++g) {
+        float region = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4 / kRegions; ++i) region += size[g][i];
+        if (__all_sync(0xffffffffu, region < 0x1p-63f) && __any_sync(0xffffffffu, region > 0.f)) small |= 1u << g;
+        all += region;
+      }
+      if (small != 0 || __any_sync(0xffffffffu, !(all < INFINITY))) {
 #pragma unroll 1
-      for (int j = 0; j < kCols; ++j) {
-        const int m = m0 + quad * 32 + lane, n = n0 + half * kCols + j;
-        if (m < M && n < N && ((small >> (j / kRegion) & 1u) || !isfinite(mine[lane * kPitch + j])))
-          mine[lane * kPitch + j] = args.alpha * plain_sum<kAContig, kBContig>(args, m, n);
+        for (int j = 0; j < kCols; ++j) {
+          const int m = m0 + quad * 32 + lane, n = n0 + part * kCols + j;
+          if (m < M && n < N && ((small >> (j / kRegion) & 1u) || !isfinite(mine[lane * kPitch + j])))
+            mine[lane * kPitch + j] = args.alpha * plain_sum<kAContig, kBContig>(args, m, n);
+        }
       }
-    }
-    __syncwarp();
-    float* C = args.C + args.stride_c * blockIdx.y;
-    const int mw = m0 + quad * 32, nw = n0 + half * kCols;
-    const bool whole = !bad && !args.symmetric && n0 + kTile <= N && (args.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
-    if (whole) {  // 16 bytes a lane
-      constexpr int kLanes = kCols / 4, kAtOnce = 32 / kLanes;   // of a row; rows
-      const int j = lane % kLanes * 4;
+      __syncwarp();
+      float* C = args.C + args.stride_c * blockIdx.y;
+      const int mw = m0 + quad * 32, nw = n0 + part * kCols;
+      const bool whole = !bad && !args.symmetric && n0 + kTile <= N && (args.ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+      if (whole) {  // 16 bytes a lane
+        constexpr int kLanes = kCols / 4, kAtOnce = 32 / kLanes;   // of a row; rows
+        const int j = lane % kLanes * 4;
 #pragma unroll 4
-      for (int r = lane / kLanes; r < 32; r += kAtOnce)
-        if (mw + r < M) *reinterpret_cast<float4*>(C + static_cast<size_t>(mw + r) * args.ldc + nw + j) = *reinterpret_cast<const float4*>(mine + r * kPitch + j);
-    }
-    for (int r = 0; r < 32 && !whole; ++r) {
-      const int m = mw + r;
-      if (m >= M) break;
+        for (int r = lane / kLanes; r < 32; r += kAtOnce)
+          if (mw + r < M) *reinterpret_cast<float4*>(C + static_cast<size_t>(mw + r) * args.ldc + nw + j) = *reinterpret_cast<const float4*>(mine + r * kPitch + j);
+      }
+      for (int r = 0; r < 32 && !whole; ++r) {
+        const int m = mw + r;
+        if (m >= M) break;
 #pragma unroll
-      for (int j = lane; j < kCols; j += 32) {
-        const int n = nw + j;
-        if (n < N && (!args.symmetric || n <= m)) C[static_cast<size_t>(m) * args.ldc + n] = bad ? __int_as_float(0x7fffffff) : mine[r * kPitch + j];
+        for (int j = lane; j < kCols; j += 32) {
+          const int n = nw + j;
+          if (n < N && (!args.symmetric || n <= m)) C[static_cast<size_t>(m) * args.ldc + n] = bad ? __int_as_float(0x7fffffff) : mine[r * kPitch + j];
+        }
       }
-    }
-    if (args.symmetric) {
-      const int m = mw + lane;
-      for (int j = 0; j < kCols; ++j) {
-        const int n = nw + j;
-        if (n < m && m < M) C[static_cast<size_t>(n) * args.ldc + m] = bad ? __int_as_float(0x7fffffff) : mine[lane * kPitch + j];
+      if (args.symmetric) {
+        const int m = mw + lane;
+        for (int j = 0; j < kCols; ++j) {
+          const int n = nw + j;
+          if (n < m && m < M) C[static_cast<size_t>(n) * args.ldc + m] = bad ? __int_as_float(0x7fffffff) : mine[lane * kPitch + j];
+        }
       }
+    };
+    if constexpr (kOneKind) {
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kBothRegs));
+      float acc[kCols];
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) acc[j] = 0.f;
+      const int group = warp >> 3;  // two groups of eight warps take the chunks in turn
+      int drained = 0;
+      if (group < chunks) load(group);
+      for (int c = group; c < chunks; c += 2) {
+        convert(c);
+        if (c + 2 < chunks) load(c + 2);
+        while (drained + 2 <= c) drain(drained++, acc);
+      }
+      while (drained < chunks) drain(drained++, acc);
+      write_out(acc);
+    } else if (warp < kConverters / 32) {
+      constexpr int kRegs = RegisterSplit<kCtas>::kConverter;
+      if constexpr (kRegs < kLaunchRegs) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs));
+      else asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
+#pragma unroll
+      for (int s = 0; s < kAhead; ++s)
+        if (s < chunks) load(s, s);
+      for (int c0 = 0; c0 < chunks; c0 += kAhead) {
+#pragma unroll
+        for (int s = 0; s < kAhead; ++s) {
+          const int c = c0 + s;
+          if (c >= chunks) break;
+          convert(c, s);
+          if (c + kAhead < chunks) load(c + kAhead, s);
+        }
+      }
+    } else {
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(RegisterSplit<kCtas>::kAdder));
+      float acc[kCols];
+#pragma unroll
+      for (int j = 0; j < kCols; ++j) acc[j] = 0.f;
+      for (int d = 0; d < chunks; ++d) drain(d, acc);
+      write_out(acc);
     }
   }
   tc_fence_before();
@@ -515,8 +554,10 @@ cudaError_t launch_size(GemmArgs args, int batch, cudaStream_t stream) {
     gemm_short_kernel<kAContig, kBContig><<<dim3(static_cast<unsigned>(tiles), batch), 256, 0, stream>>>(args);
     return cudaGetLastError();
   }
-  // A pair's chunk takes about 8/7 of a single CTA's and does four times the work with two CTAs; the single one pays where
-  // it fills the device better.
+  // A pair does four times the work of a single CTA with two CTAs; the single one pays where it fills the device better.  Single
+  // CTAs / pairs, K = 2048, orders tb, ta, none: 2 waves of either (2700 x 1600) 132 / 148, 139 / 153, 138 / 152 us; 5 waves against 4 (30000
+  // x 301) 328 / 348, 369 / 358, 393 / 361; 4 against 3 (13000 x 520) 253 / 248, 261 / 243, 266 / 236; 3 against 2 (3100 x 1600) 181 / 152, 195 / 154,
+  // 185 / 154; 2 against 1 (2048 x 2048, K = 4096) 235 / 158.  So the line lies between 1 and 1.25.
   constexpr long long kSms = 148;
   auto waves = [&](int tile, long long at_once) {
     const long long tm = (args.M + tile - 1) / tile, tn = (args.N + tile - 1) / tile;
