@@ -316,6 +316,11 @@ transmla_status_t transmla_selftest_step_gives_up(const transmla_params_t* param
                                                   const void* w_dkv_kr, const void* w_uk, const void* w_uv, void* cache,
                                                   void* workspace, size_t workspace_bytes, void* out, int32_t* dev_status, void* stream);
 
+/* Diagnostic: the inverse square root of the Cholesky factor's pivots on device doubles d [n]: out [n][3] = its value, CUDA's
+ * rsqrt and the hardware approximation it begins with.  TRANSMLA_DEV_NUMERIC in *dev_status (required) where a d is not
+ * positive (its value is then that of 1). */
+transmla_status_t transmla_selftest_conv_inverse_root(const double* d, int n, double* out, int32_t* dev_status, void* stream);
+
 /* Diagnostic: transmla_conv_top_subspace with the cluster of its Cholesky factor limited to most_ctas CTAs (1, 2, 4, 8 or
  * 16), as on a device or partition that holds no larger one. */
 transmla_status_t transmla_selftest_conv_subspace(const float* Cmat, int m, int r, int iters, float* Q, void* scratch,

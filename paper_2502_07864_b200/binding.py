@@ -16,6 +16,7 @@ EXPORTS = ('transmla_workspace_layout', 'transmla_latent_append', 'transmla_mla_
            'transmla_decode_step', 'transmla_profile_decode_kernel', 'transmla_status_string',
            'transmla_static_workspace_capacity', 'transmla_mla_attention_static', 'transmla_selftest_bounded_wait',
            'transmla_selftest_conv_gemm', 'transmla_selftest_conv_subspace', 'transmla_selftest_step_gives_up',
+           'transmla_selftest_conv_inverse_root',
            'transmla_layer_scratch_bytes', 'transmla_layer_decode_step', 'transmla_stream_probe', 'transmla_page_claims_at_run_time', 'transmla_latent_append_fp8',
            'transmla_mla_decode_fp8', 'transmla_prefill_scratch_bytes', 'transmla_prefill_decompress',
            'transmla_prefill_attention', 'transmla_mla_prefill', 'transmla_conv_gemm',
@@ -91,6 +92,7 @@ def lib():
         ci, cf = ctypes.c_int, ctypes.c_float
         L.transmla_conv_gemm.argtypes = [ci, ci, ci, ci, ci, cf, vp, ci, vp, ci, vp, ci, vp]
         L.transmla_selftest_conv_subspace.argtypes = [vp, ci, ci, ci, vp, vp, sz, ci, i32p, vp]
+        L.transmla_selftest_conv_inverse_root.argtypes = [vp, ci, vp, i32p, vp]
         L.transmla_selftest_conv_gemm.argtypes = [ci, ci, ci, ci, vp, vp, vp, i32p, vp]
         L.transmla_conv_rorope_scratch_bytes.argtypes = [ci, ci, ci, ci]
         L.transmla_conv_rorope_scratch_bytes.restype = sz
@@ -258,6 +260,11 @@ def transmla_selftest_conv_subspace(cmat, q, iters, scratch, most_ctas, dev_stat
     m, r = q.shape
     _check(lib().transmla_selftest_conv_subspace(_ptr(cmat), m, r, iters, _ptr(q), _ptr(scratch), _nbytes(scratch), int(most_ctas),
                                                  _ptr(dev_status), _stream(stream)), 'transmla_selftest_conv_subspace')
+
+
+def transmla_selftest_conv_inverse_root(d, out, dev_status, stream=None):
+    _check(lib().transmla_selftest_conv_inverse_root(_ptr(d), d.numel(), _ptr(out), _ptr(dev_status), _stream(stream)),
+           'transmla_selftest_conv_inverse_root')
 
 
 def transmla_latent_append_fp8(params, x, w_dkv_kr, positions, page_table, cache_fp8, scratch, dev_status=None, stream=None):

@@ -40,5 +40,8 @@ cudaError_t cholesky_qr(const float* Y, int m, int r, double* partial, double* G
 cudaError_t cholesky_qr_last(float* Q, int m, int r, double* partial, double* G, double* X, float* X32, float* P,
                              int32_t* dev_status, cudaStream_t stream, int most_ctas = kOrthCluster);
 
+// For a test: out [n][3] = the factor's 1 / sqrt(d), CUDA's rsqrt(d), the approximation that the first begins with.
+cudaError_t inverse_roots(const double* d, int n, double* out, int32_t* dev_status, cudaStream_t stream);
+
 }  // namespace conv
 }  // namespace transmla

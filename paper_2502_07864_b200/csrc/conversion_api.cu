@@ -127,6 +127,12 @@ transmla_status_t transmla_conv_top_subspace(const float* Cmat, int m, int r, in
   return top_subspace(Cmat, m, r, iters, Q, scratch, scratch_bytes, conv::kOrthCluster, dev_status, stream);
 }
 
+transmla_status_t transmla_selftest_conv_inverse_root(const double* d, int n, double* out, int32_t* dev_status, void* stream) {
+  if (!d || !out || !dev_status) return TRANSMLA_ERR_NULL;
+  if (n < 1) return TRANSMLA_ERR_SHAPE;
+  return done(conv::inverse_roots(d, n, out, dev_status, static_cast<cudaStream_t>(stream)));
+}
+
 transmla_status_t transmla_selftest_conv_subspace(const float* Cmat, int m, int r, int iters, float* Q, void* scratch,
                                                   size_t scratch_bytes, int most_ctas, int32_t* dev_status, void* stream) {
   if (most_ctas < 1 || most_ctas > conv::kOrthCluster || (most_ctas & (most_ctas - 1))) return TRANSMLA_ERR_SHAPE;

@@ -318,6 +318,49 @@ def test_the_basis_is_orthonormal_to_one_rounding_an_element(m, r):
     assert int(status.item()) == 0 and np.abs(q.T @ q - np.eye(r)).max() < 2.0 ** -23
 
 
+def test_inverse_root_of_the_factor_over_all_exponents():
+    # The result's roundings: d y by 2^-53, e by 2^-54 more, half of which reaches the result, and the last one 2^-53; the method
+    # leaves 5/16 e^3, which an approximation to 2^-18 would bring to 2^-52.7 and the one there is (2^-20) to 2^-58.
+    gu.ensure_built()
+    rng = np.random.default_rng(95)
+    mant = np.concatenate([[1.0, np.nextafter(1, 2), np.nextafter(2, 1), 1.5], 1 + rng.random(60)])
+    d = np.ldexp(mant[None, :], np.arange(-1022, 1024)[:, None]).ravel()
+    out = torch.empty(d.size, 3, dtype=torch.float64, device='cuda')
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    binding.transmla_selftest_conv_inverse_root(torch.tensor(d, device='cuda'), out, status)
+    got = out.cpu().numpy().astype(np.longdouble)
+    off = np.abs(got * np.sqrt(d.astype(np.longdouble))[:, None] - 1).max(axis=0)
+    assert int(status.item()) == 0
+    assert off[0] <= 2.0 ** -52 and off[1] <= 2.0 ** -52 and off[2] <= 2.0 ** -20, np.log2(off.astype(np.float64))
+    for bad in (0.0, -0.0, -1.0, np.nan, -np.inf):
+        status.zero_()
+        binding.transmla_selftest_conv_inverse_root(torch.tensor([bad], dtype=torch.float64, device='cuda'), out, status)
+        assert int(status.item()) == 8 and float(out[0, 0]) == 1.0, bad       # TRANSMLA_DEV_NUMERIC
+    binding.transmla_selftest_conv_inverse_root(torch.tensor([np.inf], dtype=torch.float64, device='cuda'), out, status)
+    assert not np.isfinite(float(out[0, 0]))                                  # which the next pivot or pass reports
+
+
+@pytest.mark.parametrize('m,r', [(100, 1), (200, 33), (200, 64), (300, 70), (600, 301), (1100, 1024)])
+@pytest.mark.parametrize('what', [0.0, float('nan'), float('inf')])
+def test_a_basis_without_full_rank_is_reported(m, r, what):
+    # a column of zeros, and one value that is not finite, in the first column, inside a step of four and in the last column
+    gu.ensure_built()
+    rng = np.random.default_rng(96)
+    x = rng.standard_normal((2 * m, m))
+    C, q0 = _dev(x.T @ x), _dev(rng.standard_normal((m, r)))
+    scratch = torch.empty(binding.transmla_conv_subspace_scratch_bytes(m, r), dtype=torch.uint8, device='cuda')
+    status = torch.zeros(1, dtype=torch.int32, device='cuda')
+    for column in sorted({0, r // 2, r - 1}):
+        q = q0.clone()
+        q[slice(None) if what == 0.0 else 5, column] = what
+        status.zero_()
+        binding.transmla_conv_top_subspace(C, q, 1, scratch, status)
+        assert int(status.item()) & 8, column                                 # TRANSMLA_DEV_NUMERIC
+    status.zero_()
+    binding.transmla_conv_top_subspace(C, q0, 1, scratch, status)
+    assert int(status.item()) == 0 and bool(torch.isfinite(q0).all())
+
+
 def test_whole_conversion_step_by_step_against_the_oracle():
     # activations -> per-group covariances -> rotations -> rotated W_K -> alpha -> joint second moment -> basis -> rewrite
     gu.ensure_built()
