@@ -11,7 +11,7 @@ l = G*M .. G*M+M-1; within a group the segment index of (frequency p = l - G*M, 
 After the rotation, component q of group G is stored at head q // M, frequency G*M + q % M, so that the
 M strongest components of every group land in head 0 - the head that keeps RoPE.
 
-Readings where the paper leaves room (all listed in the design doc): the covariance is the plain second
+Readings where the paper leaves room: the covariance is the plain second
 moment K^T K (App. B writes sigma = K^T K with no centring); with FreqFold the real parts of all M
 frequencies of a group rotate together, and the imaginary parts by the same matrix (App. B's
 constraint carried over to App. C's concatenated segments); alpha is a ratio of mean L2 norms

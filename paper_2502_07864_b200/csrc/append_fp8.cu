@@ -1,6 +1,6 @@
 // Latent append into the FP8 cache (Eq. 7 left, then this library's FP8 row format): the projection and RoPE run as in
 // the bf16 append but leave fp32 rows in a scratch buffer, because a row's scale is the maximum over all of its 512
-// latent values, which 64 different blocks of the projection produce; a second, tiny launch quantises the rows.
+// latent values, which eight feature tiles of the projection produce; a second, tiny launch quantises the rows.
 #include <cuda_fp16.h>
 
 #include "common.cuh"

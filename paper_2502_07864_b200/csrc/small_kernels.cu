@@ -367,7 +367,9 @@ __global__ void __launch_bounds__(256, kPrefetch ? 1 : 2) combine_kernel(const i
   const bool dense = T >= G;  // then every partition owns at least one slot (of G at most)
   const int32_t* seq_parts = cum + B + 1;  // only 4-byte aligned: B + 1 may be odd
 
-  // (The merge is merge_rows of combine.cuh written out: called from here the step of 16 x 8192 tokens took 47.7 us instead of 46.9.)
+  // (The merge is merge_rows of combine.cuh written out, and what changes in one changes in both.  As one routine, with the sums handed
+  // back or taken by a callback, the compiler's schedule costs 2 to 10 % of the launch: the step of 16 x 8192 45.7 -> 46.0 and 46.1 us, of 32
+  // ragged sequences 127.2 -> 128.9 and 128.5.)
 #pragma unroll 1
   for (int r0 = warp / kWarpsPerRow; r0 < kRows; r0 += 8 * kAtOnce) {
     const int c0 = kWarpsPerRow > 1 ? warp % kWarpsPerRow * (kChunks * 128) + lane * 4 : lane * 4;  // the lane's first latent
@@ -542,16 +544,17 @@ cudaError_t launch_combine(const transmla_params_t& p, int G, const int32_t* cum
     return launch_pdl(kernel, dim3(H, (BS + rows - 1) / rows, halves), dim3(256), smem, stream, cum, plan, partial_o, partial_lse, w_uv,
                       out, lse_out, p.batch, p.q_len, H, p.kv_lora_rank, p.v_dim, G);
   };
-  // Up to one wave of blocks.  Two halves of dv a row where that leaves room: a block then reads half of W_UV_h, which is what
-  // is left to wait for where the merge is short.  Four rows a block merge sooner than eight while two halves of them fit;
-  // beyond that eight rows and halves instead of four rows and all of dv.  The step of 32 heads, dv = 128, at 9 / 12 / 16
-  // sequences of 1000: 25.6 / 26.2 / 24.6 us -> 22.6 / 22.8 / 23.7; of 300: 25.0 / 25.6 / 27.3 -> 24.4 / 25.3 / 26.1; of 8192: 32.8 / 36.7 /
-  // 42.0 -> 33.5 / 36.6 / 42.1; 64 heads at 6 of 300 and 8192: 26.0 and 34.4 -> 24.6 and 34.3.  With dv <= 64 a warp has one tile of columns
-  // as it is, and few rows leave more SMs to the launches either side: dv = 64, append + decode + combine of 4 sequences of
-  // 100 27.8 us (4 rows, all of dv), 26.7 (halves), 25.2.
+  // Up to one wave of blocks.  Four rows a block, two warps a row, merge sooner than eight; two halves of dv read half of W_UV_h each,
+  // which is what is left to wait for where the merge is short.  Both while twice the blocks of four fit; beyond that eight rows and
+  // halves where a row has few partials, otherwise four rows and all of dv.  The step of 32 heads, dv = 128, 4 rows / 8 rows: 9
+  // sequences (at most G / batch = 4, 8, 16, 16 partials) of 1000 25.3 / 22.4 us, 2000 23.4 / 23.2, 4000 25.6 / 26.1, 16384 44.4 / 45.1; 13 (3, 11) of 300
+  // 26.6 / 25.1, 16384 55.0 / 55.0; 16 (9) of 8192 46.5 / 45.8; S = 2, 5 sequences (4, 30) of 1000 25.4 / 22.5, 16384 39.3 / 41.1; 64 heads, 8 of 300 (1)
+  // 26.7 / 25.4, 40000 (18) 77.1 / 77.8.  (The table's room stands for the lengths: with room for 128K 9 x 300 takes 23.2 where 8 rows
+  // would take 21.6.)  With dv <= 64 a warp has one tile of columns as it is, and few rows leave more SMs to the launches either
+  // side: dv = 64, append + decode + combine of 4 sequences of 100 27.8 us (4 rows, all of dv), 26.7 (halves), 25.2.
   if (p.v_dim >= 128 && 2 * blocks(4) <= kSms) return launch(combine_kernel<4, 1, true>, 4, 2);
   if (p.v_dim <= 64 && BS <= 32 && blocks(8) <= kSms) return launch(combine_kernel<8, 1, true>, 8, 1);
-  if (2 * blocks(8) <= kSms) return launch(combine_kernel<8, 1, true>, 8, 2);
+  if (2 * blocks(8) <= kSms && (G <= 12LL * p.batch || blocks(4) > kSms)) return launch(combine_kernel<8, 1, true>, 8, 2);
   if (blocks(4) <= kSms) return launch(combine_kernel<4, 2, true>, 4, 1);
   if (blocks(8) <= kSms) return launch(combine_kernel<8, 2, true>, 8, 1);
   if (combine_sm100_supported(p)) return launch_combine_sm100(p, G, cum, plan, partial_o, partial_lse, w_uv, out, lse_out, dev_status, stream);
