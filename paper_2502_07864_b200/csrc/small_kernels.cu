@@ -229,9 +229,11 @@ int append_token_splits(const transmla_params_t& p) {
 // r = 64, dR = 16, D = 256 1 sequence 14.0 / 15.2 us, 16 (64 heads) 16.6 / 19.0, 64 18.0 to 23.2 / 19.3 to 25.3; the same with D = 4096 16
 // 20.6 / 21.9, 64 27.7 / 21.2; r = 512, dR = 64, dn = 64 1 20.6 / 22.2, 16 22.2 / 24.6, 160 46.1 / 39.5 and (64 heads) 75.4 / 69.8.  With
 // r = 128, dR = 0 blocks of 32 features x 16 tokens are as many as clusters have CTAs: 16 19.1 / 22.2, 64 22.5 / 22.9, 160 23.8 / 26.3.
-// (The two forms add a value's products in other orders, both in fp32.)
-static bool append_in_clusters(const transmla_params_t& p) {
-  return p.batch * p.q_len > 32 && (p.kv_lora_rank + p.qk_rope_dim) % 128 != 0;
+// The append by itself with r = 512 (wide blocks), alone and in append + decode + combine of 100 cached tokens: 64 6.4 / 8.3 and 40.4 / 41.1 us, 128
+// 6.8 / 10.0 and 44.8 / 46.4, 256 13.3 / 16.6, 512 26.1 / 25.6.  (The two forms add a value's products in other orders, both in fp32.)
+static bool append_in_clusters(const transmla_params_t& p, bool alone) {
+  const int K = p.kv_lora_rank + p.qk_rope_dim;
+  return p.batch * p.q_len > (alone && K % 32 == 0 ? 256 : 32) && K % 128 != 0;
 }
 
 cudaError_t launch_append(const transmla_params_t& p, const __nv_bfloat16* x, const __nv_bfloat16* w,
@@ -240,7 +242,7 @@ cudaError_t launch_append(const transmla_params_t& p, const __nv_bfloat16* x, co
   const int K = p.kv_lora_rank + p.qk_rope_dim;
   if (prologue_sm100_supported(p))
     return launch_append_sm100(p, x, w, positions, page_table, cache, nullptr, dev_status, stream);
-  if (append_in_clusters(p)) {
+  if (append_in_clusters(p, true)) {
     static PerDeviceFlag smem_set;
     if (cudaError_t e = ensure_dynamic_smem(append_cluster_kernel, static_cast<int>(kSliceSmem), smem_set); e != cudaSuccess) return e;
     return launch_slices(append_cluster_kernel, append_clusters(p) * kSliceCtas, kSliceSmem, stream, x, w, positions, page_table, cache,
@@ -282,7 +284,7 @@ cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& part
                             cudaStream_t stream) {
   if (prologue_sm100_supported(p))
     return launch_absorb_sm100(p, parts, x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan, dev_status, stream);
-  const bool clusters = append_in_clusters(p);
+  const bool clusters = append_in_clusters(p, false);
   const int ts = append_token_splits(p), wide = append_wide(p) ? 1 : 0;
   const int n_append = clusters ? append_clusters(p) : (p.kv_lora_rank + p.qk_rope_dim) / (wide ? 32 : 8) * ts;
   const int nt = clusters ? 1 : absorb_tiles_per_block(p, 1 + n_append);

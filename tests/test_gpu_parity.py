@@ -356,7 +356,11 @@ def test_waits_that_give_up_around_the_attention_leave_no_unfinished_values(shap
 @pytest.mark.parametrize('shape,positions', [(synth.TINY, [16, 63, 64, 0]), (synth.LLAMA2_7B, [8191, 0, 77, 131071]),
                                              (synth.QWEN25_72B, [126, 63, 4000]),
                                              (synth.TINY, [(7 * i) % 200 for i in range(150)]),       # several token splits
-                                             (synth.LLAMA2_7B, [(64 * i + i) % 700 for i in range(70)])])
+                                             (synth.LLAMA2_7B, [(64 * i + i) % 700 for i in range(70)]),
+                                             # blocks of 32 features x 16 tokens, and the clusters beyond them, D / 8 in pieces of 128
+                                             (dataclasses.replace(synth.LLAMA2_7B, dn=64), [(64 * i + i) % 300 for i in range(70)]),
+                                             (dataclasses.replace(synth.LLAMA2_7B, dn=64, D=1280), [(7 * i) % 200 for i in range(257)]),
+                                             (synth.MLAShape(H=8, dn=32, dR=16, dv=32, r=64, D=4352), [(7 * i) % 200 for i in range(65)])])
 def test_append_values_slots_and_untouched_bytes(shape, positions):
     B, S, P = len(positions), shape.S, shape.page_size
     seqlens = [p + S for p in positions]
