@@ -32,15 +32,17 @@ __device__ __forceinline__ int kperm(int p) { return ((p & 7) >> 1) * 8 + (p >> 
 // ------------------------------------------------------------------------------------------------
 constexpr int kAbsorbRows = 128;  // query rows staged per pass
 
-__device__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q_pe,
+template <int nt>
+__device__ __forceinline__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q_pe,
                              const __nv_bfloat16* __restrict__ w_uk, __nv_bfloat16* q_hat, int BS, int H,
-                             int dn, int dR, int r, int h, int rt0, int nt, unsigned char* smem_raw) {
-  const int apitch = dn + 8, wpitch = nt * 128 + 8;
+                             int dn, int dR, int r, int h, int rt0, unsigned char* smem_raw) {
+  constexpr int wpitch = nt * 128 + 8, vec_per_row = nt * 16;
+  const int apitch = dn + 8;
   __nv_bfloat16* w_s = reinterpret_cast<__nv_bfloat16*>(smem_raw);  // [dn][wpitch]
   __nv_bfloat16* a_s = w_s + dn * wpitch;                            // [kAbsorbRows][dn + 8]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
-  const int n0 = rt0 * 128, K = r + dR, vec_per_row = nt * 16;
+  const int n0 = rt0 * 128, K = r + dR;
   for (int i = tid; i < dn * vec_per_row; i += 256) {  // columns beyond r are zero-filled
     const int k = i / vec_per_row, c = i % vec_per_row;
     const bool in = n0 + c * 8 < r;
@@ -89,6 +91,7 @@ __device__ void absorb_block(const __nv_bfloat16* q_nope, const __nv_bfloat16* q
     cp_async_wait<0>();
     __syncthreads();
     for (int m0 = 0; m0 < rows16; m0 += 16) {
+#pragma unroll 1
       for (int wc = warp * 16 * nt; wc < (warp + 1) * 16 * nt; wc += 16) {  // this warp's 16-column steps
         float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll 4
@@ -164,19 +167,20 @@ __global__ void __launch_bounds__(256) append_kernel(const __nv_bfloat16* x,
 }
 
 // Absorb blocks followed by one plan block: everything transmla_mla_decode needs before the split-KV kernel.
+template <int nt>
 __global__ void __launch_bounds__(256) absorb_plan_kernel(const __nv_bfloat16* q_nope,
                                                           const __nv_bfloat16* q_pe,
                                                           const __nv_bfloat16* __restrict__ w_uk,
                                                           __nv_bfloat16* q_hat,
                                                           const int32_t* seqlens, int32_t* cum,
                                                           int32_t* plan, int32_t* dev_status, int B, int S, int H,
-                                                          int dn, int dR, int r, Partitioning parts, int max_pages, int nt) {
+                                                          int dn, int dR, int r, Partitioning parts, int max_pages) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
   const int per_head = (r + 127) / 128 / nt;  // absorb blocks per head, nt tiles each
   const int n_absorb = H * per_head;
   if (static_cast<int>(blockIdx.x) < n_absorb) {
-    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, blockIdx.x / per_head, blockIdx.x % per_head * nt, nt, smem_raw);
+    absorb_block<nt>(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, blockIdx.x / per_head, blockIdx.x % per_head * nt, smem_raw);
   } else {
     plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
   }
@@ -184,13 +188,13 @@ __global__ void __launch_bounds__(256) absorb_plan_kernel(const __nv_bfloat16* q
 
 // The whole prologue of a decode step in one launch: append clusters or blocks, plan block, absorb blocks.
 // The appended token of sequence b sits at seqlens[b] - S + s.  n_append: clusters, or blocks of t_splits token splits.
-template <bool kClusters>
+template <bool kClusters, int nt>
 __global__ void __launch_bounds__(256, kClusters ? 2 : 1) prologue_kernel(
     const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w_dkv_kr,
     const int32_t* page_table, __nv_bfloat16* cache, const __nv_bfloat16* q_nope,
     const __nv_bfloat16* q_pe, const __nv_bfloat16* __restrict__ w_uk, __nv_bfloat16* q_hat,
     const int32_t* seqlens, int32_t* cum, int32_t* plan, int32_t* dev_status, int B, int S, int H, int D,
-    int dn, int dR, int r, int num_pages, int max_pages, float theta, Partitioning parts, int n_append, int t_splits, int wide, int nt) {
+    int dn, int dR, int r, int num_pages, int max_pages, float theta, Partitioning parts, int n_append, int t_splits, int wide) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_trigger();
   const int per_head = (r + 127) / 128 / nt;  // absorb blocks per head, nt tiles each
@@ -208,7 +212,7 @@ __global__ void __launch_bounds__(256, kClusters ? 2 : 1) prologue_kernel(
   } else if (bid == 0) {
     plan_block(seqlens, B, parts, (S * H + kRowBlock - 1) / kRowBlock, max_pages, cum, plan, dev_status, smem_raw);
   } else if (bid <= H * per_head) {  // (a grid of clusters is whole: a few blocks at its end have nothing to do)
-    absorb_block(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, (bid - 1) / per_head, (bid - 1) % per_head * nt, nt, smem_raw);
+    absorb_block<nt>(q_nope, q_pe, w_uk, q_hat, B * S, H, dn, dR, r, (bid - 1) / per_head, (bid - 1) % per_head * nt, smem_raw);
   }
 }
 
@@ -269,12 +273,13 @@ cudaError_t launch_absorb_plan(const transmla_params_t& p, const Partitioning& p
   const int nt = sm100 ? 1 : absorb_tiles_per_block(p, 1);
   size_t smem = absorb_smem(p.qk_nope_dim, nt);
   if (smem < kPlanSmemSeqs * sizeof(int32_t)) smem = kPlanSmemSeqs * sizeof(int32_t);
-  static PerDeviceFlag smem_set;  // zero-initialised; one slot per device
-  if (cudaError_t e = ensure_dynamic_smem(absorb_plan_kernel, kPrologueMaxSmem, smem_set); e != cudaSuccess) return e;
+  static PerDeviceFlag smem_set[2];  // zero-initialised; one slot per device
+  auto kernel = nt == 2 ? absorb_plan_kernel<2> : absorb_plan_kernel<1>;
+  if (cudaError_t e = ensure_dynamic_smem(kernel, kPrologueMaxSmem, smem_set[nt - 1]); e != cudaSuccess) return e;
   const int blocks = p.num_heads * ((p.kv_lora_rank + 127) / 128 / nt) + 1;
-  return launch_pdl(absorb_plan_kernel, dim3(blocks), dim3(256), smem, stream, q_nope, q_pe, w_uk, q_hat, seqlens, cum,
+  return launch_pdl(kernel, dim3(blocks), dim3(256), smem, stream, q_nope, q_pe, w_uk, q_hat, seqlens, cum,
                     plan, dev_status, p.batch, p.q_len, p.num_heads, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, parts,
-                    p.max_pages_per_seq, nt);
+                    p.max_pages_per_seq);
 }
 
 cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& parts, const __nv_bfloat16* x, const __nv_bfloat16* w_dkv_kr,
@@ -292,18 +297,17 @@ cudaError_t launch_prologue(const transmla_params_t& p, const Partitioning& part
   const size_t smem_append = clusters ? kSliceSmem : kAppendSmem;
   size_t smem = absorb_smem(p.qk_nope_dim, nt);
   if (smem < smem_append) smem = smem_append;
-  static PerDeviceFlag smem_set[2];  // zero-initialised; one slot per device
-  if (cudaError_t e = ensure_dynamic_smem(clusters ? prologue_kernel<true> : prologue_kernel<false>, kPrologueMaxSmem, smem_set[clusters]); e != cudaSuccess) return e;
+  static PerDeviceFlag smem_set[3];  // zero-initialised; one slot per device
+  auto kernel = clusters ? prologue_kernel<true, 1> : nt == 2 ? prologue_kernel<false, 2> : prologue_kernel<false, 1>;
+  if (cudaError_t e = ensure_dynamic_smem(kernel, kPrologueMaxSmem, smem_set[clusters ? 2 : nt - 1]); e != cudaSuccess) return e;
   auto with_args = [&](auto launch) {
     return launch(x, w_dkv_kr, page_table, cache, q_nope, q_pe, w_uk, q_hat, seqlens, cum, plan, dev_status, p.batch, p.q_len,
                   p.num_heads, p.hidden_dim, p.qk_nope_dim, p.qk_rope_dim, p.kv_lora_rank, p.num_pages, p.max_pages_per_seq,
-                  p.rope_theta, parts, n_append, ts, wide, nt);
+                  p.rope_theta, parts, n_append, ts, wide);
   };
   if (clusters)
-    return with_args([&](auto... a) {
-      return launch_slices(prologue_kernel<true>, (n_append + (others + kSliceCtas - 1) / kSliceCtas) * kSliceCtas, smem, stream, a...);
-    });
-  return with_args([&](auto... a) { return launch_pdl(prologue_kernel<false>, dim3(n_append + others), dim3(256), smem, stream, a...); });
+    return with_args([&](auto... a) { return launch_slices(kernel, (n_append + (others + kSliceCtas - 1) / kSliceCtas) * kSliceCtas, smem, stream, a...); });
+  return with_args([&](auto... a) { return launch_pdl(kernel, dim3(n_append + others), dim3(256), smem, stream, a...); });
 }
 
 // ------------------------------------------------------------------------------------------------
