@@ -233,11 +233,13 @@ int append_token_splits(const transmla_params_t& p) {
 // r = 64, dR = 16, D = 256 1 sequence 14.0 / 15.2 us, 16 (64 heads) 16.6 / 19.0, 64 18.0 to 23.2 / 19.3 to 25.3; the same with D = 4096 16
 // 20.6 / 21.9, 64 27.7 / 21.2; r = 512, dR = 64, dn = 64 1 20.6 / 22.2, 16 22.2 / 24.6, 160 46.1 / 39.5 and (64 heads) 75.4 / 69.8.  With
 // r = 128, dR = 0 blocks of 32 features x 16 tokens are as many as clusters have CTAs: 16 19.1 / 22.2, 64 22.5 / 22.9, 160 23.8 / 26.3.
-// The append by itself with r = 512 (wide blocks), alone and in append + decode + combine of 100 cached tokens: 64 6.4 / 8.3 and 40.4 / 41.1 us, 128
-// 6.8 / 10.0 and 44.8 / 46.4, 256 13.3 / 16.6, 512 26.1 / 25.6.  (The two forms add a value's products in other orders, both in fp32.)
+// An append call is followed by the decode's absorb, which starts earlier beside clusters: with it and the combine, 100 cached tokens,
+// blocks / clusters: r = 512, dn = 64 16 tokens 25.7 / 30.7, 32 31.2 / 30.2, 128 51.2 / 46.2; r = 128 16 21.1 / 23.7, 32 26.3 / 24.2; r = 64, D = 4096
+// 16 20.1 / 23.4, 32 26.9 / 23.4; D = 256 16 18.9 / 19.7, 32 19.4 / 20.0.  (By themselves blocks stay ahead up to 256 tokens of r = 512: 128
+// tokens 6.8 / 10.0.  The two forms add a value's products in other orders, both in fp32.)
 static bool append_in_clusters(const transmla_params_t& p, bool alone) {
-  const int K = p.kv_lora_rank + p.qk_rope_dim;
-  return p.batch * p.q_len > (alone && K % 32 == 0 ? 256 : 32) && K % 128 != 0;
+  const int T = p.batch * p.q_len;
+  return alone ? T > 16 : T > 32 && (p.kv_lora_rank + p.qk_rope_dim) % 128 != 0;
 }
 
 cudaError_t launch_append(const transmla_params_t& p, const __nv_bfloat16* x, const __nv_bfloat16* w,

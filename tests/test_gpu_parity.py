@@ -357,9 +357,10 @@ def test_waits_that_give_up_around_the_attention_leave_no_unfinished_values(shap
                                              (synth.QWEN25_72B, [126, 63, 4000]),
                                              (synth.TINY, [(7 * i) % 200 for i in range(150)]),       # several token splits
                                              (synth.LLAMA2_7B, [(64 * i + i) % 700 for i in range(70)]),
-                                             # blocks of 32 features x 16 tokens, and the clusters beyond them, D / 8 in pieces of 128
-                                             (dataclasses.replace(synth.LLAMA2_7B, dn=64), [(64 * i + i) % 300 for i in range(70)]),
-                                             (dataclasses.replace(synth.LLAMA2_7B, dn=64, D=1280), [(7 * i) % 200 for i in range(257)]),
+                                             # blocks, and the clusters beyond 16 tokens, D / 8 in pieces of 128
+                                             (dataclasses.replace(synth.LLAMA2_7B, dn=64), [(64 * i + i) % 300 for i in range(16)]),
+                                             (dataclasses.replace(synth.LLAMA2_7B, dn=64, D=1280), [(7 * i) % 200 for i in range(17)]),
+                                             (synth.MLAShape(H=8, dn=64, dR=0, dv=64, r=128, D=768), [(7 * i) % 200 for i in range(130)]),
                                              (synth.MLAShape(H=8, dn=32, dR=16, dv=32, r=64, D=4352), [(7 * i) % 200 for i in range(65)])])
 def test_append_values_slots_and_untouched_bytes(shape, positions):
     B, S, P = len(positions), shape.S, shape.page_size
@@ -401,7 +402,7 @@ def test_append_with_pieces_of_the_hidden_dimension_that_are_not_whole(D):
 @pytest.mark.parametrize('shape', [synth.LLAMA2_7B, synth.TINY])
 @pytest.mark.parametrize('B', [17, 32, 33, 65])
 def test_append_of_many_tokens_writes_the_bytes_of_few(shape, B):
-    # a cluster takes up to 64 tokens, its ring four pieces up to 32 and three beyond (TINY: blocks up to 32 tokens, which at
+    # a cluster takes up to 64 tokens, its ring four pieces up to 32 and three beyond (TINY: blocks up to 16 tokens, which at
     # D = 256 add in the clusters' order); a value's sum and its order do not change
     positions = [3 + 5 * (i % 40) for i in range(B)]
     ac = gu.to_dev(synth.make_append_case(shape, positions, 46))
@@ -432,8 +433,8 @@ def _seqlens(n):
     # positions, more than 128 query rows
     (synth.LLAMA2_7B, 1), (synth.LLAMA2_7B, 33), (synth.LLAMA2_7B, 65), (synth.LLAMA2_7B, 130), (synth.QWEN25_72B, 3),
     (synth.QWEN25_72B, 70), (dataclasses.replace(synth.LLAMA2_7B, D=1280), 17), (dataclasses.replace(synth.LLAMA2_7B, D=4352), 40),
-    # other shapes: append blocks up to 32 new tokens, then clusters (r + dR a multiple of 128: blocks), whose CTAs take D / 8 in
-    # pieces of 128; one and two tiles of 128 latents an absorb block
+    # other shapes: append blocks up to 32 new tokens, then clusters (r + dR a multiple of 128: blocks; by themselves: clusters
+    # from 17 tokens on), whose CTAs take D / 8 in pieces of 128; one and two tiles of 128 latents an absorb block
     (synth.TINY, 3), (synth.TINY, 33), (synth.MLAShape(H=16, dn=64, dR=0, dv=64, r=128, D=768), 20),
     (synth.MLAShape(H=16, dn=64, dR=0, dv=64, r=128, D=768), 70), (dataclasses.replace(synth.LLAMA2_7B, dn=64), 32),
     (dataclasses.replace(synth.LLAMA2_7B, dn=64, D=768), 33), (dataclasses.replace(synth.LLAMA2_7B, dn=64, D=1280, S=2), 35),
